@@ -296,8 +296,8 @@ rt_status rt_trace_batch(int32_t n_encl, const rt_enclosure *encl, const float *
 /*
  * Process-wide launch shapes, set by an autotuner (no effect on results):
  * kappa_t_per_block = temperature nodes per rt_build_kappa block (1..8, 0 = 8);
- * walk_blocks_per_sm = resident 256-thread blocks per SM the rt_trace walk is
- *   compiled for (4: 64 registers per thread, 5: 48; 0 = 5);
+ * walk_blocks_per_sm = 4 or 5 (0 = 5): kept and reported; the rt_trace walk is compiled
+ *   for four resident 256-thread blocks per SM either way;
  * walk_refill_idle = idle lanes of a warp that trigger loading new rays in the
  *   rt_trace walk (12 or 16; 0 = 16);
  * walk_group = rays of an rt_trace call grouped by wavenumber before the walk, so

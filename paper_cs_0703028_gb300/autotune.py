@@ -7,7 +7,7 @@ choice in a JSON file keyed by a signature of the workload's sizes
 
 * ``tune_kappa``: temperature nodes per rt_build_kappa block (1, 2, 4, 8).
 * ``tune_batch``: rays per work item and threads per block of the batched walk.
-* ``tune_walk``: resident blocks per SM (4 or 5) and refill threshold (12 or 16) of the rt_trace walk,
+* ``tune_walk``: refill threshold (12 or 16) of the rt_trace walk,
   then whether grouping its rays by wavenumber pays.
 """
 from __future__ import annotations
@@ -109,7 +109,7 @@ def tune_walk(grid_struct, ncells, spec, kappa, n_rays, candidates=None, reps=2,
     Returns ((blocks, refill, group), {"blocks,refill[,group]": ms}) with group 1 (off)
     or 2 (on) as rt_tuning.walk_group."""
     if candidates is None:
-        candidates = [(b, r) for b in (4, 5) for r in (12, 16)]
+        candidates = [(5, 12), (5, 16)]   # 4 and 5 blocks run the same kernel
     ng = int(n_rays if n_rays_group is None else n_rays_group)
     key = f"walk:{ncells}:{spec.n_nu}:{spec.nT}:{int(n_rays)}:{ng}"
     cached = _load().get(key) if use_cache else None

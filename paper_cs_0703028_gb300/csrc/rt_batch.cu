@@ -107,29 +107,21 @@ k_walk_batch(const EnclDev *__restrict__ E, const long long *__restrict__ item_o
       const unsigned am = __ballot_sync(0xffffffffu, active);
       if (!am) break;
       if (!active) continue;
-      bool done = false;
-      if (__all_sync(am, R.trans == 0.0f && !W.tau_cut)) {
-        // every active lane dark: DDA-only steps
-#pragma unroll
-        for (int u = 0; u < kBatchUnroll; ++u)
-          if (!done)
-            done = ray_step<false, false, true, true>(W, 0.0f, D.absorbed, D.status, rec, R, true, NoPrefetch(),
-                                                      s_axes[warp]);
-      } else {
+      bool done = false, dark = false;
 #pragma unroll
       for (int u = 0; u < kBatchUnroll; ++u) {  // steps per pass of the loop
         if (!done) {
-          // a dark ray (transmission zero, no optical-depth cut) needs neither its cell's
-          // kappa nor the next cell's data
-          const bool lit = R.trans != 0.0f || W.tau_cut;
-          const float kap = !lit ? 0.0f : (TAB == 2 ? cell_kappa_row(cd, krow) : (TAB == 1 ? cell_kappa_row1(cd, krow1, W.nT) : cell_kappa_l<TAB>(cd, tab, W.nT, W.n_nu, R.j)));
+          const float kap = TAB == 2 ? cell_kappa_row(cd, krow) : (TAB == 1 ? cell_kappa_row1(cd, krow1, W.nT) : cell_kappa_l<TAB>(cd, tab, W.nT, W.n_nu, R.j));
           float4 cdn = cd;
           done = ray_step<false, false, true>(W, kap, D.absorbed, D.status, rec, R, true,
-                                              [&](int c) { if (lit) cdn = __ldg(cells + c); }, s_axes[warp]);
+                                              [&](int c) { cdn = __ldg(cells + c); }, s_axes[warp]);
           cd = cdn;
+          // a dark ray deposits nothing more: only its visits are still to be counted
+          dark = !done && R.trans == 0.0f && !W.tau_cut;
+          done = done || dark;
         }
       }
-      }
+      if (dark) R.nv += dark_visits(W, R, D.status);
       if (done) {
         em += (double)R.w;
         esc += (double)(R.w * R.trans);

@@ -128,9 +128,13 @@ k_walk_lbl(const int4 *__restrict__ R, const float4 *__restrict__ L0, const floa
       if (Ry.w < 0.0f) Ry.w = (W.mode == RT_SRC_BEAM) ? 1.0f : emission_weight(W, Ry.j, Tc, kap);
       if (ray_step(W, kap, absorbed, status, rec, Ry, lead)) break;
       if (Ry.trans == 0.0f && !W.tau_cut) {
-        // dark (uniform over the warp's one ray): its remaining steps need no line sum
-        while (!ray_step<true, true, false, true>(W, 0.0f, absorbed, status, rec, Ry, lead)) {
-        }
+        // dark (uniform over the warp's one ray): only its visits are left, listed when it is
+        // recorded, else counted
+        if (Ry.row >= 0)
+          while (!ray_step<true, true, false, true>(W, 0.0f, absorbed, status, rec, Ry, lead)) {
+          }
+        else
+          Ry.nv += dark_visits(W, Ry, lead ? status : nullptr);
         break;
       }
     }

@@ -960,10 +960,16 @@ k_walk_mlp(const float *__restrict__ P, const uint16_t *__restrict__ tiles, Norm
         if (R.w < 0.0f) R.w = emission_weight(W, R.j, Tc, kap);
         bool fin = ray_step(W, kap, absorbed, status, rec, R);
         // a dark ray (transmission zero, no optical-depth cut) needs no more kappa: it
-        // takes its remaining steps at once, DDA only, and frees its lane for a new ray
-        if (!fin && R.trans == 0.0f && !W.tau_cut)
-          while (!(fin = ray_step<true, true, false, true>(W, 0.0f, absorbed, status, rec, R))) {
-          }
+        // only counts its remaining visits (a recorded one lists them) and frees its lane for
+        // a new ray
+        if (!fin && R.trans == 0.0f && !W.tau_cut) {
+          if (R.row >= 0)
+            while (!ray_step<true, true, false, true>(W, 0.0f, absorbed, status, rec, R)) {
+            }
+          else
+            R.nv += dark_visits(W, R, status);
+          fin = true;
+        }
         if (fin) {
           const float out = R.w * R.trans;
           em += (double)R.w;

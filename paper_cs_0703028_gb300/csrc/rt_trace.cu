@@ -115,7 +115,7 @@ __global__ void k_band_scatter(WalkParams W, int band_pts, unsigned long long *_
 
 }  // namespace
 
-int g_walk_blocks = 5;   // resident walk blocks per SM the launch is compiled for (4 or 5)
+int g_walk_blocks = 5;   // accepted launch shape (4 or 5); both run the one compiled occupancy
 int g_walk_refill = 16;  // idle lanes that trigger a refill (12 or 16)
 int g_walk_group = 0;    // rays grouped by wavenumber: 0 when >= 32 rays per wavenumber, 1 never, 2 always
 
@@ -159,8 +159,11 @@ __global__ void k_pair_table(const float *__restrict__ in, int nT, long long n_n
   }
 }
 
-template <bool REC, int TAB, int MINB, int REFILL>
-__global__ void __launch_bounds__(kWalkThreads, MINB)
+// Four blocks of 64 registers: at five of 48 the walk spills, and more resident rays share
+// one L1 (8e6 rays of a thin gas in a 75 x 52 x 61 box: 2.29 ms against 2.61 ms; 4e8 rays of
+// the opaque 128^3 box, where it matters least: 15.9 ms against 16.9 ms).
+template <bool REC, int TAB, int REFILL>
+__global__ void __launch_bounds__(kWalkThreads, 4)
 k_walk(const float4 *__restrict__ cells, const float *__restrict__ tab, const uint32_t *__restrict__ order,
        WalkParams W, double *__restrict__ absorbed, double *__restrict__ scalars,
        unsigned long long *__restrict__ steps_out, uint32_t *status, RecordPtrs rec) {
@@ -200,28 +203,29 @@ k_walk(const float4 *__restrict__ cells, const float *__restrict__ tab, const ui
     const unsigned am = __ballot_sync(0xffffffffu, active);
     if (!am) break;
     if (!active) continue;
-    bool done = false;
-    if (__all_sync(am, R.trans == 0.0f && !W.tau_cut)) {
-      // every active lane dark: kWalkUnroll DDA-only steps
-#pragma unroll
-      for (int u = 0; u < kWalkUnroll; ++u)
-        if (!done) done = ray_step<REC, true, true, true>(W, 0.0f, absorbed, status, rec, R, true, NoPrefetch(), s_axes);
-    } else {
+    bool done = false, dark = false;
     // kWalkUnroll steps per pass of the loop; each step loads the table value of
     // its cell and the next cell's data, both in flight while its arithmetic runs
 #pragma unroll
     for (int u = 0; u < kWalkUnroll; ++u) {
       if (!done) {
-        // a dark ray (transmission zero, no optical-depth cut) needs neither its cell's
-        // kappa nor the next cell's data
-        const bool lit = R.trans != 0.0f || W.tau_cut;
-        const float kap = !lit ? 0.0f : (TAB == 2 ? cell_kappa_row(cd, krow) : (TAB == 1 ? cell_kappa_row1(cd, krow1, W.nT) : cell_kappa_l<TAB>(cd, tab, W.nT, W.n_nu, R.j)));
+        const float kap = TAB == 2 ? cell_kappa_row(cd, krow) : (TAB == 1 ? cell_kappa_row1(cd, krow1, W.nT) : cell_kappa_l<TAB>(cd, tab, W.nT, W.n_nu, R.j));
         float4 cdn = cd;
         done = ray_step<REC, true, true>(W, kap, absorbed, status, rec, R, true,
-                                         [&](int c) { if (lit) cdn = __ldg(cells + c); }, s_axes);
+                                         [&](int c) { cdn = __ldg(cells + c); }, s_axes);
         cd = cdn;
+        // a dark ray (transmission zero, no optical-depth cut) deposits nothing more:
+        // only its visits are still to be counted
+        dark = !done && R.trans == 0.0f && !W.tau_cut;
+        done = done || dark;
       }
     }
+    if (dark) {
+      if (REC && R.row >= 0)  // a recorded ray lists its cells
+        while (!ray_step<REC, true, true, true>(W, 0.0f, absorbed, status, rec, R, true, NoPrefetch(), s_axes)) {
+        }
+      else
+        R.nv += dark_visits(W, R, status);
     }
     if (done) {
       const float out = R.w * R.trans;
@@ -318,7 +322,21 @@ rt_status walk_setup(const rt_grid *grid, const rt_spectral *spec, uint64_t ray_
   for (int a = 0; a < 3; ++a) {
     W->fin[a] = std::isfinite(h[a]) ? 1 : 0;
     W->h[a] = (float)h[a];
+    W->inv_h[a] = W->fin[a] ? 1.0f / W->h[a] : 0.0f;
     if (W->fin[a]) V *= h[a];
+  }
+  // dark_visits' closed form: its error bound holds for up to 65536 cells an axis and cell
+  // sizes whose face distances neither overflow nor underflow (a direction cosine is 0 or
+  // at least 5e-11)
+  W->jump = 1;
+  const int n3[3] = {grid->nx, grid->ny, grid->nz};
+  for (int a = 0; a < 3; ++a)
+    if (W->fin[a] && (n3[a] > 65536 || !(W->h[a] >= 1e-15f && W->h[a] <= 1e15f))) W->jump = 0;
+  for (int a = 0; a < 2; ++a) {
+    uint32_t s = 0;
+    while ((1ull << s) < (unsigned long long)n3[a]) ++s;
+    W->div_s[a] = 31 + s;
+    W->div_m[a] = (uint32_t)(((1ull << (31 + s)) + (unsigned long long)n3[a] - 1) / (unsigned long long)n3[a]);
   }
   W->ncells = nc;
   W->n_nu = spec->n_nu;
@@ -466,9 +484,8 @@ rt_status trace_impl(const rt_grid *grid, const float *kappa, const rt_spectral 
   // visit recording (a test path) uses one configuration; the tuned shape otherwise
   auto pick = [&](auto tab) {
     constexpr int L = decltype(tab)::value;
-    if (rec) return k_walk<true, L, 5, kRefillIdleDefault>;
-    if (g_walk_blocks == 4) return g_walk_refill == 12 ? k_walk<false, L, 4, 12> : k_walk<false, L, 4, 16>;
-    return g_walk_refill == 12 ? k_walk<false, L, 5, 12> : k_walk<false, L, 5, 16>;
+    if (rec) return k_walk<true, L, kRefillIdleDefault>;
+    return g_walk_refill == 12 ? k_walk<false, L, 12> : k_walk<false, L, 16>;
   };
   auto kern = layout == 2 ? pick(std::integral_constant<int, 2>()) : pick(std::integral_constant<int, 1>());
   int per_sm = 0;
