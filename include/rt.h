@@ -302,9 +302,9 @@ rt_status rt_trace_batch(int32_t n_encl, const rt_enclosure *encl, const float *
  *   rt_trace walk (12 or 16; 0 = 16);
  * walk_group = rays of an rt_trace call grouped by wavenumber before the walk, so
  *   that the lanes of a warp read one row of the table (a counting pass over the
- *   rays' Philox draws; scratch of 4 bytes per ray + 8 per wavenumber): 1 never,
- *   2 always, 0 = when there are at least 32 rays per wavenumber.  Tallies are
- *   sums, so the grouping changes only their binary64 summation order.
+ *   rays' Philox draws; scratch of 4 bytes per ray + 8 per wavenumber): 2 always,
+ *   0 and 1 never.  Tallies are sums, so the grouping changes only their binary64
+ *   summation order.
  */
 typedef struct {
   int32_t kappa_t_per_block;

@@ -117,7 +117,11 @@ __global__ void k_band_scatter(WalkParams W, int band_pts, unsigned long long *_
 
 int g_walk_blocks = 5;   // accepted launch shape (4 or 5); both run the one compiled occupancy
 int g_walk_refill = 16;  // idle lanes that trigger a refill (12 or 16)
-int g_walk_group = 0;    // rays grouped by wavenumber: 0 when >= 32 rays per wavenumber, 1 never, 2 always
+// Rays grouped by wavenumber only when asked for (2; 0 and 1 never): the counting passes
+// cost more than the shared table rows save.  Off / on: 1e7 rays of the opaque 32^3 box
+// 0.39 / 0.87 ms; 4e8 of the opaque 128^3 box 15.9 / 30.0 ms; 2e7 rays of a thin gas there
+// 6.7 / 10.1 ms; thin gas with a 410 MB table and 1e8 rays (62 a wavenumber) 32.5 / 48.8 ms.
+int g_walk_group = 0;
 
 namespace {
 
@@ -453,8 +457,7 @@ rt_status trace_impl(const rt_grid *grid, const float *kappa, const rt_spectral 
   const size_t cbytes = ((size_t)W.ncells * sizeof(float4) + 255) & ~size_t(255);
   const size_t tbytes = (walk_table_bytes(layout, spec->nT, spec->n_nu) + 255) & ~size_t(255);
   // rays grouped by wavenumber (one band per wavenumber): counts, band and item starts, order
-  const bool group = n_rays <= 0xFFFFFFFFull &&
-                     (g_walk_group == 2 || (g_walk_group == 0 && n_rays >= 32ull * (unsigned long long)spec->n_nu));
+  const bool group = n_rays <= 0xFFFFFFFFull && g_walk_group == 2;
   const long long nb = spec->n_nu;
   const size_t pbytes = group ? (((size_t)nb * 8 * 3 + 64 + 255) & ~size_t(255)) : 0;
   const size_t obytes = group ? (size_t)n_rays * sizeof(uint32_t) : 0;
