@@ -9,15 +9,15 @@
 //                     arithmetic for the Boltzmann exponent; for Voigt lines
 //                     also the far-wing polynomial coefficients.
 //   k_tile_lines    : per 256-point wavenumber tile, the range of lines whose
-//                     windows reach it, split into segments by kind: far lines
-//                     (degree-1 or degree-2 far-wing series, masked where the
-//                     window ends inside the tile), covering lines with the
-//                     degree-4 series, and the general path (near-centre zone).
+//                     windows reach it, split into segments by kind: lines far from
+//                     the tile (summed at a few nodes and interpolated), lines whose
+//                     window ends inside it, covering lines with the degree-4 series,
+//                     and the general path (near-centre zone).
 //   k_kappa         : per (tile, up to 8 T nodes), the line sum.  The tile's
 //                     lines are staged in shared memory by bulk asynchronous
 //                     copies (cp.async.bulk + mbarrier), double buffered; each
 //                     lane owns 8 consecutive points (two float4 stores) and
-//                     Kahan-sums over lines in ascending nu0.
+//                     Kahan-sums over lines.
 //   k_kappa_ppl     : with a fixed number of points per line, one thread per
 //                     point and eight T nodes over the few lines whose windows hold it.
 #include <cmath>
@@ -32,8 +32,10 @@ namespace {
 constexpr int kPtsPerThread = 8;
 constexpr int kTilePts = 32 * kPtsPerThread;  // 256 wavenumbers per block, one warp per T node
 constexpr int kMaxTPerBlock = 8;              // warps (T nodes) per block
-constexpr int kChunk = 96;                    // lines per staged chunk
+constexpr int kChunk = 192;                   // lines per staged chunk that need P only
+constexpr int kChunkP2 = 96;                  // ... that need P and P2
 constexpr int kGroup = 8;                     // fast-path lines summed before one compensated add
+constexpr int kNodeGroup = 4;                 // interpolated lines a lane sums before one compensated add
 constexpr unsigned kWaitLimit = 1u << 22;     // bounded mbarrier waits
 
 // CODATA 2018 (SI); derived quantities are formed on the host in binary64.
@@ -42,7 +44,7 @@ constexpr double kAmu = 1.66053906660e-27, kAtm = 101325.0;
 constexpr double kPi = 3.14159265358979323846;
 
 struct GeomParams {
-  double nu_min, dnu, cutoff;
+  double nu_min, dnu, inv_dnu, cutoff;
   long long n_nu, n_lines;
   int nT, check, ppl;
 };
@@ -77,15 +79,18 @@ __global__ void k_line_geometry(const double *__restrict__ nu0, const double *__
         status_or(status, RT_DEV_NONFINITE);
       if (l > 0 && !(nu0[l - 1] <= v)) status_or(status, RT_DEV_UNSORTED);
     }
-    // nearest grid index: the origin of the line's local coordinate
-    double fc = (v - P.nu_min) / P.dnu;
+    // nearest grid index: the origin of the line's local coordinate (any index within a
+    // grid step of the centre serves, the offset below is exact for it)
+    double fc = (v - P.nu_min) * P.inv_dnu;
     fc = fmin(fmax(isfinite(fc) ? fc : 0.0, -536870912.0), 536870912.0);
     const long long jc = llrint(fc);
     const double dc = __dsub_rn(grid_nu(P.nu_min, jc, P.dnu), v);  // nu_jc - nu0
-    const float dg = __double2float_rn(dc / P.dnu);                 // grid units
-    // inclusive cutoff window: -cutoff <= nu_j - nu0 <= cutoff, in binary64
-    double flo = floor((v - P.cutoff - P.nu_min) / P.dnu) - 1.0;
-    double fhi = ceil((v + P.cutoff - P.nu_min) / P.dnu) + 1.0;
+    const float dg = __double2float_rn(dc * P.inv_dnu);             // grid units
+    // inclusive cutoff window: -cutoff <= nu_j - nu0 <= cutoff, decided in binary64 below
+    // from an estimate (a multiplication by 1 / dnu: the two divisions it replaces took half
+    // of the kernel's time)
+    double flo = ceil((v - P.cutoff - P.nu_min) * P.inv_dnu);
+    double fhi = floor((v + P.cutoff - P.nu_min) * P.inv_dnu);
     flo = fmin(fmax(isfinite(flo) ? flo : 0.0, -1.0), (double)P.n_nu + 1.0);
     fhi = fmin(fmax(isfinite(fhi) ? fhi : 0.0, -2.0), (double)P.n_nu + 1.0);
     long long lo = (long long)flo, hi = (long long)fhi;
@@ -98,12 +103,22 @@ __global__ void k_line_geometry(const double *__restrict__ nu0, const double *__
     if (lo < 0) lo = 0;
     if (hi > P.n_nu - 1) hi = P.n_nu - 1;
     if (P.ppl <= 0) {
+      auto below = [&](long long j) { return __dsub_rn(grid_nu(P.nu_min, j, P.dnu), v) < -P.cutoff; };
+      auto above = [&](long long j) { return __dsub_rn(grid_nu(P.nu_min, j, P.dnu), v) > P.cutoff; };
+      int it = 0;
 #pragma unroll 1
-      for (int it = 0; it < 6 && lo < P.n_nu; ++it)
-        if (__dsub_rn(grid_nu(P.nu_min, lo, P.dnu), v) < -P.cutoff) ++lo;
+      for (; it < 6 && lo < P.n_nu && below(lo); ++it) ++lo;
+      if (it == 0) {
 #pragma unroll 1
-      for (int it = 0; it < 6 && hi >= 0; ++it)
-        if (__dsub_rn(grid_nu(P.nu_min, hi, P.dnu), v) > P.cutoff) --hi;
+        for (; it < 6 && lo > 0 && !below(lo - 1); ++it) --lo;
+      }
+      it = 0;
+#pragma unroll 1
+      for (; it < 6 && hi >= 0 && above(hi); ++it) --hi;
+      if (it == 0) {
+#pragma unroll 1
+        for (; it < 6 && hi < P.n_nu - 1 && !above(hi + 1); ++it) ++hi;
+      }
     }
     R[l] = make_int4((int)lo, (int)hi, (int)jc, __float_as_int(dg));
     if (hi >= lo) cnt = (unsigned long long)(hi - lo + 1) * (unsigned long long)P.nT;
@@ -115,13 +130,11 @@ __global__ void k_line_geometry(const double *__restrict__ nu0, const double *__
 }
 
 // Eq. (S) times the number density, and the profile's coefficients, for line l
-// at T node k.  Voigt: P = {c0, s dnu, y^2, c2}, P2 = {c3, c4, half-widths of |z| < 20 and < 10}
+// at T node k.  Voigt: P = {c0, s dnu, y^2, c2}, P2 = {c3, c4, half-widths of |z| < 20 and < 8}
 // with the far-wing series c0 t + c1 t^2 + c2 t^3 + c3 t^4 + c4 t^5 (c1 = 1.5 c0).
-// Writes the line's far-zone distances in grid units (float bits): beyond far[0]
-// the t^4 and t^5 terms are below 2^-24 of the value (27 y^2 t^3 <= 2^-24 with
-// t <= 1/x^2), so a degree-2 series is within one binary32 rounding of the full
-// one; beyond far[1] (>= far[0]) also (3.75 + 2 y^2) t^2 <= 2^-25, so the degree-1
-// series drops at most 1.25 * 2^-24 of the value.
+// Returns the line's far-zone distance in grid units (float bits): beyond it the t^3, t^4
+// and t^5 terms drop at most 1.25 * 2^-24 of the value, so the degree-1 series
+// c0 t (1 + 1.5 t) stands for the full one.
 // The quantities of T node k that every line shares.
 struct PrefNode {
   df Tk, iT, iTref;
@@ -152,7 +165,7 @@ __device__ __forceinline__ void prefactor_one(const double *__restrict__ nu0, co
                                                   const double *__restrict__ g, const double *__restrict__ E,
                                                   const PrefParams &Q, const PrefNode &N,
                                                   float4 *__restrict__ Pout, float4 *__restrict__ P2out,
-                                                  long long l, int k, unsigned (&far)[2]) {
+                                                  long long l, int k, unsigned &far) {
   const df iT = N.iT, iTref = N.iTref;
   const float iTf = iT.hi;
   // Eq. (S): Q ratio, Boltzmann ratio (exponent in double-float), stimulated emission
@@ -166,7 +179,7 @@ __device__ __forceinline__ void prefactor_one(const double *__restrict__ nu0, co
   const float A = (Q.u_coef * iTf) * S_T;  // u(T) S(T), cm^-1 per unit profile
   const float gam = __double2float_rn(g[l]) * Q.p_ref * N.wratio;
   float4 out;
-  far[0] = far[1] = 0;
+  far = 0;
   if (Q.profile == RT_PROFILE_LORENTZ) {
     const float gg = gam * Q.inv_dnu;  // half-width in grid units
     out = make_float4(A * gg * (float)(1.0 / kPi) * Q.inv_dnu, gg * gg, 0.0f, 0.0f);
@@ -181,15 +194,14 @@ __device__ __forceinline__ void prefactor_one(const double *__restrict__ nu0, co
     // far wing: c0 t (1 + 1.5 t + (3.75 - 2 y^2) t^2 - 15 y^2 t^3 + 12 y^4 t^4), t = 1/|z|^2
     const float c0 = A * s * (float)(1.0 / kPi) * y;
     out = make_float4(c0, sd, y2, __fmaf_rn(-2.0f, y2, 3.75f) * c0);
-    // half-width (grid units) of |z| < 10, inside which the general path takes the near form
-    const float u_core = sqrtf(fmaxf(100.0f - y2, 0.0f)) / sd;
+    // half-width (grid units) of |z| < 8, inside which the general path takes the rational form
+    const float u_core = sqrtf(fmaxf(64.0f - y2, 0.0f)) / sd;
     P2out[(long long)k * Q.n_lines + l] = make_float4(-15.0f * y2 * c0, 12.0f * y2 * y2 * c0, u_near, u_core);
-    // (27 y^2 / 2^-24)^(1/6) = 27.66 y^(1/3) and (2^25 (3.75 + 2 y^2))^(1/4), with 5 %
-    // margin, in grid units
+    // (27 y^2 / 2^-24)^(1/6) = 27.66 y^(1/3), beyond which 27 y^2 t^3 <= 2^-24 (t <= 1/x^2),
+    // and (2^25 (3.75 + 2 y^2))^(1/4), with 5 % margin, in grid units
     const float d2 = 29.1f * cbrtf(y) / sd;
     const float d1 = fmaxf(1.05f * sqrtf(sqrtf(33554432.0f * (3.75f + 2.0f * y2))) / sd, d2);
-    far[0] = (d2 >= 0.0f && d2 < 1e9f) ? __float_as_uint(d2) : __float_as_uint(1e9f);
-    far[1] = (d1 >= 0.0f && d1 < 1e9f) ? __float_as_uint(d1) : __float_as_uint(1e9f);
+    far = (d1 >= 0.0f && d1 < 1e9f) ? __float_as_uint(d1) : __float_as_uint(1e9f);
   }
   Pout[(long long)k * Q.n_lines + l] = out;
 }
@@ -204,19 +216,17 @@ __global__ void k_prefactor(const double *__restrict__ nu0, const double *__rest
   if (threadIdx.x == 0) s_node = pref_node(Q, k);
   __syncthreads();
   const PrefNode N = s_node;
-  unsigned fb[2] = {0, 0};  // this line's far-zone distances (grid units, float bits)
+  unsigned fb = 0;  // this line's far-zone distance (grid units, float bits)
   if (l < Q.n_lines) prefactor_one(nu0, S, g, E, Q, N, Pout, P2out, l, k, fb);
-  // block maxima, one atomic each per block (non-negative floats order like their bits)
-  __shared__ unsigned s_max[2][32];
-  for (int d = 0; d < 2; ++d) {
-    const unsigned m = __reduce_max_sync(0xffffffffu, fb[d]);
-    if ((threadIdx.x & 31) == 0) s_max[d][threadIdx.x >> 5] = m;
-  }
+  // block maximum, one atomic per block (non-negative floats order like their bits)
+  __shared__ unsigned s_max[32];
+  const unsigned wm = __reduce_max_sync(0xffffffffu, fb);
+  if ((threadIdx.x & 31) == 0) s_max[threadIdx.x >> 5] = wm;
   __syncthreads();
-  if (threadIdx.x < 2) {
+  if (threadIdx.x == 0) {
     unsigned m = 0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) m = max(m, s_max[threadIdx.x][w]);
-    if (m) atomicMax(far_bits + threadIdx.x, m);
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) m = max(m, s_max[w]);
+    if (m) atomicMax(far_bits, m);
   }
 }
 
@@ -263,106 +273,181 @@ __device__ __forceinline__ long long lower_bound_lo(const int4 *R, long long n, 
   return a;
 }
 
+// ---- interpolation of far lines
+// The sum of the lines far from a tile is smooth over it: it is evaluated at a few nodes
+// and interpolated to the tile's points (the line-by-line interpolation technique of Fomin,
+// JQSRT 53 (1995) 663, and Kuntz and Hoepfner, JQSRT 63 (1999) 97, here on Chebyshev
+// nodes).  A Lorentz-like wing 1/(u^2 + g^2) whose centre is D half-widths from the middle of
+// an interval has its poles on or outside the Bernstein ellipse of
+// rho = D + sqrt(D^2 - 1), so M nodes leave an error of order M rho^-M of the value.
+// Largest relative error of one line's value at any point (computed, g = 0 .. 20 grid
+// points; the nodes are Chebyshev's rounded to 1/16 grid point, so that u is exact):
+//   8 nodes on the tile (half-width 128 points), centre >= 704 points from it: 3.4e-8
+//  16 nodes on the tile, centre >= 141 points from it:                        1.4e-8
+//   4 nodes on a 32-point sub-block, centre >= 928 points from it:            4.9e-8
+// (an eighth of that on average over a line's points), against 6e-8 for one binary32
+// rounding.
+template <int M>
+struct Nodes {
+  double u[M];
+};
+constexpr Nodes<8> kNodes8{{1.9375, 21.0625, 56.375, 102.5, 152.5, 198.625, 233.9375, 253.0625}};
+constexpr Nodes<16> kNodes16{{0.125, 5.0, 14.625, 28.5625, 46.3125, 67.1875, 90.3125, 114.9375, 140.0625, 164.6875,
+                              187.8125, 208.6875, 226.4375, 240.375, 250.0, 254.875}};
+constexpr Nodes<4> kNodes4{{0.6875, 9.375, 21.625, 30.3125}};
+constexpr int kDist8 = 704, kDist16 = 141, kDistEdge = 928;  // grid points from the tile's nearest point
+
+// Lagrange weights w[m][j] of the M nodes at N positions, and the nodes in binary32
+template <int M, int N>
+struct NodeTable {
+  float u[M];
+  float w[M][N];
+};
+template <int M, int N, class At>
+constexpr NodeTable<M, N> node_table(const Nodes<M> &nd, At at) {
+  NodeTable<M, N> t{};
+  for (int m = 0; m < M; ++m) t.u[m] = (float)nd.u[m];
+  for (int j = 0; j < N; ++j)
+    for (int m = 0; m < M; ++m) {
+      double p = 1.0;
+      for (int q = 0; q < M; ++q)
+        if (q != m) p *= (at(j) - nd.u[q]) / (nd.u[m] - nd.u[q]);
+      t.w[m][j] = (float)p;
+    }
+  return t;
+}
+struct AtPoint {
+  constexpr double operator()(int j) const { return (double)j; }
+};
+struct AtNode16 {
+  constexpr double operator()(int j) const { return kNodes16.u[j]; }
+};
+__device__ constexpr NodeTable<16, kTilePts> kTab16 = node_table<16, kTilePts>(kNodes16, AtPoint{});
+__device__ constexpr NodeTable<8, 16> kTab8 = node_table<8, 16>(kNodes8, AtNode16{});
+__device__ constexpr NodeTable<4, 32> kTab4 = node_table<4, 32>(kNodes4, AtPoint{});
+
 // Kinds of line ranges within a tile (see k_tile_lines).
 enum SegKind : int {
-  kSegGeneral = 0,   // window masking and near-centre test per line
-  kSegFast = 1,      // covering, degree-4 far-wing series
-  kSegFar2 = 2,      // covering, degree-2 series
-  kSegFar1 = 3,      // covering, degree-1 series
-  kSegFar2Masked = 4,
-  kSegFar1Masked = 5,
+  kSegGeneral = 0,     // window masking and near-centre test per line
+  kSegFast = 1,        // covering, degree-4 far-wing series at every point
+  kSegNodes16 = 2,     // covering, degree-4 series at 16 nodes
+  kSegNodes8 = 3,      // covering, degree-1 series at 8 nodes
+  kSegEdge = 4,        // window ends inside the tile: degree-1 series at 4 nodes of each covered
+                       // 32-point sub-block and at the points of the one it ends in
+  kSegFar1Masked = 5,  // window ends inside the tile, degree-1 series at every point
 };
+__device__ __forceinline__ bool degree1_kind(int kd) { return kd >= kSegNodes8; }
 constexpr int kMaxSegs = 12;
 constexpr int kTileInts = 5;  // int4 per tile: {lb, ub, nseg, 0}, 12 ends, 16 kind bytes
 
 // Per tile of kTilePts wavenumbers [jw0, jw0 + kTilePts): the lines [lb, ub)
 // whose windows reach it, split into ranges by kind.  Windows and centres are
 // monotone in the (sorted) line index, so every set below is an index range:
-//   cover : j_lo <= jw0 and j_hi >= jw0 + kTilePts - 1 (no masking needed);
+//   cover : the window holds every point of the tile that is on the grid (no masking);
 //   near  : j_c within W + 4 grid points of the tile, W bounding the near-centre
 //           half-width of every line (lines outside it have no point |z| < 20);
-//   far2 / far1 : j_c more than D2 / D1 grid points from the tile, D1 >= D2 >= W + 4
-//           bounding every line's far-zone distances (degree-2 / degree-1 series).
-// Covering lines are far1, far2, fast or (near) general; partially covering
-// lines are far1-masked, far2-masked or general.
+//   n16, n8, edge : j_c at least kDist16 (and W + 4), kDist8 or kDistEdge (and D1) grid
+//           points from the tile, D1 bounding every line's far-zone distance (degree-1
+//           series).
+// Covering lines are nodes-8, nodes-16, fast or (near) general; partially covering lines
+// are edge, far1-masked or general.
+__device__ __forceinline__ int clamp_int(long long v) {
+  return (int)min(max(v, -0x40000000LL), 0x40000000LL);  // centres lie within 2^29 grid steps
+}
+
 __global__ void k_tile_lines(const int4 *__restrict__ R, long long n, long long n_nu, int W,
                              const unsigned *__restrict__ far_bits, long long n_tiles,
                              int4 *__restrict__ out) {
-  // one warp per tile: lanes 0..9 run the tile's ten binary searches side by side
+  // One warp per tile.  The 14 searches run side by side, 32 lanes a search: each round reads
+  // 32 lines spread over the remaining range of every search at once and keeps the gap the
+  // key lies in, so that a list of 500 lines takes two dependent reads and one of 1e6 four
+  // (a lane per search took 9 and 20; with the warp-parallel split below instead of one
+  // lane's insertion sort the kernel's time fell from 8.4 to 5.3 us for 500 lines).
   const long long t = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (t >= n_tiles) return;  // warp-uniform
-  const long long D2 = max((long long)W + 4, (long long)ceilf(fminf(__uint_as_float(far_bits[0]), 1e9f)) + 2);
-  const long long D1 = max(D2, (long long)ceilf(fminf(__uint_as_float(far_bits[1]), 1e9f)) + 2);
+  const long long near = (long long)W + 4;
+  const long long D1 = max(near, (long long)ceilf(fminf(__uint_as_float(far_bits[0]), 1e9f)) + 2);
+  const long long d16 = max(near, (long long)kDist16), d8 = max(D1, (long long)kDist8), dE = max(D1, (long long)kDistEdge);
   const long long jw0 = t * kTilePts, jw1 = jw0 + kTilePts - 1;
-  const long long jend = min(jw0 + (long long)kTilePts, n_nu);
-  // search i: the first line whose field (0: window start, 1: window end, 2: centre) >= key
-  const int fld = (lane == 1 || lane == 3) ? 0 : ((lane == 0 || lane == 2) ? 1 : 2);
-  const long long key = lane == 0 ? jw0 : lane == 1 ? jend : lane == 2 ? jw1 : lane == 3 ? jw0 + 1
-                        : lane == 4 ? jw0 - D1 : lane == 5 ? jw0 - D2 : lane == 6 ? jw0 - W - 4
-                        : lane == 7 ? jw1 + W + 5 : lane == 8 ? jw1 + D2 + 1 : jw1 + D1 + 1;
-  long long a = 0, e = n;
-  if (lane < 10) {
-    while (a < e) {
-      const long long m = (a + e) >> 1;
-      const int4 r = __ldg(R + m);
-      const long long v = fld == 0 ? r.x : (fld == 1 ? r.y : r.z);
-      if (v < key) a = m + 1; else e = m;
-    }
-  }
-  long long sr[10];
+  // search i: the first line whose field (0: window start, 1: window end, 2: centre) >= key;
+  // 0, 1: the tile's lines [lb, ub); 2, 3: covering ones; 4 .. 8: centres left of the tile by
+  // dE, D1, d8, d16, near; 9 .. 13: right of it by near, d16, d8, D1, dE
+  constexpr int kSearches = 14;
+  const int key[kSearches] = {(int)jw0, (int)min(jw0 + (long long)kTilePts, n_nu), (int)min(jw1, n_nu - 1), (int)jw0 + 1,
+                              clamp_int(jw0 - dE), clamp_int(jw0 - D1), clamp_int(jw0 - d8), clamp_int(jw0 - d16),
+                              clamp_int(jw0 - near), clamp_int(jw1 + near + 1), clamp_int(jw1 + d16 + 1),
+                              clamp_int(jw1 + d8 + 1), clamp_int(jw1 + D1 + 1), clamp_int(jw1 + dE + 1)};
+  int pos[kSearches];  // the answer lies in [pos, pos + len]
 #pragma unroll
-  for (int i = 0; i < 10; ++i) sr[i] = __shfl_sync(0xffffffffu, a, i);
-  if (lane != 0) return;
-  const long long lb = sr[0];
-  const long long ub = max(lb, sr[1]);
-  auto cl = [&](long long v) { return min(max(v, lb), ub); };
-  const long long ca = cl(sr[2]);   // cover = [ca, cb)
-  const long long cb = cl(sr[3]);
-  const long long f1a = cl(sr[4]);  // far1: l < f1a or l >= f1b
-  const long long f2a = cl(sr[5]);  // far2: l < f2a or l >= f2b
-  const long long na = cl(sr[6]);   // near: [na, nb)
-  const long long nb = cl(sr[7]);
-  const long long f2b = cl(sr[8]);
-  const long long f1b = cl(sr[9]);
-  auto kind = [&](long long l) -> int {
-    const bool far1 = l < f1a || l >= f1b, far2 = l < f2a || l >= f2b;
-    if (l < ca || l >= cb) return far1 ? kSegFar1Masked : (far2 ? kSegFar2Masked : kSegGeneral);
-    if (far1) return kSegFar1;
-    if (far2) return kSegFar2;
-    if (l < na || l >= nb) return kSegFast;
-    return kSegGeneral;
-  };
-  // the change points, sorted; one segment per maximal run of equal kind
-  long long b[9] = {ca, cb, f1a, f2a, na, nb, f2b, f1b, ub};
-  for (int i = 1; i < 8; ++i)
-    for (int j = i; j > 0 && b[j - 1] > b[j]; --j) {
-      const long long x = b[j - 1]; b[j - 1] = b[j]; b[j] = x;
+  for (int i = 0; i < kSearches; ++i) pos[i] = 0;
+  for (long long len = n; len > 0;) {
+    // probes at pos + (lane + 1) step - 1: those below the key are a prefix of the lanes
+    const long long step = (len + 31) / 32;
+    int v[kSearches];
+#pragma unroll
+    for (int i = 0; i < kSearches; ++i) {
+      const long long q = (long long)pos[i] + (long long)(lane + 1) * step - 1;
+      const int *f = reinterpret_cast<const int *>(R + min(q, n - 1)) + ((i == 1 || i == 3) ? 0 : ((i == 0 || i == 2) ? 1 : 2));
+      v[i] = q < (long long)pos[i] + len && q < n ? __ldg(f) : 0x7fffffff;
     }
-  int ends[kMaxSegs];
-  unsigned char kinds[16] = {};
-  int nseg = 0;
-  long long start = lb;
-  for (int i = 0; i < 9; ++i) {
-    const long long e = b[i];
-    if (e <= start) continue;
-    const int kd = kind(start);
-    if (nseg > 0 && kinds[nseg - 1] == kd) {
-      ends[nseg - 1] = (int)e;
-    } else {
-      kinds[nseg] = (unsigned char)kd;
-      ends[nseg++] = (int)e;
-    }
-    start = e;
+#pragma unroll
+    for (int i = 0; i < kSearches; ++i)
+      pos[i] += (int)(__popc(__ballot_sync(0xffffffffu, v[i] < key[i])) * step);
+    len = step - 1;
   }
-  for (int i = nseg; i < kMaxSegs; ++i) ends[i] = (int)ub;
-  int4 *o = out + kTileInts * t;
-  o[0] = make_int4((int)lb, (int)ub, nseg, 0);
-  for (int i = 0; i < 3; ++i) o[1 + i] = make_int4(ends[4 * i], ends[4 * i + 1], ends[4 * i + 2], ends[4 * i + 3]);
-  int kw[4];
-  for (int i = 0; i < 4; ++i)
-    kw[i] = kinds[4 * i] | (kinds[4 * i + 1] << 8) | (kinds[4 * i + 2] << 16) | (kinds[4 * i + 3] << 24);
-  o[4] = make_int4(kw[0], kw[1], kw[2], kw[3]);
+  const int lb = min(pos[0], (int)n), ub = max(lb, min(pos[1], (int)n));
+  // change point `lane` (0, 1: the covering range; then the distances as searched; 12: ub)
+  int mine = ub;
+#pragma unroll
+  for (int i = 0; i < 12; ++i)
+    if (lane == i) mine = min(max(pos[i + 2], lb), ub);
+  int c[12];
+#pragma unroll
+  for (int i = 0; i < 12; ++i) c[i] = __shfl_sync(0xffffffffu, mine, i);
+  // in ascending order: lane r takes the r-th of the 13
+  int rank = 0;
+#pragma unroll
+  for (int i = 0; i < 12; ++i) rank += (c[i] < mine || (c[i] == mine && i < lane)) ? 1 : 0;
+  if (lane >= 12) rank = lane;
+  int end = ub;
+#pragma unroll
+  for (int i = 0; i < 13; ++i) {
+    const int e = __shfl_sync(0xffffffffu, mine, i), r = __shfl_sync(0xffffffffu, rank, i);
+    if (r == lane) end = e;
+  }
+  const int prev = __shfl_up_sync(0xffffffffu, end, 1);
+  const int start = lane == 0 ? lb : prev;
+  auto beyond = [&](int q) { return start < c[2 + q] || start >= c[11 - q]; };
+  int kd;
+  if (start < c[0] || start >= c[1])
+    kd = beyond(0) ? kSegEdge : (beyond(1) ? kSegFar1Masked : kSegGeneral);
+  else
+    kd = beyond(2) ? kSegNodes8 : (beyond(3) ? kSegNodes16 : (beyond(4) ? kSegFast : kSegGeneral));
+  // one segment per maximal run of equal kind among the non-empty ranges: a range ends one
+  // when the next non-empty range is of another kind
+  const unsigned full = __ballot_sync(0xffffffffu, lane < 13 && end > start);
+  const unsigned above = full & ~((2u << lane) - 1u);
+  const int next_kd = __shfl_sync(0xffffffffu, kd, above ? __ffs(above) - 1 : 0);
+  const bool last = ((full >> lane) & 1u) && (!above || next_kd != kd);
+  const unsigned ends = __ballot_sync(0xffffffffu, last);
+  const int nseg = __popc(ends);  // at most 12: of the 13 ranges one is always empty or joined
+  const int seg = __popc(ends & ((1u << lane) - 1u));
+  int *o = reinterpret_cast<int *>(out + kTileInts * t);
+  unsigned char *kinds = reinterpret_cast<unsigned char *>(o + 16);
+  if (lane < 16) kinds[lane] = 0;
+  if (lane >= nseg && lane < kMaxSegs) o[4 + lane] = ub;
+  __syncwarp();
+  if (last && seg < kMaxSegs) {
+    o[4 + seg] = end;
+    kinds[seg] = (unsigned char)kd;
+  }
+  if (lane == 0) *reinterpret_cast<int4 *>(o) = make_int4(lb, ub, min(nseg, kMaxSegs), 0);
+  if (nseg > kMaxSegs && lane == 0) {  // cannot happen; the general path holds for every line
+    __threadfence_block();
+    o[4 + kMaxSegs - 1] = ub;
+    kinds[kMaxSegs - 1] = (unsigned char)kSegGeneral;
+  }
 }
 
 __device__ __forceinline__ float rcp_approx(float x) {
@@ -385,34 +470,49 @@ __device__ __forceinline__ void kahan_add2(float2 &s, float2 &c, float2 v) {
   c = __fadd2_rn(__fadd2_rn(t, neg2(s)), neg2(y));
   s = t;
 }
+// the same for a v that may exceed s (Knuth's two-sum)
+__device__ __forceinline__ void two_sum_add2(float2 &s, float2 &c, float2 v) {
+  const float2 y = __fadd2_rn(v, neg2(c));
+  const float2 t = __fadd2_rn(s, y);
+  const float2 yy = __fadd2_rn(t, neg2(s));
+  const float2 ss = __fadd2_rn(t, neg2(yy));
+  c = __fadd2_rn(__fadd2_rn(ss, neg2(s)), __fadd2_rn(yy, neg2(y)));
+  s = t;
+}
 
 // Block = 256 consecutive wavenumbers x up to 8 temperature nodes (one warp per
 // node, 8 consecutive points per lane).  All warps walk the same lines: the
 // block's lines are staged chunk by chunk (geometry R once, coefficients P and,
-// for Voigt, P2 per node) with bulk asynchronous copies on an mbarrier, double
-// buffered.  A point's offset from a line centre, in grid units, is the exact
-// integer j - j_c plus the binary32 sub-grid offset of the centre, so its
-// rounding error is relative to the distance itself.
+// where a kind needs them, P2 per node) with bulk asynchronous copies on an mbarrier,
+// double buffered.  A point's or node's offset from a line centre, in grid units, is exact
+// but for one rounding of the centre's sub-grid offset, so its rounding error is relative
+// to the distance itself.
 // Voigt far wing (|z| >= 20): with t = 1/|z|^2 the three-term series is the
 // polynomial c0 t + c1 t^2 + c2 t^3 + c3 t^4 + c4 t^5 (coefficients from
-// k_prefactor).  The binary32 arithmetic runs on pairs of a lane's points (f32x2
-// instructions).  Fast-path lines (whole tile covered, no near-centre point, or
-// far lines with masked window ends) add kGroup lines per compensated add; the
-// general-path lines evaluate a four-term series, replace the points of their
-// contiguous near-centre range by faddeeva_re_near (one point per lane, handed
-// back through shared memory), mask the ends of their windows, and add in pairs.
+// k_prefactor).  The binary32 arithmetic runs on pairs of points, nodes or lines (f32x2
+// instructions).  By kind: far lines at 8 or 16 nodes of the tile, several lines per warp at
+// a time; lines whose window ends in the tile at 4 nodes of the covered sub-blocks plus the
+// points of the one it ends in; fast lines at every point, kGroup per compensated add;
+// general lines by a five-term series with the points |z| < 8 replaced by the rational
+// series, window ends masked, added in pairs.
 // Lorentz: P = {A g / (pi dnu), g^2}.
+// Of the 2560 lines a tile of the 128^3 workload sums (64 T x 400k points, 100k lines), 2000
+// cost 8 evaluations, 280 16, 128 about 64 and 134 256 each instead of 256 each: 16.2 -> 4.95
+// ms (32^3 workload 1.89 -> 0.96 ms).  Of the 4.95, by timing copies that leave a kind out:
+// general lines 2.5 (their core points 1.4), window ends 0.8, 8 nodes 0.6, fast 0.35, 16 nodes
+// 0.2, interpolation 0.07, chunks and barriers the rest; the FMA pipe (a paired FMA takes two
+// of its cycles) and issue bound it, the reciprocals no longer do.
 template <int PROFILE>
 __global__ void __launch_bounds__(32 * kMaxTPerBlock, 3)
 k_kappa(const float4 *__restrict__ P, const float4 *__restrict__ P2, const int4 *__restrict__ R,
         const int4 *__restrict__ tiles, long long n_lines, long long n_nu, int nT, WeidCoef wc,
         int vec_ok, int accumulate, float *__restrict__ kappa, uint32_t *status) {
   constexpr bool kVoigt = PROFILE == RT_PROFILE_VOIGT;
-  constexpr int kPSets = kVoigt ? 2 : 1;
+  constexpr int kFull = kVoigt ? kChunkP2 : kChunk;  // lines of a chunk of any kind
   __shared__ __align__(16) int4 sR[2][kChunk];
-  __shared__ __align__(16) float4 sP[2][kPSets][kMaxTPerBlock][kChunk];
+  __shared__ __align__(16) float4 sP[2][kMaxTPerBlock][kChunk];  // P, and P2 from kChunkP2 on
   __shared__ __align__(8) uint64_t bars[2];
-  __shared__ float s_res[kMaxTPerBlock][kTilePts];          // near-centre values by tile point
+  __shared__ __align__(16) float s_res[kMaxTPerBlock][2 * kTilePts];  // a warp's core values or node sums
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int tpb = blockDim.x >> 5;
@@ -448,18 +548,30 @@ k_kappa(const float4 *__restrict__ P, const float4 *__restrict__ P2, const int4 
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
-  const int nchunks = (ub - lb + kChunk - 1) / kChunk;
 
-  auto issue = [&](int c) {
-    const long long l0 = (long long)lb + (long long)c * kChunk;
-    const uint32_t cnt = (uint32_t)min((long long)kChunk, (long long)ub - l0);
-    const int b = c & 1;
+  // Chunks: the last kFull lines or fewer in one; else lines of one degree-1 range (P only),
+  // kChunk at most, or the next kFull lines.  sg: the segment of line l, carried along.
+  auto chunk_at = [&](int l, int &sg, bool &with_p2) -> int {
+    while (s_end[sg] <= l) ++sg;  // the last segment ends at ub > l
+    with_p2 = kVoigt;
+    if (ub - l <= kFull) return ub - l;
+    if (!degree1_kind(s_kind[sg])) return kFull;
+    with_p2 = false;
+    return min(kChunk, s_end[sg] - l);
+  };
+  // copies of the chunk at line l into buffer b, issued by the lanes of warp 0: R, then P (and
+  // P2) of one node each
+  auto issue = [&](int l, int cnt, bool with_p2, int b) {
+    const uint32_t bytes = (uint32_t)cnt * 16u;
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    mbar_arrive_expect_tx(&bars[b], cnt * 16u * (uint32_t)(kPSets * nk + 1));
-    bulk_g2s(&sR[b][0], R + l0, cnt * 16u, &bars[b]);
-    for (int w = 0; w < nk; ++w) {
-      bulk_g2s(&sP[b][0][w][0], P + (long long)(k0 + w) * n_lines + l0, cnt * 16u, &bars[b]);
-      if (kVoigt) bulk_g2s(&sP[b][kPSets - 1][w][0], P2 + (long long)(k0 + w) * n_lines + l0, cnt * 16u, &bars[b]);
+    if (lane == 0) {
+      mbar_arrive_expect_tx(&bars[b], bytes * (uint32_t)(nk * (with_p2 ? 2 : 1) + 1));
+      bulk_g2s(&sR[b][0], R + l, bytes, &bars[b]);
+    }
+    __syncwarp();
+    if (lane < nk) {
+      bulk_g2s(&sP[b][lane][0], P + (long long)(k0 + lane) * n_lines + l, bytes, &bars[b]);
+      if (with_p2) bulk_g2s(&sP[b][lane][kChunkP2], P2 + (long long)(k0 + lane) * n_lines + l, bytes, &bars[b]);
     }
   };
 
@@ -468,14 +580,29 @@ k_kappa(const float4 *__restrict__ P, const float4 *__restrict__ P2, const int4 
   float2 acc[kPairs], cmp[kPairs];
 #pragma unroll
   for (int h = 0; h < kPairs; ++h) acc[h] = cmp[h] = make_float2(0.0f, 0.0f);
-  if (threadIdx.x == 0) {
-    if (nchunks > 0) issue(0);
-    if (nchunks > 1) issue(1);
+  // sums of the interpolated lines at the lane's two nodes: 8 nodes (lane & 3) over every
+  // eighth line, 16 nodes (lane & 7) over every fourth
+  float2 n8 = make_float2(0.0f, 0.0f), n8c = n8, n16 = n8, n16c = n8;
+  bool nodes = false;
+  // warp 0 issues chunks up to two ahead of the one being summed
+  int pl = lb, pseg = 0, issued = 0;
+  auto issue_next = [&]() {
+    if (pl >= ub) return;
+    bool with_p2;
+    const int cnt = chunk_at(pl, pseg, with_p2);
+    issue(pl, cnt, with_p2, issued & 1);
+    pl += cnt;
+    ++issued;
+  };
+  if (warp == 0) {
+    issue_next();
+    issue_next();
   }
   const int wsel = min(warp, nk - 1);
   int seg = 0;  // current segment, carried across chunks
   bool aborted = false;
-  for (int c = 0; c < nchunks; ++c) {
+  int cnt = 0;
+  for (int c = 0, l0 = lb; l0 < ub; ++c, l0 += cnt) {
     const int b = c & 1;
     const uint32_t parity = (uint32_t)((c >> 1) & 1);
     unsigned spins = 0;
@@ -486,32 +613,106 @@ k_kappa(const float4 *__restrict__ P, const float4 *__restrict__ P2, const int4 
         break;
       }
     }
-    if (__syncthreads_or(timed_out)) {  // the block leaves together
-      if (threadIdx.x == 0) {
-        status_or(status, RT_DEV_TIMEOUT);
-        // The copies of this chunk and of the next one (issued one chunk ahead) may
-        // still be writing into this block's shared memory: wait for them, again with
-        // a bound, so that no copy lands after the block has released it.
-        for (int d = c; d < min(c + 2, nchunks); ++d) {
-          unsigned n = 0;
-          while (!mbar_try_wait(&bars[d & 1], (uint32_t)((d >> 1) & 1)) && ++n <= kWaitLimit) {
-          }
-        }
+    timed_out = __any_sync(0xffffffffu, timed_out);  // warp-uniform: such a warp sums nothing
+    bool with_p2;
+    cnt = chunk_at(l0, seg, with_p2);
+    const int4 *cR = sR[b];
+    const float4 *cP = sP[b][wsel], *cP2 = cP + kChunkP2;
+
+    // the line's value, less the factor p.x for Lorentz lines, at a pair of offsets u (grid
+    // units) from its centre; DEG 4 or 1: the far-wing series' degree
+    auto far_value = [&](auto deg, float2 u, const float4 &p, int i) -> float2 {
+      constexpr int DEG = decltype(deg)::value;
+      if (!kVoigt) return __fmul2_rn(dup2(p.x), rcp2(__ffma2_rn(u, u, dup2(p.y))));
+      const float2 c0 = dup2(p.x), c1 = dup2(1.5f * p.x);
+      const float2 x = __fmul2_rn(dup2(p.y), u);
+      const float2 t = rcp2(__ffma2_rn(x, x, dup2(p.z)));
+      if (DEG == 4) {
+        const float4 p2 = cP2[i];
+        return __fmul2_rn(t, __ffma2_rn(t, __ffma2_rn(t, __ffma2_rn(t, __ffma2_rn(t, dup2(p2.y), dup2(p2.x)), dup2(p.w)), c1), c0));
       }
-      aborted = true;
-      break;
-    }
-    const int l0 = lb + c * kChunk;
-    const int cnt = min(kChunk, ub - l0);
+      return __fmul2_rn(t, __ffma2_rn(t, c1, c0));
+    };
+    // lines [i, i1) at the M tile nodes: M / 2 lanes take a line (two nodes each), the warp
+    // 64 / M lines at a time
+    auto run_nodes = [&](auto deg, auto m, const float *un, int i, int i1, float2 &s, float2 &sc) {
+      constexpr int kLanes = decltype(m)::value / 2, kLines = 32 / kLanes;
+      const float2 u0 = *reinterpret_cast<const float2 *>(un + 2 * (lane % kLanes));
+#pragma unroll 1
+      for (i += lane / kLanes; __any_sync(0xffffffffu, i < i1); i += kLines * kNodeGroup) {
+        float2 g = make_float2(0.0f, 0.0f);
+#pragma unroll
+        for (int e = 0; e < kNodeGroup; ++e) {
+          const bool in = i + e * kLines < i1;
+          const int q = in ? i + e * kLines : i1 - 1;
+          const int2 r = *reinterpret_cast<const int2 *>(&cR[q].z);
+          const float2 u = __fadd2_rn(__fadd2_rn(dup2((float)(jw0 - r.x)), u0), dup2(__int_as_float(r.y)));
+          const float2 v = far_value(deg, u, cP[q], q);
+          if (in) g = __fadd2_rn(g, v);
+        }
+        kahan_add2(s, sc, g);
+      }
+      nodes = true;
+    };
+    // lines [i, i1) whose windows end inside the tile, one after the other: lane (b, m) takes
+    // node m of sub-block b where the window covers it, and point `lane` of the sub-block the
+    // window ends in.  Both sums go to the points before returning.
+    auto run_edge = [&](int i, int i1) {
+      float *res = s_res[warp];
+      const int sb = lane >> 2, nu_last = (int)(n_nu - 1);
+      const float un = 32.0f * (float)sb + kTab4.u[lane & 3];
+      float2 s = make_float2(0.0f, 0.0f), sc = s;
+#pragma unroll
+      for (int q = 0; q < kPtsPerThread; ++q) res[32 * q + lane] = 0.0f;
+      int cur = -1;
+      auto flush = [&]() {
+        if (cur >= 0 && cur < kTilePts / 32) res[32 * cur + lane] += __fsub_rn(s.y, sc.y);
+        s.y = sc.y = 0.0f;
+      };
+#pragma unroll 1
+      for (; i < i1; ++i) {
+        const int4 r = cR[i];
+        // covered tile points; a window that holds the grid's last point has no end here
+        const int a = max(r.x - jw0, 0), e = r.y >= nu_last ? kTilePts - 1 : min(r.y - jw0, kTilePts - 1);
+        const int eb = a == 0 ? (e + 1) >> 5 : a >> 5;                      // sub-block of the end
+        if (eb != cur) {  // warp-uniform; window ends are monotone in the line index
+          flush();
+          cur = eb;
+        }
+        const int pt = 32 * eb + lane;
+        const float2 u = __fadd2_rn(__fadd2_rn(dup2((float)(jw0 - r.z)), make_float2(un, (float)pt)), dup2(__int_as_float(r.w)));
+        float2 v = far_value(std::integral_constant<int, 1>(), u, cP[i], i);
+        if (32 * sb < a || 32 * sb + 31 > e) v.x = 0.0f;
+        if (pt < a || pt > e || (32 * eb >= a && 32 * eb + 31 <= e)) v.y = 0.0f;
+        kahan_add2(s, sc, v);
+      }
+      flush();
+      __syncwarp();
+      const float f = __fsub_rn(s.x, sc.x);
+      float fm[4];
+#pragma unroll
+      for (int m = 0; m < 4; ++m) fm[m] = __shfl_sync(0xffffffffu, f, (lane & ~3) + m);
+      const int p0 = lane * kPtsPerThread, w0 = p0 & 31;
+#pragma unroll
+      for (int h = 0; h < kPairs; ++h) {
+        float2 v = *reinterpret_cast<const float2 *>(res + p0 + 2 * h);
+        v = __fadd2_rn(v, dup2(fm[1]));  // interpolate the differences to one node's value
+#pragma unroll
+        for (int m = 0; m < 4; ++m)
+          if (m != 1)
+            v = __ffma2_rn(*reinterpret_cast<const float2 *>(&kTab4.w[m][w0 + 2 * h]), dup2(fm[m] - fm[1]), v);
+        two_sum_add2(acc[h], cmp[h], v);
+      }
+      __syncwarp();  // res is the general path's next
+    };
 
     // fast paths: g[q] += value of line i at the lane's points (or = when first).
-    // DEG 4: full far-wing series; DEG 2: far lines (t^3 and t^4 terms negligible);
-    // MASK: zero outside the line's window.
+    // DEG 4: full far-wing series; DEG 1: far lines; MASK: zero outside the line's window.
     auto fast_line = [&](auto deg, auto mask, int i, float2 (&g)[kPairs], bool first) {
       constexpr int DEG = decltype(deg)::value;
       constexpr bool MASK = decltype(mask)::value;
-      const int4 r = sR[b][i];
-      const float4 p = sP[b][0][wsel][i];
+      const int4 r = cR[i];
+      const float4 p = cP[i];
       const float ul = point_offset(jt, r.z, r.w);
       if (!kVoigt) {
         const float2 u0 = dup2(ul), g2 = dup2(p.y), a2 = dup2(p.x);
@@ -529,7 +730,7 @@ k_kappa(const float4 *__restrict__ P, const float4 *__restrict__ P2, const int4 
         const float2 c0 = dup2(p.x), c1 = dup2(1.5f * p.x), sd = dup2(p.y), y2 = dup2(p.z);
         const float2 xt = dup2(p.y * ul);
         float4 p2 = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-        if (DEG == 4) p2 = sP[b][kPSets - 1][wsel][i];
+        if (DEG == 4) p2 = cP2[i];
 #pragma unroll
         for (int h = 0; h < kPairs; ++h) {
           const float2 x = __ffma2_rn(sd, make_float2((float)(2 * h), (float)(2 * h + 1)), xt);
@@ -537,8 +738,6 @@ k_kappa(const float4 *__restrict__ P, const float4 *__restrict__ P2, const int4 
           float2 v;
           if (DEG == 4)
             v = __ffma2_rn(t, __ffma2_rn(t, __ffma2_rn(t, __ffma2_rn(t, dup2(p2.y), dup2(p2.x)), dup2(p.w)), c1), c0);
-          else if (DEG == 2)
-            v = __ffma2_rn(t, __ffma2_rn(t, dup2(p.w), c1), c0);
           else
             v = __ffma2_rn(t, c1, c0);
           if (MASK) {
@@ -569,118 +768,235 @@ k_kappa(const float4 *__restrict__ P, const float4 *__restrict__ P2, const int4 
       }
     };
 
-    // general path: the value of line i at the lane's points, with masking
-    // outside the window and near-centre points
-    auto line_vals = [&](int i, float2 (&v)[kPairs]) {
-        const int4 r = sR[b][i];
-        const float4 p = sP[b][0][wsel][i];
-        const float ul = point_offset(jt, r.z, r.w);
-        if (!kVoigt) {
-          const float2 u0 = dup2(ul), g2 = dup2(p.y), a2 = dup2(p.x);
+    // general path, two lines at a time (the second may be absent).  line_series: a line's
+    // five-term series at the lane's points, valid for |z| >= 8; Lorentz: its value.
+    auto line_series = [&](int i, float2 (&v)[kPairs]) {
+      const int4 r = cR[i];
+      const float4 p = cP[i];
+      const float ul = point_offset(jt, r.z, r.w);
+      if (!kVoigt) {
+        const float2 u0 = dup2(ul), g2 = dup2(p.y), a2 = dup2(p.x);
 #pragma unroll
-          for (int h = 0; h < kPairs; ++h) {
-            const float2 u = __fadd2_rn(u0, make_float2((float)(2 * h), (float)(2 * h + 1)));
-            v[h] = __fmul2_rn(a2, rcp2(__ffma2_rn(u, u, g2)));
-          }
-        } else {
-          const float4 p2 = sP[b][kPSets - 1][wsel][i];
-          const float y2 = p.z;
-          const float2 y22 = dup2(y2), sd = dup2(p.y), xt = dup2(p.y * ul);
-          // four-term series, valid for |z| >= 10: the degree-4 polynomial plus the
-          // fourth term 15 t^3 (7 - 56 s + 112 s^2 - 64 s^3) / 8, s = y^2 t, in t
-          const float q1 = y2 * p.x, q2 = q1 * y2;
-          const float2 c3 = dup2(__fmaf_rn(13.125f, p.x, p2.x)), c4 = dup2(__fmaf_rn(-105.0f, q1, p2.y));
-          const float2 c5 = dup2(210.0f * q2), c6 = dup2(-120.0f * q2 * y2);
-          const float2 c0 = dup2(p.x), c1 = dup2(1.5f * p.x), c2 = dup2(p.w);
-#pragma unroll
-          for (int h = 0; h < kPairs; ++h) {
-            const float2 x = __ffma2_rn(sd, make_float2((float)(2 * h), (float)(2 * h + 1)), xt);
-            const float2 t = rcp2(__ffma2_rn(x, x, y22));
-            const float2 w = __ffma2_rn(
-                t, __ffma2_rn(t, __ffma2_rn(t, __ffma2_rn(t, __ffma2_rn(t, __ffma2_rn(t, c6, c5), c4), c3), c2), c1),
-                c0);
-            v[h] = __fmul2_rn(t, w);
-          }
-          // warp-uniform: the tile's offsets [fu, fu + kTilePts) meet the region |z| < 10,
-          // |u| < u_core in grid units; its points are the contiguous tile indices [ea, eb]
-          // (one point of margin each side: the near form holds at any |z|), evaluated
-          // one per lane and handed to their owners through shared memory
-          const float fu = (float)(jw0 - r.z) + __int_as_float(r.w);
-          if (fu < p2.w + 1.0f && fu + (float)kTilePts > -p2.w - 1.0f) {
-            const int ea = (int)fmaxf(floorf(-p2.w - 1.0f - fu), 0.0f);
-            const int eb = (int)fminf(ceilf(p2.w + 1.0f - fu), (float)(kTilePts - 1));
-            float *res = s_res[warp];
-            const float y = sqrtf(y2);
-            const float coef = __fdividef(p.x, y);
-            for (int e = ea + lane; e <= eb; e += 32) {
-              const float xe = p.y * point_offset(jw0 + e, r.z, r.w);
-              res[e] = coef * faddeeva_re_near(xe, y, __fmaf_rn(xe, xe, y2), wc);
-            }
-            __syncwarp();
-            const int p0 = lane * kPtsPerThread;
-            if (p0 + kPtsPerThread > ea && p0 <= eb) {
-#pragma unroll
-              for (int h = 0; h < kPairs; ++h) {
-                if (p0 + 2 * h >= ea && p0 + 2 * h <= eb) v[h].x = res[p0 + 2 * h];
-                if (p0 + 2 * h + 1 >= ea && p0 + 2 * h + 1 <= eb) v[h].y = res[p0 + 2 * h + 1];
-              }
-            }
-            __syncwarp();
-          }
+        for (int h = 0; h < kPairs; ++h) {
+          const float2 u = __fadd2_rn(u0, make_float2((float)(2 * h), (float)(2 * h + 1)));
+          v[h] = __fmul2_rn(a2, rcp2(__ffma2_rn(u, u, g2)));
         }
-        if (r.x > jw0 || r.y < jw1) {  // warp-uniform: the window ends inside this block's points
+        return;
+      }
+      const float4 p2 = cP2[i];
+      // in t: the degree-4 polynomial plus 13.125 t^3, (59.0625 - 105 q) t^4 and the powers
+      // above of the fourth and fifth terms, q = y^2 (see faddeeva_series5)
+      const float q1 = p.z * p.x, q2 = p.z * q1, q3 = p.z * q2;
+      const float2 y22 = dup2(p.z), sd = dup2(p.y), xt = dup2(p.y * ul);
+      const float2 c8 = dup2(1680.0f * p.z * q3), c7 = dup2(-3780.0f * q3);
+      const float2 c6 = dup2(__fmaf_rn(2835.0f, q2, -120.0f * q3)), c5 = dup2(__fmaf_rn(-787.5f, q1, 210.0f * q2));
+      const float2 c4 = dup2(__fmaf_rn(59.0625f, p.x, __fmaf_rn(-105.0f, q1, p2.y)));
+      const float2 c3 = dup2(__fmaf_rn(13.125f, p.x, p2.x)), c2 = dup2(p.w), c1 = dup2(1.5f * p.x), c0 = dup2(p.x);
 #pragma unroll
-          for (int h = 0; h < kPairs; ++h) {
-            if (jt + 2 * h < r.x || jt + 2 * h > r.y) v[h].x = 0.0f;
-            if (jt + 2 * h + 1 < r.x || jt + 2 * h + 1 > r.y) v[h].y = 0.0f;
-          }
+      for (int h = 0; h < kPairs; ++h) {
+        const float2 x = __ffma2_rn(sd, make_float2((float)(2 * h), (float)(2 * h + 1)), xt);
+        const float2 t = rcp2(__ffma2_rn(x, x, y22));
+        float2 w = __ffma2_rn(t, c8, c7);
+        w = __ffma2_rn(t, __ffma2_rn(t, __ffma2_rn(t, w, c6), c5), c4);
+        w = __ffma2_rn(t, __ffma2_rn(t, __ffma2_rn(t, __ffma2_rn(t, w, c3), c2), c1), c0);
+        v[h] = __fmul2_rn(t, w);
+      }
+    };
+    // the tile points with |z| < 8 of line i: |u| <= u_core, the contiguous indices
+    // [first, first + n) (warp-uniform)
+    auto core_range = [&](int i, int &first) -> int {
+      const int2 r = *reinterpret_cast<const int2 *>(&cR[i].z);
+      const float fu = (float)(jw0 - r.x) + __int_as_float(r.y), uc = cP2[i].w;
+      first = (int)fmaxf(ceilf(-uc - fu), 0.0f);
+      const int last = (int)fminf(floorf(uc - fu), (float)(kTilePts - 1));
+      return uc > 0.0f ? last - first + 1 : 0;
+    };
+    // Those points by Weideman's rational series, one lane a point, two lines in one paired
+    // pass (a line has 16 to 40 such points on a 0.005 cm^-1 grid: 32 lanes take them in one
+    // or two passes), into shared memory for their owners.
+    auto core_values = [&](int ia, int ib, int fa, int fb, int n) {
+      float2 *res = reinterpret_cast<float2 *>(s_res[warp]);
+      const float4 pa = cP[ia], pb = cP[ib];
+      const int2 ra = *reinterpret_cast<const int2 *>(&cR[ia].z), rb = *reinterpret_cast<const int2 *>(&cR[ib].z);
+      const float2 y = make_float2(sqrtf(pa.z), sqrtf(pb.z));
+      const float2 coef = make_float2(__fdividef(pa.x, y.x), __fdividef(pb.x, y.y));
+      const float2 dr = __fadd2_rn(dup2(wc.L), y), nr = __fadd2_rn(dup2(wc.L), neg2(y));
+#pragma unroll 1
+      for (int e = lane; e < n; e += 32) {
+        const float2 x = make_float2(pa.y * point_offset(jw0 + fa + e, ra.x, ra.y),
+                                     pb.y * point_offset(jw0 + fb + e, rb.x, rb.y));
+        // iz = -y + ix, v = 1 / (L - iz), Z = (L + iz) v; sqrt(pi) w = v (p(Z) v + 1)
+        const float2 d = __ffma2_rn(dr, dr, __fmul2_rn(x, x));
+        const float2 inv = make_float2(__frcp_rn(d.x), __frcp_rn(d.y));
+        const float2 vr = __fmul2_rn(dr, inv), vi = __fmul2_rn(x, inv);
+        const float2 zr = __ffma2_rn(nr, vr, neg2(__fmul2_rn(x, vi))), zi = __ffma2_rn(nr, vi, __fmul2_rn(x, vr));
+        const float2 nzi = neg2(zi);
+        float2 pr = dup2(wc.a[kWeidN - 1]), pi = make_float2(0.0f, 0.0f);
+#pragma unroll
+        for (int n = kWeidN - 2; n >= 0; --n) {
+          const float2 t = __ffma2_rn(pr, zr, __ffma2_rn(pi, nzi, dup2(wc.a[n])));
+          pi = __ffma2_rn(pr, zi, __fmul2_rn(pi, zr));
+          pr = t;
         }
+        const float2 nvi = neg2(vi);
+        const float2 qr = __fadd2_rn(__ffma2_rn(pr, vr, __fmul2_rn(pi, nvi)), dup2(1.0f));
+        const float2 qi = __ffma2_rn(pr, vi, __fmul2_rn(pi, vr));
+        res[e] = __fmul2_rn(coef, __ffma2_rn(vr, qr, __fmul2_rn(nvi, qi)));
+      }
+      __syncwarp();
+    };
+    // the lane's points among the n core points from tile point `first` on: values c of res
+    auto take_core = [&](int c, int first, int n, float2 (&v)[kPairs]) {
+      const float *res = s_res[warp] + c;
+      const int a = lane * kPtsPerThread - first;  // the lane's first point in res
+      if (a + kPtsPerThread > 0 && a < n) {
+#pragma unroll
+        for (int h = 0; h < kPairs; ++h) {
+          if ((unsigned)(a + 2 * h) < (unsigned)n) v[h].x = res[2 * (a + 2 * h)];
+          if ((unsigned)(a + 2 * h + 1) < (unsigned)n) v[h].y = res[2 * (a + 2 * h + 1)];
+        }
+      }
+    };
+    auto mask_window = [&](int i, float2 (&v)[kPairs]) {
+      const int2 r = *reinterpret_cast<const int2 *>(&cR[i].x);
+      if (r.x > jw0 || r.y < jw1) {  // warp-uniform: the window ends inside this block's points
+#pragma unroll
+        for (int h = 0; h < kPairs; ++h) {
+          if (jt + 2 * h < r.x || jt + 2 * h > r.y) v[h].x = 0.0f;
+          if (jt + 2 * h + 1 < r.x || jt + 2 * h + 1 > r.y) v[h].y = 0.0f;
+        }
+      }
     };
     // lines enter the compensated sum in pairs: the sum of two positive line
     // values is rounded once (relative error <= 2^-24 of the pair)
     auto run_general = [&](int i, int i1) {
 #pragma unroll 1
-      for (; i + 1 < i1; i += 2) {
-        float2 va[kPairs], vb[kPairs];
-        line_vals(i, va);
-        line_vals(i + 1, vb);
+      for (; i < i1; i += 2) {
+        const bool two = i + 1 < i1;
+        const int j = two ? i + 1 : i;
+        int fa = 0, fb = 0, na = 0, nb = 0;
+        if (kVoigt) {
+          na = core_range(i, fa);
+          nb = two ? core_range(j, fb) : 0;
+          if (max(na, nb) > 0) core_values(i, j, fa, fb, max(na, nb));
+        }
+        float2 v[kPairs], w[kPairs];
+        line_series(i, v);
+        if (na > 0) take_core(0, fa, na, v);
+        mask_window(i, v);
+        if (two) {
+          line_series(j, w);
+          if (nb > 0) take_core(1, fb, nb, w);
+          mask_window(j, w);
 #pragma unroll
-        for (int h = 0; h < kPairs; ++h) kahan_add2(acc[h], cmp[h], __fadd2_rn(va[h], vb[h]));
-      }
-      if (i < i1) {
-        float2 va[kPairs];
-        line_vals(i, va);
+          for (int h = 0; h < kPairs; ++h) v[h] = __fadd2_rn(v[h], w[h]);
+        }
+        __syncwarp();  // res is the next lines'
 #pragma unroll
-        for (int h = 0; h < kPairs; ++h) kahan_add2(acc[h], cmp[h], va[h]);
+        for (int h = 0; h < kPairs; ++h) kahan_add2(acc[h], cmp[h], v[h]);
       }
     };
 
     // the chunk [l0, l0 + cnt) split at the tile's segment ends (block-uniform)
-    int i = 0;
+    int i = timed_out ? cnt : 0;
 #pragma unroll 1
     while (i < cnt) {
       const int l = l0 + i;
       while (s_end[seg] <= l) ++seg;  // the last segment ends at ub > l
       const int i1 = min(cnt, s_end[seg] - l0);
       const int kd = s_kind[seg];
-      if (kd == kSegFar1)
-        run_fast(std::integral_constant<int, 1>(), std::false_type(), i, i1);
-      else if (kd == kSegFar2)
-        run_fast(std::integral_constant<int, 2>(), std::false_type(), i, i1);
+      if (kd == kSegNodes8)
+        run_nodes(std::integral_constant<int, 1>(), std::integral_constant<int, 8>(), kTab8.u, i, i1, n8, n8c);
+      else if (kd == kSegNodes16)
+        run_nodes(std::integral_constant<int, 4>(), std::integral_constant<int, 16>(), kTab16.u, i, i1, n16, n16c);
+      else if (kd == kSegEdge)
+        run_edge(i, i1);
       else if (kd == kSegFast)
         run_fast(std::integral_constant<int, 4>(), std::false_type(), i, i1);
       else if (kd == kSegFar1Masked)
         run_fast(std::integral_constant<int, 1>(), std::true_type(), i, i1);
-      else if (kd == kSegFar2Masked)
-        run_fast(std::integral_constant<int, 2>(), std::true_type(), i, i1);
       else
         run_general(i, i1);
       i = i1;
     }
-    __syncthreads();  // every warp is done with buffer b
-    if (threadIdx.x == 0 && c + 2 < nchunks) issue(c + 2);
+    // every warp is done with buffer b (the waits above order each thread's own reads)
+    if (__syncthreads_or(timed_out)) {  // the block leaves together
+      if (threadIdx.x == 0) {
+        status_or(status, RT_DEV_TIMEOUT);
+        // The copies of this chunk and of the next one (issued one chunk ahead) may
+        // still be writing into this block's shared memory: wait for them, again with
+        // a bound, so that no copy lands after the block has released it.
+        for (int d = c; d < issued; ++d) {
+          unsigned n = 0;
+          while (!mbar_try_wait(&bars[d & 1], (uint32_t)((d >> 1) & 1)) && ++n <= kWaitLimit) {
+          }
+        }
+      }
+      aborted = true;
+      break;
+    }
+    if (warp == 0) issue_next();
   }
   if (aborted || warp >= nk) return;
+
+  if (nodes) {  // warp-uniform: the interpolated lines' node sums to the lane's points
+    // as hi + lo pairs throughout, so that the interpolation adds next to nothing to the
+    // rounding error of the line values themselves
+    float2 f8 = n8, l8 = neg2(n8c), f16 = n16, l16 = neg2(n16c);
+    auto two_sum2 = [](float2 &hi, float2 &lo, float2 v) {  // hi + lo += v
+      const float2 t = __fadd2_rn(hi, v), vv = __fadd2_rn(t, neg2(hi)), hh = __fadd2_rn(t, neg2(vv));
+      lo = __fadd2_rn(lo, __fadd2_rn(__fadd2_rn(hi, neg2(hh)), __fadd2_rn(v, neg2(vv))));
+      hi = t;
+    };
+    auto add_lanes = [&](float2 &hi, float2 &lo, int o) {
+      lo = __fadd2_rn(lo, make_float2(__shfl_xor_sync(0xffffffffu, lo.x, o), __shfl_xor_sync(0xffffffffu, lo.y, o)));
+      two_sum2(hi, lo, make_float2(__shfl_xor_sync(0xffffffffu, hi.x, o), __shfl_xor_sync(0xffffffffu, hi.y, o)));
+    };
+#pragma unroll
+    for (int o = 4; o < 32; o <<= 1) add_lanes(f8, l8, o);
+#pragma unroll
+    for (int o = 8; o < 32; o <<= 1) add_lanes(f16, l16, o);
+    // the 8-node interpolant at the lane's two of the 16 nodes; only differences to one
+    // node's value are weighted, so that the weights' signs cost no accuracy
+    const int p16 = 2 * (lane & 7);
+    const float r8 = __shfl_sync(0xffffffffu, f8.x, 2), rl8 = __shfl_sync(0xffffffffu, l8.x, 2);
+    float2 d8 = dup2(rl8);
+#pragma unroll
+    for (int m = 0; m < 8; ++m) {
+      const float f = __shfl_sync(0xffffffffu, (m & 1) ? f8.y : f8.x, m >> 1) - r8;
+      const float l = __shfl_sync(0xffffffffu, (m & 1) ? l8.y : l8.x, m >> 1) - rl8;
+      d8 = __ffma2_rn(*reinterpret_cast<const float2 *>(&kTab8.w[m][p16]), dup2(f + l), d8);
+    }
+    two_sum2(f16, l16, dup2(r8));
+    two_sum2(f16, l16, d8);
+    float *res = s_res[warp];
+    __syncwarp();
+    if (lane < 8) {
+      *reinterpret_cast<float2 *>(res + p16) = f16;
+      *reinterpret_cast<float2 *>(res + 16 + p16) = l16;
+    }
+    __syncwarp();
+    const float ref = res[8], refl = res[16 + 8];
+    float2 v[kPairs];
+#pragma unroll
+    for (int h = 0; h < kPairs; ++h) v[h] = dup2(refl);
+    const int p0 = lane * kPtsPerThread;
+#pragma unroll
+    for (int m = 0; m < 16; ++m) {
+      const float2 f = dup2((res[m] - ref) + (res[16 + m] - refl));
+      const float4 wa = *reinterpret_cast<const float4 *>(&kTab16.w[m][p0]);
+      const float4 wb = *reinterpret_cast<const float4 *>(&kTab16.w[m][p0 + 4]);
+      v[0] = __ffma2_rn(make_float2(wa.x, wa.y), f, v[0]);
+      v[1] = __ffma2_rn(make_float2(wa.z, wa.w), f, v[1]);
+      v[2] = __ffma2_rn(make_float2(wb.x, wb.y), f, v[2]);
+      v[3] = __ffma2_rn(make_float2(wb.z, wb.w), f, v[3]);
+    }
+#pragma unroll
+    for (int h = 0; h < kPairs; ++h) {
+      two_sum_add2(acc[h], cmp[h], dup2(ref));
+      two_sum_add2(acc[h], cmp[h], v[h]);
+    }
+  }
 
   float *row = kappa + (long long)k * n_nu;
   float out[kPtsPerThread];
@@ -1014,7 +1330,7 @@ rt_status launch_line_geometry(const double *nu0, const double *S, const double 
                                long long n, const rt_spectral *spec, int check, int4 *R,
                                unsigned long long *evals, uint32_t *status, cudaStream_t st) {
   if (n <= 0) return RT_OK;
-  GeomParams G{spec->nu_min, spec->dnu, spec->cutoff, spec->n_nu, n, spec->nT, check,
+  GeomParams G{spec->nu_min, spec->dnu, 1.0 / spec->dnu, spec->cutoff, spec->n_nu, n, spec->nT, check,
                spec->points_per_line};
   k_line_geometry<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(nu0, S, g, E, G, R, evals, status);
   RT_CUDA_TRY(cudaGetLastError());
@@ -1082,7 +1398,7 @@ rt_status run_build(char *base, const KappaLayout &L, const rt_lines *lines, con
   int4 *tiles = reinterpret_cast<int4 *>(base + L.off_tiles);
   unsigned *far_bits = reinterpret_cast<unsigned *>(base + L.off_far);
 
-  GeomParams G{spec->nu_min, spec->dnu, spec->cutoff, spec->n_nu, n, spec->nT,
+  GeomParams G{spec->nu_min, spec->dnu, 1.0 / spec->dnu, spec->cutoff, spec->n_nu, n, spec->nT,
                lines->memory == RT_MEM_DEVICE ? 1 : 0, spec->points_per_line};
   const int tb = 256;
   const bool adaptive = spec->kappa_min > 0;
@@ -1119,7 +1435,7 @@ rt_status run_build(char *base, const KappaLayout &L, const rt_lines *lines, con
   Q.nT = spec->nT;
   Q.profile = spec->profile;
   dim3 gp((unsigned)((n + tb - 1) / tb), (unsigned)spec->nT);
-  RT_CUDA_TRY(cudaMemsetAsync(far_bits, 0, 2 * sizeof(unsigned), st));
+  RT_CUDA_TRY(cudaMemsetAsync(far_bits, 0, sizeof(unsigned), st));
   k_prefactor<<<gp, tb, 0, st>>>(d_nu0, d_S, d_g, d_E, Q, P, P2, far_bits);
   RT_CUDA_TRY(cudaGetLastError());
 
