@@ -32,8 +32,7 @@ namespace {
 constexpr int kPtsPerThread = 8;
 constexpr int kTilePts = 32 * kPtsPerThread;  // 256 wavenumbers per block, one warp per T node
 constexpr int kMaxTPerBlock = 8;              // warps (T nodes) per block
-constexpr int kChunk = 192;                   // lines per staged chunk that need P only
-constexpr int kChunkP2 = 96;                  // ... that need P and P2
+constexpr int kChunk = 192;                   // lines per staged chunk that need P only (half that with P2)
 constexpr int kGroup = 8;                     // fast-path lines summed before one compensated add
 constexpr int kNodeGroup = 4;                 // interpolated lines a lane sums before one compensated add
 constexpr unsigned kWaitLimit = 1u << 22;     // bounded mbarrier waits
@@ -502,15 +501,26 @@ __device__ __forceinline__ void two_sum_add2(float2 &s, float2 &c, float2 v) {
 // general lines 2.5 (their core points 1.4), window ends 0.8, 8 nodes 0.6, fast 0.35, 16 nodes
 // 0.2, interpolation 0.07, chunks and barriers the rest; the FMA pipe (a paired FMA takes two
 // of its cycles) and issue bound it, the reciprocals no longer do.
-template <int PROFILE>
+// ADAPT: every line has its own window at each node (AW, within the cutoff window), staged
+// with the coefficients.  A warp sorts each range's lines by its node's windows (ballots):
+// lines whose window holds the tile go the range's way, lines whose window ends in it the
+// masked or window-end way, the others cost nothing more.  64 T x 100k points, 20k lines,
+// kappa_min 1e-3: 1.04 ms, where a gather over each tile's kept lines took 4.24.
+template <int PROFILE, bool ADAPT>
 __global__ void __launch_bounds__(32 * kMaxTPerBlock, 3)
 k_kappa(const float4 *__restrict__ P, const float4 *__restrict__ P2, const int4 *__restrict__ R,
+        const int2 *__restrict__ AW,
         const int4 *__restrict__ tiles, long long n_lines, long long n_nu, int nT, WeidCoef wc,
         int vec_ok, int accumulate, float *__restrict__ kappa, uint32_t *status) {
   constexpr bool kVoigt = PROFILE == RT_PROFILE_VOIGT;
-  constexpr int kFull = kVoigt ? kChunkP2 : kChunk;  // lines of a chunk of any kind
-  __shared__ __align__(16) int4 sR[2][kChunk];
-  __shared__ __align__(16) float4 sP[2][kMaxTPerBlock][kChunk];  // P, and P2 from kChunkP2 on
+  constexpr int kCap = ADAPT ? 128 : kChunk, kCapP2 = kCap / 2;  // lines of a chunk: P only, P and P2
+  constexpr int kFull = kVoigt ? kCapP2 : kCap;                  // lines of a chunk of any kind
+  __shared__ __align__(16) int4 sR[2][kCap];
+  __shared__ __align__(16) float4 sP[2][kMaxTPerBlock][kCap];  // P, and P2 from kCapP2 on
+  // windows at the node (16-byte copies: one element of margin each side); a warp's lists of
+  // chunk lines: covering; ending in the tile from the front, masked ones from the back
+  __shared__ __align__(16) int2 sW[2][ADAPT ? kMaxTPerBlock : 1][ADAPT ? kCap + 2 : 2];
+  __shared__ unsigned char s_list[ADAPT ? kMaxTPerBlock : 1][2][ADAPT ? kCap : 1];
   __shared__ __align__(8) uint64_t bars[2];
   __shared__ __align__(16) float s_res[kMaxTPerBlock][2 * kTilePts];  // a warp's core values or node sums
 
@@ -550,28 +560,33 @@ k_kappa(const float4 *__restrict__ P, const float4 *__restrict__ P2, const int4 
   __syncthreads();
 
   // Chunks: the last kFull lines or fewer in one; else lines of one degree-1 range (P only),
-  // kChunk at most, or the next kFull lines.  sg: the segment of line l, carried along.
+  // kCap at most, or the next kFull lines.  sg: the segment of line l, carried along.
   auto chunk_at = [&](int l, int &sg, bool &with_p2) -> int {
     while (s_end[sg] <= l) ++sg;  // the last segment ends at ub > l
     with_p2 = kVoigt;
     if (ub - l <= kFull) return ub - l;
     if (!degree1_kind(s_kind[sg])) return kFull;
     with_p2 = false;
-    return min(kChunk, s_end[sg] - l);
+    return min(kCap, s_end[sg] - l);
   };
   // copies of the chunk at line l into buffer b, issued by the lanes of warp 0: R, then P (and
   // P2) of one node each
   auto issue = [&](int l, int cnt, bool with_p2, int b) {
     const uint32_t bytes = (uint32_t)cnt * 16u;
+    // windows: from the 16-byte boundary at or below the node's first to the one past its last
+    const long long w0 = (long long)(k0 + lane) * n_lines + l;
+    const uint32_t wbytes = ADAPT && lane < nk ? (uint32_t)(((int)(w0 & 1) + cnt + 1) >> 1) * 16u : 0u;
+    const uint32_t wall = ADAPT ? __reduce_add_sync(0xffffffffu, wbytes) : 0u;
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     if (lane == 0) {
-      mbar_arrive_expect_tx(&bars[b], bytes * (uint32_t)(nk * (with_p2 ? 2 : 1) + 1));
+      mbar_arrive_expect_tx(&bars[b], bytes * (uint32_t)(nk * (with_p2 ? 2 : 1) + 1) + wall);
       bulk_g2s(&sR[b][0], R + l, bytes, &bars[b]);
     }
     __syncwarp();
     if (lane < nk) {
       bulk_g2s(&sP[b][lane][0], P + (long long)(k0 + lane) * n_lines + l, bytes, &bars[b]);
-      if (with_p2) bulk_g2s(&sP[b][lane][kChunkP2], P2 + (long long)(k0 + lane) * n_lines + l, bytes, &bars[b]);
+      if (ADAPT) bulk_g2s(&sW[b][lane][0], AW + (w0 & ~1LL), wbytes, &bars[b]);
+      if (with_p2) bulk_g2s(&sP[b][lane][kCapP2], P2 + (long long)(k0 + lane) * n_lines + l, bytes, &bars[b]);
     }
   };
 
@@ -617,7 +632,10 @@ k_kappa(const float4 *__restrict__ P, const float4 *__restrict__ P2, const int4 
     bool with_p2;
     cnt = chunk_at(l0, seg, with_p2);
     const int4 *cR = sR[b];
-    const float4 *cP = sP[b][wsel], *cP2 = cP + kChunkP2;
+    const float4 *cP = sP[b][wsel], *cP2 = cP + kCapP2;
+    const int2 *cW = sW[b][ADAPT ? wsel : 0] + (ADAPT ? (((long long)k * n_lines + l0) & 1) : 0);
+    // line i's window: its own at this node, or the cutoff's
+    auto window = [&](int i) -> int2 { return ADAPT ? cW[i] : *reinterpret_cast<const int2 *>(&cR[i].x); };
 
     // the line's value, less the factor p.x for Lorentz lines, at a pair of offsets u (grid
     // units) from its centre; DEG 4 or 1: the far-wing series' degree
@@ -633,18 +651,19 @@ k_kappa(const float4 *__restrict__ P, const float4 *__restrict__ P2, const int4 
       }
       return __fmul2_rn(t, __ffma2_rn(t, c1, c0));
     };
-    // lines [i, i1) at the M tile nodes: M / 2 lanes take a line (two nodes each), the warp
+    // Below, a range's lines are at(0) .. at(n - 1), chunk indices.
+    // run_nodes: at the M tile nodes: M / 2 lanes take a line (two nodes each), the warp
     // 64 / M lines at a time
-    auto run_nodes = [&](auto deg, auto m, const float *un, int i, int i1, float2 &s, float2 &sc) {
+    auto run_nodes = [&](auto deg, auto m, const float *un, auto at, int n, float2 &s, float2 &sc) {
       constexpr int kLanes = decltype(m)::value / 2, kLines = 32 / kLanes;
       const float2 u0 = *reinterpret_cast<const float2 *>(un + 2 * (lane % kLanes));
 #pragma unroll 1
-      for (i += lane / kLanes; __any_sync(0xffffffffu, i < i1); i += kLines * kNodeGroup) {
+      for (int i = lane / kLanes; __any_sync(0xffffffffu, i < n); i += kLines * kNodeGroup) {
         float2 g = make_float2(0.0f, 0.0f);
 #pragma unroll
         for (int e = 0; e < kNodeGroup; ++e) {
-          const bool in = i + e * kLines < i1;
-          const int q = in ? i + e * kLines : i1 - 1;
+          const bool in = i + e * kLines < n;
+          const int q = at(in ? i + e * kLines : n - 1);
           const int2 r = *reinterpret_cast<const int2 *>(&cR[q].z);
           const float2 u = __fadd2_rn(__fadd2_rn(dup2((float)(jw0 - r.x)), u0), dup2(__int_as_float(r.y)));
           const float2 v = far_value(deg, u, cP[q], q);
@@ -654,10 +673,10 @@ k_kappa(const float4 *__restrict__ P, const float4 *__restrict__ P2, const int4 
       }
       nodes = true;
     };
-    // lines [i, i1) whose windows end inside the tile, one after the other: lane (b, m) takes
+    // lines whose windows end inside the tile (on one side), one after the other: lane (b, m) takes
     // node m of sub-block b where the window covers it, and point `lane` of the sub-block the
     // window ends in.  Both sums go to the points before returning.
-    auto run_edge = [&](int i, int i1) {
+    auto run_edge = [&](auto at, int n) {
       float *res = s_res[warp];
       const int sb = lane >> 2, nu_last = (int)(n_nu - 1);
       const float un = 32.0f * (float)sb + kTab4.u[lane & 3];
@@ -670,12 +689,14 @@ k_kappa(const float4 *__restrict__ P, const float4 *__restrict__ P2, const int4 
         s.y = sc.y = 0.0f;
       };
 #pragma unroll 1
-      for (; i < i1; ++i) {
+      for (int q = 0; q < n; ++q) {
+        const int i = at(q);
         const int4 r = cR[i];
+        const int2 win = window(i);
         // covered tile points; a window that holds the grid's last point has no end here
-        const int a = max(r.x - jw0, 0), e = r.y >= nu_last ? kTilePts - 1 : min(r.y - jw0, kTilePts - 1);
+        const int a = max(win.x - jw0, 0), e = win.y >= nu_last ? kTilePts - 1 : min(win.y - jw0, kTilePts - 1);
         const int eb = a == 0 ? (e + 1) >> 5 : a >> 5;                      // sub-block of the end
-        if (eb != cur) {  // warp-uniform; window ends are monotone in the line index
+        if (eb != cur) {  // warp-uniform; cutoff windows' ends are monotone in the line index
           flush();
           cur = eb;
         }
@@ -711,7 +732,8 @@ k_kappa(const float4 *__restrict__ P, const float4 *__restrict__ P2, const int4 
     auto fast_line = [&](auto deg, auto mask, int i, float2 (&g)[kPairs], bool first) {
       constexpr int DEG = decltype(deg)::value;
       constexpr bool MASK = decltype(mask)::value;
-      const int4 r = cR[i];
+      int4 r = cR[i];
+      if (MASK && ADAPT) r.x = cW[i].x, r.y = cW[i].y;
       const float4 p = cP[i];
       const float ul = point_offset(jt, r.z, r.w);
       if (!kVoigt) {
@@ -748,21 +770,22 @@ k_kappa(const float4 *__restrict__ P, const float4 *__restrict__ P2, const int4 
         }
       }
     };
-    auto run_fast = [&](auto deg, auto mask, int i, int i1) {
+    auto run_fast = [&](auto deg, auto mask, auto at, int n) {
+      int i = 0;
 #pragma unroll 1
-      for (; i + kGroup <= i1; i += kGroup) {
+      for (; i + kGroup <= n; i += kGroup) {
         float2 g[kPairs];
-        fast_line(deg, mask, i, g, true);
+        fast_line(deg, mask, at(i), g, true);
 #pragma unroll
-        for (int e = 1; e < kGroup; ++e) fast_line(deg, mask, i + e, g, false);
+        for (int e = 1; e < kGroup; ++e) fast_line(deg, mask, at(i + e), g, false);
 #pragma unroll
         for (int h = 0; h < kPairs; ++h) kahan_add2(acc[h], cmp[h], g[h]);
       }
-      if (i < i1) {
+      if (i < n) {
         float2 g[kPairs];
-        fast_line(deg, mask, i, g, true);
+        fast_line(deg, mask, at(i), g, true);
 #pragma unroll 1
-        for (int e = i + 1; e < i1; ++e) fast_line(deg, mask, e, g, false);
+        for (int e = i + 1; e < n; ++e) fast_line(deg, mask, at(e), g, false);
 #pragma unroll
         for (int h = 0; h < kPairs; ++h) kahan_add2(acc[h], cmp[h], g[h]);
       }
@@ -858,7 +881,7 @@ k_kappa(const float4 *__restrict__ P, const float4 *__restrict__ P2, const int4 
       }
     };
     auto mask_window = [&](int i, float2 (&v)[kPairs]) {
-      const int2 r = *reinterpret_cast<const int2 *>(&cR[i].x);
+      const int2 r = window(i);
       if (r.x > jw0 || r.y < jw1) {  // warp-uniform: the window ends inside this block's points
 #pragma unroll
         for (int h = 0; h < kPairs; ++h) {
@@ -869,11 +892,11 @@ k_kappa(const float4 *__restrict__ P, const float4 *__restrict__ P2, const int4 
     };
     // lines enter the compensated sum in pairs: the sum of two positive line
     // values is rounded once (relative error <= 2^-24 of the pair)
-    auto run_general = [&](int i, int i1) {
+    auto run_general = [&](auto at, int n) {
 #pragma unroll 1
-      for (; i < i1; i += 2) {
-        const bool two = i + 1 < i1;
-        const int j = two ? i + 1 : i;
+      for (int q = 0; q < n; q += 2) {
+        const bool two = q + 1 < n;
+        const int i = at(q), j = two ? at(q + 1) : i;
         int fa = 0, fb = 0, na = 0, nb = 0;
         if (kVoigt) {
           na = core_range(i, fa);
@@ -905,18 +928,65 @@ k_kappa(const float4 *__restrict__ P, const float4 *__restrict__ P2, const int4 
       while (s_end[seg] <= l) ++seg;  // the last segment ends at ub > l
       const int i1 = min(cnt, s_end[seg] - l0);
       const int kd = s_kind[seg];
-      if (kd == kSegNodes8)
-        run_nodes(std::integral_constant<int, 1>(), std::integral_constant<int, 8>(), kTab8.u, i, i1, n8, n8c);
-      else if (kd == kSegNodes16)
-        run_nodes(std::integral_constant<int, 4>(), std::integral_constant<int, 16>(), kTab16.u, i, i1, n16, n16c);
-      else if (kd == kSegEdge)
-        run_edge(i, i1);
-      else if (kd == kSegFast)
-        run_fast(std::integral_constant<int, 4>(), std::false_type(), i, i1);
-      else if (kd == kSegFar1Masked)
-        run_fast(std::integral_constant<int, 1>(), std::true_type(), i, i1);
-      else
-        run_general(i, i1);
+      const std::integral_constant<int, 1> d1;
+      const std::integral_constant<int, 4> d4;
+      const std::integral_constant<int, 8> m8;
+      const std::integral_constant<int, 16> m16;
+      const std::false_type all;
+      const std::true_type masked;
+      if (!ADAPT) {
+        const int n = i1 - i;
+        auto at = [i](int e) { return i + e; };
+        if (kd == kSegNodes8) run_nodes(d1, m8, kTab8.u, at, n, n8, n8c);
+        else if (kd == kSegNodes16) run_nodes(d4, m16, kTab16.u, at, n, n16, n16c);
+        else if (kd == kSegEdge) run_edge(at, n);
+        else if (kd == kSegFast) run_fast(d4, all, at, n);
+        else if (kd == kSegFar1Masked) run_fast(d1, masked, at, n);
+        else run_general(at, n);
+      } else {
+        // a general line goes with the covering ones (its path masks), a degree-1 line far
+        // enough for the sub-blocks' nodes with the window ends, the rest are masked
+        unsigned char *lc = s_list[warp][0], *lp = s_list[warp][1];
+        int nc = 0, ne = 0, nm = 0;
+        const int last = (int)min((long long)jw1, n_nu - 1);
+        for (int q0 = i; q0 < i1; q0 += 32) {
+          const int q = q0 + lane;
+          int to = 0;  // 0 none, 1 covering, 2 window end, 3 masked
+          if (q < i1) {
+            const int2 w = cW[q];
+            const int jc = cR[q].z;
+            if (w.y >= w.x && w.y >= jw0 && w.x <= last) {
+              if (kd == kSegGeneral || (w.x <= jw0 && w.y >= last)) to = 1;
+              else to = degree1_kind(kd) && max(jw0 - jc, jc - jw1) >= kDistEdge ? 2 : 3;
+            }
+          }
+          const unsigned lt = (1u << lane) - 1u;
+          const unsigned c = __ballot_sync(0xffffffffu, to == 1), e = __ballot_sync(0xffffffffu, to == 2),
+                         m = __ballot_sync(0xffffffffu, to == 3);
+          if (to == 1) lc[nc + __popc(c & lt)] = (unsigned char)q;
+          if (to == 2) lp[ne + __popc(e & lt)] = (unsigned char)q;
+          if (to == 3) lp[kCap - 1 - nm - __popc(m & lt)] = (unsigned char)q;
+          nc += __popc(c);
+          ne += __popc(e);
+          nm += __popc(m);
+        }
+        __syncwarp();
+        auto cover = [lc](int e) { return (int)lc[e]; };
+        auto ends = [lp](int e) { return (int)lp[e]; };
+        auto rest = [lp](int e) { return (int)lp[kCap - 1 - e]; };
+        if (kd == kSegGeneral) {
+          run_general(cover, nc);
+        } else if (degree1_kind(kd)) {
+          if (nc > 0) run_nodes(d1, m8, kTab8.u, cover, nc, n8, n8c);
+          if (ne > 0) run_edge(ends, ne);
+          run_fast(d1, masked, rest, nm);
+        } else {
+          if (kd == kSegFast) run_fast(d4, all, cover, nc);
+          else if (nc > 0) run_nodes(d4, m16, kTab16.u, cover, nc, n16, n16c);
+          run_fast(d4, masked, rest, nm);
+        }
+        __syncwarp();  // the lists are the next range's
+      }
       i = i1;
     }
     // every warp is done with buffer b (the waits above order each thread's own reads)
@@ -1093,131 +1163,99 @@ struct AdaptParams {
   int nT;
 };
 
-__global__ void k_adaptive_windows(const double *__restrict__ nu0, const double *__restrict__ S,
-                                   const double *__restrict__ g, const double *__restrict__ E, AdaptParams P,
-                                   int2 *__restrict__ AW, unsigned long long *evals) {
-  const long long l = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  const int k = blockIdx.y;
+__device__ __noinline__ int2 adaptive_window64(double v, double S, double g, double E, const AdaptParams &P, int k) {
+  const double T = P.nT > 1 ? P.T_min + (double)k * ((P.T_max - P.T_min) / (double)(P.nT - 1)) : P.T_min;
+  const double q = pow(P.T_ref / T, P.q_exp);
+  const double boltz = exp(-P.c2 * E / T) / exp(-P.c2 * E / P.T_ref);
+  const double stim = (-expm1(-P.c2 * v / T)) / (-expm1(-P.c2 * v / P.T_ref));
+  const double ST = S * q * boltz * stim;
+  const double A = P.x_ref * P.p_ref * kAtm / (kKB * T) * 1e-6 * ST;
+  const double gam = g * P.p_ref * pow(P.T_ref / T, P.n_T);
+  double w = sqrt(A * gam / (kPi * P.kappa_min));
+  if (!(w <= P.cutoff)) w = P.cutoff;
+  double flo = floor((v - w - P.nu_min) / P.dnu) - 1.0;
+  double fhi = ceil((v + w - P.nu_min) / P.dnu) + 1.0;
+  flo = fmin(fmax(isfinite(flo) ? flo : 0.0, -1.0), (double)P.n_nu + 1.0);
+  fhi = fmin(fmax(isfinite(fhi) ? fhi : 0.0, -2.0), (double)P.n_nu + 1.0);
+  long long lo = (long long)flo, hi = (long long)fhi;
+  if (lo < 0) lo = 0;
+  if (hi > P.n_nu - 1) hi = P.n_nu - 1;
+#pragma unroll 1
+  for (int it = 0; it < 6 && lo < P.n_nu; ++it)
+    if (__dsub_rn(grid_nu(P.nu_min, lo, P.dnu), v) < -w) ++lo;
+#pragma unroll 1
+  for (int it = 0; it < 6 && hi >= 0; ++it)
+    if (__dsub_rn(grid_nu(P.nu_min, hi, P.dnu), v) > w) --hi;
+  return make_int2((int)lo, (int)hi);
+}
+
+// Windows of 256 lines at kWinNodes nodes per block, after k_prefactor.  The binary32
+// coefficients give the half-width in grid units, sqrt(c0 / kappa_min) / (s dnu) for Voigt and
+// sqrt(P.x / kappa_min) for Lorentz lines, to a relative error below kWinTol (half that of
+// A gamma: two roundings of expf, four of powf each for q and gamma, a dozen others, 2e-6 in
+// all).  An end further than that from any grid point's edge, and a half-width further than
+// that from the cutoff, is decided already (a window at the cutoff is the line's cutoff
+// window); the others, about 2 % of the pairs, are queued and decided in binary64 as
+// stated.  The binary64 form for every pair took 1060 us for 64 nodes x 20k lines, this 54 us.
+constexpr int kWinNodes = 8;
+constexpr float kWinTol = 4e-6f;
+struct WinParams {
+  float inv_kmin, cut_grid, tol;  // 1 / kappa_min, cutoff in grid units, relative tolerance
+  float min_w2;                   // half-widths^2 above min_w2 gamma_ref: S(T) is above 1e-36
+  double min_S;                   // intensities whose product with the partition ratio is
+};
+template <int PROFILE>
+__global__ void __launch_bounds__(256)
+k_adaptive_windows(const double *__restrict__ nu0, const double *__restrict__ S, const double *__restrict__ g,
+                   const double *__restrict__ E, AdaptParams P, const float4 *__restrict__ coef,
+                   const int4 *__restrict__ R, WinParams Q, int2 *__restrict__ AW,
+                   unsigned long long *evals) {
+  __shared__ unsigned short s_queue[256 * kWinNodes];
+  __shared__ int s_n;
+  const long long l = (long long)blockIdx.x * 256 + threadIdx.x;
+  const int k0 = blockIdx.y * kWinNodes, k1 = min(k0 + kWinNodes, P.nT);
+  if (threadIdx.x == 0) s_n = 0;
+  __syncthreads();
   unsigned long long cnt = 0;
   if (l < P.n_lines) {
-    const double T = P.nT > 1 ? P.T_min + (double)k * ((P.T_max - P.T_min) / (double)(P.nT - 1)) : P.T_min;
-    const double v = nu0[l];
-    const double q = pow(P.T_ref / T, P.q_exp);
-    const double boltz = exp(-P.c2 * E[l] / T) / exp(-P.c2 * E[l] / P.T_ref);
-    const double stim = (-expm1(-P.c2 * v / T)) / (-expm1(-P.c2 * v / P.T_ref));
-    const double ST = S[l] * q * boltz * stim;
-    const double A = P.x_ref * P.p_ref * kAtm / (kKB * T) * 1e-6 * ST;
-    const double gam = g[l] * P.p_ref * pow(P.T_ref / T, P.n_T);
-    double w = sqrt(A * gam / (kPi * P.kappa_min));
-    if (!(w <= P.cutoff)) w = P.cutoff;
-    double flo = floor((v - w - P.nu_min) / P.dnu) - 1.0;
-    double fhi = ceil((v + w - P.nu_min) / P.dnu) + 1.0;
-    flo = fmin(fmax(isfinite(flo) ? flo : 0.0, -1.0), (double)P.n_nu + 1.0);
-    fhi = fmin(fmax(isfinite(fhi) ? fhi : 0.0, -2.0), (double)P.n_nu + 1.0);
-    long long lo = (long long)flo, hi = (long long)fhi;
-    if (lo < 0) lo = 0;
-    if (hi > P.n_nu - 1) hi = P.n_nu - 1;
-#pragma unroll 1
-    for (int it = 0; it < 6 && lo < P.n_nu; ++it)
-      if (__dsub_rn(grid_nu(P.nu_min, lo, P.dnu), v) < -w) ++lo;
-#pragma unroll 1
-    for (int it = 0; it < 6 && hi >= 0; ++it)
-      if (__dsub_rn(grid_nu(P.nu_min, hi, P.dnu), v) > w) --hi;
-    AW[(long long)k * P.n_lines + l] = make_int2((int)lo, (int)hi);
-    if (hi >= lo) cnt = (unsigned long long)(hi - lo + 1);
+    const int4 r = R[l];
+    const float dg = __int_as_float(r.w);
+    const bool plain = S[l] > Q.min_S;  // no binary32 underflow on the way to the coefficients
+    const float w2_min = Q.min_w2 * __double2float_ru(g[l]);
+    for (int k = k0; k < k1; ++k) {
+      const float4 c = __ldg(coef + (long long)k * P.n_lines + l);
+      const float w = PROFILE == RT_PROFILE_LORENTZ ? sqrtf(c.x * Q.inv_kmin) : sqrtf(c.x * Q.inv_kmin) / c.y;
+      const float tol = __fmaf_rn(Q.tol, w, 1e-6f);
+      int2 win = make_int2(r.x, r.y);
+      const bool known = plain && c.x > 1e-30f && w * w > w2_min && w < 1e18f;
+      bool sure = known && w - tol > Q.cut_grid;
+      if (known && w + tol < Q.cut_grid && w < 1e6f) {
+        // points j with |j - j_c + dg| <= w
+        const float a = -w - dg, b = w - dg;
+        const float ca = ceilf(a), fb = floorf(b);
+        sure = ca - a > tol && a - (ca - 1.0f) > tol && b - fb > tol && fb + 1.0f - b > tol;
+        win.x = max(r.z + (int)ca, 0);
+        win.y = (int)min((long long)r.z + (long long)fb, P.n_nu - 1);
+      }
+      if (sure) {
+        AW[(long long)k * P.n_lines + l] = win;
+        if (win.y >= win.x) cnt += (unsigned long long)(win.y - win.x + 1);
+      } else {
+        s_queue[atomicAdd(&s_n, 1)] = (unsigned short)((k - k0) * 256 + threadIdx.x);
+      }
+    }
+  }
+  __syncthreads();
+  for (int q = threadIdx.x; q < s_n; q += 256) {
+    const int k = k0 + (s_queue[q] >> 8);
+    const long long m = (long long)blockIdx.x * 256 + (s_queue[q] & 255);
+    const int2 win = adaptive_window64(nu0[m], S[m], g[m], E[m], P, k);
+    AW[(long long)k * P.n_lines + m] = win;
+    if (win.y >= win.x) cnt += (unsigned long long)(win.y - win.x + 1);
   }
   if (evals) {
     for (int o = 16; o > 0; o >>= 1) cnt += __shfl_down_sync(0xffffffffu, cnt, o);
     if ((threadIdx.x & 31) == 0 && cnt) atomicAdd(evals, cnt);
-  }
-}
-
-// The line sum with adaptive windows: a block per (256-point tile, T node).  The lines
-// whose cutoff windows touch the tile are a contiguous index range; the block takes it
-// in chunks of 256 lines, keeps (ballot compaction, in ascending nu0) those whose
-// adaptive window at this node meets the tile, and each point then sums the kept
-// lines whose window holds it (Kahan, ascending nu0).  A kept line can be far from
-// the point (strong lines keep the whole cutoff window), so values take the full-range
-// form: the Lorentz reciprocal, or the Faddeeva function in all its regions.
-template <int PROFILE>
-__global__ void __launch_bounds__(kTilePts)
-k_kappa_adaptive(const float4 *__restrict__ P, const int4 *__restrict__ R, const int2 *__restrict__ AW,
-                 long long n_lines, long long n_nu, WeidCoef wc, int accumulate, float *__restrict__ kappa) {
-  __shared__ long long s_range[2];
-  __shared__ int2 s_win[kTilePts];     // kept lines' windows at this node
-  __shared__ float4 s_par[kTilePts];   // their {centre index bits, centre offset, coefficient, g^2 or y}
-  __shared__ float s_sd[kTilePts];     // Voigt: s dnu (grid units to x)
-  __shared__ int s_warp[kTilePts / 32];
-  const long long jw0 = (long long)blockIdx.x * kTilePts;
-  const long long jend = min(jw0 + (long long)kTilePts, n_nu);
-  const int k = blockIdx.y;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (threadIdx.x == 0) s_range[0] = lower_bound_hi(R, n_lines, (int)jw0);
-  if (threadIdx.x == 1) s_range[1] = lower_bound_lo(R, n_lines, (int)jend);
-  __syncthreads();
-  const long long a = s_range[0], b = max(s_range[0], s_range[1]);
-  const long long j = jw0 + threadIdx.x;
-  const float4 *Pk = P + (long long)k * n_lines;
-  const int2 *Wk = AW + (long long)k * n_lines;
-  float acc = 0.0f, cmp = 0.0f;
-#pragma unroll 1
-  for (long long c0 = a; c0 < b; c0 += kTilePts) {
-    const long long l = c0 + threadIdx.x;
-    int2 w = make_int2(1, 0);
-    bool keep = false;
-    if (l < b) {
-      w = __ldg(Wk + l);
-      keep = w.y >= w.x && w.y >= (int)jw0 && (long long)w.x < jend;
-    }
-    const unsigned m = __ballot_sync(0xffffffffu, keep);
-    if (lane == 0) s_warp[warp] = __popc(m);
-    __syncthreads();
-    int off = 0, total = 0;
-#pragma unroll
-    for (int q = 0; q < kTilePts / 32; ++q) {
-      const int c = s_warp[q];
-      off += q < warp ? c : 0;
-      total += c;
-    }
-    if (keep) {  // the kept line's constants, formed once for all the tile's points
-      const int pos = off + __popc(m & ((1u << lane) - 1u));
-      const int4 r = __ldg(R + l);
-      const float4 p = __ldg(Pk + l);
-      s_win[pos] = w;
-      if (PROFILE == RT_PROFILE_LORENTZ) {
-        s_par[pos] = make_float4(__int_as_float(r.z), __int_as_float(r.w), p.x, p.y);
-      } else {
-        const float y = sqrtf(p.z);
-        s_par[pos] = make_float4(__int_as_float(r.z), __int_as_float(r.w), __fdividef(p.x, y), y);
-        s_sd[pos] = p.y;
-      }
-    }
-    __syncthreads();
-    if (j < jend) {
-#pragma unroll 1
-      for (int i = 0; i < total; ++i) {
-        const int2 ww = s_win[i];
-        if ((int)j < ww.x || (int)j > ww.y) continue;
-        const float4 q = s_par[i];
-        const float u = __fadd_rn((float)((int)j - __float_as_int(q.x)), q.y);
-        float v;
-        if (PROFILE == RT_PROFILE_LORENTZ) {
-          v = q.z * rcp_approx(__fmaf_rn(u, u, q.w));
-        } else {
-          v = q.z * faddeeva_re(s_sd[i] * u, q.w, wc);
-        }
-        const float yk = __fsub_rn(v, cmp);
-        const float t = __fadd_rn(acc, yk);
-        cmp = __fsub_rn(__fsub_rn(t, acc), yk);
-        acc = t;
-      }
-    }
-    __syncthreads();  // the kept list is rewritten by the next chunk
-  }
-  if (j < jend) {
-    float *dst = kappa + (long long)k * n_nu + j;
-    const float out = __fsub_rn(acc, cmp);
-    *dst = accumulate ? *dst + out : out;
   }
 }
 
@@ -1230,18 +1268,6 @@ rt_status launch_kappa(const float4 *P, const float4 *P2, const int4 *R, int4 *t
   static WeidCoef wc;
   static std::once_flag wc_once;
   std::call_once(wc_once, [] { weideman_coefficients(&wc); });
-  const long long n_tiles_a = (spec->n_nu + kTilePts - 1) / kTilePts;
-  if (AW) {  // adaptive points per line: the windows' gather kernel
-    dim3 g((unsigned)n_tiles_a, (unsigned)spec->nT);
-    if (spec->profile == RT_PROFILE_LORENTZ)
-      k_kappa_adaptive<RT_PROFILE_LORENTZ><<<g, kTilePts, 0, st>>>(P, R, AW, n, spec->n_nu, wc,
-                                                                   spec->accumulate ? 1 : 0, kappa);
-    else
-      k_kappa_adaptive<RT_PROFILE_VOIGT><<<g, kTilePts, 0, st>>>(P, R, AW, n, spec->n_nu, wc,
-                                                                 spec->accumulate ? 1 : 0, kappa);
-    RT_CUDA_TRY(cudaGetLastError());
-    return RT_OK;
-  }
   // W bounds every line's near-centre half-width sqrt(400 - y^2) / (s dnu) <= 20 alpha /
   // (sqrt(ln 2) dnu), alpha the largest Doppler half-width of a line that reaches the grid
   int W = 0;
@@ -1271,8 +1297,10 @@ rt_status launch_kappa(const float4 *P, const float4 *P2, const int4 *R, int4 *t
   if (want < 1 || want > kMaxTPerBlock) want = kMaxTPerBlock;
   const int tpb = spec->nT < want ? spec->nT : want;
   dim3 gk((unsigned)n_tiles, (unsigned)((spec->nT + tpb - 1) / tpb));
-  auto kernel = spec->profile == RT_PROFILE_LORENTZ ? k_kappa<RT_PROFILE_LORENTZ> : k_kappa<RT_PROFILE_VOIGT>;
-  kernel<<<gk, 32 * tpb, 0, st>>>(P, P2, R, tiles, n, spec->n_nu, spec->nT, wc, vec_ok,
+  auto kernel = spec->profile == RT_PROFILE_LORENTZ
+                    ? (AW ? k_kappa<RT_PROFILE_LORENTZ, true> : k_kappa<RT_PROFILE_LORENTZ, false>)
+                    : (AW ? k_kappa<RT_PROFILE_VOIGT, true> : k_kappa<RT_PROFILE_VOIGT, false>);
+  kernel<<<gk, 32 * tpb, 0, st>>>(P, P2, R, AW, tiles, n, spec->n_nu, spec->nT, wc, vec_ok,
                                   spec->accumulate ? 1 : 0, kappa, status);
   RT_CUDA_TRY(cudaGetLastError());
   return RT_OK;
@@ -1406,17 +1434,6 @@ rt_status run_build(char *base, const KappaLayout &L, const rt_lines *lines, con
   k_line_geometry<<<(unsigned)((n + tb - 1) / tb), tb, 0, st>>>(d_nu0, d_S, d_g, d_E, G, R,
                                                                 adaptive ? nullptr : evals_out, status);
   RT_CUDA_TRY(cudaGetLastError());
-  int2 *AW = nullptr;
-  if (adaptive) {
-    AW = reinterpret_cast<int2 *>(base + L.off_AW);
-    AdaptParams A{spec->nu_min, spec->dnu, spec->cutoff, spec->T_min, spec->T_max, lines->T_ref,
-                  100.0 * (kH * kC / kKB), spec->x_ref, spec->p_ref_atm, lines->n_T, lines->q_exp,
-                  spec->kappa_min, spec->n_nu, n, spec->nT};
-    dim3 ga((unsigned)((n + tb - 1) / tb), (unsigned)spec->nT);
-    k_adaptive_windows<<<ga, tb, 0, st>>>(d_nu0, d_S, d_g, d_E, A, AW, evals_out);
-    RT_CUDA_TRY(cudaGetLastError());
-  }
-
   PrefParams Q;
   Q.T_min = spec->T_min;
   Q.T_max = spec->T_max;
@@ -1438,6 +1455,31 @@ rt_status run_build(char *base, const KappaLayout &L, const rt_lines *lines, con
   RT_CUDA_TRY(cudaMemsetAsync(far_bits, 0, sizeof(unsigned), st));
   k_prefactor<<<gp, tb, 0, st>>>(d_nu0, d_S, d_g, d_E, Q, P, P2, far_bits);
   RT_CUDA_TRY(cudaGetLastError());
+
+  int2 *AW = nullptr;
+  if (adaptive) {
+    AW = reinterpret_cast<int2 *>(base + L.off_AW);
+    AdaptParams A{spec->nu_min, spec->dnu, spec->cutoff, spec->T_min, spec->T_max, lines->T_ref,
+                  100.0 * (kH * kC / kKB), spec->x_ref, spec->p_ref_atm, lines->n_T, lines->q_exp,
+                  spec->kappa_min, spec->n_nu, n, spec->nT};
+    dim3 ga((unsigned)((n + tb - 1) / tb), (unsigned)((spec->nT + kWinNodes - 1) / kWinNodes));
+    auto windows = spec->profile == RT_PROFILE_LORENTZ ? k_adaptive_windows<RT_PROFILE_LORENTZ>
+                                                       : k_adaptive_windows<RT_PROFILE_VOIGT>;
+    // gamma <= gamma_ref p G and u <= u_max over the nodes; A gamma / pi = kappa_min (w dnu)^2
+    const double ra = lines->T_ref / spec->T_min, rb = lines->T_ref / spec->T_max;
+    const double G = std::fmax(std::pow(ra, lines->n_T), std::pow(rb, lines->n_T)) * spec->p_ref_atm;
+    const double qmin = std::fmin(std::pow(ra, lines->q_exp), std::pow(rb, lines->q_exp));
+    const double u_max = spec->x_ref * spec->p_ref_atm * kAtm / (kKB * spec->T_min) * 1e-6;
+    WinParams wp;
+    wp.inv_kmin = (float)(1.0 / spec->kappa_min);
+    wp.cut_grid = (float)(spec->cutoff / spec->dnu);
+    // the ratio T_ref / T carries 2^-23 into its powers
+    wp.tol = kWinTol + 2e-7f * (float)(std::fabs(lines->q_exp) + std::fabs(lines->n_T));
+    wp.min_w2 = (float)(1e-36 * u_max * G / (kPi * spec->dnu * spec->dnu * spec->kappa_min));
+    wp.min_S = 1e-36 / std::fmin(qmin, 1.0);
+    windows<<<ga, tb, 0, st>>>(d_nu0, d_S, d_g, d_E, A, P, R, wp, AW, evals_out);
+    RT_CUDA_TRY(cudaGetLastError());
+  }
 
   // largest |nu0| of a line whose window (cutoff or fixed points) reaches the grid
   const double reach = spec->cutoff + (spec->points_per_line + 2.0) * spec->dnu;

@@ -64,3 +64,31 @@ def test_many_lines_per_tile(rt):
     lines.nu0[1000:1400] = lines.nu0[1000]
     spec = synth.Spectral(nu_min=2000.0, dnu=0.004, n_nu=520, cutoff=9.0, profile="voigt", nT=1, T_min=600.0, T_max=600.0)
     _check(rt, lines, spec)
+
+
+# Windows per line and node: odd and even line counts and nodes (the windows' copies are
+# aligned to pairs), thresholds from keeping everything to next to nothing, intensities and
+# partition exponents that leave the binary32 estimate's range.  The evaluation counts are
+# integers and equal.
+@pytest.mark.parametrize("n,nT,kappa_min,profile,S,q_exp", [
+    (301, 1, 1e-2, "voigt", 1e-20, 1.0), (300, 9, 1.0, "voigt", 1e-20, 1.0), (77, 3, 1e-6, "lorentz", 1e-20, 1.0),
+    (301, 8, 30.0, "lorentz", 1e-19, 1.0), (128, 2, 1e-24, "voigt", 1e-40, 1.0), (65, 2, 1e-3, "voigt", 1e-20, 30.0),
+    (1, 1, 1e-1, "voigt", 1e-20, 1.0)])
+def test_adaptive_windows_match_oracle(rt, n, nT, kappa_min, profile, S, q_exp):
+    import torch
+    rng = synth.rng_for(34, n)
+    lines = synth.make_lines(n, 1995.0, 2035.0, rng, S_lo=S, S_hi=30.0 * S)
+    lines.q_exp = q_exp
+    spec = synth.Spectral(nu_min=2000.0, dnu=0.01, n_nu=3001, cutoff=20.0, profile=profile, nT=nT, T_min=400.0,
+                          T_max=400.0 if nT == 1 else 900.0, kappa_min=kappa_min)
+    ev = torch.zeros(1, dtype=torch.int64, device="cuda")
+    got = rt.build_kappa(lines, spec, evals=ev).cpu().numpy().astype(np.float64)
+    ref = okappa.kappa_table(lines, spec)
+    assert int(ev) == okappa.profile_evals(lines, spec)
+    if S < 1e-38:
+        return  # the values themselves are below binary32's range there
+    assert np.array_equal(got > 0, ref > 0)
+    nz = ref > 0
+    assert nz.any()
+    # an exponent of 30 multiplies the rounding of T_ref / T, 1.2e-7, into the ratio
+    assert (np.abs(got[nz] - ref[nz]) / ref[nz]).max() <= (TOL if q_exp == 1.0 else 4.0 * TOL)
