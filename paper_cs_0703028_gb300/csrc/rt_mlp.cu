@@ -13,6 +13,8 @@
 //   k_grad_adam : the gradient, the tiles' partials summed in tile order, and
 //                the Adam update of the FP32 masters (Kingma and Ba); within a
 //                run of steps also the next step's BF16 tiles.
+//   k_mlp_fused : a run of training steps whose batch is one 128-row tile, all three
+//                in one kernel, a network per block.
 //   k_walk_mlp : the Monte-Carlo walk with the network in place of the table
 //                (three 128-ray tiles per block; every layer, biases included,
 //                on the tensor cores).
@@ -114,6 +116,18 @@ __device__ __forceinline__ void stage_small(SmallParams &S, const float *__restr
     S.w5[c] = P[oW5 + c];
   }
   if (threadIdx.x == 0) S.b5 = P[oB5];
+}
+
+// moments of the same parameters, in the order kSmallW1 .. kSmallB5
+constexpr int kSmallW1 = 0, kSmallB1 = 4 * kH, kSmallB = 5 * kH, kSmallW5 = 8 * kH, kSmallB5 = 9 * kH, kSmall = 9 * kH + 1;
+__device__ __forceinline__ int small_index(int i) {  // the i-th small parameter's place in the vector
+  return i < kSmallB ? i : (i < kSmallB + kH ? i - kSmallB + oB2
+                            : (i < kSmallB + 2 * kH ? i - kSmallB - kH + oB3
+                               : (i < kSmallW5 ? i - kSmallB - 2 * kH + oB4 : i - kSmallW5 + oW5)));
+}
+static_assert(oB1 == kSmallB1 && oB5 == oW5 + kH, "small_index follows the parameter layout");
+__device__ __forceinline__ void stage_moments(float *s, const float *__restrict__ g) {
+  for (int i = threadIdx.x; i < kSmall; i += blockDim.x) s[i] = g[small_index(i)];
 }
 
 __device__ __forceinline__ float layer1(const SmallParams &S, int c, const float (&u)[4]) {
@@ -627,6 +641,443 @@ k_grad_adam(const float *__restrict__ part, int nparts, float *__restrict__ grad
     const float pi = pv[q] - lr * (mi / c1) / (sqrtf(vi / c2) + eps);
     P[i] = pi;
     if (tiles) adam_tile_write(tiles, i, pi);
+  }
+}
+
+// ---------------------------------------------------------------- fused training steps
+// A run of steps of an ensemble whose batch is one 128-sample tile: a block trains one network
+// at a time through all the launch's steps, forward, backward and Adam in one kernel, so that
+//  - the pre-activations stay in tensor memory (Z2..Z4, 384 columns, raw accumulators; z1 is
+//    recomputed from the four inputs), the gradients go from tensor memory straight into Adam,
+//    and the BF16 weight tiles stay in shared memory (dZ W reads the forward tile MN-major, so
+//    there are no transposed tiles): of the per-step traffic of the separate kernels (Z 0.26 MB
+//    written and read 3 times, partials 0.2 MB twice, tiles 0.2 MB three times) only the masters
+//    and moments are left, 0.6 MB read and 0.6 MB written;
+//  - those stay in L2 from step to step (0.6 MB of one network per SM, 92 MB in all).
+// 8 steps of 1024 networks x 128 samples: 5.09 -> 2.26 ms (the separate kernels spent 0.32 ms on
+// the tiles and 0.075 + 0.22 + 0.286 ms a step on forward, backward and Adam); one network
+// 60 -> 36 us a step. Of a step's 33 us per network and SM the products take 3, the
+// elementwise passes and barriers between them 14, Adam 13; issue (16 warps an SM) and the latency
+// of Adam's loads bound it.
+// Every value is formed by the same operations in the same order as in k_mlp_fwd, k_mlp_bwd
+// and k_grad_adam, so the parameters are bitwise those of the separate kernels.
+// The weight gradient is taken transposed (rows = input unit), so that a warp's 32 lanes hold
+// 32 consecutive parameters of a row of W.  512 threads: warp w has row quarter w mod 4 and
+// column quarter w / 4.
+constexpr int kFusedThreads = 4 * kH;
+constexpr int kFusedSteps = 240;  // steps per launch (their Adam constants are kernel parameters)
+
+struct StepConsts {
+  int n_steps;
+  long long first;           // 0-based number of the first step
+  float lr[kFusedSteps], c1[kFusedSteps], c2[kFusedSteps];
+};
+
+struct FusedSmem {
+  uint16_t W[3][kTileElems];  // W2..W4, rows = out
+  uint16_t H[kTileElems];     // the current layer's input, rows = samples
+  uint16_t dZ[kTileElems];    // rows = samples, k = out
+  SmallParams sp[2];          // this step's and the next step's
+  float sm[kSmall], sv[kSmall];  // their moments: the small parameters live here during a launch
+  float colred[5][4][kH];     // as in BwdSmem
+  float yp[2][kH], yh[kH], dy[kH];
+  float dyred[4], red[4];
+  uint64_t bar;
+  uint32_t tmem;
+};
+static_assert(sizeof(FusedSmem) <= 227 * 1024, "fused training shared memory exceeds 227 KB per block");
+
+// Paired binary32 (f32x2) forms of the elementwise steps: each half rounds as the scalar
+// operation, half the instructions.
+__device__ __forceinline__ float2 dup2(float a) { return make_float2(a, a); }
+__device__ __forceinline__ float2 sigmoid2(float2 z) {
+  const float2 h = __fmul2_rn(dup2(0.5f), z);
+  return __ffma2_rn(dup2(0.5f), make_float2(tanh_approx(h.x), tanh_approx(h.y)), dup2(0.5f));
+}
+// silu'(z) = s (1 + z (1 - s)), s = sigmoid(z)
+__device__ __forceinline__ float2 silu_grad2(float2 z, float2 s) {
+  return __fmul2_rn(s, __ffma2_rn(z, __fadd2_rn(dup2(1.0f), make_float2(-s.x, -s.y)), dup2(1.0f)));
+}
+__device__ __forceinline__ uint32_t pack2(float2 a) {  // {a.x low, a.y high}
+  const __nv_bfloat162 b = __floats2bfloat162_rn(a.x, a.y);
+  return *reinterpret_cast<const uint32_t *>(&b);
+}
+// elements (r, k0 .. k0 + 7) of a K-major tile
+__device__ __forceinline__ void put_pairs(uint16_t *tile, int r, int k0, const float2 *v) {
+  *reinterpret_cast<uint4 *>(&tile[tile_index(r, k0)]) = make_uint4(pack2(v[0]), pack2(v[1]), pack2(v[2]), pack2(v[3]));
+}
+// z = acc + bias for N units from 16-byte aligned biases
+template <int N>
+__device__ __forceinline__ void add_bias(float2 (&z)[N / 2], const float (&acc)[N], const float *bias) {
+#pragma unroll
+  for (int i = 0; i < N; i += 4) {
+    const float4 b = *reinterpret_cast<const float4 *>(bias + i);
+    z[i / 2] = __fadd2_rn(make_float2(acc[i], acc[i + 1]), make_float2(b.x, b.y));
+    z[i / 2 + 1] = __fadd2_rn(make_float2(acc[i + 2], acc[i + 3]), make_float2(b.z, b.w));
+  }
+}
+__device__ __forceinline__ float2 layer1_pair(const SmallParams &S, int c, const float (&u)[4]) {
+  return make_float2(layer1(S, c, u), layer1(S, c + 1, u));
+}
+__device__ __forceinline__ float column_sum(const float2 (&v)[8], int lane) {
+  float w[16];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    w[2 * i] = v[i].x;
+    w[2 * i + 1] = v[i].y;
+  }
+  return warp_column_sum16(w, lane);
+}
+
+// the Adam update of k_grad_adam; a bias correction of exactly 1 needs no division
+__device__ __forceinline__ float2 adam_update2(float2 g, float2 p, float2 &m, float2 &v, float lr, float c1, float c2) {
+  constexpr float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
+  m = __ffma2_rn(dup2(b1), m, __fmul2_rn(dup2(1.0f - b1), g));
+  v = __ffma2_rn(dup2(b2), v, __fmul2_rn(__fmul2_rn(dup2(1.0f - b2), g), g));
+  const float2 mh = c1 == 1.0f ? m : make_float2(m.x / c1, m.y / c1);
+  const float2 vh = c2 == 1.0f ? v : make_float2(v.x / c2, v.y / c2);
+  const float2 num = __fmul2_rn(dup2(lr), mh), den = __fadd2_rn(make_float2(sqrtf(vh.x), sqrtf(vh.y)), dup2(eps));
+  return __fadd2_rn(p, make_float2(-(num.x / den.x), -(num.y / den.y)));
+}
+__device__ __forceinline__ float adam_update(float g, float p, float &m, float &v, float lr, float c1, float c2) {
+  float2 mm = make_float2(m, 0.0f), vv = make_float2(v, 1.0f);
+  const float r = adam_update2(make_float2(g, 0.0f), make_float2(p, 0.0f), mm, vv, lr, c1, c2).x;
+  m = mm.x;
+  v = vv.x;
+  return r;
+}
+
+__global__ void __launch_bounds__(kFusedThreads, 1)
+k_mlp_fused(float *__restrict__ P, float *__restrict__ M, float *__restrict__ V, float *__restrict__ grad, Norm N1,
+            const Norm *__restrict__ norms, const float *__restrict__ inputs, const float *__restrict__ targets,
+            int n, long long in_stride, long long n_batches, int n_nets, __grid_constant__ const StepConsts C,
+            int store_grad, float *__restrict__ loss, int loss_stride, float loss_scale, uint32_t *status) {
+  extern __shared__ __align__(1024) unsigned char smem_raw[];
+  FusedSmem &S = *reinterpret_cast<FusedSmem *>(smem_raw);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int q4 = warp & 3, r = q4 * 32 + lane;  // sample row (activations) or input unit (gradients)
+  const int cq = warp >> 2, cb = cq * 32;       // column quarter
+  const uint32_t lanes = (uint32_t)(q4 * 32) << 16;
+  const bool valid = r < n;
+  if (tid == 0) {
+    tc::mbar_init(&S.bar, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 0) tc::tmem_alloc(&S.tmem, 512);
+  tc::fence_before_sync();
+  __syncthreads();
+  tc::fence_after_sync();
+  const uint32_t tmem = S.tmem;
+  const uint32_t tZ[3] = {tmem, tmem + 128, tmem + 256}, tX = tmem + 384;
+  uint32_t phase = 0;
+  int pending = 0;  // block-uniform: a product's wait gave up
+  // all threads: the committed products are complete (false: a bounded wait ran out)
+  auto wait_products = [&]() -> bool {
+    const int late = tc::mbar_wait(&S.bar, phase, kWaitLimit) ? 0 : 1;
+    phase ^= 1u;
+    if (__syncthreads_or(late)) {
+      pending = 1;
+      return false;
+    }
+    tc::fence_after_sync();
+    return true;
+  };
+  // all threads: what they wrote to shared memory and read from tensor memory is ordered
+  // before thread 0's next products
+  auto ready = [&]() {
+    tc::fence_smem_to_async();
+    tc::fence_before_sync();
+    __syncthreads();
+  };
+  // small parameter q (kSmall order) with value p: its gradient, four row-quarter partials in
+  // order, and the Adam update; returns the new value
+  auto small_adam = [&](int set, int i, int q, float p, float *GN, float lr, float c1, float c2) -> float {
+    const float gi = S.colred[set][0][i] + S.colred[set][1][i] + S.colred[set][2][i] + S.colred[set][3][i];
+    if (GN) GN[small_index(q)] = gi;
+    return adam_update(gi, p, S.sm[q], S.sv[q], lr, c1, c2);
+  };
+
+#pragma unroll 1
+  for (int net = blockIdx.x; net < n_nets && !pending; net += gridDim.x) {
+    const Norm N = net_norm(norms, N1, net);
+    float *PN = P + (long long)net * kNParam, *MN = M + (long long)net * kNParam, *VN = V + (long long)net * kNParam;
+    // the network's weights into BF16 tiles (rows of 128 consecutive parameters: coalesced)
+#pragma unroll 1
+    for (int l = 0; l < 3; ++l) {
+      const float *w = PN + (l == 0 ? oW2 : (l == 1 ? oW3 : oW4)) + tid;
+#pragma unroll
+      for (int i0 = 0; i0 < kTileElems; i0 += 16 * kFusedThreads) {
+        float v[16];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) v[i] = w[i0 + i * kFusedThreads];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) put_bf16(S.W[l], (i0 + i * kFusedThreads + tid) / kH, tid % kH, v[i]);
+      }
+    }
+    stage_small(S.sp[0], PN);
+    stage_moments(S.sm, MN);
+    stage_moments(S.sv, VN);
+    __syncthreads();
+#pragma unroll 1
+    for (int it = 0; it < C.n_steps; ++it) {
+      SmallParams &sp = S.sp[it & 1], &spn = S.sp[(it + 1) & 1];
+      const float lr = C.lr[it], c1 = C.c1[it], c2 = C.c2[it];
+      float *GN = store_grad && it == C.n_steps - 1 ? grad + (long long)net * kNParam : nullptr;
+      const long long row0 = net * in_stride + ((C.first + it) % n_batches) * n;
+      float u[4];
+      normalise(inputs + 4 * row0, r, valid, N, u);
+      // ---- forward
+#pragma unroll 1
+      for (int c0 = cb; c0 < cb + 32; c0 += 8) {
+        float2 h[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const float2 z = layer1_pair(sp, c0 + 2 * i, u);
+          h[i] = __fmul2_rn(z, sigmoid2(z));
+        }
+        put_pairs(S.H, r, c0, h);
+      }
+      float2 h4[16];
+#pragma unroll 1
+      for (int l = 0; l < 3; ++l) {
+        ready();
+        if (tid == 0) {
+          tc::fence_after_sync();
+          tc::mma_128x128x128(tZ[0] + 128u * l, S.H, S.W[l]);
+          tc::mma_commit(&S.bar);
+        }
+        if (!wait_products()) break;
+        float acc[32];
+        tc::tmem_ld32(tZ[0] + 128u * l + lanes + (uint32_t)cb, acc);
+        add_bias<32>(h4, acc, &sp.b[l][cb]);
+#pragma unroll
+        for (int i = 0; i < 16; ++i) h4[i] = __fmul2_rn(h4[i], sigmoid2(h4[i]));
+        if (l < 2) {
+#pragma unroll
+          for (int i = 0; i < 16; i += 4) put_pairs(S.H, r, cb + 2 * i, h4 + i);
+        }
+      }
+      if (pending) break;
+      // the head: a row's first (second) 64 units in one chain, by column quarters 0 and 1 (2, 3)
+      float y = 0.0f;
+      if ((cq & 1) == 0) {
+#pragma unroll
+        for (int i = 0; i < 16; ++i) y = fmaf(sp.w5[cb + 2 * i + 1], h4[i].y, fmaf(sp.w5[cb + 2 * i], h4[i].x, y));
+        S.yp[cq >> 1][r] = y;
+      }
+      __syncthreads();
+      if (cq & 1) {
+        y = S.yp[cq >> 1][r];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) y = fmaf(sp.w5[cb + 2 * i + 1], h4[i].y, fmaf(sp.w5[cb + 2 * i], h4[i].x, y));
+        if (cq == 3) S.yh[r] = y;
+      }
+      __syncthreads();
+      if (cq == 1) {
+        y += S.yh[r];
+        y += sp.b5;
+        const float ts = valid ? (targets[row0 + r] - N.mean) / N.scale : 0.0f;
+        const float res = valid ? (y - ts) : 0.0f;
+        const float dyv = valid ? res / (float)n : 0.0f;
+        S.dy[r] = dyv;
+        float l2 = 0.5f * res * res / (float)n * loss_scale;
+        for (int o = 16; o > 0; o >>= 1) l2 += __shfl_down_sync(0xffffffffu, l2, o);
+        if (lane == 0) S.red[q4] = l2;
+        float d = dyv;
+        for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
+        if (lane == 0) S.dyred[q4] = d;
+      }
+      __syncthreads();
+      if (tid == 0) atomicAdd(loss + (long long)it * loss_stride, S.red[0] + S.red[1] + S.red[2] + S.red[3]);
+      const float dyv = S.dy[r];
+      // ---- backward.  Head: dw5 = sum_s dy h4; dz4 = dy w5 silu'(z4), db4; H still holds h3
+      // (rows past the batch: dz is zero there)
+      {
+#pragma unroll 1
+        for (int c0 = cb; c0 < cb + 32; c0 += 16) {
+          float acc[16];
+          float2 z[8], v[8];
+          tc::tmem_ld16(tZ[2] + lanes + (uint32_t)c0, acc);
+          add_bias<16>(z, acc, &sp.b[2][c0]);
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            if (!valid) z[i] = make_float2(0.0f, 0.0f);
+            const float2 s = sigmoid2(z[i]), w = *reinterpret_cast<const float2 *>(&sp.w5[c0 + 2 * i]);
+            v[i] = __fmul2_rn(__fmul2_rn(dup2(dyv), z[i]), s);
+            z[i] = __fmul2_rn(__fmul2_rn(dup2(dyv), w), silu_grad2(z[i], s));
+          }
+          put_pairs(S.dZ, r, c0, z);
+          put_pairs(S.dZ, r, c0 + 8, z + 4);
+          float cs = column_sum(v, lane);
+          if (lane < 16) S.colred[0][q4][c0 + lane] = cs;
+          cs = column_sum(z, lane);
+          if (lane < 16) S.colred[1][q4][c0 + lane] = cs;
+        }
+      }
+      ready();
+      if (tid == 0) {
+        tc::fence_after_sync();
+        tc::mma_128x128x128_mn(tX, S.H, S.dZ);           // dW4^T[in][out]
+        tc::mma_128x128x128_kn(tZ[2], S.dZ, S.W[2]);     // dH3[sample][in]
+        tc::mma_commit(&S.bar);
+      }
+      if (cq == 0) spn.w5[r] = small_adam(0, r, kSmallW5 + r, sp.w5[r], GN, lr, c1, c2);
+      if (cq == 1) spn.b[2][r] = small_adam(1, r, kSmallB + 2 * kH + r, sp.b[2][r], GN, lr, c1, c2);
+      if (tid == kFusedThreads - 1) {  // b5
+        const float gi = S.dyred[0] + S.dyred[1] + S.dyred[2] + S.dyred[3];
+        if (GN) GN[oB5] = gi;
+        spn.b5 = adam_update(gi, sp.b5, S.sm[kSmallB5], S.sv[kSmallB5], lr, c1, c2);
+      }
+#pragma unroll 1
+      for (int l = 4; l >= 2; --l) {
+        const int oW = l == 4 ? oW4 : (l == 3 ? oW3 : oW2);
+        auto load_adam = [&](int at, float2 (&p)[2], float2 (&m)[2], float2 (&v)[2]) {
+#pragma unroll
+          for (int j = 0; j < 2; ++j) {
+            p[j] = make_float2(PN[at + 2 * j * kH], PN[at + (2 * j + 1) * kH]);
+            m[j] = make_float2(MN[at + 2 * j * kH], MN[at + (2 * j + 1) * kH]);
+            v[j] = make_float2(VN[at + 2 * j * kH], VN[at + (2 * j + 1) * kH]);
+          }
+        };
+        float2 pv[2], mv[2], vv[2];  // W_l's first four of this thread, in flight until Adam needs them
+        load_adam(oW + cb * kH + r, pv, mv, vv);
+        if (!wait_products()) break;
+        // tensor memory: l = 4: dW in X, dH in Z4's columns; 3: Z4's, Z3's; 2: X, Z4's again
+        // (dW3 has been read by then: ready() below)
+        const uint32_t tW = l == 3 ? tZ[2] : tX, tH = l == 4 ? tZ[2] : (l == 3 ? tZ[1] : tZ[1]);
+        // dz_{l-1} and, for l > 2, h_{l-2}
+#pragma unroll 1
+        for (int hc = 0; hc < 32; hc += 16) {
+          const int c0 = cb + hc;
+          // pre-activations of layer q (1..4) at this thread's 16 units
+          auto pre = [&](int q, float2 (&z)[8]) {
+            if (q > 1) {
+              float acc[16];
+              tc::tmem_ld16(tZ[0] + 128u * (q - 2) + lanes + (uint32_t)c0, acc);
+              add_bias<16>(z, acc, &sp.b[q - 2][c0]);
+            } else {
+#pragma unroll
+              for (int i = 0; i < 8; ++i) z[i] = layer1_pair(sp, c0 + 2 * i, u);
+            }
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+              if (!valid) z[i] = make_float2(0.0f, 0.0f);
+          };
+          float2 z[8], dz[8];
+          pre(l - 1, z);
+          {
+            float acc[16];
+            tc::tmem_ld16(tH + lanes + (uint32_t)c0, acc);
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+              dz[i] = __fmul2_rn(make_float2(acc[2 * i], acc[2 * i + 1]), silu_grad2(z[i], sigmoid2(z[i])));
+          }
+          if (l > 2) {
+            put_pairs(S.dZ, r, c0, dz);
+            put_pairs(S.dZ, r, c0 + 8, dz + 4);
+            pre(l - 2, z);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) z[i] = __fmul2_rn(z[i], sigmoid2(z[i]));
+            put_pairs(S.H, r, c0, z);
+            put_pairs(S.H, r, c0 + 8, z + 4);
+          }
+          float cs = column_sum(dz, lane);
+          if (lane < 16) S.colred[0][q4][c0 + lane] = cs;
+          if (l == 2) {  // first layer: dW1[c][k] = sum_s dz1[s][c] u[s][k]
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+#pragma unroll
+              for (int i = 0; i < 8; ++i) z[i] = __fmul2_rn(dz[i], dup2(u[k]));
+              cs = column_sum(z, lane);
+              if (lane < 16) S.colred[1 + k][q4][c0 + lane] = cs;
+            }
+          }
+        }
+        ready();
+        if (l > 2 && tid == 0) {  // the next layer's products run under this one's Adam
+          tc::fence_after_sync();
+          tc::mma_128x128x128_mn(l == 4 ? tZ[2] : tX, S.H, S.dZ);
+          tc::mma_128x128x128_kn(tZ[1], S.dZ, S.W[l - 3]);
+          tc::mma_commit(&S.bar);
+        }
+        // Adam of W_l: this thread's input unit r, output units cb .. cb + 31, four at a time
+        // with the next four's loads in flight
+        uint16_t *te = S.W[l - 2] + tile_index(cb, r);  // output unit cb; the next ones by tile_index(j, 0)
+#pragma unroll 1
+        for (int hc = 0; hc < 32; hc += 16) {
+          float g[16];
+          tc::tmem_ld16(tW + lanes + (uint32_t)(cb + hc), g);
+#pragma unroll
+          for (int j0 = 0; j0 < 16; j0 += 4) {
+            const int at = oW + (cb + hc + j0) * kH + r;
+            float2 np[2], nm[2], nv[2];
+            if (j0 < 12 || hc == 0) load_adam(at + 4 * kH, np, nm, nv);
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+              const float2 gi = make_float2(g[j0 + 2 * j], g[j0 + 2 * j + 1]);
+              const int a0 = at + 2 * j * kH, a1 = a0 + kH;
+              if (GN) {
+                GN[a0] = gi.x;
+                GN[a1] = gi.y;
+              }
+              const float2 pn = adam_update2(gi, pv[j], mv[j], vv[j], lr, c1, c2);
+              PN[a0] = pn.x;
+              PN[a1] = pn.y;
+              MN[a0] = mv[j].x;
+              MN[a1] = mv[j].y;
+              VN[a0] = vv[j].x;
+              VN[a1] = vv[j].y;
+              const uint32_t h = pack2(pn);
+              te[tile_index(hc + j0 + 2 * j, 0)] = (uint16_t)h;
+              te[tile_index(hc + j0 + 2 * j + 1, 0)] = (uint16_t)(h >> 16);
+            }
+            if (j0 < 12 || hc == 0) {
+#pragma unroll
+              for (int j = 0; j < 2; ++j) {
+                pv[j] = np[j];
+                mv[j] = nm[j];
+                vv[j] = nv[j];
+              }
+            }
+          }
+        }
+        if (cq == 0) {
+          float *bn = l > 2 ? spn.b[l - 3] : spn.b1;
+          const float *bp = l > 2 ? sp.b[l - 3] : sp.b1;
+          bn[r] = small_adam(0, r, (l > 2 ? kSmallB + (l - 3) * kH : kSmallB1) + r, bp[r], GN, lr, c1, c2);
+        }
+        if (l == 2)  // W1: four gradients a unit, one by each column quarter
+          reinterpret_cast<float *>(&spn.w1[r])[cq] =
+              small_adam(1 + cq, r, kSmallW1 + 4 * r + cq, reinterpret_cast<const float *>(&sp.w1[r])[cq], GN, lr, c1, c2);
+        tc::fence_before_sync();
+      }
+      if (pending) break;
+      __syncthreads();  // the next step reads spn, H and the tiles
+      tc::fence_after_sync();
+    }
+    if (!pending) {  // the small parameters and their moments back to memory
+      const SmallParams &sp = S.sp[C.n_steps & 1];
+      for (int i = tid; i < kSmall; i += kFusedThreads) {
+        const int at = small_index(i);
+        PN[at] = i < kSmallB1 ? reinterpret_cast<const float *>(sp.w1)[i]
+                 : i < kSmallB ? sp.b1[i - kSmallB1]
+                 : i < kSmallW5 ? sp.b[0][i - kSmallB]
+                 : i < kSmallB5 ? sp.w5[i - kSmallW5] : sp.b5;
+        MN[at] = S.sm[i];
+        VN[at] = S.sv[i];
+      }
+      __syncthreads();  // the next network's are staged over them
+    }
+  }
+  if (pending && tid == 0) {
+    status_or(status, RT_DEV_TIMEOUT);
+    tc::mbar_wait(&S.bar, phase ^ 1u, kWaitLimit);  // bounded: let the products land
+  }
+  tc::fence_before_sync();
+  __syncthreads();
+  if (warp == 0) {
+    tc::fence_after_sync();
+    tc::tmem_dealloc(tmem, 512);
   }
 }
 
@@ -1245,6 +1696,43 @@ rt_status mlp_train_steps_impl(float *params, float *m, float *v, float *grad, c
     return fail(RT_E_INVAL, "rt_mlp_train_steps: finite learning rates >= 0 required");
   if (n_nets < 1) return fail(RT_E_INVAL, "rt_mlp_train_steps_nets: n_nets must be >= 1");
   if (n_steps == 0) return RT_OK;
+  const Norm N1 = norm_on_device ? Norm{} : to_norm(nm);
+  const Norm *norms = norm_on_device ? reinterpret_cast<const Norm *>(nm) : nullptr;
+  const int64_t nb = n / batch;
+  const double span = (double)std::max(1, total_steps - 1);
+  auto rate = [&](int64_t s) { return (float)(lr1 + 0.5 * (lr0 - lr1) * (1.0 + std::cos(kPiD * (double)s / span))); };
+  if (batch <= kH) {  // one tile a step: the fused kernel
+    Scratch scr;
+    rt_status r = scr.alloc(256, st);
+    if (r != RT_OK) return r;
+    float *loss = losses ? losses : scr.as<float>();
+    r = validate_train(params, m, v, grad, inputs, targets, batch, n_nets, nm, norm_on_device, 0, loss);
+    if (r != RT_OK) return r;
+    static std::once_flag once;
+    static rt_status attr = RT_OK;
+    std::call_once(once, [] { attr = set_smem((const void *)k_mlp_fused, sizeof(FusedSmem)); });
+    if (attr != RT_OK) return attr;
+    int dev = 0, sms = 0;
+    RT_CUDA_TRY(cudaGetDevice(&dev));
+    RT_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    if (losses) RT_CUDA_TRY(cudaMemsetAsync(losses, 0, (size_t)n_steps * sizeof(float), st));
+    for (int32_t i0 = 0; i0 < n_steps; i0 += kFusedSteps) {
+      StepConsts C;
+      C.n_steps = std::min<int32_t>(kFusedSteps, n_steps - i0);
+      C.first = (long long)step_first - 1 + i0;
+      for (int32_t i = 0; i < C.n_steps; ++i) {
+        const int64_t s = C.first + i;
+        C.lr[i] = rate(s);
+        C.c1[i] = (float)(1.0 - std::pow(0.9, (double)(s + 1)));
+        C.c2[i] = (float)(1.0 - std::pow(0.999, (double)(s + 1)));
+      }
+      k_mlp_fused<<<std::min(n_nets, sms), kFusedThreads, sizeof(FusedSmem), st>>>(
+          params, m, v, grad, N1, norms, inputs, targets, (int)batch, n, nb, n_nets, C, i0 + C.n_steps == n_steps,
+          losses ? losses + i0 : loss, losses ? 1 : 0, 1.0f / (float)n_nets, status);
+      RT_CUDA_TRY(cudaGetLastError());
+    }
+    return RT_OK;
+  }
   // one scratch for all steps: the step's buffers, then a loss slot if none is given
   const size_t sb = (train_scratch_bytes(batch, n_nets) + 255) & ~size_t(255);
   Scratch scr;
@@ -1254,23 +1742,18 @@ rt_status mlp_train_steps_impl(float *params, float *m, float *v, float *grad, c
   r = validate_train(params, m, v, grad, inputs, targets, batch, n_nets, nm, norm_on_device, 0,
                      losses ? losses : loss1);
   if (r != RT_OK) return r;
-  const Norm N1 = norm_on_device ? Norm{} : to_norm(nm);
-  const Norm *norms = norm_on_device ? reinterpret_cast<const Norm *>(nm) : nullptr;
   // the steps after the first take their BF16 tiles from the previous step's Adam
   // kernel, and a given loss buffer is zeroed once for all steps
   if (losses) RT_CUDA_TRY(cudaMemsetAsync(losses, 0, (size_t)n_steps * sizeof(float), st));
   r = mlp_prep_tiles(params, scr.as<uint16_t>(), n_nets, 6, st);
   if (r != RT_OK) return r;
-  const int64_t nb = n / batch;
-  const double span = (double)std::max(1, total_steps - 1);
   for (int32_t i = 0; i < n_steps; ++i) {
     const int64_t s = (int64_t)step_first - 1 + i;
     const int64_t b = s % nb;
-    const double lr = lr1 + 0.5 * (lr0 - lr1) * (1.0 + std::cos(kPiD * (double)s / span));
     if (!losses) RT_CUDA_TRY(cudaMemsetAsync(loss1, 0, sizeof(float), st));
     // every network's batch b: rows b * batch .. of its own n rows
     r = mlp_train_core(params, m, v, grad, inputs + 4 * b * batch, targets + b * batch, batch, n, n_nets, N1,
-                       norms, (float)lr, (int32_t)(s + 1), 0, losses ? losses + i : loss1, status, scr.as<char>(),
+                       norms, rate(s), (int32_t)(s + 1), 0, losses ? losses + i : loss1, status, scr.as<char>(),
                        true, i == n_steps - 1, st);
     if (r != RT_OK) return r;
   }

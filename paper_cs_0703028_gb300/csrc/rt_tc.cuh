@@ -169,5 +169,17 @@ __device__ __forceinline__ void mma_128x128x128_mn(uint32_t d_tmem, const void *
              idesc, s > 0 ? 1u : 0u);
 }
 
+// The same with A K-major (rows = m) and B MN-major: D[m][n] = sum_k A[m][k] B[k][n], B
+// written with one row per contraction index, so that a weight tile W[out][in] serves both
+// H W^T (K-major) and dZ W.
+__device__ __forceinline__ void mma_128x128x128_kn(uint32_t d_tmem, const void *A, const void *B) {
+  constexpr uint32_t idesc = idesc_bf16_f32(128, 128) | (1u << 16);
+  const uint32_t a0 = smem_addr(A), b0 = smem_addr(B);
+#pragma unroll
+  for (int s = 0; s < 8; ++s)
+    mma_bf16(d_tmem, smem_desc(a0 + 256u * s, 128u, 2048u), smem_desc(b0 + 4096u * s, 2048u, 128u),
+             idesc, s > 0 ? 1u : 0u);
+}
+
 }  // namespace tc
 }  // namespace rt
