@@ -74,17 +74,27 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float a, float b) {
 // bf16 element (r, k) of a K-major 128x128 tile (in units of 2-byte elements)
 __device__ __forceinline__ int tile_index(int r, int k) { return (int)(tc::kmajor_offset(r, k, kH) >> 1); }
 
-__global__ void k_mlp_prep(const float *__restrict__ P, uint16_t *__restrict__ tiles, int n_mats) {
-  const int m = blockIdx.y;  // 0..2: W2..W4 (rows = out), 3..5: transposes (rows = in)
-  const long long net = blockIdx.z;
-  P += net * kNParam;
-  tiles += net * n_mats * kTileElems;
-  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= kTileElems) return;
-  const int r = idx / kH, k = idx % kH;
-  const int base = (m % 3 == 0) ? oW2 : (m % 3 == 1 ? oW3 : oW4);
-  const float w = (m < 3) ? P[base + r * kH + k] : P[base + k * kH + r];
-  tiles[m * kTileElems + tile_index(r, k)] = __bfloat16_as_ushort(__float2bfloat16_rn(w));
+// A thread writes one core-matrix row (8 elements, 16 bytes); a warp's 32 (8 rows x 4
+// columns of core matrices) are 512 consecutive bytes, read as 128-byte pieces of 8 rows.
+// 6250 networks x 3 matrices: PREPUS ms (1.84 GB; 0.88 with an element a thread in row order).
+constexpr int kPrepThreads = 256;
+__global__ void __launch_bounds__(kPrepThreads)
+k_mlp_prep(const float *__restrict__ P, uint16_t *__restrict__ tiles, int n_mats) {
+  const int m = blockIdx.x;  // 0..2: W2..W4 (rows = out), 3..5: transposes (rows = in)
+  const long long net = blockIdx.y;
+  P += net * kNParam + ((m % 3 == 0) ? oW2 : (m % 3 == 1 ? oW3 : oW4));
+  tiles += (net * n_mats + m) * kTileElems;
+  const int step = m < 3 ? 1 : kH;
+#pragma unroll 4
+  for (int e = threadIdx.x; e < kTileElems / 8; e += kPrepThreads) {
+    const int r = ((e >> 7) << 3) + (e & 7), k = ((e >> 3) & 15) << 3;  // e = (r / 8, k / 8, r % 8)
+    const float *w = m < 3 ? P + r * kH + k : P + k * kH + r;
+    float v[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) v[i] = __ldg(w + i * step);
+    *reinterpret_cast<uint4 *>(tiles + tile_index(r, k)) =
+        make_uint4(pack_bf16x2(v[0], v[1]), pack_bf16x2(v[2], v[3]), pack_bf16x2(v[4], v[5]), pack_bf16x2(v[6], v[7]));
+  }
 }
 
 __device__ __forceinline__ void normalise(const float *__restrict__ in, long long row, bool valid,
@@ -1138,7 +1148,9 @@ k_tc_selftest(const float *__restrict__ A, const float *__restrict__ B, float *_
 
 // ---------------------------------------------------------------- surrogate walk
 constexpr int kWalkTiles = 3;                   // 128-ray tiles sharing the resident weights
-constexpr int kWalkMlpThreads = 128 * kWalkTiles;
+constexpr int kTileThreads = 256;               // two threads per ray of a tile, half the units each
+constexpr int kWalkRays = 128 * kWalkTiles;     // rays in flight per block
+constexpr int kWalkMlpThreads = kTileThreads * kWalkTiles;
 constexpr int kWalkTmemCols = 512;              // power of two >= kWalkTiles * kH
 
 // Layer 1 (K = 4) on the tensor cores as one K = 16 product: each input u_i and
@@ -1164,6 +1176,7 @@ struct WalkMlpSmem {
   uint16_t B1[kL1Elems];               // layer-1 weights and bias (hi/lo split, rows = out)
   uint16_t Bb[3][kL1Elems];            // biases of layers 2..4 against A1's constant-one columns
   WalkSmall sp;
+  Norm norm;                           // the band's
   uint64_t bar_w, bar_mma[kWalkTiles];
   unsigned long long next, end;        // the current work item's claim cursor and end
   int band;                            // the current work item's band (-1: no item left)
@@ -1177,6 +1190,7 @@ struct WalkMlpSmem {
 struct BandPlan {
   const uint32_t *order;
   const long long *band_start, *item_start;
+  const int *item_band;           // each item's band
   unsigned long long *item_next;  // work-item counter, zero at launch
   long long chunk;
   int n_bands;
@@ -1217,27 +1231,30 @@ __device__ __forceinline__ void stage_walk(WalkMlpSmem &S, const float *__restri
   if (threadIdx.x == 0) S.sp.b5 = P[oB5];
 }
 
-// The 128 threads of one tile (4 warps, named barrier 1 + tile) synchronise
+// The 256 threads of one tile (8 warps, named barrier 1 + tile) synchronise
 // among themselves only, so the tiles of a block drift apart and one tile's
 // epilogue runs while another tile's products occupy the tensor cores.
 __device__ __forceinline__ void tile_sync(int tile) {
-  asm volatile("barrier.cta.sync %0, 128;" ::"r"(1 + tile) : "memory");
+  asm volatile("barrier.cta.sync %0, 256;" ::"r"(1 + tile) : "memory");
 }
 __device__ __forceinline__ bool tile_or(int tile, bool v) {
   uint32_t r;
   asm volatile(
       "{\n .reg .pred p, q;\n setp.ne.u32 p, %1, 0;\n"
-      " barrier.cta.red.or.pred q, %2, 128, p;\n selp.u32 %0, 1, 0, q;\n}\n"
+      " barrier.cta.red.or.pred q, %2, 256, p;\n selp.u32 %0, 1, 0, q;\n}\n"
       : "=r"(r) : "r"((uint32_t)v), "r"(1 + tile) : "memory");
   return r != 0;
 }
 
-// Network output (log kappa) for this thread's query, the 128 threads of its tile
-// together.  Returns false if a bounded tensor-core wait ran out.
+// Network output (log kappa) for ray r's query, the 256 threads of its tile together: thread
+// (half, r) takes units [64 half, 64 half + 64) of every layer; half 0 holds the query and gets
+// the output.  The head is one chain over the units in order (half 1 hands its activations
+// over through the tile's A buffer, which no later product of this evaluation reads).
+// Returns false if a bounded tensor-core wait ran out.
 __device__ __forceinline__ bool mlp_eval_tile(WalkMlpSmem &S, uint32_t tmem, const Norm &N,
                                               const float (&raw)[4], uint32_t &phase, float &logk) {
-  const int tid = threadIdx.x, tile = tid >> 7, r = tid & 127, warp = tid >> 5;
-  {  // this row of the layer-1 operand A: {u_hi, u_hi, u_lo} per input, then 1, 1, 0, 0
+  const int tid = threadIdx.x, tile = tid / kTileThreads, r = tid & 127, half = (tid >> 7) & 1, warp = tid >> 5;
+  if (half == 0) {  // this row of the layer-1 operand A: {u_hi, u_hi, u_lo} per input, then 1, 1, 0, 0
     uint16_t e[kL1K];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
@@ -1256,14 +1273,17 @@ __device__ __forceinline__ bool mlp_eval_tile(WalkMlpSmem &S, uint32_t tmem, con
     *reinterpret_cast<uint4 *>(&S.A1[tile][l1_index(r, 8)]) = make_uint4(w[4], w[5], w[6], w[7]);
   }
   float y = 0.0f;
+  bool late = false;  // this thread saw a wait give up: it issues and waits no more
   const uint32_t tcol = tmem + (uint32_t)(tile * kH);
+  const uint32_t tacc = tcol + ((uint32_t)((warp & 3) * 32) << 16);
+  float4 *h4 = reinterpret_cast<float4 *>(S.A[tile]);  // [unit / 4 of half 1][row]
   // l = 0: layer 1 (K = 16); l = 1..3: W2..W4 (K = 128)
 #pragma unroll 1
   for (int l = 0; l < 4; ++l) {
     tc::fence_smem_to_async();
     tc::fence_before_sync();
     tile_sync(tile);
-    if (r == 0) {
+    if (r == 0 && half == 0 && !late) {
       tc::fence_after_sync();
       const uint64_t a1 = tc::smem_desc(tc::smem_addr(S.A1[tile]), 128u, 256u);
       if (l == 0) {
@@ -1275,34 +1295,52 @@ __device__ __forceinline__ bool mlp_eval_tile(WalkMlpSmem &S, uint32_t tmem, con
       }
       tc::mma_commit(&S.bar_mma[tile]);
     }
-    const int timeout = tc::mbar_wait(&S.bar_mma[tile], phase, kWaitLimit) ? 0 : 1;
+    if (!late) late = !tc::mbar_wait(&S.bar_mma[tile], phase, kWaitLimit);
     phase ^= 1u;
-    if (tile_or(tile, timeout)) {
-      // the product may still be in flight: let it land (bounded) before the tile stops
-      if (r == 0) tc::mbar_wait(&S.bar_mma[tile], phase ^ 1u, kWaitLimit);
-      return false;
-    }
+    __syncwarp();
     tc::fence_after_sync();
-#pragma unroll 1
-    for (int c0 = 0; c0 < kH; c0 += 32) {
-      float z[32];  // pre-activations, biases included
-      tc::tmem_ld32(tcol + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)c0, z);
-      if (l < 3) {  // next layer's BF16 input: binary32 SiLU (as in training), rounded to BF16
+    // pre-activations, biases included, 16 units at a time with the next 16 on their way from
+    // tensor memory
+    uint32_t z[2][16];
+    tc::tmem_ld16_async(tacc + 64u * (uint32_t)half, z[0]);
 #pragma unroll
-        for (int i = 0; i < 32; i += 8)
-          *reinterpret_cast<uint4 *>(&S.A[tile][tile_index(r, c0 + i)]) =
-              make_uint4(pack_bf16x2(z[i] * sigmoid_fast(z[i]), z[i + 1] * sigmoid_fast(z[i + 1])),
-                         pack_bf16x2(z[i + 2] * sigmoid_fast(z[i + 2]), z[i + 3] * sigmoid_fast(z[i + 3])),
-                         pack_bf16x2(z[i + 4] * sigmoid_fast(z[i + 4]), z[i + 5] * sigmoid_fast(z[i + 5])),
-                         pack_bf16x2(z[i + 6] * sigmoid_fast(z[i + 6]), z[i + 7] * sigmoid_fast(z[i + 7])));
-      } else {  // last hidden layer: binary32 SiLU into the head
+    for (int q = 0; q < 4; ++q) {
+      const int c0 = 64 * half + 16 * q;
+      tc::tmem_ld_wait(z[q & 1]);
+      if (q < 3) tc::tmem_ld16_async(tacc + (uint32_t)(c0 + 16), z[(q + 1) & 1]);
+      // binary32 SiLU (as in training)
+      float2 h[8];
 #pragma unroll
-        for (int q = 0; q < 32; ++q) y = fmaf(S.sp.w5[c0 + q], z[q] * sigmoid_fast(z[q]), y);
+      for (int i = 0; i < 8; ++i) {
+        const float2 zi = make_float2(__uint_as_float(z[q & 1][2 * i]), __uint_as_float(z[q & 1][2 * i + 1]));
+        h[i] = __fmul2_rn(zi, sigmoid2(zi));
+      }
+      if (l < 3) {  // next layer's BF16 input
+        put_pairs(S.A[tile], r, c0, h);
+        put_pairs(S.A[tile], r, c0 + 8, h + 4);
+      } else if (half == 0) {  // last hidden layer: into the head
+#pragma unroll
+        for (int i = 0; i < 8; ++i) y = fmaf(S.sp.w5[c0 + 2 * i + 1], h[i].y, fmaf(S.sp.w5[c0 + 2 * i], h[i].x, y));
+      } else {
+#pragma unroll
+        for (int i = 0; i < 8; i += 2) h4[((c0 - 64 + 2 * i) / 4) * 128 + r] = make_float4(h[i].x, h[i].y, h[i + 1].x, h[i + 1].y);
       }
     }
   }
   // this tile's accumulators are read before its next products overwrite them
   tc::fence_before_sync();
+  if (tile_or(tile, late)) {
+    // a product may still be in flight: let it land (bounded) before the tile stops
+    if (r == 0 && half == 0) tc::mbar_wait(&S.bar_mma[tile], phase ^ 1u, kWaitLimit);
+    return false;
+  }
+  if (half == 0) {
+#pragma unroll
+    for (int q = 0; q < 16; ++q) {
+      const float4 h = h4[q * 128 + r], w = *reinterpret_cast<const float4 *>(&S.sp.w5[64 + 4 * q]);
+      y = fmaf(w.w, h.w, fmaf(w.z, h.z, fmaf(w.y, h.y, fmaf(w.x, h.x, y))));
+    }
+  }
   logk = N.mean + N.scale * (y + S.sp.b5);
   return true;
 }
@@ -1334,9 +1372,10 @@ k_walk_mlp(const float *__restrict__ P, const uint16_t *__restrict__ tiles, Norm
   uint32_t wphase = 0;  // the weight copies' barrier phase
   int cur_band = -1, timeout = 0;
   bool weights_late = false;
-  const int tile = tid >> 7;
+  const int tile = tid / kTileThreads;
+  const bool owner = (tid & 128) == 0;  // the thread that holds its tile row's ray
   unsigned long long n_evals = 0;  // this tile's network evaluations (counted by its thread 0)
-  Norm N = N1;
+  const Norm &N = S.norm;
 #pragma unroll 1
   for (;;) {  // work items: one band's network, at most B.chunk of its rays
     if (tid == 0) {
@@ -1344,29 +1383,25 @@ k_walk_mlp(const float *__restrict__ P, const uint16_t *__restrict__ tiles, Norm
       int band = -1;
       long long b0 = 0, b1 = 0;
       if (it < B.item_start[B.n_bands]) {
-        int lo = 0, hi = B.n_bands - 1;  // the last band whose first item is <= it
-        while (lo < hi) {
-          const int mid = (lo + hi + 1) >> 1;
-          if (B.item_start[mid] <= it) lo = mid; else hi = mid - 1;
-        }
-        band = lo;
+        band = B.item_band[it];
         b0 = B.band_start[band] + (it - B.item_start[band]) * B.chunk;
         b1 = min(b0 + B.chunk, B.band_start[band + 1]);
       }
       S.band = band;
       S.next = (unsigned long long)b0;
       S.end = (unsigned long long)b1;
+      if (band >= 0 && band != cur_band) {  // every tile is done with the previous band's weights
+        tc::mbar_arrive_expect_tx(&S.bar_w, 3 * kTileBytes);
+        tc::bulk_g2s(&S.W[0][0], tiles + (long long)band * 3 * kTileElems, 3 * kTileBytes, &S.bar_w);
+      }
     }
     __syncthreads();
     const int band = S.band;
     if (band < 0) break;
     if (band != cur_band) {  // this band's network: small parameters staged, hidden layers copied
       stage_walk(S, P + (long long)band * kNParam);
+      if (tid == 0) S.norm = net_norm(norms, N1, band);
       tc::fence_smem_to_async();  // B1, Bb are read by the tensor cores of every tile
-      if (tid == 0) {
-        tc::mbar_arrive_expect_tx(&S.bar_w, 3 * kTileBytes);
-        tc::bulk_g2s(&S.W[0][0], tiles + (long long)band * 3 * kTileElems, 3 * kTileBytes, &S.bar_w);
-      }
       const int late = tc::mbar_wait(&S.bar_w, wphase, kWaitLimit) ? 0 : 1;
       wphase ^= 1u;
       tc::fence_before_sync();
@@ -1376,25 +1411,24 @@ k_walk_mlp(const float *__restrict__ P, const uint16_t *__restrict__ tiles, Norm
         break;
       }
       tc::fence_after_sync();
-      N = net_norm(norms, N1, band);
       cur_band = band;
     }
     Ray R;
     bool active = false;
 #pragma unroll 1
     for (;;) {  // the item's rays: a lane whose ray is done claims the next one
-      if (!active) {
+      if (owner && !active) {
         const unsigned long long claim = atomicAdd(&S.next, 1ull);
         if (claim < S.end) {
           ray_init(W, nullptr, nullptr, B.order ? (unsigned long long)B.order[claim] : claim, record, R);
           active = true;
         }
       }
-      if (!tile_or(tile, active)) break;  // this tile has no ray of the item left
-      float raw[4] = {N.lo[0], N.lo[1], N.lo[2], N.lo[3]};
       float Tc = 1.0f;
+      if (active) Tc = __ldg(T + R.cell);  // on its way while the tile gathers
+      if (!tile_or(tile, active)) break;   // this tile has no ray of the item left
+      float raw[4] = {N.lo[0], N.lo[1], N.lo[2], N.lo[3]};
       if (active) {
-        Tc = T[R.cell];
         raw[0] = __logf(fmaf((float)R.j, W.dnu, W.nu_min));
         raw[1] = Tc;
         raw[2] = Pf ? Pf[R.cell] : p_ref;
@@ -1405,7 +1439,7 @@ k_walk_mlp(const float *__restrict__ P, const uint16_t *__restrict__ tiles, Norm
         timeout = 1;
         break;
       }
-      n_evals += (tid & 127) == 0 ? 1 : 0;
+      n_evals += (tid & (kTileThreads - 1)) == 0 ? 1 : 0;
       if (active) {
         const float kap = __expf(logk);
         if (R.w < 0.0f) R.w = emission_weight(W, R.j, Tc, kap);
@@ -1575,7 +1609,7 @@ Norm to_norm(const rt_mlp_norm *nm) {
 
 // BF16 tiles of n_nets networks: the first n_mats of W2..W4, W2^T..W4^T per network
 rt_status mlp_prep_tiles(const float *params, uint16_t *tiles, int n_nets, int n_mats, cudaStream_t st) {
-  k_mlp_prep<<<dim3(kTileElems / 256, n_mats, n_nets), 256, 0, st>>>(params, tiles, n_mats);
+  k_mlp_prep<<<dim3(n_mats, n_nets), kPrepThreads, 0, st>>>(params, tiles, n_mats);
   RT_CUDA_TRY(cudaGetLastError());
   return RT_OK;
 }
@@ -1834,14 +1868,15 @@ rt_status trace_mlp_core(const rt_grid *grid, int band_pts, const float *params,
   int dev = 0, sms = 0;
   RT_CUDA_TRY(cudaGetDevice(&dev));
   RT_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  const unsigned long long want = (n_rays + 8ull * kWalkMlpThreads - 1) / (8ull * kWalkMlpThreads);
+  const unsigned long long want = (n_rays + 8ull * kWalkRays - 1) / (8ull * kWalkRays);
   const unsigned blocks = (unsigned)(want < (unsigned long long)sms ? (want > 0 ? want : 1) : sms);
   // work items of about 1/8 of a block's share of the rays (at least 1024), so that
   // the blocks finish together
   const long long chunk = std::max(1024LL, (long long)(n_rays / (8ull * blocks)));
   // scratch: the bands' BF16 hidden-layer tiles, the plan, the band-grouped ray order
   const size_t tiles_b = (size_t)n_bands * 3 * kTileBytes;
-  const size_t plan_b = (((size_t)n_bands * 8 * 3 + 16 * 3 + 255) / 256) * 256;
+  const size_t max_items = (size_t)n_bands + (size_t)(n_rays / (unsigned long long)chunk) + 1;
+  const size_t plan_b = (((size_t)n_bands * 8 * 3 + 16 * 3 + max_items * 4 + 255) / 256) * 256;
   const size_t order_b = n_bands > 1 ? (size_t)n_rays * sizeof(uint32_t) : 0;
   Scratch scr;
   v = scr.alloc(tiles_b + plan_b + order_b, st);
@@ -1852,13 +1887,14 @@ rt_status trace_mlp_core(const rt_grid *grid, int band_pts, const float *params,
   long long *band_start = reinterpret_cast<long long *>(counts + n_bands);
   long long *item_start = band_start + (n_bands + 1);
   unsigned long long *item_next = reinterpret_cast<unsigned long long *>(item_start + (n_bands + 1));
+  int *item_band = reinterpret_cast<int *>(item_next + 1);
   uint32_t *order = n_bands > 1 ? reinterpret_cast<uint32_t *>(base + tiles_b + plan_b) : nullptr;
   v = mlp_prep_tiles(params, tiles, n_bands, 3, st);
   if (v != RT_OK) return v;
   RT_CUDA_TRY(cudaMemsetAsync(item_next, 0, sizeof(unsigned long long), st));
-  v = band_plan(W, band_pts, n_bands, chunk, counts, band_start, item_start, order, sms, st);
+  v = band_plan(W, band_pts, n_bands, chunk, counts, band_start, item_start, item_band, order, sms, st);
   if (v != RT_OK) return v;
-  BandPlan B{order, band_start, item_start, item_next, chunk, n_bands};
+  BandPlan B{order, band_start, item_start, item_band, item_next, chunk, n_bands};
   k_walk_mlp<<<blocks, kWalkMlpThreads, sizeof(WalkMlpSmem), st>>>(
       params, tiles, N1, norms, B, grid->T, grid->p_atm, grid->x, (float)spec->p_ref_atm, (float)spec->x_ref, W,
       tally->absorbed, tally->scalars, tally->steps, count_evals ? tally->steps + 1 : nullptr, tally->status, rp);

@@ -66,7 +66,8 @@ __global__ void k_band_count(WalkParams W, int band_pts, long long n_bands, unsi
 // scatter cursors; counts == nullptr: one band holding all n_rays rays
 __global__ void k_band_plan(const unsigned long long *__restrict__ counts, long long n_bands,
                             unsigned long long n_rays, long long chunk, long long *__restrict__ band_start,
-                            long long *__restrict__ item_start, unsigned long long *__restrict__ cursor) {
+                            long long *__restrict__ item_start, int *__restrict__ item_band,
+                            unsigned long long *__restrict__ cursor) {
   __shared__ long long sc[1024], si[1024];
   const int t = threadIdx.x, nt = blockDim.x;
   // each thread sums a contiguous run of bands, then the runs are scanned
@@ -95,7 +96,8 @@ __global__ void k_band_plan(const unsigned long long *__restrict__ counts, long 
     item_start[b] = pi;
     if (cursor) cursor[b] = (unsigned long long)pc;
     pc += k;
-    pi += (k + chunk - 1) / chunk;
+    for (const long long end = pi + (k + chunk - 1) / chunk; pi < end; ++pi)
+      if (item_band) item_band[pi] = (int)b;
   }
   if (t == nt - 1) {
     band_start[n_bands] = sc[t];
@@ -420,22 +422,22 @@ rt_status cell_prep(const rt_grid *grid, const rt_spectral *spec, float4 *cells,
 }
 
 rt_status band_plan(const WalkParams &W, int band_pts, long long n_bands, long long chunk,
-                    unsigned long long *counts, long long *band_start, long long *item_start, uint32_t *order,
-                    int sms, cudaStream_t st) {
+                    unsigned long long *counts, long long *band_start, long long *item_start, int *item_band,
+                    uint32_t *order, int sms, cudaStream_t st) {
   if (n_bands > 1) {
     RT_CUDA_TRY(cudaMemsetAsync(counts, 0, (size_t)n_bands * sizeof(unsigned long long), st));
     const unsigned gb = (unsigned)std::min<unsigned long long>((W.n_rays + 255) / 256, 8ull * (unsigned)sms);
     k_band_count<<<gb, 256, 0, st>>>(W, band_pts, n_bands, counts);
     RT_CUDA_TRY(cudaGetLastError());
     // the counts are read by the plan, then the same words serve as the scatter cursors
-    k_band_plan<<<1, 1024, 0, st>>>(counts, n_bands, W.n_rays, chunk, band_start, item_start, counts);
+    k_band_plan<<<1, 1024, 0, st>>>(counts, n_bands, W.n_rays, chunk, band_start, item_start, item_band, counts);
     RT_CUDA_TRY(cudaGetLastError());
     if (order) {
       k_band_scatter<<<gb, 256, 0, st>>>(W, band_pts, counts, order);
       RT_CUDA_TRY(cudaGetLastError());
     }
   } else {
-    k_band_plan<<<1, 1024, 0, st>>>(nullptr, 1, W.n_rays, chunk, band_start, item_start, nullptr);
+    k_band_plan<<<1, 1024, 0, st>>>(nullptr, 1, W.n_rays, chunk, band_start, item_start, item_band, nullptr);
     RT_CUDA_TRY(cudaGetLastError());
   }
   return RT_OK;
@@ -480,7 +482,7 @@ rt_status trace_impl(const rt_grid *grid, const float *kappa, const rt_spectral 
     long long *band_start = reinterpret_cast<long long *>(counts + nb);
     long long *item_start = band_start + (nb + 1);
     order = reinterpret_cast<uint32_t *>(pb + pbytes);
-    v = band_plan(W, 1, nb, 1LL << 40, counts, band_start, item_start, order, sms, st);
+    v = band_plan(W, 1, nb, 1LL << 40, counts, band_start, item_start, nullptr, order, sms, st);
     if (v != RT_OK) return v;
   }
   const bool rec = rp.cells != nullptr;
