@@ -122,15 +122,4 @@ rt_status rt_status_read(const uint32_t *status, void *stream) {
   return rt::status_from_bits(bits);
 }
 
-rt_status rt_tally_zero(const rt_tally_buf *t, int64_t ncells, void *stream) {
-  if (!t || !t->absorbed || !t->scalars || !t->steps || !t->status || ncells < 1)
-    return rt::fail(RT_E_INVAL, "rt_tally_zero: bad tally buffer");
-  cudaStream_t s = (cudaStream_t)stream;
-  RT_CUDA_TRY(cudaMemsetAsync(t->absorbed, 0, sizeof(double) * (size_t)ncells, s));
-  RT_CUDA_TRY(cudaMemsetAsync(t->scalars, 0, sizeof(double) * 4, s));
-  RT_CUDA_TRY(cudaMemsetAsync(t->steps, 0, sizeof(unsigned long long), s));
-  RT_CUDA_TRY(cudaMemsetAsync(t->status, 0, sizeof(uint32_t), s));
-  return RT_OK;
-}
-
 }  // extern "C"

@@ -2,8 +2,9 @@
 // final tally reduction.
 //   k_cell_prep : per cell, the binary32 temperature bracket (k, frac) of the
 //                 kappa table, the density scale (p x)/(p_ref x_ref) and T.
-//   k_pair_table: the walk's copy of the table, {kappa_k, kappa_k+1} per
-//                 (wavenumber, node), so a step's interpolation is one 8-byte load.
+//   k_walk_setup: the cells (as k_cell_prep) and the walk's copy of the table in one launch:
+//                 {kappa_k, kappa_k+1} per (wavenumber, node), so a step's interpolation is
+//                 one 8-byte load, or wavenumber-major.
 //   k_walk      : per ray, Philox draws -> emission cell, wavenumber, position,
 //                 isotropic direction -> cell-by-cell walk with Beer-Lambert
 //                 attenuation (Eq. I, first term), binary64 atomic deposits;
@@ -23,7 +24,7 @@ rt_status validate_spec(const rt_spectral *s);
 
 namespace {
 
-constexpr int kWalkThreads = 256;
+constexpr int kWalkThreads = 256, kWalkBlocks = 4;  // resident blocks per SM
 constexpr int kReduceBlocks = 256;
 
 __global__ void k_cell_prep(const float *__restrict__ T, const float *__restrict__ p,
@@ -127,49 +128,69 @@ int g_walk_group = 0;
 
 namespace {
 
-// [nT][n_nu] -> [n_nu][nT] through 32 x 33 shared tiles
-__global__ void k_transpose(const float *__restrict__ in, int rows, long long cols, float *__restrict__ out) {
-  __shared__ float t[32][33];
-  const long long c0 = (long long)blockIdx.x * 32;
-  const int r0 = blockIdx.y * 32;
-  for (int i = threadIdx.y; i < 32; i += blockDim.y) {
-    const int r = r0 + i;
-    const long long c = c0 + threadIdx.x;
-    if (r < rows && c < cols) t[i][threadIdx.x] = in[(long long)r * cols + c];
-  }
-  __syncthreads();
-  for (int i = threadIdx.y; i < 32; i += blockDim.y) {
-    const long long c = c0 + i;
-    const int r = r0 + threadIdx.x;
-    if (r < rows && c < cols) out[c * rows + r] = t[threadIdx.x][i];
+constexpr int kSetupThreads = 256;
+constexpr int kPairRows = 64;
+// Blocks of the walk's copy of a T-major table: bx over 32-wavenumber slices, by over nodes.
+// Layout 1, [nT][n_nu] -> [n_nu][nT]: 32 x 32 tiles.  Layout 2, node pairs out[j (nT - 1) + k] =
+// {in[k][j], in[k + 1][j]}: each block stages kPairRows + 1 rows of 32 wavenumbers and writes
+// the pairs wavenumber by wavenumber.
+template <int LAYOUT>
+__device__ __forceinline__ void table_block(const float *__restrict__ in, int nT, long long n_nu,
+                                            float *__restrict__ out, long long bx, int by) {
+  __shared__ float t[LAYOUT == 2 ? kPairRows + 1 : 32][33];
+  const long long j0 = bx * 32;
+  if (LAYOUT == 2) {
+    const int k0 = by * kPairRows;
+    const int rows = min(kPairRows + 1, nT - k0);
+    for (int idx = threadIdx.x; idx < rows * 32; idx += kSetupThreads) {
+      const int r = idx >> 5, c = idx & 31;
+      if (j0 + c < n_nu) t[r][c] = in[(long long)(k0 + r) * n_nu + j0 + c];
+    }
+    __syncthreads();
+    const int np = rows - 1;
+    for (int idx = threadIdx.x; idx < np * 32; idx += kSetupThreads) {
+      const int c = idx / np, r = idx - c * np;
+      if (j0 + c < n_nu)
+        reinterpret_cast<float2 *>(out)[(j0 + c) * (long long)(nT - 1) + k0 + r] = make_float2(t[r][c], t[r + 1][c]);
+    }
+  } else {
+    const int r0 = by * 32, x = threadIdx.x & 31;
+    for (int i = threadIdx.x >> 5; i < 32; i += kSetupThreads / 32)
+      if (r0 + i < nT && j0 + x < n_nu) t[i][x] = in[(long long)(r0 + i) * n_nu + j0 + x];
+    __syncthreads();
+    for (int i = threadIdx.x >> 5; i < 32; i += kSetupThreads / 32)
+      if (r0 + x < nT && j0 + i < n_nu) out[(j0 + i) * nT + r0 + x] = t[x][i];
   }
 }
 
-// [nT][n_nu] -> node pairs out[j * (nT - 1) + k] = {in[k][j], in[k + 1][j]}: each block
-// stages kPairRows + 1 rows of 32 wavenumbers and writes the pairs wavenumber by wavenumber.
-constexpr int kPairRows = 64;
-__global__ void k_pair_table(const float *__restrict__ in, int nT, long long n_nu, float2 *__restrict__ out) {
-  __shared__ float t[kPairRows + 1][33];
-  const long long j0 = (long long)blockIdx.x * 32;
-  const int k0 = blockIdx.y * kPairRows;
-  const int rows = min(kPairRows + 1, nT - k0);
-  for (int idx = threadIdx.x; idx < rows * 32; idx += blockDim.x) {
-    const int r = idx >> 5, c = idx & 31;
-    if (j0 + c < n_nu) t[r][c] = in[(long long)(k0 + r) * n_nu + j0 + c];
+template <int LAYOUT>
+__global__ void __launch_bounds__(kSetupThreads)
+k_walk_table(const float *__restrict__ in, int nT, long long n_nu, float *__restrict__ out) {
+  table_block<LAYOUT>(in, nT, n_nu, out, blockIdx.x, blockIdx.y);
+}
+
+// The set-up of a table walk in one launch: the first cell_blocks blocks prepare the cells, the
+// others copy the table.
+template <int LAYOUT>
+__global__ void __launch_bounds__(kSetupThreads)
+k_walk_setup(const float *__restrict__ T, const float *__restrict__ p, const float *__restrict__ x, CellParams C,
+             float4 *__restrict__ cells, uint32_t *status, long long cell_blocks, const float *__restrict__ in, int nT,
+             long long n_nu, long long slices, float *__restrict__ out) {
+  const long long b = blockIdx.x;
+  if (b < cell_blocks) {
+    const long long c = b * kSetupThreads + threadIdx.x;
+    if (c < C.ncells) cells[c] = cell_prep_one(T, p, x, c, C, status);
+    return;
   }
-  __syncthreads();
-  const int np = rows - 1;
-  for (int idx = threadIdx.x; idx < np * 32; idx += blockDim.x) {
-    const int c = idx / np, r = idx - c * np;
-    if (j0 + c < n_nu) out[(j0 + c) * (long long)(nT - 1) + k0 + r] = make_float2(t[r][c], t[r + 1][c]);
-  }
+  const long long q = b - cell_blocks;
+  table_block<LAYOUT>(in, nT, n_nu, out, q % slices, (int)(q / slices));
 }
 
 // Four blocks of 64 registers: at five of 48 the walk spills, and more resident rays share
 // one L1 (8e6 rays of a thin gas in a 75 x 52 x 61 box: 2.29 ms against 2.61 ms; 4e8 rays of
 // the opaque 128^3 box, where it matters least: 15.9 ms against 16.9 ms).
 template <bool REC, int TAB, int REFILL>
-__global__ void __launch_bounds__(kWalkThreads, 4)
+__global__ void __launch_bounds__(kWalkThreads, kWalkBlocks)
 k_walk(const float4 *__restrict__ cells, const float *__restrict__ tab, const uint32_t *__restrict__ order,
        WalkParams W, double *__restrict__ absorbed, double *__restrict__ scalars,
        unsigned long long *__restrict__ steps_out, uint32_t *status, RecordPtrs rec) {
@@ -258,29 +279,61 @@ k_walk(const float4 *__restrict__ cells, const float *__restrict__ tab, const ui
   }
 }
 
-__global__ void k_reduce(const double *__restrict__ a, long long n, double *__restrict__ partial) {
+// sum over the block of each thread's s, in thread 0 (a fixed tree)
+__device__ __forceinline__ double block_sum(double s) {
   __shared__ double sh[32];
-  double s = 0.0;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (long long)gridDim.x * blockDim.x)
-    s += a[i];
   for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
   if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = s;
   __syncthreads();
   if (threadIdx.x < 32) {
     s = threadIdx.x < (blockDim.x >> 5) ? sh[threadIdx.x] : 0.0;
     for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-    if (threadIdx.x == 0) partial[blockIdx.x] = s;
   }
+  return s;
 }
 
-__global__ void k_final(const double *__restrict__ partial, int np, double *__restrict__ scalars) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
+__global__ void k_reduce(const double *__restrict__ a, long long n, double *__restrict__ partial) {
   double s = 0.0;
-  for (int i = 0; i < np; ++i) s += partial[i];
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
+       i += (long long)gridDim.x * blockDim.x)
+    s += a[i];
+  s = block_sum(s);
+  if (threadIdx.x == 0) partial[blockIdx.x] = s;
+}
+
+// One block: the sum of a[0 .. n) (the partials of k_reduce, or a small tally itself), the
+// energy balance into scalars, and what the host reads in one copy: out = {scalars[0..3],
+// status bits, then copy_n values of a}.  (One thread adding 256 partials took 17 us.)
+__global__ void __launch_bounds__(1024) k_final(const double *__restrict__ a, long long n, double *__restrict__ scalars,
+                                                const uint32_t *__restrict__ status, double *__restrict__ out,
+                                                int copy_n) {
+  double s = 0.0;
+  for (long long i = threadIdx.x; i < n; i += blockDim.x) {
+    const double v = a[i];
+    s += v;
+    if (i < copy_n) out[5 + i] = v;
+  }
+  s = block_sum(s);
+  if (threadIdx.x != 0) return;
+  const double e = scalars[0], w = scalars[2], r = e != 0.0 ? fabs(e - s - w) / e : 0.0;
   scalars[1] = s;
-  const double e = scalars[0];
-  scalars[3] = e != 0.0 ? fabs(e - s - scalars[2]) / e : 0.0;
+  scalars[3] = r;
+  out[0] = e;
+  out[1] = s;
+  out[2] = w;
+  out[3] = r;
+  out[4] = (double)*status;
+}
+
+__global__ void k_tally_zero(double *__restrict__ absorbed, long long n, double *__restrict__ scalars,
+                             unsigned long long *__restrict__ steps, uint32_t *__restrict__ status) {
+  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  for (long long c = i; c < n; c += (long long)gridDim.x * blockDim.x) absorbed[c] = 0.0;
+  if (i < 4) scalars[i] = 0.0;
+  if (i == 0) {
+    steps[0] = 0;
+    *status = 0;
+  }
 }
 
 rt_status validate_grid(const rt_grid *g) {
@@ -375,13 +428,6 @@ rt_status walk_setup(const rt_grid *grid, const rt_spectral *spec, uint64_t ray_
   return RT_OK;
 }
 
-rt_status launch_transpose(const float *tab, int nT, long long n_nu, float *tabt, cudaStream_t st) {
-  dim3 tg((unsigned)((n_nu + 31) / 32), (unsigned)((nT + 31) / 32));
-  k_transpose<<<tg, dim3(32, 8), 0, st>>>(tab, nT, n_nu, tabt);
-  RT_CUDA_TRY(cudaGetLastError());
-  return RT_OK;
-}
-
 int walk_table_layout(int nT, long long n_nu) {
   return (nT >= 2 && (size_t)n_nu * (size_t)(nT - 1) * 8 <= kPairTableBytes) ? 2 : 1;
 }
@@ -391,9 +437,10 @@ size_t walk_table_bytes(int layout, int nT, long long n_nu) {
 }
 
 rt_status launch_walk_table(int layout, const float *tab, int nT, long long n_nu, float *out, cudaStream_t st) {
-  if (layout != 2) return launch_transpose(tab, nT, n_nu, out, st);
-  dim3 g((unsigned)((n_nu + 31) / 32), (unsigned)((nT - 1 + kPairRows - 1) / kPairRows));
-  k_pair_table<<<g, 256, 0, st>>>(tab, nT, n_nu, reinterpret_cast<float2 *>(out));
+  const int ny = layout == 2 ? (nT - 1 + kPairRows - 1) / kPairRows : (nT + 31) / 32;
+  const dim3 g((unsigned)((n_nu + 31) / 32), (unsigned)ny);
+  if (layout == 2) k_walk_table<2><<<g, kSetupThreads, 0, st>>>(tab, nT, n_nu, out);
+  else k_walk_table<1><<<g, kSetupThreads, 0, st>>>(tab, nT, n_nu, out);
   RT_CUDA_TRY(cudaGetLastError());
   return RT_OK;
 }
@@ -467,10 +514,23 @@ rt_status trace_impl(const rt_grid *grid, const float *kappa, const rt_spectral 
   if (v != RT_OK) return v;
   float4 *cells = scr.as<float4>();
   float *tabw = reinterpret_cast<float *>(scr.as<char>() + cbytes);
-  v = cell_prep(grid, spec, cells, tally->status, st);
-  if (v != RT_OK) return v;
-  v = launch_walk_table(layout, kappa, spec->nT, spec->n_nu, tabw, st);
-  if (v != RT_OK) return v;
+  {
+    const CellParams C = cell_params(spec, W.ncells, (grid->p_atm || grid->x) ? 1 : 0);
+    const long long cb = (W.ncells + kSetupThreads - 1) / kSetupThreads, slices = (spec->n_nu + 31) / 32;
+    const long long ny = layout == 2 ? (spec->nT - 1 + kPairRows - 1) / kPairRows : (spec->nT + 31) / 32;
+    const long long nblocks = cb + slices * ny;
+    if (nblocks <= 0x7FFFFFFFLL) {
+      auto setup = layout == 2 ? k_walk_setup<2> : k_walk_setup<1>;
+      setup<<<(unsigned)nblocks, kSetupThreads, 0, st>>>(grid->T, grid->p_atm, grid->x, C, cells, tally->status, cb,
+                                                         kappa, spec->nT, spec->n_nu, slices, tabw);
+      RT_CUDA_TRY(cudaGetLastError());
+    } else {  // more blocks than one grid axis holds
+      v = cell_prep(grid, spec, cells, tally->status, st);
+      if (v != RT_OK) return v;
+      v = launch_walk_table(layout, kappa, spec->nT, spec->n_nu, tabw, st);
+      if (v != RT_OK) return v;
+    }
+  }
   W.nu_major = layout;
   int dev = 0, sms = 0;
   RT_CUDA_TRY(cudaGetDevice(&dev));
@@ -493,13 +553,11 @@ rt_status trace_impl(const rt_grid *grid, const float *kappa, const rt_spectral 
     return g_walk_refill == 12 ? k_walk<false, L, 12> : k_walk<false, L, 16>;
   };
   auto kern = layout == 2 ? pick(std::integral_constant<int, 2>()) : pick(std::integral_constant<int, 1>());
-  int per_sm = 0;
-  RT_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kWalkThreads, 0));
-  if (per_sm < 1) per_sm = 1;
-  // persistent warps, each with a contiguous ray range of at least 64 rays
-  unsigned long long want = (n_rays + 64ull * (kWalkThreads / 32) - 1) / (64ull * (kWalkThreads / 32));
-  const unsigned long long cap = (unsigned long long)sms * (unsigned long long)per_sm;
-  const unsigned blocks = (unsigned)(want < cap ? (want > 0 ? want : 1) : cap);
+  // persistent warps, each with a contiguous ray range, at least one ray a lane (a call of 1e5
+  // rays is over sooner with a ray on every lane than with two on half of them)
+  const unsigned long long want = (n_rays + kWalkThreads - 1) / kWalkThreads;
+  const unsigned long long cap = (unsigned long long)sms * kWalkBlocks;
+  const unsigned blocks = (unsigned)(want < cap ? want : cap);
   kern<<<blocks, kWalkThreads, 0, st>>>(cells, tabw, order, W, tally->absorbed, tally->scalars, tally->steps,
                                         tally->status, rp);
   RT_CUDA_TRY(cudaGetLastError());
@@ -512,21 +570,38 @@ rt_status tally_impl(const rt_tally_buf *t, int64_t ncells, double *host_absorbe
     return fail(RT_E_INVAL, "rt_tally: bad tally buffer");
   if (ncells < 1) return fail(RT_E_INVAL, "rt_tally: ncells must be >= 1");
   if (!host_scalars) return fail(RT_E_INVAL, "rt_tally: host_scalars is NULL");
+  // a small tally is summed by one block and comes back with the scalars in one copy
+  constexpr int kSmall = 4096;
+  const bool small = ncells <= kSmall;
+  const int back = small && host_absorbed ? (int)ncells : 0;
   Scratch scr;
-  rt_status v = scr.alloc(sizeof(double) * kReduceBlocks, st);
+  rt_status v = scr.alloc(sizeof(double) * (size_t)(kReduceBlocks + 5 + back), st);
   if (v != RT_OK) return v;
-  k_reduce<<<kReduceBlocks, 256, 0, st>>>(t->absorbed, ncells, scr.as<double>());
+  double *partial = scr.as<double>(), *out = partial + kReduceBlocks;
+  if (!small) {
+    k_reduce<<<kReduceBlocks, 256, 0, st>>>(t->absorbed, ncells, partial);
+    RT_CUDA_TRY(cudaGetLastError());
+  }
+  k_final<<<1, small && ncells > 256 ? 1024 : 256, 0, st>>>(small ? t->absorbed : partial, small ? ncells : kReduceBlocks,
+                                                            t->scalars, t->status, out, back);
   RT_CUDA_TRY(cudaGetLastError());
-  k_final<<<1, 32, 0, st>>>(scr.as<double>(), kReduceBlocks, t->scalars);
-  RT_CUDA_TRY(cudaGetLastError());
-  uint32_t bits = 0;
-  RT_CUDA_TRY(cudaMemcpyAsync(host_scalars, t->scalars, 4 * sizeof(double), cudaMemcpyDeviceToHost, st));
-  if (host_absorbed)
+  double buf[5 + kSmall];
+  if (host_absorbed && !back)
     RT_CUDA_TRY(cudaMemcpyAsync(host_absorbed, t->absorbed, (size_t)ncells * sizeof(double),
                                 cudaMemcpyDeviceToHost, st));
-  RT_CUDA_TRY(cudaMemcpyAsync(&bits, t->status, sizeof(bits), cudaMemcpyDeviceToHost, st));
+  RT_CUDA_TRY(cudaMemcpyAsync(buf, out, (size_t)(5 + back) * sizeof(double), cudaMemcpyDeviceToHost, st));
   RT_CUDA_TRY(cudaStreamSynchronize(st));
-  return status_from_bits(bits);
+  for (int i = 0; i < 4; ++i) host_scalars[i] = buf[i];
+  for (int i = 0; i < back; ++i) host_absorbed[i] = buf[5 + i];
+  return status_from_bits((uint32_t)buf[4]);
+}
+
+rt_status tally_zero_impl(const rt_tally_buf *t, int64_t ncells, cudaStream_t st) {
+  if (!t || !t->absorbed || !t->scalars || !t->steps || !t->status || ncells < 1)
+    return fail(RT_E_INVAL, "rt_tally_zero: bad tally buffer");
+  k_tally_zero<<<(unsigned)std::min<int64_t>((ncells + 255) / 256, 1 << 16), 256, 0, st>>>(t->absorbed, ncells, t->scalars, t->steps, t->status);
+  RT_CUDA_TRY(cudaGetLastError());
+  return RT_OK;
 }
 
 }  // namespace rt
@@ -539,6 +614,10 @@ rt_status rt_trace(const rt_grid *grid, const float *kappa, const rt_spectral *s
                    const rt_record *record, void *stream) {
   return rt::trace_impl(grid, kappa, spec, ray_begin, n_rays, n_rays_total, seed, enclosure, flags,
                         tally, record, (cudaStream_t)stream);
+}
+
+rt_status rt_tally_zero(const rt_tally_buf *tally, int64_t ncells, void *stream) {
+  return rt::tally_zero_impl(tally, ncells, (cudaStream_t)stream);
 }
 
 rt_status rt_tally(const rt_tally_buf *tally, int64_t ncells, double *host_absorbed,

@@ -416,8 +416,6 @@ rt_status walk_setup(const rt_grid *grid, const rt_spectral *spec, uint64_t ray_
                      uint64_t n_rays, uint64_t n_total, uint64_t seed, uint32_t enclosure,
                      int32_t flags, const rt_tally_buf *tally, const rt_record *record,
                      WalkParams *W, RecordPtrs *rp);
-// Host: wavenumber-major copy tabt[j * nT + k] of a T-major table.
-rt_status launch_transpose(const float *tab, int nT, long long n_nu, float *tabt, cudaStream_t st);
 // Host: the walk's copy of a T-major table: node pairs (layout 2) when nT >= 2 and the
 // pair table fits kPairTableBytes (so that it can stay in L2), else wavenumber-major (1).
 constexpr size_t kPairTableBytes = size_t(64) << 20;
