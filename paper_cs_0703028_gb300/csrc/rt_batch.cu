@@ -52,6 +52,7 @@ __global__ void k_cell_prep_batch(const EnclDev *__restrict__ E, const long long
 
 constexpr int kRefillIdleBatch = 16;
 constexpr int kBatchUnroll = 4;
+constexpr int kPassLanesBatch = 14;
 
 template <int TAB>
 __global__ void __launch_bounds__(256, 4)
@@ -94,15 +95,17 @@ k_walk_batch(const EnclDev *__restrict__ E, const long long *__restrict__ item_o
     bool active = false;
     for (;;) {
       const unsigned idle = __ballot_sync(0xffffffffu, !active);
+      bool fresh = false;  // rays loaded for this pass
       if (next < last && (idle == 0xffffffffu || __popc(idle) >= kRefillIdleBatch)) {
         const unsigned rank = __popc(idle & ((1u << lane) - 1u));
         if (!active && next + rank < last) {
-          ray_init(W, cells, tab, next + rank, false, R, &cd);
+          ray_init<TAB>(W, cells, tab, next + rank, false, R, &cd);
           if (TAB == 2) krow = reinterpret_cast<const float2 *>(tab) + (long long)R.j * (W.nT - 1);
           if (TAB == 1) krow1 = tab + (long long)R.j * W.nT;
           active = true;
         }
         next += __popc(idle);
+        fresh = true;
       }
       const unsigned am = __ballot_sync(0xffffffffu, active);
       if (!am) break;
@@ -110,8 +113,10 @@ k_walk_batch(const EnclDev *__restrict__ E, const long long *__restrict__ item_o
       bool done = false, dark = false;
 #pragma unroll
       for (int u = 0; u < kBatchUnroll; ++u) {  // steps per pass of the loop
+        // few lanes left of newly loaded rays (an opaque gas): load the next ones
+        if (u == 1 && fresh && __popc(__ballot_sync(am, !done)) < kPassLanesBatch) break;
         if (!done) {
-          const float kap = TAB == 2 ? cell_kappa_row(cd, krow) : (TAB == 1 ? cell_kappa_row1(cd, krow1, W.nT) : cell_kappa_l<TAB>(cd, tab, W.nT, W.n_nu, R.j));
+          const float kap = TAB == 2 ? cell_kappa_row(cd, krow) : cell_kappa_row1(cd, krow1, W.nT);
           float4 cdn = cd;
           done = ray_step<false, false, true>(W, kap, D.absorbed, D.status, rec, R, true,
                                               [&](int c) { cdn = __ldg(cells + c); }, s_axes[warp]);
@@ -191,7 +196,6 @@ static rt_status batch_build(int32_t n_encl, const rt_enclosure *encl, const rt_
       snprintf(msg, sizeof(msg), "%s", rt_last_error());
       return fail(v, "enclosure %d: %s", e, msg);
     }
-    H[e].W.nu_major = walk_table_layout(spec->nT, spec->n_nu);
     H[e].T = encl[e].grid.T;
     H[e].p = encl[e].grid.p_atm;
     H[e].x = encl[e].grid.x;

@@ -117,7 +117,7 @@ k_walk_lbl(const int4 *__restrict__ R, const float4 *__restrict__ L0, const floa
   unsigned long long nsteps = 0;
   for (unsigned long long rr = wid; rr < W.n_rays; rr += nwarps) {
     Ray Ry;
-    ray_init(W, nullptr, nullptr, rr, record, Ry);
+    ray_init<0>(W, nullptr, nullptr, rr, record, Ry);
     const long long l0 = first_hi_ge(R, n_lines, Ry.j);
     const long long l1 = first_lo_gt(R, n_lines, Ry.j);
     for (;;) {

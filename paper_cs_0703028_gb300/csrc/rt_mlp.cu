@@ -1420,7 +1420,7 @@ k_walk_mlp(const float *__restrict__ P, const uint16_t *__restrict__ tiles, Norm
       if (owner && !active) {
         const unsigned long long claim = atomicAdd(&S.next, 1ull);
         if (claim < S.end) {
-          ray_init(W, nullptr, nullptr, B.order ? (unsigned long long)B.order[claim] : claim, record, R);
+          ray_init<0>(W, nullptr, nullptr, B.order ? (unsigned long long)B.order[claim] : claim, record, R);
           active = true;
         }
       }

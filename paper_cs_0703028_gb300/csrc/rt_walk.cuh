@@ -50,7 +50,6 @@ struct WalkParams {
   uint32_t div_m[2], div_s[2];  // c / n[0], c / n[1] as (c * div_m) >> div_s, c < 2^31
   long long ncells, n_nu;
   int nT, mode, tau_cut, step_cap;
-  int nu_major;  // walk table layout: 0 T-major, 1 wavenumber-major, 2 wavenumber-major node pairs
   unsigned long long ray_begin, n_rays;
   uint32_t seed_lo, seed_hi, enclosure;
   float nu_min, dnu;
@@ -83,57 +82,20 @@ __device__ __forceinline__ bool marsaglia(uint32_t ua, uint32_t ub, float &dx, f
   return true;
 }
 
-// kappa of a cell from the table, linear in T between its bracketing nodes, times
-// the density scale.  T-major table: tab[k * n_nu + j].
-__device__ __forceinline__ float cell_kappa(const float4 cd, const float *__restrict__ tab,
-                                            long long n_nu, int nT, long long j) {
-  const int k = __float_as_int(cd.w);
-  const float v0 = __ldg(tab + (long long)k * n_nu + j);
-  if (nT < 2) return cd.y * v0;
-  const float v1 = __ldg(tab + (long long)(k + 1) * n_nu + j);
-  return cd.y * fmaf(cd.x, v1, (1.0f - cd.x) * v0);
-}
-
-// The same from a wavenumber-major copy tabt[j * nT + k]: both nodes share a cache line.
-__device__ __forceinline__ float cell_kappa_t(const float4 cd, const float *__restrict__ tabt, int nT,
-                                              long long j) {
-  const int k = __float_as_int(cd.w);
-  const float *c = tabt + j * (long long)nT + k;
-  const float v0 = __ldg(c);
-  if (nT < 2) return cd.y * v0;
-  const float v1 = __ldg(c + 1);
-  return cd.y * fmaf(cd.x, v1, (1.0f - cd.x) * v0);
-}
-
-// The same from node pairs tabp[j * (nT - 1) + k] = {kappa_k, kappa_k+1}: one 8-byte load.
-__device__ __forceinline__ float cell_kappa_p(const float4 cd, const float *__restrict__ tabp, int nT,
-                                              long long j) {
-  const int k = __float_as_int(cd.w);
-  const float2 v = __ldg(reinterpret_cast<const float2 *>(tabp) + j * (long long)(nT - 1) + k);
-  return cd.y * fmaf(cd.x, v.y, (1.0f - cd.x) * v.x);
-}
-
-// The same from the ray's row of node pairs, row = tabp + j (nT - 1).
+// kappa of a cell from the walk table, linear in T between its bracketing nodes, times the
+// density scale.
+// From the ray's row of node pairs (layout 2), row = tabp + j (nT - 1).
 __device__ __forceinline__ float cell_kappa_row(const float4 cd, const float2 *__restrict__ row) {
   const float2 v = __ldg(row + __float_as_int(cd.w));
   return cd.y * fmaf(cd.x, v.y, (1.0f - cd.x) * v.x);
 }
 
-// The same from the ray's row of a wavenumber-major table, row = tabt + j nT.
+// From the ray's row of a wavenumber-major table (layout 1), row = tabt + j nT.
 __device__ __forceinline__ float cell_kappa_row1(const float4 cd, const float *__restrict__ row, int nT) {
   const float *c = row + __float_as_int(cd.w);
   const float v0 = __ldg(c);
   if (nT < 2) return cd.y * v0;
   return cd.y * fmaf(cd.x, __ldg(c + 1), (1.0f - cd.x) * v0);
-}
-
-// kappa of a cell from the walk table in layout L (0 T-major, 1 wavenumber-major, 2 pairs).
-template <int L>
-__device__ __forceinline__ float cell_kappa_l(const float4 cd, const float *__restrict__ tab, int nT,
-                                              long long n_nu, long long j) {
-  if (L == 2) return cell_kappa_p(cd, tab, nT, j);
-  if (L == 1) return cell_kappa_t(cd, tab, nT, j);
-  return cell_kappa(cd, tab, n_nu, nT, j);
 }
 
 __device__ __forceinline__ float tmax_of(int i, int step, float h, float pos, float invd) {
@@ -159,6 +121,10 @@ struct Ray {
 
 // Philox draws -> emission cell, wavenumber, position, direction, weight; DDA set-up.
 // *cd_out (if given; walks with a table) receives the data of the first cell.
+// TAB: the walk table's layout (1 or 2; 0: no table).  The cell's record is loaded as soon as
+// the first draw names it and the table as soon as the record is there, so that the
+// direction's draws and the set-up arithmetic run under the two dependent gathers.
+template <int TAB>
 __device__ __forceinline__ void ray_init(const WalkParams &W, const float4 *__restrict__ cells,
                                          const float *__restrict__ tab, unsigned long long rr,
                                          bool record, Ray &R, float4 *cd_out = nullptr) {
@@ -179,6 +145,8 @@ __device__ __forceinline__ void ray_init(const WalkParams &W, const float4 *__re
     const long long c = (long long)(((unsigned long long)v.x * (unsigned long long)W.ncells) >> 32);
     R.j = (int)(((unsigned long long)v.y * (unsigned long long)W.n_nu) >> 32);
     const float fx = u24(v.z), fy = u24(v.w);
+    float4 cd = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    if (TAB) cd = __ldg(cells + c);
     ctr.z = 1u;
     v = philox4x32_10(ctr, W.seed_lo, W.seed_hi);
     const float fz = u24(v.x);
@@ -190,6 +158,14 @@ __device__ __forceinline__ void ray_init(const WalkParams &W, const float4 *__re
       if (!ok) ok = marsaglia(v.z, v.w, dx, dy, dz);
     }
     if (!ok) { dx = 0.0f; dy = 0.0f; dz = 1.0f; }
+    float2 node = make_float2(0.0f, 0.0f);  // kappa of the cell's two nodes
+    if (TAB == 2) {
+      node = __ldg(reinterpret_cast<const float2 *>(tab) + (long long)R.j * (W.nT - 1) + __float_as_int(cd.w));
+    } else if (TAB == 1) {
+      const float *p = tab + (long long)R.j * W.nT + __float_as_int(cd.w);
+      node.x = __ldg(p);
+      if (W.nT >= 2) node.y = __ldg(p + 1);
+    }
     // cell index -> (ix, iy, iz) in 32-bit unsigned arithmetic (c < ncells < 2^31)
     // with the divisors' reciprocals (exact for 31-bit dividends)
     const uint32_t cu = (uint32_t)c, n0 = (uint32_t)W.n[0], n1 = (uint32_t)W.n[1];
@@ -202,11 +178,8 @@ __device__ __forceinline__ void ray_init(const WalkParams &W, const float4 *__re
     R.py = W.fin[1] ? __fmul_rn(__fadd_rn((float)R.iy, fy), W.h[1]) : 0.0f;
     R.pz = W.fin[2] ? __fmul_rn(__fadd_rn((float)R.iz, fz), W.h[2]) : 0.0f;
     // emission weight from the table; walks without a table set it at their first step
-    if (tab) {
-      const float4 cd = cells[c];
-      const float ke = W.nu_major == 2 ? cell_kappa_p(cd, tab, W.nT, R.j)
-                       : (W.nu_major == 1 ? cell_kappa_t(cd, tab, W.nT, R.j)
-                                          : cell_kappa(cd, tab, W.n_nu, W.nT, R.j));
+    if (TAB) {
+      const float ke = W.nT < 2 ? cd.y * node.x : cd.y * fmaf(cd.x, node.y, (1.0f - cd.x) * node.x);
       R.w = emission_weight(W, R.j, cd.z, ke);
       if (cd_out) *cd_out = cd;
     } else {
