@@ -62,12 +62,13 @@ rt_status Scratch::alloc(size_t bytes, cudaStream_t stream) {
 // then w(z) = 2 sum_{n>=0} a_{n+1} Z^n / (L - iz)^2 + (1/sqrt(pi)) / (L - iz),
 // Z = (L + iz)/(L - iz), L = (N / sqrt 2)^(1/2).  The a_n are the trapezoidal
 // Fourier coefficients on 2M = 4N equispaced angles (psi = 0 at theta = pi).
-void weideman_coefficients(WeidCoef *out) {
-  const int N = kWeidN, M = 2 * N;
+void weideman_coefficients(int N, float *L_out, float *a_out) {
+  constexpr int kMaxM = 4 * kWeidN;  // 2 M for the largest N used
+  const int M = 2 * N;
   const double L = std::sqrt(N / std::sqrt(2.0));
   const double pi = 3.14159265358979323846;
-  double psi[2 * M];
-  double th[2 * M];
+  double psi[kMaxM];
+  double th[kMaxM];
   for (int k = -M; k < M; ++k) {
     double theta = k * pi / M;
     th[k + M] = theta;
@@ -78,12 +79,12 @@ void weideman_coefficients(WeidCoef *out) {
       psi[k + M] = std::exp(-t * t) * (L * L + t * t);
     }
   }
-  out->L = (float)L;
+  *L_out = (float)L;
   const double scale = 2.0 * std::sqrt(pi);
   for (int n = 1; n <= N; ++n) {
     double acc = 0.0;
     for (int k = 0; k < 2 * M; ++k) acc += psi[k] * std::cos(n * th[k]);
-    out->a[n - 1] = (float)(scale * acc / (2 * M));
+    a_out[n - 1] = (float)(scale * acc / (2 * M));
   }
 }
 

@@ -117,10 +117,12 @@ __device__ __forceinline__ df df_from_double(double v) {
 // Measured relative error against binary64: <= 5.3e-7 for |z| >= 8, <= 2.2e-6 for
 // 5 <= |z| < 8, <= 1.5e-6 for |z| < 5 with y >= 0.5 (degrading toward 1e-4 as y -> 0).
 constexpr int kWeidN = 24;
-struct WeidCoef {
+template <int N>
+struct WeidSeries {
   float L;
-  float a[kWeidN];  // 2 sqrt(pi) a_n, n = 1..N
+  float a[N];  // 2 sqrt(pi) a_n, n = 1..N
 };
+using WeidCoef = WeidSeries<kWeidN>;
 
 // bracket of the three-term series; sqrt(pi) Re w = y t S3
 __device__ __forceinline__ float faddeeva_series3(float t, float s) {
@@ -177,8 +179,14 @@ __device__ __forceinline__ float faddeeva_re(float x, float y, const WeidCoef &c
   return faddeeva_re_near(x, y, r2, c);
 }
 
-// Host: Weideman coefficients for N = kWeidN (binary64 DFT, then binary32).
-void weideman_coefficients(WeidCoef *out);
+// Host: Weideman's L and coefficients for N terms (binary64 DFT, then binary32).
+void weideman_coefficients(int N, float *L, float *a);
+template <int N>
+WeidSeries<N> weideman_series() {
+  WeidSeries<N> w;
+  weideman_coefficients(N, &w.L, w.a);
+  return w;
+}
 
 // ---------------------------------------------------------------- misc
 __device__ __forceinline__ void status_or(uint32_t *status, uint32_t bits) {

@@ -129,7 +129,7 @@ __global__ void k_line_geometry(const double *__restrict__ nu0, const double *__
 }
 
 // Eq. (S) times the number density, and the profile's coefficients, for line l
-// at T node k.  Voigt: P = {c0, s dnu, y^2, c2}, P2 = {c3, c4, half-widths of |z| < 20 and < 8}
+// at T node k.  Voigt: P = {c0, s dnu, y^2, c2}, P2 = {c3, c4, y, half-width of |z| < 8}
 // with the far-wing series c0 t + c1 t^2 + c2 t^3 + c3 t^4 + c4 t^5 (c1 = 1.5 c0).
 // Returns the line's far-zone distance in grid units (float bits): beyond it the t^3, t^4
 // and t^5 terms drop at most 1.25 * 2^-24 of the value, so the degree-1 series
@@ -187,15 +187,13 @@ __device__ __forceinline__ void prefactor_one(const double *__restrict__ nu0, co
     const float s = 0.83255461f / alpha;                  // sqrt(ln 2) / alpha
     const float y = s * gam;
     const float sd = s * Q.dnu;
-    // half-width (grid units) of the region |z| < 20 where the far-wing series does not hold
     const float y2 = y * y;
-    const float u_near = sqrtf(fmaxf(400.0f - y2, 0.0f)) / sd;
     // far wing: c0 t (1 + 1.5 t + (3.75 - 2 y^2) t^2 - 15 y^2 t^3 + 12 y^4 t^4), t = 1/|z|^2
     const float c0 = A * s * (float)(1.0 / kPi) * y;
     out = make_float4(c0, sd, y2, __fmaf_rn(-2.0f, y2, 3.75f) * c0);
     // half-width (grid units) of |z| < 8, inside which the general path takes the rational form
     const float u_core = sqrtf(fmaxf(64.0f - y2, 0.0f)) / sd;
-    P2out[(long long)k * Q.n_lines + l] = make_float4(-15.0f * y2 * c0, 12.0f * y2 * y2 * c0, u_near, u_core);
+    P2out[(long long)k * Q.n_lines + l] = make_float4(-15.0f * y2 * c0, 12.0f * y2 * y2 * c0, y, u_core);
     // (27 y^2 / 2^-24)^(1/6) = 27.66 y^(1/3), beyond which 27 y^2 t^3 <= 2^-24 (t <= 1/x^2),
     // and (2^25 (3.75 + 2 y^2))^(1/4), with 5 % margin, in grid units
     const float d2 = 29.1f * cbrtf(y) / sd;
@@ -324,6 +322,15 @@ struct AtNode16 {
 __device__ constexpr NodeTable<16, kTilePts> kTab16 = node_table<16, kTilePts>(kNodes16, AtPoint{});
 __device__ constexpr NodeTable<8, 16> kTab8 = node_table<8, 16>(kNodes8, AtNode16{});
 __device__ constexpr NodeTable<4, 32> kTab4 = node_table<4, 32>(kNodes4, AtPoint{});
+
+// Weideman's series for the core points.  Its error falls fast with y: relative to Re w over
+// |z| < 8.2 (against binary64), 24 terms give 2e-8 at y = 0.1 and 4e-10 at 0.75, 16 terms 2.5e-8
+// at y = 2.3, 12 terms 1.4e-8 at y = 5; each is used from there on.
+struct WeidSet {
+  WeidSeries<24> n24;
+  WeidSeries<16> n16;
+  WeidSeries<12> n12;
+};
 
 // Kinds of line ranges within a tile (see k_tile_lines).
 enum SegKind : int {
@@ -510,7 +517,8 @@ template <int PROFILE, bool ADAPT>
 __global__ void __launch_bounds__(32 * kMaxTPerBlock, 3)
 k_kappa(const float4 *__restrict__ P, const float4 *__restrict__ P2, const int4 *__restrict__ R,
         const int2 *__restrict__ AW,
-        const int4 *__restrict__ tiles, long long n_lines, long long n_nu, int nT, WeidCoef wc,
+        const int4 *__restrict__ tiles, long long n_lines, long long n_nu, int nT,
+        const __grid_constant__ WeidSet ws,
         int vec_ok, int accumulate, float *__restrict__ kappa, uint32_t *status) {
   constexpr bool kVoigt = PROFILE == RT_PROFILE_VOIGT;
   constexpr int kCap = ADAPT ? 128 : kChunk, kCapP2 = kCap / 2;  // lines of a chunk: P only, P and P2
@@ -838,46 +846,58 @@ k_kappa(const float4 *__restrict__ P, const float4 *__restrict__ P2, const int4 
     // pass (a line has 16 to 40 such points on a 0.005 cm^-1 grid: 32 lanes take them in one
     // or two passes), into shared memory for their owners.
     auto core_values = [&](int ia, int ib, int fa, int fb, int n) {
-      float2 *res = reinterpret_cast<float2 *>(s_res[warp]);
       const float4 pa = cP[ia], pb = cP[ib];
       const int2 ra = *reinterpret_cast<const int2 *>(&cR[ia].z), rb = *reinterpret_cast<const int2 *>(&cR[ib].z);
-      const float2 y = make_float2(sqrtf(pa.z), sqrtf(pb.z));
+      const float2 y = make_float2(cP2[ia].z, cP2[ib].z);
       const float2 coef = make_float2(__fdividef(pa.x, y.x), __fdividef(pb.x, y.y));
-      const float2 dr = __fadd2_rn(dup2(wc.L), y), nr = __fadd2_rn(dup2(wc.L), neg2(y));
+      const float2 sd = make_float2(pa.y, pb.y), dg = make_float2(__int_as_float(ra.y), __int_as_float(rb.y));
+      const float2 first = make_float2((float)(jw0 + fa - ra.x), (float)(jw0 + fb - rb.x));
+      float *res = s_res[warp];  // the first line's at 0, the second's at kTilePts
+      auto points = [&](auto &wc) {
+        constexpr int N = sizeof(wc.a) / sizeof(float);
+        const float2 dr = __fadd2_rn(dup2(wc.L), y), nr = __fadd2_rn(dup2(wc.L), neg2(y));
 #pragma unroll 1
-      for (int e = lane; e < n; e += 32) {
-        const float2 x = make_float2(pa.y * point_offset(jw0 + fa + e, ra.x, ra.y),
-                                     pb.y * point_offset(jw0 + fb + e, rb.x, rb.y));
-        // iz = -y + ix, v = 1 / (L - iz), Z = (L + iz) v; sqrt(pi) w = v (p(Z) v + 1)
-        const float2 d = __ffma2_rn(dr, dr, __fmul2_rn(x, x));
-        const float2 inv = make_float2(__frcp_rn(d.x), __frcp_rn(d.y));
-        const float2 vr = __fmul2_rn(dr, inv), vi = __fmul2_rn(x, inv);
-        const float2 zr = __ffma2_rn(nr, vr, neg2(__fmul2_rn(x, vi))), zi = __ffma2_rn(nr, vi, __fmul2_rn(x, vr));
-        const float2 nzi = neg2(zi);
-        float2 pr = dup2(wc.a[kWeidN - 1]), pi = make_float2(0.0f, 0.0f);
+        for (int e = lane; e < n; e += 32) {
+          const float2 x = __fmul2_rn(sd, __fadd2_rn(__fadd2_rn(first, dup2((float)e)), dg));
+          // iz = -y + ix, v = 1 / (L - iz), Z = (L + iz) v; sqrt(pi) w = v (p(Z) v + 1)
+          const float2 d = __ffma2_rn(dr, dr, __fmul2_rn(x, x));
+          float2 inv = rcp2(d);  // one Newton step: within a rounding of 1 / d
+          inv = __ffma2_rn(inv, __ffma2_rn(neg2(d), inv, dup2(1.0f)), inv);
+          const float2 vr = __fmul2_rn(dr, inv), vi = __fmul2_rn(x, inv);
+          const float2 zr = __ffma2_rn(nr, vr, neg2(__fmul2_rn(x, vi))), zi = __ffma2_rn(nr, vi, __fmul2_rn(x, vr));
+          const float2 nzi = neg2(zi);
+          float2 pr = dup2(wc.a[N - 1]), pi = make_float2(0.0f, 0.0f);
 #pragma unroll
-        for (int n = kWeidN - 2; n >= 0; --n) {
-          const float2 t = __ffma2_rn(pr, zr, __ffma2_rn(pi, nzi, dup2(wc.a[n])));
-          pi = __ffma2_rn(pr, zi, __fmul2_rn(pi, zr));
-          pr = t;
+          for (int n = N - 2; n >= 0; --n) {
+            const float2 t = __ffma2_rn(pr, zr, __ffma2_rn(pi, nzi, dup2(wc.a[n])));
+            pi = __ffma2_rn(pr, zi, __fmul2_rn(pi, zr));
+            pr = t;
+          }
+          const float2 nvi = neg2(vi);
+          const float2 qr = __fadd2_rn(__ffma2_rn(pr, vr, __fmul2_rn(pi, nvi)), dup2(1.0f));
+          const float2 qi = __ffma2_rn(pr, vi, __fmul2_rn(pi, vr));
+          const float2 w = __fmul2_rn(coef, __ffma2_rn(vr, qr, __fmul2_rn(nvi, qi)));
+          res[e] = w.x;
+          res[kTilePts + e] = w.y;
         }
-        const float2 nvi = neg2(vi);
-        const float2 qr = __fadd2_rn(__ffma2_rn(pr, vr, __fmul2_rn(pi, nvi)), dup2(1.0f));
-        const float2 qi = __ffma2_rn(pr, vi, __fmul2_rn(pi, vr));
-        res[e] = __fmul2_rn(coef, __ffma2_rn(vr, qr, __fmul2_rn(nvi, qi)));
-      }
+      };
+      // fewer terms where the line is broad (warp-uniform; see WeidSet)
+      const float ymin = fminf(y.x, y.y);
+      if (ymin >= 5.0f) points(ws.n12);
+      else if (ymin >= 2.3f) points(ws.n16);
+      else points(ws.n24);
       __syncwarp();
     };
-    // the lane's points among the n core points from tile point `first` on: values c of res
+    // the lane's points among the n core points from tile point `first` on, from res + c
     auto take_core = [&](int c, int first, int n, float2 (&v)[kPairs]) {
-      const float *res = s_res[warp] + c;
       const int a = lane * kPtsPerThread - first;  // the lane's first point in res
-      if (a + kPtsPerThread > 0 && a < n) {
+      if (a + kPtsPerThread <= 0 || a >= n) return;
+      const float *res = s_res[warp] + c + a;
+      const unsigned in = (n - a >= kPtsPerThread ? 0xffu : (1u << (n - a)) - 1u) & (a >= 0 ? 0xffu : 0xffu << -a);
 #pragma unroll
-        for (int h = 0; h < kPairs; ++h) {
-          if ((unsigned)(a + 2 * h) < (unsigned)n) v[h].x = res[2 * (a + 2 * h)];
-          if ((unsigned)(a + 2 * h + 1) < (unsigned)n) v[h].y = res[2 * (a + 2 * h + 1)];
-        }
+      for (int h = 0; h < kPairs; ++h) {
+        if ((in >> (2 * h)) & 1u) v[h].x = res[2 * h];
+        if ((in >> (2 * h + 1)) & 1u) v[h].y = res[2 * h + 1];
       }
     };
     auto mask_window = [&](int i, float2 (&v)[kPairs]) {
@@ -909,7 +929,7 @@ k_kappa(const float4 *__restrict__ P, const float4 *__restrict__ P2, const int4 
         mask_window(i, v);
         if (two) {
           line_series(j, w);
-          if (nb > 0) take_core(1, fb, nb, w);
+          if (nb > 0) take_core(kTilePts, fb, nb, w);
           mask_window(j, w);
 #pragma unroll
           for (int h = 0; h < kPairs; ++h) v[h] = __fadd2_rn(v[h], w[h]);
@@ -1265,9 +1285,8 @@ rt_status launch_kappa(const float4 *P, const float4 *P2, const int4 *R, int4 *t
                        const unsigned *far_bits, const int2 *AW, long long n, const rt_spectral *spec,
                        double nu_abs_max, double mass_amu, float *kappa, uint32_t *status,
                        cudaStream_t st) {
-  static WeidCoef wc;
-  static std::once_flag wc_once;
-  std::call_once(wc_once, [] { weideman_coefficients(&wc); });
+  static const WeidSet ws{weideman_series<24>(), weideman_series<16>(), weideman_series<12>()};
+  const WeidCoef &wc = ws.n24;
   // W bounds every line's near-centre half-width sqrt(400 - y^2) / (s dnu) <= 20 alpha /
   // (sqrt(ln 2) dnu), alpha the largest Doppler half-width of a line that reaches the grid
   int W = 0;
@@ -1300,7 +1319,7 @@ rt_status launch_kappa(const float4 *P, const float4 *P2, const int4 *R, int4 *t
   auto kernel = spec->profile == RT_PROFILE_LORENTZ
                     ? (AW ? k_kappa<RT_PROFILE_LORENTZ, true> : k_kappa<RT_PROFILE_LORENTZ, false>)
                     : (AW ? k_kappa<RT_PROFILE_VOIGT, true> : k_kappa<RT_PROFILE_VOIGT, false>);
-  kernel<<<gk, 32 * tpb, 0, st>>>(P, P2, R, AW, tiles, n, spec->n_nu, spec->nT, wc, vec_ok,
+  kernel<<<gk, 32 * tpb, 0, st>>>(P, P2, R, AW, tiles, n, spec->n_nu, spec->nT, ws, vec_ok,
                                   spec->accumulate ? 1 : 0, kappa, status);
   RT_CUDA_TRY(cudaGetLastError());
   return RT_OK;

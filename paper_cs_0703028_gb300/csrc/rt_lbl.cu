@@ -216,8 +216,7 @@ rt_status trace_lbl_impl(const rt_grid *grid, const rt_lines *lines, const rt_sp
   K.u_coef = (float)(kAtm / kKB * 1e-6);
   K.sqrt_ln2 = (float)std::sqrt(std::log(2.0));
   K.inv_pi = (float)(1.0 / kPi);
-  WeidCoef wc;
-  weideman_coefficients(&wc);
+  const WeidCoef wc = weideman_series<kWeidN>();
   int dev = 0, sms = 0;
   RT_CUDA_TRY(cudaGetDevice(&dev));
   RT_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
