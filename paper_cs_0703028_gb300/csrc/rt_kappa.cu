@@ -21,6 +21,7 @@
 //   k_kappa_ppl     : with a fixed number of points per line, one thread per
 //                     point and eight T nodes over the few lines whose windows hold it.
 #include <cmath>
+#include <cstring>
 #include <mutex>
 #include <type_traits>
 
@@ -33,6 +34,8 @@ constexpr int kPtsPerThread = 8;
 constexpr int kTilePts = 32 * kPtsPerThread;  // 256 wavenumbers per block, one warp per T node
 constexpr int kMaxTPerBlock = 8;              // warps (T nodes) per block
 constexpr int kChunk = 192;                   // lines per staged chunk that need P only (half that with P2)
+constexpr int kStagedLines = 2048;            // host lists up to this go through pinned memory
+constexpr int kDirectPairs = 8192;            // (node, line) pairs up to which the kernels read them there
 constexpr int kGroup = 8;                     // fast-path lines summed before one compensated add
 constexpr int kNodeGroup = 4;                 // interpolated lines a lane sums before one compensated add
 constexpr unsigned kWaitLimit = 1u << 22;     // bounded mbarrier waits
@@ -63,11 +66,10 @@ __device__ __forceinline__ double grid_nu(double nu_min, long long j, double dnu
   return __dadd_rn(nu_min, __dmul_rn((double)j, dnu));
 }
 
-__global__ void k_line_geometry(const double *__restrict__ nu0, const double *__restrict__ S,
-                                const double *__restrict__ g, const double *__restrict__ E,
-                                GeomParams P, int4 *__restrict__ R,
-                                unsigned long long *evals, uint32_t *status) {
-  const long long l = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+__device__ __forceinline__ void line_geometry(const double *__restrict__ nu0, const double *__restrict__ S,
+                                              const double *__restrict__ g, const double *__restrict__ E,
+                                              const GeomParams &P, int4 *__restrict__ R,
+                                              unsigned long long *evals, uint32_t *status, long long l) {
   unsigned long long cnt = 0;
   if (l < P.n_lines) {
     const double v = nu0[l];
@@ -126,6 +128,13 @@ __global__ void k_line_geometry(const double *__restrict__ nu0, const double *__
     for (int o = 16; o > 0; o >>= 1) cnt += __shfl_down_sync(0xffffffffu, cnt, o);
     if ((threadIdx.x & 31) == 0 && cnt) atomicAdd(evals, cnt);
   }
+}
+
+__global__ void k_line_geometry(const double *__restrict__ nu0, const double *__restrict__ S,
+                                const double *__restrict__ g, const double *__restrict__ E,
+                                GeomParams P, int4 *__restrict__ R,
+                                unsigned long long *evals, uint32_t *status) {
+  line_geometry(nu0, S, g, E, P, R, evals, status, (long long)blockIdx.x * blockDim.x + threadIdx.x);
 }
 
 // Eq. (S) times the number density, and the profile's coefficients, for line l
@@ -203,12 +212,10 @@ __device__ __forceinline__ void prefactor_one(const double *__restrict__ nu0, co
   Pout[(long long)k * Q.n_lines + l] = out;
 }
 
-__global__ void k_prefactor(const double *__restrict__ nu0, const double *__restrict__ S,
-                            const double *__restrict__ g, const double *__restrict__ E,
-                            PrefParams Q, float4 *__restrict__ Pout, float4 *__restrict__ P2out,
-                            unsigned *__restrict__ far_bits) {
-  const long long l = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  const int k = blockIdx.y;
+__device__ __forceinline__ void prefactors(const double *__restrict__ nu0, const double *__restrict__ S,
+                                           const double *__restrict__ g, const double *__restrict__ E,
+                                           const PrefParams &Q, float4 *__restrict__ Pout, float4 *__restrict__ P2out,
+                                           unsigned *__restrict__ far_bits, long long l, int k) {
   __shared__ PrefNode s_node;  // T node k's shared quantities, formed once per block
   if (threadIdx.x == 0) s_node = pref_node(Q, k);
   __syncthreads();
@@ -227,6 +234,26 @@ __global__ void k_prefactor(const double *__restrict__ nu0, const double *__rest
   }
 }
 
+// The lines' set-up in one launch: line_blocks blocks of k_line_geometry's work, then as many
+// for each T node's prefactors (neither reads what the other writes).
+__global__ void k_line_setup(const double *__restrict__ nu0, const double *__restrict__ S,
+                             const double *__restrict__ g, const double *__restrict__ E, GeomParams G, PrefParams Q,
+                             unsigned line_blocks, int4 *__restrict__ R, float4 *__restrict__ Pout,
+                             float4 *__restrict__ P2out, unsigned *__restrict__ far_bits,
+                             unsigned long long *evals, uint32_t *status) {
+  const unsigned y = blockIdx.x / line_blocks;
+  const long long l = (long long)(blockIdx.x - y * line_blocks) * blockDim.x + threadIdx.x;
+  if (y == 0) line_geometry(nu0, S, g, E, G, R, evals, status, l);
+  else prefactors(nu0, S, g, E, Q, Pout, P2out, far_bits, l, (int)y - 1);
+}
+
+// The prefactors alone, nodes along grid.y (sizes whose blocks exceed one grid axis).
+__global__ void k_prefactor(const double *__restrict__ nu0, const double *__restrict__ S,
+                            const double *__restrict__ g, const double *__restrict__ E,
+                            PrefParams Q, float4 *__restrict__ Pout, float4 *__restrict__ P2out,
+                            unsigned *__restrict__ far_bits) {
+  prefactors(nu0, S, g, E, Q, Pout, P2out, far_bits, (long long)blockIdx.x * blockDim.x + threadIdx.x, blockIdx.y);
+}
 
 // ---- bulk asynchronous copies global -> shared, completed on an mbarrier
 __device__ __forceinline__ uint32_t smem_u32(const void *p) {
@@ -1426,33 +1453,124 @@ rt_status validate_build_args(const rt_lines *lines, const rt_spectral *spec, fl
   return RT_OK;
 }
 
-// Everything after validation, on scratch laid out by kappa_layout.
-rt_status run_build(char *base, const KappaLayout &L, const rt_lines *lines, const rt_spectral *spec,
+// Small host lists are handed to the GPU through pinned memory: read from there by the set-up
+// kernels where few (node, line) pairs do, else in one copy, instead of four copies out of
+// pageable memory (about 2 us of device time each; a 500-line table 41 -> 33 us).  Per host
+// thread, kSlots buffers of kStagedLines lines (64 KB each) in turn, each with an event that
+// tells when the work of its last call has read it; freed when the thread ends.
+class LineStage {
+ public:
+  ~LineStage() { release(); }
+  // The four arrays packed into a slot (n values each), or nullptr: a capturing stream, whose
+  // replays would read the slot again; a list too long; no pinned memory.
+  const double *pack(const double *const (&src)[4], long long n, cudaStream_t st) {
+    const Relaxed relaxed;
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    int dev = 0;
+    if (n > kStagedLines || cudaStreamIsCapturing(st, &capture) != cudaSuccess ||
+        capture != cudaStreamCaptureStatusNone || cudaGetDevice(&dev) != cudaSuccess || !ready(dev))
+      return nullptr;
+    if (cudaEventSynchronize(ev_[next_]) != cudaSuccess) {  // its device was reset: start over
+      cudaGetLastError();
+      release();
+      return nullptr;
+    }
+    double *b = buf_ + (size_t)next_ * 4 * kStagedLines;
+    for (int q = 0; q < 4; ++q) std::memcpy(b + q * n, src[q], (size_t)n * sizeof(double));
+    return b;
+  }
+  // Everything that reads the packed slot is queued on st.
+  void queued(cudaStream_t st) {
+    const Relaxed relaxed;
+    if (cudaEventRecord(ev_[next_], st) != cudaSuccess) {
+      cudaGetLastError();
+      cudaStreamSynchronize(st);
+    }
+    next_ = (next_ + 1) % kSlots;
+  }
+
+ private:
+  // another thread's capture is not disturbed by what this one does to its own buffers
+  struct Relaxed {
+    mutable cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    Relaxed() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~Relaxed() { cudaThreadExchangeStreamCaptureMode(&mode); }
+  };
+  static constexpr int kSlots = 4;
+  bool ready(int dev) {
+    if (buf_ && dev == dev_) return true;
+    release();  // events belong to a device
+    if (cudaHostAlloc(&buf_, kSlots * 4 * kStagedLines * sizeof(double), cudaHostAllocPortable) != cudaSuccess) {
+      cudaGetLastError();
+      buf_ = nullptr;
+      return false;
+    }
+    for (n_ev_ = 0; n_ev_ < kSlots; ++n_ev_)
+      if (cudaEventCreateWithFlags(&ev_[n_ev_], cudaEventDisableTiming) != cudaSuccess) {
+        cudaGetLastError();
+        release();
+        return false;
+      }
+    dev_ = dev;
+    return true;
+  }
+  void release() {
+    for (int i = 0; i < n_ev_; ++i) {
+      cudaEventSynchronize(ev_[i]);
+      cudaEventDestroy(ev_[i]);
+    }
+    n_ev_ = 0;
+    if (buf_) cudaFreeHost(buf_);
+    buf_ = nullptr;
+    cudaGetLastError();
+  }
+  double *buf_ = nullptr;
+  cudaEvent_t ev_[kSlots] = {};
+  int n_ev_ = 0, next_ = 0, dev_ = -1;
+};
+
+// Everything after validation, on scratch laid out by kappa_layout.  staged: small host lists
+// may go through the thread's pinned buffers (the allocation-free entry has none).
+rt_status run_build(char *base, const KappaLayout &L, const rt_lines *lines, const rt_spectral *spec, bool staged,
                     float *kappa, unsigned long long *evals_out, uint32_t *status, cudaStream_t st) {
   const long long n = lines->n;
   const double *d_nu0 = lines->nu0, *d_S = lines->S_ref, *d_g = lines->gamma_ref, *d_E = lines->E_lower;
+  unsigned *far_bits = reinterpret_cast<unsigned *>(base + L.off_far);
+  // a packed slot is given back once everything below that reads it is queued
+  struct SlotUser {
+    LineStage *stage = nullptr;
+    cudaStream_t st = nullptr;
+    ~SlotUser() {
+      if (stage) stage->queued(st);
+    }
+  } user;
   if (lines->memory == RT_MEM_HOST) {
+    static thread_local LineStage stage;
     double *d = reinterpret_cast<double *>(base);
-    RT_CUDA_TRY(cudaMemcpyAsync(d, lines->nu0, n * sizeof(double), cudaMemcpyHostToDevice, st));
-    RT_CUDA_TRY(cudaMemcpyAsync(d + n, lines->S_ref, n * sizeof(double), cudaMemcpyHostToDevice, st));
-    RT_CUDA_TRY(cudaMemcpyAsync(d + 2 * n, lines->gamma_ref, n * sizeof(double), cudaMemcpyHostToDevice, st));
-    RT_CUDA_TRY(cudaMemcpyAsync(d + 3 * n, lines->E_lower, n * sizeof(double), cudaMemcpyHostToDevice, st));
+    const double *src[4] = {lines->nu0, lines->S_ref, lines->gamma_ref, lines->E_lower};
+    const double *slot = staged ? stage.pack(src, n, st) : nullptr;
+    if (slot) {
+      user.stage = &stage;
+      user.st = st;
+      if (n * spec->nT <= kDirectPairs)
+        d = const_cast<double *>(slot);  // read by the kernels (the address is the same on the device)
+      else
+        RT_CUDA_TRY(cudaMemcpyAsync(d, slot, 4 * (size_t)n * sizeof(double), cudaMemcpyHostToDevice, st));
+    } else {
+      for (int q = 0; q < 4; ++q)
+        RT_CUDA_TRY(cudaMemcpyAsync(d + q * n, src[q], (size_t)n * sizeof(double), cudaMemcpyHostToDevice, st));
+    }
     d_nu0 = d; d_S = d + n; d_g = d + 2 * n; d_E = d + 3 * n;
   }
   int4 *R = reinterpret_cast<int4 *>(base + L.off_R);
   float4 *P = reinterpret_cast<float4 *>(base + L.off_P);
   float4 *P2 = reinterpret_cast<float4 *>(base + L.off_P2);
   int4 *tiles = reinterpret_cast<int4 *>(base + L.off_tiles);
-  unsigned *far_bits = reinterpret_cast<unsigned *>(base + L.off_far);
 
   GeomParams G{spec->nu_min, spec->dnu, 1.0 / spec->dnu, spec->cutoff, spec->n_nu, n, spec->nT,
                lines->memory == RT_MEM_DEVICE ? 1 : 0, spec->points_per_line};
   const int tb = 256;
   const bool adaptive = spec->kappa_min > 0;
-  // with adaptive points the evaluations are counted per (node, line) window below
-  k_line_geometry<<<(unsigned)((n + tb - 1) / tb), tb, 0, st>>>(d_nu0, d_S, d_g, d_E, G, R,
-                                                                adaptive ? nullptr : evals_out, status);
-  RT_CUDA_TRY(cudaGetLastError());
   PrefParams Q;
   Q.T_min = spec->T_min;
   Q.T_max = spec->T_max;
@@ -1470,10 +1588,20 @@ rt_status run_build(char *base, const KappaLayout &L, const rt_lines *lines, con
   Q.n_lines = n;
   Q.nT = spec->nT;
   Q.profile = spec->profile;
-  dim3 gp((unsigned)((n + tb - 1) / tb), (unsigned)spec->nT);
   RT_CUDA_TRY(cudaMemsetAsync(far_bits, 0, sizeof(unsigned), st));
-  k_prefactor<<<gp, tb, 0, st>>>(d_nu0, d_S, d_g, d_E, Q, P, P2, far_bits);
-  RT_CUDA_TRY(cudaGetLastError());
+  // with adaptive points the evaluations are counted per (node, line) window below
+  unsigned long long *ev = adaptive ? nullptr : evals_out;
+  const unsigned line_blocks = (unsigned)((n + tb - 1) / tb);
+  if ((unsigned long long)line_blocks * (spec->nT + 1ull) <= 0x7FFFFFFFull) {
+    k_line_setup<<<line_blocks * (spec->nT + 1u), tb, 0, st>>>(d_nu0, d_S, d_g, d_E, G, Q, line_blocks, R, P, P2,
+                                                               far_bits, ev, status);
+    RT_CUDA_TRY(cudaGetLastError());
+  } else {
+    k_line_geometry<<<line_blocks, tb, 0, st>>>(d_nu0, d_S, d_g, d_E, G, R, ev, status);
+    RT_CUDA_TRY(cudaGetLastError());
+    k_prefactor<<<dim3(line_blocks, (unsigned)spec->nT), tb, 0, st>>>(d_nu0, d_S, d_g, d_E, Q, P, P2, far_bits);
+    RT_CUDA_TRY(cudaGetLastError());
+  }
 
   int2 *AW = nullptr;
   if (adaptive) {
@@ -1527,7 +1655,7 @@ rt_status build_kappa_impl(const rt_lines *lines, const rt_spectral *spec, float
   Scratch scr;
   v = scr.alloc(L.total, st);
   if (v != RT_OK) return v;
-  return run_build(scr.as<char>(), L, lines, spec, kappa, evals_out, status, st);
+  return run_build(scr.as<char>(), L, lines, spec, true, kappa, evals_out, status, st);
 }
 
 // ---------------------------------------------------------------------------
@@ -1579,7 +1707,7 @@ rt_status build_kappa_static_impl(const rt_lines *lines, const rt_spectral *spec
   void *scratch = nullptr;
   v = static_scratch_address(&scratch);
   if (v != RT_OK) return v;
-  return run_build(reinterpret_cast<char *>(scratch), L, lines, spec, kappa, evals_out, status, st);
+  return run_build(reinterpret_cast<char *>(scratch), L, lines, spec, false, kappa, evals_out, status, st);
 }
 
 }  // namespace rt
