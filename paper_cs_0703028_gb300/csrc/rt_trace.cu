@@ -190,7 +190,13 @@ k_walk_setup(const float *__restrict__ T, const float *__restrict__ p, const flo
 // Four blocks of 64 registers: at five of 48 the walk spills, and more resident rays share
 // one L1 (8e6 rays of a thin gas in a 75 x 52 x 61 box: 2.29 ms against 2.61 ms; 4e8 rays of
 // the opaque 128^3 box, where it matters least: 15.9 ms against 16.9 ms).
-template <bool REC, int TAB, int REFILL>
+// FEW: a tally of at most kFewCells cells is kept per block in shared memory and added to the
+// caller's at the end; otherwise the rays' deposits queue on few addresses of L2.  Whole trace,
+// global / shared tally: 1e5 rays of a 64-cell slab 64 / 42 us; 3e6 rays of a thin gas in 8^3
+// cells 1049 / 260 us, 12^3 603 / 296, 16^3 561 / 343; 1e5 rays of an opaque gas in 16^3 49 / 54
+// (zeroing and adding 4096 cells a block), so the line lies between 12^3 and 16^3.
+constexpr int kFewCells = 2048;
+template <bool REC, int TAB, int REFILL, bool FEW = false>
 __global__ void __launch_bounds__(kWalkThreads, kWalkBlocks)
 k_walk(const float4 *__restrict__ cells, const float *__restrict__ tab, const uint32_t *__restrict__ order,
        WalkParams W, double *__restrict__ absorbed, double *__restrict__ scalars,
@@ -201,6 +207,10 @@ k_walk(const float4 *__restrict__ cells, const float *__restrict__ tab, const ui
   unsigned long long next = W.n_rays * wid / nwarps;
   const unsigned long long last = W.n_rays * (wid + 1) / nwarps;
   const bool record = REC;
+  __shared__ double s_tally[FEW ? kFewCells : 1];
+  if (FEW)
+    for (int c = threadIdx.x; c < (int)W.ncells; c += kWalkThreads) s_tally[c] = 0.0;
+  double *const tally = FEW ? s_tally : absorbed;
   __shared__ int4 s_axes[3];  // per axis {n, cell stride, h bits}
   if (threadIdx.x < 3) {
     const int a = threadIdx.x;
@@ -244,7 +254,7 @@ k_walk(const float4 *__restrict__ cells, const float *__restrict__ tab, const ui
       if (!done) {
         const float kap = TAB == 2 ? cell_kappa_row(cd, krow) : cell_kappa_row1(cd, krow1, W.nT);
         float4 cdn = cd;
-        done = ray_step<REC, true, true>(W, kap, absorbed, status, rec, R, true,
+        done = ray_step<REC, true, true>(W, kap, tally, status, rec, R, true,
                                          [&](int c) { cdn = __ldg(cells + c); }, s_axes);
         cd = cdn;
         // a dark ray (transmission zero, no optical-depth cut) deposits nothing more:
@@ -255,7 +265,7 @@ k_walk(const float4 *__restrict__ cells, const float *__restrict__ tab, const ui
     }
     if (dark) {
       if (REC && R.row >= 0)  // a recorded ray lists its cells
-        while (!ray_step<REC, true, true, true>(W, 0.0f, absorbed, status, rec, R, true, NoPrefetch(), s_axes)) {
+        while (!ray_step<REC, true, true, true>(W, 0.0f, tally, status, rec, R, true, NoPrefetch(), s_axes)) {
         }
       else
         R.nv += dark_visits(W, R, status);
@@ -282,6 +292,11 @@ k_walk(const float4 *__restrict__ cells, const float *__restrict__ tab, const ui
     if (em != 0.0) atomicAdd(scalars + 0, em);
     if (esc != 0.0) atomicAdd(scalars + 2, esc);
     if (nsteps) atomicAdd(steps_out, nsteps);
+  }
+  if (FEW) {
+    __syncthreads();
+    for (int c = threadIdx.x; c < (int)W.ncells; c += kWalkThreads)
+      if (s_tally[c] != 0.0) atomicAdd(absorbed + c, s_tally[c]);
   }
 }
 
@@ -554,6 +569,7 @@ rt_status trace_impl(const rt_grid *grid, const float *kappa, const rt_spectral 
   auto pick = [&](auto tab) {
     constexpr int L = decltype(tab)::value;
     if (rec) return k_walk<true, L, kRefillIdleDefault>;
+    if (W.ncells <= kFewCells) return k_walk<false, L, 16, true>;
     return g_walk_refill == 12 ? k_walk<false, L, 12> : k_walk<false, L, 16>;
   };
   auto kern = layout == 2 ? pick(std::integral_constant<int, 2>()) : pick(std::integral_constant<int, 1>());
