@@ -452,7 +452,7 @@ rt_status rt_mlp_make_samples(const float *tables, int32_t n_p, const float *p_n
  * range and output scale).  The caller owns every buffer; the calls allocate only
  * stream-ordered scratch (BF16 weight tiles: 96 KB per network for a walk, 192 KB
  * for training, plus the training step's activations and gradient partials, none of
- * these where a step is at most 128 samples; a banded walk also 4 bytes per ray for the band-grouped order).  Bad sizes, NULL
+ * these where the steps run fused; a banded walk also 4 bytes per ray for the band-grouped order).  Bad sizes, NULL
  * buffers or out-of-range arguments return RT_E_INVAL before any launch; a bounded
  * device wait that gives up sets RT_DEV_TIMEOUT in the status word.  The norms are
  * read on the device and are not validated.

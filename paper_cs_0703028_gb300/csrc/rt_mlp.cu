@@ -13,8 +13,7 @@
 //   k_grad_adam : the gradient, the tiles' partials summed in tile order, and
 //                the Adam update of the FP32 masters (Kingma and Ba); within a
 //                run of steps also the next step's BF16 tiles.
-//   k_mlp_fused : a run of training steps whose batch is one 128-row tile, all three
-//                in one kernel, a network per block.
+//   k_mlp_fused : a run of training steps, all three in one kernel, a network per block.
 //   k_walk_mlp : the Monte-Carlo walk with the network in place of the table
 //                (three 128-ray tiles per block; every layer, biases included,
 //                on the tensor cores).
@@ -655,8 +654,8 @@ k_grad_adam(const float *__restrict__ part, int nparts, float *__restrict__ grad
 }
 
 // ---------------------------------------------------------------- fused training steps
-// A run of steps of an ensemble whose batch is one 128-sample tile: a block trains one network
-// at a time through all the launch's steps, forward, backward and Adam in one kernel, so that
+// A run of steps of an ensemble: a block trains one network at a time through all the launch's
+// steps, the batch's 128-sample tiles one after the other, forward, backward and Adam in one kernel, so that
 //  - the pre-activations stay in tensor memory (Z2..Z4, 384 columns, raw accumulators; z1 is
 //    recomputed from the four inputs), the gradients go from tensor memory straight into Adam,
 //    and the BF16 weight tiles stay in shared memory (dZ W reads the forward tile MN-major, so
@@ -664,7 +663,8 @@ k_grad_adam(const float *__restrict__ part, int nparts, float *__restrict__ grad
 //    written and read 3 times, partials 0.2 MB twice, tiles 0.2 MB three times) only the masters
 //    and moments are left, 0.6 MB read and 0.6 MB written;
 //  - those stay in L2 from step to step (0.6 MB of one network per SM, 92 MB in all).
-// 8 steps of 1024 networks x 128 samples: 5.09 -> 2.26 ms (the separate kernels spent 0.32 ms on
+// 8 steps of 1024 networks x 128 samples: 5.09 -> 2.26 ms, x 256 samples 7.47 -> 3.84 (the
+// separate kernels spent 0.32 ms on
 // the tiles and 0.075 + 0.22 + 0.286 ms a step on forward, backward and Adam); one network
 // 60 -> 36 us a step. Of a step's 33 us per network and SM the products take 3, the
 // elementwise passes and barriers between them 14, Adam 13; issue (16 warps an SM) and the latency
@@ -689,6 +689,7 @@ struct FusedSmem {
   uint16_t dZ[kTileElems];    // rows = samples, k = out
   SmallParams sp[2];          // this step's and the next step's
   float sm[kSmall], sv[kSmall];  // their moments: the small parameters live here during a launch
+  float sg[kSmall];              // their gradients over the batch's tiles so far
   float colred[5][4][kH];     // as in BwdSmem
   float yp[2][kH], yh[kH], dy[kH];
   float dyred[4], red[4];
@@ -757,10 +758,13 @@ __device__ __forceinline__ float adam_update(float g, float p, float &m, float &
   return r;
 }
 
+// TILES: batches of more than one tile
+template <bool TILES>
 __global__ void __launch_bounds__(kFusedThreads, 1)
 k_mlp_fused(float *__restrict__ P, float *__restrict__ M, float *__restrict__ V, float *__restrict__ grad, Norm N1,
             const Norm *__restrict__ norms, const float *__restrict__ inputs, const float *__restrict__ targets,
-            int n, long long in_stride, long long n_batches, int n_nets, __grid_constant__ const StepConsts C,
+            int batch, long long in_stride, long long n_batches, int n_nets, float *__restrict__ gsum,
+            __grid_constant__ const StepConsts C,
             int store_grad, float *__restrict__ loss, int loss_stride, float loss_scale, uint32_t *status) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   FusedSmem &S = *reinterpret_cast<FusedSmem *>(smem_raw);
@@ -768,7 +772,7 @@ k_mlp_fused(float *__restrict__ P, float *__restrict__ M, float *__restrict__ V,
   const int q4 = warp & 3, r = q4 * 32 + lane;  // sample row (activations) or input unit (gradients)
   const int cq = warp >> 2, cb = cq * 32;       // column quarter
   const uint32_t lanes = (uint32_t)(q4 * 32) << 16;
-  const bool valid = r < n;
+  gsum += (long long)blockIdx.x * kGradStride;  // weight gradients over the batch's tiles so far
   if (tid == 0) {
     tc::mbar_init(&S.bar, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -799,12 +803,20 @@ k_mlp_fused(float *__restrict__ P, float *__restrict__ M, float *__restrict__ V,
     tc::fence_before_sync();
     __syncthreads();
   };
-  // small parameter q (kSmall order) with value p: its gradient, four row-quarter partials in
-  // order, and the Adam update; returns the new value
-  auto small_adam = [&](int set, int i, int q, float p, float *GN, float lr, float c1, float c2) -> float {
-    const float gi = S.colred[set][0][i] + S.colred[set][1][i] + S.colred[set][2][i] + S.colred[set][3][i];
+  // small parameter q (kSmall order) with value p: its gradient g added to the batch's earlier
+  // tiles', and after the last tile the Adam update; returns the (new) value
+  auto small_step = [&](float g, int q, float p, bool first, bool last, float *GN, float lr, float c1, float c2) -> float {
+    const float gi = first ? g : S.sg[q] + g;
+    if (!last) {
+      S.sg[q] = gi;
+      return p;
+    }
     if (GN) GN[small_index(q)] = gi;
     return adam_update(gi, p, S.sm[q], S.sv[q], lr, c1, c2);
+  };
+  // four row-quarter partials in order
+  auto quarters = [&](int set, int i) -> float {
+    return S.colred[set][0][i] + S.colred[set][1][i] + S.colred[set][2][i] + S.colred[set][3][i];
   };
 
 #pragma unroll 1
@@ -833,237 +845,261 @@ k_mlp_fused(float *__restrict__ P, float *__restrict__ M, float *__restrict__ V,
       SmallParams &sp = S.sp[it & 1], &spn = S.sp[(it + 1) & 1];
       const float lr = C.lr[it], c1 = C.c1[it], c2 = C.c2[it];
       float *GN = store_grad && it == C.n_steps - 1 ? grad + (long long)net * kNParam : nullptr;
-      const long long row0 = net * in_stride + ((C.first + it) % n_batches) * n;
-      float u[4];
-      normalise(inputs + 4 * row0, r, valid, N, u);
-      // ---- forward
 #pragma unroll 1
-      for (int c0 = cb; c0 < cb + 32; c0 += 8) {
-        float2 h[4];
+      for (int t0 = 0; t0 < (TILES ? batch : 1); t0 += kH) {  // the batch's tiles
+        const bool first = !TILES || t0 == 0, last = !TILES || t0 + kH >= batch;
+        const bool valid = t0 + r < batch;
+        const long long row0 = net * in_stride + ((C.first + it) % n_batches) * batch + t0;
+        float u[4];
+        normalise(inputs + 4 * row0, r, valid, N, u);
+        // ---- forward
+#pragma unroll 1
+        for (int c0 = cb; c0 < cb + 32; c0 += 8) {
+          float2 h[4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const float2 z = layer1_pair(sp, c0 + 2 * i, u);
-          h[i] = __fmul2_rn(z, sigmoid2(z));
+          for (int i = 0; i < 4; ++i) {
+            const float2 z = layer1_pair(sp, c0 + 2 * i, u);
+            h[i] = __fmul2_rn(z, sigmoid2(z));
+          }
+          put_pairs(S.H, r, c0, h);
         }
-        put_pairs(S.H, r, c0, h);
-      }
-      float2 h4[16];
+        float2 h4[16];
 #pragma unroll 1
-      for (int l = 0; l < 3; ++l) {
+        for (int l = 0; l < 3; ++l) {
+          ready();
+          if (tid == 0) {
+            tc::fence_after_sync();
+            tc::mma_128x128x128(tZ[0] + 128u * l, S.H, S.W[l]);
+            tc::mma_commit(&S.bar);
+          }
+          if (!wait_products()) break;
+          float acc[32];
+          tc::tmem_ld32(tZ[0] + 128u * l + lanes + (uint32_t)cb, acc);
+          add_bias<32>(h4, acc, &sp.b[l][cb]);
+#pragma unroll
+          for (int i = 0; i < 16; ++i) h4[i] = __fmul2_rn(h4[i], sigmoid2(h4[i]));
+          if (l < 2) {
+#pragma unroll
+            for (int i = 0; i < 16; i += 4) put_pairs(S.H, r, cb + 2 * i, h4 + i);
+          }
+        }
+        if (pending) break;
+        // the head: a row's first (second) 64 units in one chain, by column quarters 0 and 1 (2, 3)
+        float y = 0.0f;
+        if ((cq & 1) == 0) {
+#pragma unroll
+          for (int i = 0; i < 16; ++i) y = fmaf(sp.w5[cb + 2 * i + 1], h4[i].y, fmaf(sp.w5[cb + 2 * i], h4[i].x, y));
+          S.yp[cq >> 1][r] = y;
+        }
+        __syncthreads();
+        if (cq & 1) {
+          y = S.yp[cq >> 1][r];
+#pragma unroll
+          for (int i = 0; i < 16; ++i) y = fmaf(sp.w5[cb + 2 * i + 1], h4[i].y, fmaf(sp.w5[cb + 2 * i], h4[i].x, y));
+          if (cq == 3) S.yh[r] = y;
+        }
+        __syncthreads();
+        if (cq == 1) {
+          y += S.yh[r];
+          y += sp.b5;
+          const float ts = valid ? (targets[row0 + r] - N.mean) / N.scale : 0.0f;
+          const float res = valid ? (y - ts) : 0.0f;
+          const float dyv = valid ? res / (float)batch : 0.0f;
+          S.dy[r] = dyv;
+          float l2 = 0.5f * res * res / (float)batch * loss_scale;
+          for (int o = 16; o > 0; o >>= 1) l2 += __shfl_down_sync(0xffffffffu, l2, o);
+          if (lane == 0) S.red[q4] = l2;
+          float d = dyv;
+          for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
+          if (lane == 0) S.dyred[q4] = d;
+        }
+        __syncthreads();
+        if (tid == 0) atomicAdd(loss + (long long)it * loss_stride, S.red[0] + S.red[1] + S.red[2] + S.red[3]);
+        const float dyv = S.dy[r];
+        // ---- backward.  Head: dw5 = sum_s dy h4; dz4 = dy w5 silu'(z4), db4; H still holds h3
+        // (rows past the batch: dz is zero there)
+        {
+#pragma unroll 1
+          for (int c0 = cb; c0 < cb + 32; c0 += 16) {
+            float acc[16];
+            float2 z[8], v[8];
+            tc::tmem_ld16(tZ[2] + lanes + (uint32_t)c0, acc);
+            add_bias<16>(z, acc, &sp.b[2][c0]);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+              if (!valid) z[i] = make_float2(0.0f, 0.0f);
+              const float2 s = sigmoid2(z[i]), w = *reinterpret_cast<const float2 *>(&sp.w5[c0 + 2 * i]);
+              v[i] = __fmul2_rn(__fmul2_rn(dup2(dyv), z[i]), s);
+              z[i] = __fmul2_rn(__fmul2_rn(dup2(dyv), w), silu_grad2(z[i], s));
+            }
+            put_pairs(S.dZ, r, c0, z);
+            put_pairs(S.dZ, r, c0 + 8, z + 4);
+            float cs = column_sum(v, lane);
+            if (lane < 16) S.colred[0][q4][c0 + lane] = cs;
+            cs = column_sum(z, lane);
+            if (lane < 16) S.colred[1][q4][c0 + lane] = cs;
+          }
+        }
         ready();
         if (tid == 0) {
           tc::fence_after_sync();
-          tc::mma_128x128x128(tZ[0] + 128u * l, S.H, S.W[l]);
+          tc::mma_128x128x128_mn(tX, S.H, S.dZ);           // dW4^T[in][out]
+          tc::mma_128x128x128_kn(tZ[2], S.dZ, S.W[2]);     // dH3[sample][in]
           tc::mma_commit(&S.bar);
         }
-        if (!wait_products()) break;
-        float acc[32];
-        tc::tmem_ld32(tZ[0] + 128u * l + lanes + (uint32_t)cb, acc);
-        add_bias<32>(h4, acc, &sp.b[l][cb]);
-#pragma unroll
-        for (int i = 0; i < 16; ++i) h4[i] = __fmul2_rn(h4[i], sigmoid2(h4[i]));
-        if (l < 2) {
-#pragma unroll
-          for (int i = 0; i < 16; i += 4) put_pairs(S.H, r, cb + 2 * i, h4 + i);
-        }
-      }
-      if (pending) break;
-      // the head: a row's first (second) 64 units in one chain, by column quarters 0 and 1 (2, 3)
-      float y = 0.0f;
-      if ((cq & 1) == 0) {
-#pragma unroll
-        for (int i = 0; i < 16; ++i) y = fmaf(sp.w5[cb + 2 * i + 1], h4[i].y, fmaf(sp.w5[cb + 2 * i], h4[i].x, y));
-        S.yp[cq >> 1][r] = y;
-      }
-      __syncthreads();
-      if (cq & 1) {
-        y = S.yp[cq >> 1][r];
-#pragma unroll
-        for (int i = 0; i < 16; ++i) y = fmaf(sp.w5[cb + 2 * i + 1], h4[i].y, fmaf(sp.w5[cb + 2 * i], h4[i].x, y));
-        if (cq == 3) S.yh[r] = y;
-      }
-      __syncthreads();
-      if (cq == 1) {
-        y += S.yh[r];
-        y += sp.b5;
-        const float ts = valid ? (targets[row0 + r] - N.mean) / N.scale : 0.0f;
-        const float res = valid ? (y - ts) : 0.0f;
-        const float dyv = valid ? res / (float)n : 0.0f;
-        S.dy[r] = dyv;
-        float l2 = 0.5f * res * res / (float)n * loss_scale;
-        for (int o = 16; o > 0; o >>= 1) l2 += __shfl_down_sync(0xffffffffu, l2, o);
-        if (lane == 0) S.red[q4] = l2;
-        float d = dyv;
-        for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
-        if (lane == 0) S.dyred[q4] = d;
-      }
-      __syncthreads();
-      if (tid == 0) atomicAdd(loss + (long long)it * loss_stride, S.red[0] + S.red[1] + S.red[2] + S.red[3]);
-      const float dyv = S.dy[r];
-      // ---- backward.  Head: dw5 = sum_s dy h4; dz4 = dy w5 silu'(z4), db4; H still holds h3
-      // (rows past the batch: dz is zero there)
-      {
+        if (cq == 0) spn.w5[r] = small_step(quarters(0, r), kSmallW5 + r, sp.w5[r], first, last, GN, lr, c1, c2);
+        if (cq == 1) spn.b[2][r] = small_step(quarters(1, r), kSmallB + 2 * kH + r, sp.b[2][r], first, last, GN, lr, c1, c2);
+        if (tid == kFusedThreads - 1)
+          spn.b5 = small_step(S.dyred[0] + S.dyred[1] + S.dyred[2] + S.dyred[3], kSmallB5, sp.b5, first, last, GN, lr, c1, c2);
 #pragma unroll 1
-        for (int c0 = cb; c0 < cb + 32; c0 += 16) {
-          float acc[16];
-          float2 z[8], v[8];
-          tc::tmem_ld16(tZ[2] + lanes + (uint32_t)c0, acc);
-          add_bias<16>(z, acc, &sp.b[2][c0]);
-#pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            if (!valid) z[i] = make_float2(0.0f, 0.0f);
-            const float2 s = sigmoid2(z[i]), w = *reinterpret_cast<const float2 *>(&sp.w5[c0 + 2 * i]);
-            v[i] = __fmul2_rn(__fmul2_rn(dup2(dyv), z[i]), s);
-            z[i] = __fmul2_rn(__fmul2_rn(dup2(dyv), w), silu_grad2(z[i], s));
-          }
-          put_pairs(S.dZ, r, c0, z);
-          put_pairs(S.dZ, r, c0 + 8, z + 4);
-          float cs = column_sum(v, lane);
-          if (lane < 16) S.colred[0][q4][c0 + lane] = cs;
-          cs = column_sum(z, lane);
-          if (lane < 16) S.colred[1][q4][c0 + lane] = cs;
-        }
-      }
-      ready();
-      if (tid == 0) {
-        tc::fence_after_sync();
-        tc::mma_128x128x128_mn(tX, S.H, S.dZ);           // dW4^T[in][out]
-        tc::mma_128x128x128_kn(tZ[2], S.dZ, S.W[2]);     // dH3[sample][in]
-        tc::mma_commit(&S.bar);
-      }
-      if (cq == 0) spn.w5[r] = small_adam(0, r, kSmallW5 + r, sp.w5[r], GN, lr, c1, c2);
-      if (cq == 1) spn.b[2][r] = small_adam(1, r, kSmallB + 2 * kH + r, sp.b[2][r], GN, lr, c1, c2);
-      if (tid == kFusedThreads - 1) {  // b5
-        const float gi = S.dyred[0] + S.dyred[1] + S.dyred[2] + S.dyred[3];
-        if (GN) GN[oB5] = gi;
-        spn.b5 = adam_update(gi, sp.b5, S.sm[kSmallB5], S.sv[kSmallB5], lr, c1, c2);
-      }
-#pragma unroll 1
-      for (int l = 4; l >= 2; --l) {
-        const int oW = l == 4 ? oW4 : (l == 3 ? oW3 : oW2);
-        auto load_adam = [&](int at, float2 (&p)[2], float2 (&m)[2], float2 (&v)[2]) {
-#pragma unroll
-          for (int j = 0; j < 2; ++j) {
-            p[j] = make_float2(PN[at + 2 * j * kH], PN[at + (2 * j + 1) * kH]);
-            m[j] = make_float2(MN[at + 2 * j * kH], MN[at + (2 * j + 1) * kH]);
-            v[j] = make_float2(VN[at + 2 * j * kH], VN[at + (2 * j + 1) * kH]);
-          }
-        };
-        float2 pv[2], mv[2], vv[2];  // W_l's first four of this thread, in flight until Adam needs them
-        load_adam(oW + cb * kH + r, pv, mv, vv);
-        if (!wait_products()) break;
-        // tensor memory: l = 4: dW in X, dH in Z4's columns; 3: Z4's, Z3's; 2: X, Z4's again
-        // (dW3 has been read by then: ready() below)
-        const uint32_t tW = l == 3 ? tZ[2] : tX, tH = l == 4 ? tZ[2] : (l == 3 ? tZ[1] : tZ[1]);
-        // dz_{l-1} and, for l > 2, h_{l-2}
-#pragma unroll 1
-        for (int hc = 0; hc < 32; hc += 16) {
-          const int c0 = cb + hc;
-          // pre-activations of layer q (1..4) at this thread's 16 units
-          auto pre = [&](int q, float2 (&z)[8]) {
-            if (q > 1) {
-              float acc[16];
-              tc::tmem_ld16(tZ[0] + 128u * (q - 2) + lanes + (uint32_t)c0, acc);
-              add_bias<16>(z, acc, &sp.b[q - 2][c0]);
-            } else {
-#pragma unroll
-              for (int i = 0; i < 8; ++i) z[i] = layer1_pair(sp, c0 + 2 * i, u);
-            }
-#pragma unroll
-            for (int i = 0; i < 8; ++i)
-              if (!valid) z[i] = make_float2(0.0f, 0.0f);
-          };
-          float2 z[8], dz[8];
-          pre(l - 1, z);
-          {
-            float acc[16];
-            tc::tmem_ld16(tH + lanes + (uint32_t)c0, acc);
-#pragma unroll
-            for (int i = 0; i < 8; ++i)
-              dz[i] = __fmul2_rn(make_float2(acc[2 * i], acc[2 * i + 1]), silu_grad2(z[i], sigmoid2(z[i])));
-          }
-          if (l > 2) {
-            put_pairs(S.dZ, r, c0, dz);
-            put_pairs(S.dZ, r, c0 + 8, dz + 4);
-            pre(l - 2, z);
-#pragma unroll
-            for (int i = 0; i < 8; ++i) z[i] = __fmul2_rn(z[i], sigmoid2(z[i]));
-            put_pairs(S.H, r, c0, z);
-            put_pairs(S.H, r, c0 + 8, z + 4);
-          }
-          float cs = column_sum(dz, lane);
-          if (lane < 16) S.colred[0][q4][c0 + lane] = cs;
-          if (l == 2) {  // first layer: dW1[c][k] = sum_s dz1[s][c] u[s][k]
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-#pragma unroll
-              for (int i = 0; i < 8; ++i) z[i] = __fmul2_rn(dz[i], dup2(u[k]));
-              cs = column_sum(z, lane);
-              if (lane < 16) S.colred[1 + k][q4][c0 + lane] = cs;
-            }
-          }
-        }
-        ready();
-        if (l > 2 && tid == 0) {  // the next layer's products run under this one's Adam
-          tc::fence_after_sync();
-          tc::mma_128x128x128_mn(l == 4 ? tZ[2] : tX, S.H, S.dZ);
-          tc::mma_128x128x128_kn(tZ[1], S.dZ, S.W[l - 3]);
-          tc::mma_commit(&S.bar);
-        }
-        // Adam of W_l: this thread's input unit r, output units cb .. cb + 31, four at a time
-        // with the next four's loads in flight
-        uint16_t *te = S.W[l - 2] + tile_index(cb, r);  // output unit cb; the next ones by tile_index(j, 0)
-#pragma unroll 1
-        for (int hc = 0; hc < 32; hc += 16) {
-          float g[16];
-          tc::tmem_ld16(tW + lanes + (uint32_t)(cb + hc), g);
-#pragma unroll
-          for (int j0 = 0; j0 < 16; j0 += 4) {
-            const int at = oW + (cb + hc + j0) * kH + r;
-            float2 np[2], nm[2], nv[2];
-            if (j0 < 12 || hc == 0) load_adam(at + 4 * kH, np, nm, nv);
+        for (int l = 4; l >= 2; --l) {
+          const int oW = l == 4 ? oW4 : (l == 3 ? oW3 : oW2);
+          auto load_adam = [&](int at, float2 (&p)[2], float2 (&m)[2], float2 (&v)[2]) {
 #pragma unroll
             for (int j = 0; j < 2; ++j) {
-              const float2 gi = make_float2(g[j0 + 2 * j], g[j0 + 2 * j + 1]);
-              const int a0 = at + 2 * j * kH, a1 = a0 + kH;
-              if (GN) {
-                GN[a0] = gi.x;
-                GN[a1] = gi.y;
-              }
-              const float2 pn = adam_update2(gi, pv[j], mv[j], vv[j], lr, c1, c2);
-              PN[a0] = pn.x;
-              PN[a1] = pn.y;
-              MN[a0] = mv[j].x;
-              MN[a1] = mv[j].y;
-              VN[a0] = vv[j].x;
-              VN[a1] = vv[j].y;
-              const uint32_t h = pack2(pn);
-              te[tile_index(hc + j0 + 2 * j, 0)] = (uint16_t)h;
-              te[tile_index(hc + j0 + 2 * j + 1, 0)] = (uint16_t)(h >> 16);
+              p[j] = make_float2(PN[at + 2 * j * kH], PN[at + (2 * j + 1) * kH]);
+              m[j] = make_float2(MN[at + 2 * j * kH], MN[at + (2 * j + 1) * kH]);
+              v[j] = make_float2(VN[at + 2 * j * kH], VN[at + (2 * j + 1) * kH]);
             }
-            if (j0 < 12 || hc == 0) {
+          };
+          float2 pv[2], mv[2], vv[2];  // W_l's first four of this thread, in flight until Adam needs them
+          if (last) load_adam(oW + cb * kH + r, pv, mv, vv);
+          if (!wait_products()) break;
+          // tensor memory: l = 4: dW in X, dH in Z4's columns; 3: Z4's, Z3's; 2: X, Z4's again
+          // (dW3 has been read by then: ready() below)
+          const uint32_t tW = l == 3 ? tZ[2] : tX, tH = l == 4 ? tZ[2] : (l == 3 ? tZ[1] : tZ[1]);
+          // dz_{l-1} and, for l > 2, h_{l-2}
+#pragma unroll 1
+          for (int hc = 0; hc < 32; hc += 16) {
+            const int c0 = cb + hc;
+            // pre-activations of layer q (1..4) at this thread's 16 units
+            auto pre = [&](int q, float2 (&z)[8]) {
+              if (q > 1) {
+                float acc[16];
+                tc::tmem_ld16(tZ[0] + 128u * (q - 2) + lanes + (uint32_t)c0, acc);
+                add_bias<16>(z, acc, &sp.b[q - 2][c0]);
+              } else {
 #pragma unroll
-              for (int j = 0; j < 2; ++j) {
-                pv[j] = np[j];
-                mv[j] = nm[j];
-                vv[j] = nv[j];
+                for (int i = 0; i < 8; ++i) z[i] = layer1_pair(sp, c0 + 2 * i, u);
+              }
+#pragma unroll
+              for (int i = 0; i < 8; ++i)
+                if (!valid) z[i] = make_float2(0.0f, 0.0f);
+            };
+            float2 z[8], dz[8];
+            pre(l - 1, z);
+            {
+              float acc[16];
+              tc::tmem_ld16(tH + lanes + (uint32_t)c0, acc);
+#pragma unroll
+              for (int i = 0; i < 8; ++i)
+                dz[i] = __fmul2_rn(make_float2(acc[2 * i], acc[2 * i + 1]), silu_grad2(z[i], sigmoid2(z[i])));
+            }
+            if (l > 2) {
+              put_pairs(S.dZ, r, c0, dz);
+              put_pairs(S.dZ, r, c0 + 8, dz + 4);
+              pre(l - 2, z);
+#pragma unroll
+              for (int i = 0; i < 8; ++i) z[i] = __fmul2_rn(z[i], sigmoid2(z[i]));
+              put_pairs(S.H, r, c0, z);
+              put_pairs(S.H, r, c0 + 8, z + 4);
+            }
+            float cs = column_sum(dz, lane);
+            if (lane < 16) S.colred[0][q4][c0 + lane] = cs;
+            if (l == 2) {  // first layer: dW1[c][k] = sum_s dz1[s][c] u[s][k]
+#pragma unroll
+              for (int k = 0; k < 4; ++k) {
+#pragma unroll
+                for (int i = 0; i < 8; ++i) z[i] = __fmul2_rn(dz[i], dup2(u[k]));
+                cs = column_sum(z, lane);
+                if (lane < 16) S.colred[1 + k][q4][c0 + lane] = cs;
               }
             }
           }
+          ready();
+          if (l > 2 && tid == 0) {  // the next layer's products run under this one's Adam
+            tc::fence_after_sync();
+            tc::mma_128x128x128_mn(l == 4 ? tZ[2] : tX, S.H, S.dZ);
+            tc::mma_128x128x128_kn(tZ[1], S.dZ, S.W[l - 3]);
+            tc::mma_commit(&S.bar);
+          }
+          if (!last) {  // dW_l joins the batch's earlier tiles'
+#pragma unroll 1
+            for (int hc = 0; hc < 32; hc += 16) {
+              float g[16], e[16];
+              float *gs = gsum + oW + (cb + hc) * kH + r;
+              if (!first) {
+#pragma unroll
+                for (int j = 0; j < 16; ++j) e[j] = gs[j * kH];
+              }
+              tc::tmem_ld16(tW + lanes + (uint32_t)(cb + hc), g);
+#pragma unroll
+              for (int j = 0; j < 16; ++j) gs[j * kH] = first ? g[j] : e[j] + g[j];
+            }
+          } else {
+            // Adam of W_l: this thread's input unit r, output units cb .. cb + 31, four at a time
+            // with the next four's loads in flight
+            uint16_t *te = S.W[l - 2] + tile_index(cb, r);  // output unit cb; the next ones by tile_index(j, 0)
+    #pragma unroll 1
+            for (int hc = 0; hc < 32; hc += 16) {
+              float g[16];
+              tc::tmem_ld16(tW + lanes + (uint32_t)(cb + hc), g);
+              if (!first) {
+    #pragma unroll
+                for (int j = 0; j < 16; ++j) g[j] = gsum[oW + (cb + hc + j) * kH + r] + g[j];
+              }
+    #pragma unroll
+              for (int j0 = 0; j0 < 16; j0 += 4) {
+                const int at = oW + (cb + hc + j0) * kH + r;
+                float2 np[2], nm[2], nv[2];
+                if (j0 < 12 || hc == 0) load_adam(at + 4 * kH, np, nm, nv);
+    #pragma unroll
+                for (int j = 0; j < 2; ++j) {
+                  const float2 gi = make_float2(g[j0 + 2 * j], g[j0 + 2 * j + 1]);
+                  const int a0 = at + 2 * j * kH, a1 = a0 + kH;
+                  if (GN) {
+                    GN[a0] = gi.x;
+                    GN[a1] = gi.y;
+                  }
+                  const float2 pn = adam_update2(gi, pv[j], mv[j], vv[j], lr, c1, c2);
+                  PN[a0] = pn.x;
+                  PN[a1] = pn.y;
+                  MN[a0] = mv[j].x;
+                  MN[a1] = mv[j].y;
+                  VN[a0] = vv[j].x;
+                  VN[a1] = vv[j].y;
+                  const uint32_t h = pack2(pn);
+                  te[tile_index(hc + j0 + 2 * j, 0)] = (uint16_t)h;
+                  te[tile_index(hc + j0 + 2 * j + 1, 0)] = (uint16_t)(h >> 16);
+                }
+                if (j0 < 12 || hc == 0) {
+    #pragma unroll
+                  for (int j = 0; j < 2; ++j) {
+                    pv[j] = np[j];
+                    mv[j] = nm[j];
+                    vv[j] = nv[j];
+                  }
+                }
+              }
+            }
+          }
+          if (cq == 0) {
+            float *bn = l > 2 ? spn.b[l - 3] : spn.b1;
+            const float *bp = l > 2 ? sp.b[l - 3] : sp.b1;
+            bn[r] = small_step(quarters(0, r), (l > 2 ? kSmallB + (l - 3) * kH : kSmallB1) + r, bp[r], first, last, GN, lr,
+                               c1, c2);
+          }
+          if (l == 2)  // W1: four gradients a unit, one by each column quarter
+            reinterpret_cast<float *>(&spn.w1[r])[cq] =
+                small_step(quarters(1 + cq, r), kSmallW1 + 4 * r + cq, reinterpret_cast<const float *>(&sp.w1[r])[cq], first,
+                           last, GN, lr, c1, c2);
+          tc::fence_before_sync();
         }
-        if (cq == 0) {
-          float *bn = l > 2 ? spn.b[l - 3] : spn.b1;
-          const float *bp = l > 2 ? sp.b[l - 3] : sp.b1;
-          bn[r] = small_adam(0, r, (l > 2 ? kSmallB + (l - 3) * kH : kSmallB1) + r, bp[r], GN, lr, c1, c2);
-        }
-        if (l == 2)  // W1: four gradients a unit, one by each column quarter
-          reinterpret_cast<float *>(&spn.w1[r])[cq] =
-              small_adam(1 + cq, r, kSmallW1 + 4 * r + cq, reinterpret_cast<const float *>(&sp.w1[r])[cq], GN, lr, c1, c2);
-        tc::fence_before_sync();
+        if (pending) break;
+        __syncthreads();  // the next tile or step reads spn, H and the tiles
+        tc::fence_after_sync();
       }
       if (pending) break;
-      __syncthreads();  // the next step reads spn, H and the tiles
-      tc::fence_after_sync();
     }
     if (!pending) {  // the small parameters and their moments back to memory
       const SmallParams &sp = S.sp[C.n_steps & 1];
@@ -1714,6 +1750,16 @@ rt_status mlp_train_impl(float *params, float *m, float *v, float *grad, const f
                         loss, status, scr.as<char>(), false, true, st);
 }
 
+// Whether a run's steps go to the fused kernel: its blocks take their networks' tiles one after
+// the other, the separate kernels spread all tiles over the GPU.  Per step, in us, measured on
+// 1 .. 1024 networks of 1 .. 4 tiles: fused 43 for one tile and 22 for each further one, per
+// round of one network an SM; separate about 50 + 0.3 per tile (fused / separate: 1 x 1 tile 37 /
+// 59, 32 x 2 66 / 75, 32 x 4 109 / 76, 48 x 3 87 / 87, 152 x 4 119 / 248, 1024 x 2 480 / 933).
+bool fused_pays(int n_nets, int64_t tiles, int sms) {
+  const double rounds = (double)((n_nets + sms - 1) / sms);
+  return tiles == 1 || rounds * (43.0 + 22.0 * (double)(tiles - 1)) <= 50.0 + 0.3 * (double)n_nets * (double)tiles;
+}
+
 // n_steps steps of n_nets networks (one network: nm is a host norm; an ensemble: nm
 // is a device array of n_nets norms), inputs / targets [n_nets][n] rows
 rt_status mlp_train_steps_impl(float *params, float *m, float *v, float *grad, const float *inputs,
@@ -1735,20 +1781,25 @@ rt_status mlp_train_steps_impl(float *params, float *m, float *v, float *grad, c
   const int64_t nb = n / batch;
   const double span = (double)std::max(1, total_steps - 1);
   auto rate = [&](int64_t s) { return (float)(lr1 + 0.5 * (lr0 - lr1) * (1.0 + std::cos(kPiD * (double)s / span))); };
-  if (batch <= kH) {  // one tile a step: the fused kernel
+  int dev = 0, sms = 0;
+  RT_CUDA_TRY(cudaGetDevice(&dev));
+  RT_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  if (fused_pays(n_nets, (batch + kH - 1) / kH, sms)) {
+    const int blocks = std::min(n_nets, sms);
     Scratch scr;
-    rt_status r = scr.alloc(256, st);
+    rt_status r = scr.alloc(256 + (batch > kH ? (size_t)blocks * kGradStride * sizeof(float) : 0), st);
     if (r != RT_OK) return r;
     float *loss = losses ? losses : scr.as<float>();
+    float *gsum = scr.as<float>() + 64;
     r = validate_train(params, m, v, grad, inputs, targets, batch, n_nets, nm, norm_on_device, 0, loss);
     if (r != RT_OK) return r;
     static std::once_flag once;
     static rt_status attr = RT_OK;
-    std::call_once(once, [] { attr = set_smem((const void *)k_mlp_fused, sizeof(FusedSmem)); });
+    std::call_once(once, [] {
+      attr = set_smem((const void *)k_mlp_fused<false>, sizeof(FusedSmem));
+      if (attr == RT_OK) attr = set_smem((const void *)k_mlp_fused<true>, sizeof(FusedSmem));
+    });
     if (attr != RT_OK) return attr;
-    int dev = 0, sms = 0;
-    RT_CUDA_TRY(cudaGetDevice(&dev));
-    RT_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     if (losses) RT_CUDA_TRY(cudaMemsetAsync(losses, 0, (size_t)n_steps * sizeof(float), st));
     for (int32_t i0 = 0; i0 < n_steps; i0 += kFusedSteps) {
       StepConsts C;
@@ -1760,8 +1811,8 @@ rt_status mlp_train_steps_impl(float *params, float *m, float *v, float *grad, c
         C.c1[i] = (float)(1.0 - std::pow(0.9, (double)(s + 1)));
         C.c2[i] = (float)(1.0 - std::pow(0.999, (double)(s + 1)));
       }
-      k_mlp_fused<<<std::min(n_nets, sms), kFusedThreads, sizeof(FusedSmem), st>>>(
-          params, m, v, grad, N1, norms, inputs, targets, (int)batch, n, nb, n_nets, C, i0 + C.n_steps == n_steps,
+      (batch > kH ? k_mlp_fused<true> : k_mlp_fused<false>)<<<blocks, kFusedThreads, sizeof(FusedSmem), st>>>(
+          params, m, v, grad, N1, norms, inputs, targets, (int)batch, n, nb, n_nets, gsum, C, i0 + C.n_steps == n_steps,
           losses ? losses + i0 : loss, losses ? 1 : 0, 1.0f / (float)n_nets, status);
       RT_CUDA_TRY(cudaGetLastError());
     }

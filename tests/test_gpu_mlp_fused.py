@@ -1,5 +1,5 @@
-"""Training steps of at most one 128-sample tile run in one fused kernel: bit for bit the
-parameters, moments and last gradient of the separate forward, backward and Adam kernels
+"""Training steps of one 128-sample tile, or of several for enough networks, run in one fused
+kernel: bit for bit the parameters, moments and last gradient of the separate forward, backward and Adam kernels
 (rt_mlp_train_step, which keeps them)."""
 import math
 
@@ -18,9 +18,10 @@ def rt():
 
 
 # one sample, ragged rows of a warp and of the tile, a full tile; several networks and batches;
-# more steps than one launch takes, from the middle of a schedule (bias corrections not yet 1)
+# more steps than one launch takes, from the middle of a schedule (bias corrections not yet 1);
+# batches of two and three tiles with a ragged last one
 @pytest.mark.parametrize("n_nets,batch,n_batches,n_steps,first", [(1, 1, 2, 3, 1), (2, 33, 1, 3, 1), (1, 64, 3, 4, 7), (3, 127, 2, 3, 200),
-                                                                  (2, 128, 3, 5, 20000), (1, 40, 2, 243, 1)])
+                                                                  (2, 128, 3, 5, 20000), (1, 40, 2, 243, 1), (40, 129, 2, 2, 3), (50, 300, 1, 2, 1)])
 def test_fused_steps_equal_separate_kernels(rt, n_nets, batch, n_batches, n_steps, first):
     import torch
     n = batch * n_batches
