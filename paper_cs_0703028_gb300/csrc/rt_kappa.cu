@@ -530,11 +530,12 @@ __device__ __forceinline__ void two_sum_add2(float2 &s, float2 &c, float2 v) {
 // series, window ends masked, added in pairs.
 // Lorentz: P = {A g / (pi dnu), g^2}.
 // Of the 2560 lines a tile of the 128^3 workload sums (64 T x 400k points, 100k lines), 2000
-// cost 8 evaluations, 280 16, 128 about 64 and 134 256 each instead of 256 each: 16.2 -> 4.95
-// ms (32^3 workload 1.89 -> 0.96 ms).  Of the 4.95, by timing copies that leave a kind out:
-// general lines 2.5 (their core points 1.4), window ends 0.8, 8 nodes 0.6, fast 0.35, 16 nodes
+// cost 8 evaluations, 280 16, 128 about 64 and 134 256 each instead of 256 each: 16.2 -> 4.6
+// ms (32^3 workload 1.89 -> 0.91 ms).  Of the 4.6, by timing copies that leave a kind out:
+// general lines 2.2 (their core points 1.2), window ends 0.8, 8 nodes 0.35, fast 0.35, 16 nodes
 // 0.2, interpolation 0.07, chunks and barriers the rest; the FMA pipe (a paired FMA takes two
-// of its cycles) and issue bound it, the reciprocals no longer do.
+// of its cycles) and issue bound it, the reciprocals no longer do.  A barrier a chunk keeps the
+// warps on the same code: with the buffers handed on warp by warp instead 3 % slower.
 // ADAPT: every line has its own window at each node (AW, within the cutoff window), staged
 // with the coefficients.  A warp sorts each range's lines by its node's windows (ballots):
 // lines whose window holds the tile go the range's way, lines whose window ends in it the
@@ -688,20 +689,31 @@ k_kappa(const float4 *__restrict__ P, const float4 *__restrict__ P2, const int4 
     };
     // Below, a range's lines are at(0) .. at(n - 1), chunk indices.
     // run_nodes: at the M tile nodes: M / 2 lanes take a line (two nodes each), the warp
-    // 64 / M lines at a time
+    // 64 / M lines at a time; whole groups without bounds checks (with them 4.99 ms of the
+    // 128^3 workload, 4.72 without)
     auto run_nodes = [&](auto deg, auto m, const float *un, auto at, int n, float2 &s, float2 &sc) {
       constexpr int kLanes = decltype(m)::value / 2, kLines = 32 / kLanes;
       const float2 u0 = *reinterpret_cast<const float2 *>(un + 2 * (lane % kLanes));
+      auto value = [&](int e) -> float2 {
+        const int q = at(e);
+        const int2 r = *reinterpret_cast<const int2 *>(&cR[q].z);
+        const float2 u = __fadd2_rn(__fadd2_rn(dup2((float)(jw0 - r.x)), u0), dup2(__int_as_float(r.y)));
+        return far_value(deg, u, cP[q], q);
+      };
+      int i = lane / kLanes, left = n;
 #pragma unroll 1
-      for (int i = lane / kLanes; __any_sync(0xffffffffu, i < n); i += kLines * kNodeGroup) {
+      for (; left >= kLines * kNodeGroup; left -= kLines * kNodeGroup, i += kLines * kNodeGroup) {
+        float2 g = value(i);
+#pragma unroll
+        for (int e = 1; e < kNodeGroup; ++e) g = __fadd2_rn(g, value(i + e * kLines));
+        kahan_add2(s, sc, g);
+      }
+      if (left > 0) {
         float2 g = make_float2(0.0f, 0.0f);
 #pragma unroll
         for (int e = 0; e < kNodeGroup; ++e) {
           const bool in = i + e * kLines < n;
-          const int q = at(in ? i + e * kLines : n - 1);
-          const int2 r = *reinterpret_cast<const int2 *>(&cR[q].z);
-          const float2 u = __fadd2_rn(__fadd2_rn(dup2((float)(jw0 - r.x)), u0), dup2(__int_as_float(r.y)));
-          const float2 v = far_value(deg, u, cP[q], q);
+          const float2 v = value(in ? i + e * kLines : n - 1);
           if (in) g = __fadd2_rn(g, v);
         }
         kahan_add2(s, sc, g);
@@ -920,11 +932,10 @@ k_kappa(const float4 *__restrict__ P, const float4 *__restrict__ P2, const int4 
       const int a = lane * kPtsPerThread - first;  // the lane's first point in res
       if (a + kPtsPerThread <= 0 || a >= n) return;
       const float *res = s_res[warp] + c + a;
-      const unsigned in = (n - a >= kPtsPerThread ? 0xffu : (1u << (n - a)) - 1u) & (a >= 0 ? 0xffu : 0xffu << -a);
 #pragma unroll
       for (int h = 0; h < kPairs; ++h) {
-        if ((in >> (2 * h)) & 1u) v[h].x = res[2 * h];
-        if ((in >> (2 * h + 1)) & 1u) v[h].y = res[2 * h + 1];
+        if ((unsigned)(a + 2 * h) < (unsigned)n) v[h].x = res[2 * h];
+        if ((unsigned)(a + 2 * h + 1) < (unsigned)n) v[h].y = res[2 * h + 1];
       }
     };
     auto mask_window = [&](int i, float2 (&v)[kPairs]) {
