@@ -1,10 +1,9 @@
 // Monte-Carlo ray tracing through finite volumes (Section 3, Fig. ray) and the
 // final tally reduction.
-//   k_cell_prep : per cell, the binary32 temperature bracket (k, frac) of the
-//                 kappa table, the density scale (p x)/(p_ref x_ref) and T.
-//   k_walk_setup: the cells (as k_cell_prep, and 8-byte step records) and the walk's copy of the table in one launch:
-//                 {kappa_k, kappa_k+1} per (wavenumber, node), so a step's interpolation is
-//                 one 8-byte load, or wavenumber-major.
+//   k_walk_setup: per cell, the binary32 temperature bracket (k, frac) of the kappa table,
+//                 the density scale (p x)/(p_ref x_ref) and T, and an 8-byte step record; the
+//                 walk's copy of the table, {kappa_k, kappa_k+1} per (wavenumber, node), so a
+//                 step's interpolation is one 8-byte load, or wavenumber-major.
 //   k_walk      : per ray, Philox draws -> emission cell, wavenumber, position,
 //                 isotropic direction -> cell-by-cell walk with Beer-Lambert
 //                 attenuation (Eq. I, first term), binary64 atomic deposits;
@@ -26,14 +25,6 @@ namespace {
 
 constexpr int kWalkThreads = 256, kWalkBlocks = 4;  // resident blocks per SM
 constexpr int kReduceBlocks = 256;
-
-__global__ void k_cell_prep(const float *__restrict__ T, const float *__restrict__ p,
-                            const float *__restrict__ x, CellParams C, float4 *__restrict__ out,
-                            uint32_t *status) {
-  const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= C.ncells) return;
-  out[c] = cell_prep_one(T, p, x, c, C, status);
-}
 
 // Persistent walk: each warp owns a contiguous range of rays.  Lanes step their
 // own rays; when half of the warp's lanes are idle (ballot), the idle lanes take
@@ -499,16 +490,6 @@ CellParams cell_params(const rt_spectral *spec, long long ncells, int has_px) {
   C.nT = spec->nT;
   C.has_px = has_px;
   return C;
-}
-
-rt_status cell_prep(const rt_grid *grid, const rt_spectral *spec, float4 *cells, uint32_t *status,
-                    cudaStream_t st) {
-  const long long nc = (long long)grid->nx * grid->ny * grid->nz;
-  const CellParams C = cell_params(spec, nc, (grid->p_atm || grid->x) ? 1 : 0);
-  k_cell_prep<<<(unsigned)((nc + 255) / 256), 256, 0, st>>>(grid->T, grid->p_atm, grid->x, C, cells,
-                                                           status);
-  RT_CUDA_TRY(cudaGetLastError());
-  return RT_OK;
 }
 
 rt_status band_plan(const WalkParams &W, int band_pts, long long n_bands, long long chunk,

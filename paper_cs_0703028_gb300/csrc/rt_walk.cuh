@@ -405,8 +405,5 @@ CellParams cell_params(const rt_spectral *spec, long long ncells, int has_px);
 rt_status band_plan(const WalkParams &W, int band_pts, long long n_bands, long long chunk,
                     unsigned long long *counts, long long *band_start, long long *item_start, int *item_band,
                     uint32_t *order, int sms, cudaStream_t st);
-// Host: per-cell T bracket, density scale and T (float4 per cell).
-rt_status cell_prep(const rt_grid *grid, const rt_spectral *spec, float4 *cells, uint32_t *status,
-                    cudaStream_t st);
 
 }  // namespace rt
