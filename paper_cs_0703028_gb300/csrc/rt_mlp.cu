@@ -78,7 +78,7 @@ __device__ __forceinline__ int tile_index(int r, int k) { return (int)(tc::kmajo
 // 6250 networks x 3 matrices: 0.37 ms (1.84 GB; 0.88 with an element a thread in row order).
 constexpr int kPrepThreads = 256;
 __global__ void __launch_bounds__(kPrepThreads)
-k_mlp_prep(const float *__restrict__ P, uint16_t *__restrict__ tiles, int n_mats) {
+k_mlp_prep(const float *__restrict__ P, uint16_t *__restrict__ tiles, int n_mats, float scale) {
   const int m = blockIdx.x;  // 0..2: W2..W4 (rows = out), 3..5: transposes (rows = in)
   const long long net = blockIdx.y;
   P += net * kNParam + ((m % 3 == 0) ? oW2 : (m % 3 == 1 ? oW3 : oW4));
@@ -90,7 +90,7 @@ k_mlp_prep(const float *__restrict__ P, uint16_t *__restrict__ tiles, int n_mats
     const float *w = m < 3 ? P + r * kH + k : P + k * kH + r;
     float v[8];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) v[i] = __ldg(w + i * step);
+    for (int i = 0; i < 8; ++i) v[i] = scale * __ldg(w + i * step);
     *reinterpret_cast<uint4 *>(tiles + tile_index(r, k)) =
         make_uint4(pack_bf16x2(v[0], v[1]), pack_bf16x2(v[2], v[3]), pack_bf16x2(v[4], v[5]), pack_bf16x2(v[6], v[7]));
   }
@@ -1236,17 +1236,18 @@ static_assert(sizeof(WalkMlpSmem) <= 227 * 1024, "surrogate walk shared memory e
 __device__ __forceinline__ uint16_t bf16_bits(float v) { return __bfloat16_as_ushort(__float2bfloat16_rn(v)); }
 __device__ __forceinline__ float bf16_value(uint16_t b) { return __bfloat162float(__ushort_as_bfloat16(b)); }
 
-// the walk's parameters in shared memory: layer-1 operand B, biases and head
+// the walk's parameters in shared memory: layer-1 operand B, biases (both halved, as W2..W4:
+// see mlp_eval_tile) and head
 __device__ __forceinline__ void stage_walk(WalkMlpSmem &S, const float *__restrict__ P) {
   for (int e = threadIdx.x; e < kL1Elems; e += blockDim.x) {
     const int n = e / kL1K, k = e % kL1K;
     uint16_t bits = 0;
     if (k < 12) {
-      const float w = P[oW1 + 4 * n + k / 3];
+      const float w = 0.5f * P[oW1 + 4 * n + k / 3];
       const uint16_t hi = bf16_bits(w);
       bits = (k % 3 == 1) ? bf16_bits(w - bf16_value(hi)) : hi;
     } else if (k < 14) {
-      const float b = P[oB1 + n];
+      const float b = 0.5f * P[oB1 + n];
       const uint16_t hi = bf16_bits(b);
       bits = (k == 13) ? bf16_bits(b - bf16_value(hi)) : hi;
     }
@@ -1257,7 +1258,7 @@ __device__ __forceinline__ void stage_walk(WalkMlpSmem &S, const float *__restri
     const int l = e / kL1Elems, n = (e % kL1Elems) / kL1K, k = e % kL1K;
     uint16_t bits = 0;
     if (k == 12 || k == 13) {
-      const float b = P[(l == 0 ? oB2 : (l == 1 ? oB3 : oB4)) + n];
+      const float b = 0.5f * P[(l == 0 ? oB2 : (l == 1 ? oB3 : oB4)) + n];
       const uint16_t hi = bf16_bits(b);
       bits = (k == 13) ? bf16_bits(b - bf16_value(hi)) : hi;
     }
@@ -1344,12 +1345,14 @@ __device__ __forceinline__ bool mlp_eval_tile(WalkMlpSmem &S, uint32_t tmem, con
       const int c0 = 64 * half + 16 * q;
       tc::tmem_ld_wait(z[q & 1]);
       if (q < 3) tc::tmem_ld16_async(tacc + (uint32_t)(c0 + 16), z[(q + 1) & 1]);
-      // binary32 SiLU (as in training)
+      // binary32 SiLU (as in training): the accumulators hold g = z / 2, so that
+      // z sigmoid(z) = z (1 + tanh(z / 2)) / 2 = g (1 + tanh g), the same bits one paired
+      // multiply cheaper (halving is exact)
       float2 h[8];
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
-        const float2 zi = make_float2(__uint_as_float(z[q & 1][2 * i]), __uint_as_float(z[q & 1][2 * i + 1]));
-        h[i] = __fmul2_rn(zi, sigmoid2(zi));
+        const float2 g = make_float2(__uint_as_float(z[q & 1][2 * i]), __uint_as_float(z[q & 1][2 * i + 1]));
+        h[i] = __fmul2_rn(g, __fadd2_rn(dup2(1.0f), make_float2(tanh_approx(g.x), tanh_approx(g.y))));
       }
       if (l < 3) {  // next layer's BF16 input
         put_pairs(S.A[tile], r, c0, h);
@@ -1643,9 +1646,10 @@ Norm to_norm(const rt_mlp_norm *nm) {
 
 }  // namespace
 
-// BF16 tiles of n_nets networks: the first n_mats of W2..W4, W2^T..W4^T per network
-rt_status mlp_prep_tiles(const float *params, uint16_t *tiles, int n_nets, int n_mats, cudaStream_t st) {
-  k_mlp_prep<<<dim3(n_mats, n_nets), kPrepThreads, 0, st>>>(params, tiles, n_mats);
+// BF16 tiles of n_nets networks: the first n_mats of W2..W4, W2^T..W4^T per network, times scale
+// (a power of two)
+rt_status mlp_prep_tiles(const float *params, uint16_t *tiles, int n_nets, int n_mats, float scale, cudaStream_t st) {
+  k_mlp_prep<<<dim3(n_mats, n_nets), kPrepThreads, 0, st>>>(params, tiles, n_mats, scale);
   RT_CUDA_TRY(cudaGetLastError());
   return RT_OK;
 }
@@ -1708,7 +1712,7 @@ rt_status mlp_train_core(float *params, float *m, float *v, float *grad, const f
       (reinterpret_cast<uintptr_t>(dy + nn * (size_t)n) + 63) & ~uintptr_t(63));  // 64-byte aligned rows
   if (!chained) {
     RT_CUDA_TRY(cudaMemsetAsync(loss, 0, sizeof(float), st));
-    rt_status s = mlp_prep_tiles(params, tiles, n_nets, 6, st);
+    rt_status s = mlp_prep_tiles(params, tiles, n_nets, 6, 1.0f, st);
     if (s != RT_OK) return s;
   }
   const long long ts = 6LL * kTileElems;
@@ -1830,7 +1834,7 @@ rt_status mlp_train_steps_impl(float *params, float *m, float *v, float *grad, c
   // the steps after the first take their BF16 tiles from the previous step's Adam
   // kernel, and a given loss buffer is zeroed once for all steps
   if (losses) RT_CUDA_TRY(cudaMemsetAsync(losses, 0, (size_t)n_steps * sizeof(float), st));
-  r = mlp_prep_tiles(params, scr.as<uint16_t>(), n_nets, 6, st);
+  r = mlp_prep_tiles(params, scr.as<uint16_t>(), n_nets, 6, 1.0f, st);
   if (r != RT_OK) return r;
   for (int32_t i = 0; i < n_steps; ++i) {
     const int64_t s = (int64_t)step_first - 1 + i;
@@ -1862,7 +1866,7 @@ rt_status mlp_forward_impl(int n_nets, const float *params, const rt_mlp_norm *n
   Scratch scr;
   rt_status s = scr.alloc((size_t)n_nets * 3 * (size_t)kTileBytes, st);
   if (s != RT_OK) return s;
-  s = mlp_prep_tiles(params, scr.as<uint16_t>(), n_nets, 3, st);
+  s = mlp_prep_tiles(params, scr.as<uint16_t>(), n_nets, 3, 1.0f, st);
   if (s != RT_OK) return s;
   const unsigned grid = (unsigned)((n + kH - 1) / kH);
   const Norm N1 = norm_on_device ? Norm{} : to_norm(nm);
@@ -1940,7 +1944,7 @@ rt_status trace_mlp_core(const rt_grid *grid, int band_pts, const float *params,
   unsigned long long *item_next = reinterpret_cast<unsigned long long *>(item_start + (n_bands + 1));
   int *item_band = reinterpret_cast<int *>(item_next + 1);
   uint32_t *order = n_bands > 1 ? reinterpret_cast<uint32_t *>(base + tiles_b + plan_b) : nullptr;
-  v = mlp_prep_tiles(params, tiles, n_bands, 3, st);
+  v = mlp_prep_tiles(params, tiles, n_bands, 3, 0.5f, st);
   if (v != RT_OK) return v;
   RT_CUDA_TRY(cudaMemsetAsync(item_next, 0, sizeof(unsigned long long), st));
   v = band_plan(W, band_pts, n_bands, chunk, counts, band_start, item_start, item_band, order, sms, st);
