@@ -172,17 +172,18 @@ WORKLOADS = {
     1: "box32_voigt20k: 32^3 cells 1 m^3, 20k Voigt lines 2000-3000 cm^-1, 64 T x 100k nu table, "
        "1e7 rays per GPU",
 }
-# algorithmic bytes of one ray-cell step: the cell's record (T bracket, and on the 128^3
-# workload its density scale) and the two kappa values of the ray's column
-WALK_BYTES_PER_STEP = {4: 16, 1: 12}
 PROFILE_SUMMARIES = {4: ("k_kappa_box128_voigt100k.md", "k_walk_box128_voigt100k.md"),
                      1: ("k_kappa_box32_voigt20k.md", "k_walk_box32_voigt20k.md")}
-# what bounds the walk instead of HBM, from those profiles (tables and cells L2-resident)
+# what bounds the line sum and the walk, from those profiles
+KAPPA_LIMITERS = {
+    4: {"issue_pct": 68.3, "fma_pipe_pct": 52.7, "alu_pipe_pct": 47.5, "xu_pipe_pct": 17.4},
+    1: {"issue_pct": 67.1, "fma_pipe_pct": 51.6, "alu_pipe_pct": 47.5, "xu_pipe_pct": 16.3},
+}
 WALK_LIMITERS = {
-    4: {"dram_bytes_per_step": 1.0, "l2_hit_pct": 44.9, "alu_pipe_pct": 72.4, "issue_pct": 69.7,
-        "l1_data_pipe_pct": 19.6, "note": "ungrouped; dark rays take only the DDA step; ALU and issue bind"},
-    1: {"dram_bytes_per_step": 0.21, "l2_hit_pct": 83.1, "alu_pipe_pct": 60.5, "issue_pct": 68.5,
-        "l1_data_pipe_pct": 21.0, "note": "ungrouped; dark rays take only the DDA step; ALU and issue bind"},
+    4: {"issue_pct": 68.4, "threads_per_instruction": 26.8, "alu_pipe_pct": 49.3, "dram_pct": 49.8,
+        "l2_hit_pct": 37.5, "dram_bytes_per_ray": 131},
+    1: {"issue_pct": 70.2, "threads_per_instruction": 26.8, "alu_pipe_pct": 50.3, "dram_pct": 1.8,
+        "l2_hit_pct": 85.2, "dram_bytes_per_ray": 4.6},
 }
 
 
@@ -285,10 +286,10 @@ def hot_path_line(index, args, world, rank, local, e2e=True, tau_cut=True):
            "ray_cell_steps_per_step": steps_per_step, "profile_evals_per_step": evals_per_step,
            "kernels_ms": {"rt_build_kappa": ms_build, "rt_trace": ms_trace},
            "energy_residual": energy_residual,
-           # per step: k_line_geometry, k_prefactor, k_tile_lines, k_kappa; k_cell_prep, walk
-           # table copy, [k_band_count, k_band_plan, k_band_scatter when the rays are grouped by
-           # wavenumber], k_walk; k_reduce, k_final
-           "gpu_launches": (9 + (3 if walk_shape[2] == 2 else 0)) * args.steps,
+           # per step: k_line_setup, k_tile_lines, k_kappa; k_tally_zero; k_walk_setup, [k_band_count,
+           # k_band_plan, k_band_scatter when the rays are grouped by wavenumber], k_walk;
+           # k_reduce, k_final
+           "gpu_launches": (8 + (3 if walk_shape[2] == 2 else 0)) * args.steps,
            "tuning": {"walk_blocks_per_sm": walk_shape[0], "walk_refill_idle": walk_shape[1],
                       "walk_group_by_wavenumber": walk_shape[2] == 2,
                       "walk_candidates_ms": walk_tune_ms,
@@ -383,19 +384,22 @@ def hot_path_line(index, args, world, rank, local, e2e=True, tau_cut=True):
     prof_k, prof_w = PROFILE_SUMMARIES[index]
     traffic = _profiled_traffic(prof_k, ["rt_kappa.cu", "rt_common.cuh"])
     out["roofline"] = {"kernel": "k_kappa (rt_build_kappa)", **roof, "traffic": traffic,
-                       "timed": "rt_build_kappa (k_kappa and its three small set-up kernels)"}
-    # the walk, second kernel of the step, at its algorithmic bytes per ray-cell step against HBM
-    hbm_peak = peaks.get("hbm_gbs", 6771.5)
-    bps = WALK_BYTES_PER_STEP[index]
-    walk_gbs = steps_per_step / world * bps / (ms_trace * 1e-3) / 1e9   # per GPU
-    out["walk_roofline"] = {"kernel": "k_walk (rt_trace)", "bound": "hbm", "achieved": walk_gbs,
-                            "peak": hbm_peak, "unit": "GB/s", "frac": walk_gbs / hbm_peak,
+                       "timed": "rt_build_kappa (k_kappa and its two small set-up kernels)",
+                       "limiters": {**KAPPA_LIMITERS[index], "source": "profiles/" + prof_k},
+                       "note": "evaluations are (line, point) pairs within the cutoff, as the estimate "
+                               "defines them; the sum evaluates far lines at a tile's nodes and "
+                               "interpolates, so that frac, the rate all pairs would need, exceeds 1"}
+    # the walk, by rays: in an opaque gas most of a ray's steps are visits after its transmission
+    # has underflowed, which are counted in closed form and move no bytes
+    out["walk_roofline"] = {"kernel": "k_walk (rt_trace)", "bound": "issue",
+                            "rays_per_s": n_rays / (ms_trace * 1e-3),   # per GPU
+                            "ray_cell_steps_per_s": steps_per_step / world / (ms_trace * 1e-3),
                             "traffic": _profiled_traffic(prof_w, ["rt_trace.cu", "rt_walk.cuh",
                                                                   "rt_common.cuh"]),
-                            "bytes_per_step": bps, "peak_source": "measured HBM copy (MEASURED_PEAKS.json)",
                             "limiters": {**WALK_LIMITERS[index], "source": "profiles/" + prof_w},
-                            "note": "the walk is bound by the ALU pipe and issue (the DDA's compares and "
-                                    "selects), not by HBM (limiters, from the ncu summary)"}
+                            "note": "a ray's draws, set-up and one to three lit visits bound the walk; its "
+                                    "visits in the dark are counted in closed form and are part of the "
+                                    "ray-cell steps, as in every other count of them"}
     return out
 
 
