@@ -1,6 +1,6 @@
 // Absorption-coefficient table on a temperature grid: Eqs. (S) and (tau) of
 // Section 3, for one absorbing gas, with Lorentz or Voigt line shapes and a
-// wing cutoff.  Five kernels:
+// wing cutoff.  Kernels:
 //   k_line_geometry : per line, the binary64 grid decisions (cutoff window
 //                     [j_lo, j_hi], nearest grid index j_c and offset) and the
 //                     profile-evaluation count; validates device-resident lists.
@@ -8,6 +8,8 @@
 //                     the width parameters, in binary32 with double-float
 //                     arithmetic for the Boltzmann exponent; for Voigt lines
 //                     also the far-wing polynomial coefficients.
+//   k_line_setup    : both in one launch.
+//   k_adaptive_windows : with adaptive points, per (T node, line) its own window.
 //   k_tile_lines    : per 256-point wavenumber tile, the range of lines whose
 //                     windows reach it, split into segments by kind: lines far from
 //                     the tile (summed at a few nodes and interpolated), lines whose
@@ -540,7 +542,7 @@ __device__ __forceinline__ void two_sum_add2(float2 &s, float2 &c, float2 v) {
 // with the coefficients.  A warp sorts each range's lines by its node's windows (ballots):
 // lines whose window holds the tile go the range's way, lines whose window ends in it the
 // masked or window-end way, the others cost nothing more.  64 T x 100k points, 20k lines,
-// kappa_min 1e-3: 1.04 ms, where a gather over each tile's kept lines took 4.24.
+// kappa_min 1e-3: 0.98 ms, where a gather over each tile's kept lines took 4.24.
 template <int PROFILE, bool ADAPT>
 __global__ void __launch_bounds__(32 * kMaxTPerBlock, 3)
 k_kappa(const float4 *__restrict__ P, const float4 *__restrict__ P2, const int4 *__restrict__ R,

@@ -623,7 +623,8 @@ rt_status tally_impl(const rt_tally_buf *t, int64_t ncells, double *host_absorbe
 rt_status tally_zero_impl(const rt_tally_buf *t, int64_t ncells, cudaStream_t st) {
   if (!t || !t->absorbed || !t->scalars || !t->steps || !t->status || ncells < 1)
     return fail(RT_E_INVAL, "rt_tally_zero: bad tally buffer");
-  k_tally_zero<<<(unsigned)std::min<int64_t>((ncells + 255) / 256, 1 << 16), 256, 0, st>>>(t->absorbed, ncells, t->scalars, t->steps, t->status);
+  const unsigned blocks = (unsigned)std::min<int64_t>((ncells + 255) / 256, 1 << 16);
+  k_tally_zero<<<blocks, 256, 0, st>>>(t->absorbed, ncells, t->scalars, t->steps, t->status);
   RT_CUDA_TRY(cudaGetLastError());
   return RT_OK;
 }

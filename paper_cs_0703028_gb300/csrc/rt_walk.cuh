@@ -400,8 +400,9 @@ CellParams cell_params(const rt_spectral *spec, long long ncells, int has_px);
 // Host: rays [0, W.n_rays) grouped by band = (wavenumber index) / band_pts: per-band
 // counts (n_bands words, reused as scatter cursors), band_start and item_start
 // ([n_bands + 1]: first position of each band in the grouped order and first work
-// item of `chunk` rays), item_band (if given) each item's band, and, if order is given, the rays' offsets grouped by band
-// (within a band in arrival order).  One band: band_start = {0, n_rays}, no order.
+// item of `chunk` rays), item_band (if given) each item's band, and, if order is given, the
+// rays' offsets grouped by band (within a band in arrival order).  One band: band_start =
+// {0, n_rays}, no order.
 rt_status band_plan(const WalkParams &W, int band_pts, long long n_bands, long long chunk,
                     unsigned long long *counts, long long *band_start, long long *item_start, int *item_band,
                     uint32_t *order, int sms, cudaStream_t st);
