@@ -413,17 +413,18 @@ rt_status walk_setup(const rt_grid *grid, const rt_spectral *spec, uint64_t ray_
   W->n[0] = grid->nx; W->n[1] = grid->ny; W->n[2] = grid->nz;
   const double h[3] = {grid->hx, grid->hy, grid->hz};
   double V = 1.0;
+  const int n3[3] = {grid->nx, grid->ny, grid->nz};
   for (int a = 0; a < 3; ++a) {
     W->fin[a] = std::isfinite(h[a]) ? 1 : 0;
     W->h[a] = (float)h[a];
     W->inv_h[a] = W->fin[a] ? 1.0f / W->h[a] : 0.0f;
+    W->len[a] = W->fin[a] ? (float)n3[a] * W->h[a] : 0.0f;
     if (W->fin[a]) V *= h[a];
   }
   // dark_visits' closed form: its error bound holds for up to 65536 cells an axis and cell
   // sizes whose face distances neither overflow nor underflow (a direction cosine is 0 or
   // at least 5e-11)
   W->jump = 1;
-  const int n3[3] = {grid->nx, grid->ny, grid->nz};
   for (int a = 0; a < 3; ++a)
     if (W->fin[a] && (n3[a] > 65536 || !(W->h[a] >= 1e-15f && W->h[a] <= 1e15f))) W->jump = 0;
   for (int a = 0; a < 2; ++a) {
