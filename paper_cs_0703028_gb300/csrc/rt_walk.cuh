@@ -130,11 +130,11 @@ __device__ __forceinline__ void ray_init(const WalkParams &W, const float4 *__re
                                          const float *__restrict__ tab, unsigned long long rr,
                                          bool record, Ray &R, float4 *cd_out = nullptr) {
   const unsigned long long r = W.ray_begin + rr;
-  const long long nxy = (long long)W.n[0] * W.n[1];
   float dx, dy, dz;
   if (W.mode == RT_SRC_BEAM) {
     R.j = (int)(r % (unsigned long long)W.n_nu);
     R.ix = 0; R.iy = W.n[1] / 2; R.iz = W.n[2] / 2;
+    R.cell = W.n[0] * (R.iy + W.n[1] * R.iz);
     R.px = 0.0f;
     R.py = W.fin[1] ? __fmul_rn(__fadd_rn((float)R.iy, 0.5f), W.h[1]) : 0.0f;
     R.pz = W.fin[2] ? __fmul_rn(__fadd_rn((float)R.iz, 0.5f), W.h[2]) : 0.0f;
@@ -143,8 +143,9 @@ __device__ __forceinline__ void ray_init(const WalkParams &W, const float4 *__re
   } else {
     u32x4 ctr{(uint32_t)r, (uint32_t)(r >> 32), 0u, W.enclosure};
     u32x4 v = philox4x32_10(ctr, W.seed_lo, W.seed_hi);
-    const long long c = (long long)(((unsigned long long)v.x * (unsigned long long)W.ncells) >> 32);
-    R.j = (int)(((unsigned long long)v.y * (unsigned long long)W.n_nu) >> 32);
+    // (draw * count) >> 32, the counts below 2^31
+    const uint32_t c = __umulhi(v.x, (uint32_t)W.ncells);
+    R.j = (int)__umulhi(v.y, (uint32_t)W.n_nu);
     const float fx = u24(v.z), fy = u24(v.w);
     float4 cd = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     if (TAB) cd = __ldg(cells + c);
@@ -169,10 +170,11 @@ __device__ __forceinline__ void ray_init(const WalkParams &W, const float4 *__re
     }
     // cell index -> (ix, iy, iz) in 32-bit unsigned arithmetic (c < ncells < 2^31)
     // with the divisors' reciprocals (exact for 31-bit dividends)
-    const uint32_t cu = (uint32_t)c, n0 = (uint32_t)W.n[0], n1 = (uint32_t)W.n[1];
-    const uint32_t q0 = (uint32_t)(((unsigned long long)cu * W.div_m[0]) >> W.div_s[0]);
+    const uint32_t n0 = (uint32_t)W.n[0], n1 = (uint32_t)W.n[1];
+    const uint32_t q0 = (uint32_t)(((unsigned long long)c * W.div_m[0]) >> W.div_s[0]);
     const uint32_t q1 = (uint32_t)(((unsigned long long)q0 * W.div_m[1]) >> W.div_s[1]);
-    R.ix = (int)(cu - q0 * n0);
+    R.cell = (int)c;
+    R.ix = (int)(c - q0 * n0);
     R.iy = (int)(q0 - q1 * n1);
     R.iz = (int)q1;
     R.px = W.fin[0] ? __fmul_rn(__fadd_rn((float)R.ix, fx), W.h[0]) : 0.0f;
@@ -192,7 +194,6 @@ __device__ __forceinline__ void ray_init(const WalkParams &W, const float4 *__re
   if (W.fin[0] && dx != 0.0f) { R.ivx = __frcp_rn(dx); R.tx = tmax_of(R.ix, dx > 0.0f ? 1 : -1, W.h[0], R.px, R.ivx); }
   if (W.fin[1] && dy != 0.0f) { R.ivy = __frcp_rn(dy); R.ty = tmax_of(R.iy, dy > 0.0f ? 1 : -1, W.h[1], R.py, R.ivy); }
   if (W.fin[2] && dz != 0.0f) { R.ivz = __frcp_rn(dz); R.tz = tmax_of(R.iz, dz > 0.0f ? 1 : -1, W.h[2], R.pz, R.ivz); }
-  R.cell = (int)(R.ix + (long long)W.n[0] * R.iy + nxy * R.iz);
   if (cd_out && W.mode == RT_SRC_BEAM) *cd_out = cells[R.cell];
   R.row = (record && rr < (unsigned long long)W.rec_n) ? (int)rr : -1;
   R.t = 0.0f; R.tau = 0.0f; R.tc = 0.0f; R.trans = 1.0f;
@@ -204,7 +205,7 @@ __device__ __forceinline__ void ray_init(const WalkParams &W, const float4 *__re
 __device__ __forceinline__ int ray_nu_index(const WalkParams &W, unsigned long long rr) {
   const unsigned long long r = W.ray_begin + rr;
   const u32x4 v = philox4x32_10(u32x4{(uint32_t)r, (uint32_t)(r >> 32), 0u, W.enclosure}, W.seed_lo, W.seed_hi);
-  return (int)(((unsigned long long)v.y * (unsigned long long)W.n_nu) >> 32);
+  return (int)__umulhi(v.y, (uint32_t)W.n_nu);
 }
 
 // 1 - exp(-a) for a >= 0: below 1/4 its Taylor series to a^6 (truncation
