@@ -430,7 +430,7 @@ rt_status walk_setup(const rt_grid *grid, const rt_spectral *spec, uint64_t ray_
   for (int a = 0; a < 2; ++a) {
     uint32_t s = 0;
     while ((1ull << s) < (unsigned long long)n3[a]) ++s;
-    W->div_s[a] = 31 + s;
+    W->div_s[a] = s;
     W->div_m[a] = (uint32_t)(((1ull << (31 + s)) + (unsigned long long)n3[a] - 1) / (unsigned long long)n3[a]);
   }
   W->ncells = nc;

@@ -48,7 +48,7 @@ struct WalkParams {
   float inv_h[3];  // 1 / h, 0 on an unbounded axis
   float len[3];    // n h, the far wall
   int jump;        // dark_visits may count in closed form (walk_setup)
-  uint32_t div_m[2], div_s[2];  // c / n[0], c / n[1] as (c * div_m) >> div_s, c < 2^31
+  uint32_t div_m[2], div_s[2];  // c / n[0], c / n[1] as (c * div_m) >> (31 + div_s), c < 2^31
   long long ncells, n_nu;
   int nT, mode, tau_cut, step_cap;
   unsigned long long ray_begin, n_rays;
@@ -69,17 +69,20 @@ struct RecordPtrs {
   float *weight, *escaped;
 };
 
-__device__ __forceinline__ float u24(uint32_t u) { return __fmul_rn(__uint2float_rn(u >> 8), 0x1p-24f); }
+// The draws are u = (w >> 8) 2^-24 in [0, 1).  Products with powers of two are exact, so a scaled
+// draw plus a number is one multiply-add with the same bits as the separate operations.
+__device__ __forceinline__ float draw24(uint32_t w) { return __uint2float_rn(w >> 8); }
+__device__ __forceinline__ float u24_plus(uint32_t w, float a) { return __fmaf_rn(draw24(w), 0x1p-24f, a); }
 
 __device__ __forceinline__ bool marsaglia(uint32_t ua, uint32_t ub, float &dx, float &dy, float &dz) {
-  const float a = __fsub_rn(__fmul_rn(2.0f, u24(ua)), 1.0f);
-  const float b = __fsub_rn(__fmul_rn(2.0f, u24(ub)), 1.0f);
+  const float a = __fmaf_rn(draw24(ua), 0x1p-23f, -1.0f);  // 2 u - 1
+  const float b = __fmaf_rn(draw24(ub), 0x1p-23f, -1.0f);
   const float s = __fadd_rn(__fmul_rn(a, a), __fmul_rn(b, b));
   if (s >= 1.0f || s == 0.0f) return false;
-  const float q = __fsqrt_rn(__fsub_rn(1.0f, s));
-  dx = __fmul_rn(__fmul_rn(2.0f, a), q);
-  dy = __fmul_rn(__fmul_rn(2.0f, b), q);
-  dz = __fsub_rn(1.0f, __fmul_rn(2.0f, s));
+  const float q = __fsqrt_rn(__fsub_rn(1.0f, s)), q2 = __fadd_rn(q, q);
+  dx = __fmul_rn(a, q2);
+  dy = __fmul_rn(b, q2);
+  dz = __fmaf_rn(-2.0f, s, 1.0f);
   return true;
 }
 
@@ -146,12 +149,12 @@ __device__ __forceinline__ void ray_init(const WalkParams &W, const float4 *__re
     // (draw * count) >> 32, the counts below 2^31
     const uint32_t c = __umulhi(v.x, (uint32_t)W.ncells);
     R.j = (int)__umulhi(v.y, (uint32_t)W.n_nu);
-    const float fx = u24(v.z), fy = u24(v.w);
+    const uint32_t wx = v.z, wy = v.w;
     float4 cd = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     if (TAB) cd = __ldg(cells + c);
     ctr.z = 1u;
     v = philox4x32_10(ctr, W.seed_lo, W.seed_hi);
-    const float fz = u24(v.x);
+    const uint32_t wz = v.x;
     bool ok = marsaglia(v.y, v.z, dx, dy, dz);
     for (uint32_t call = 2; !ok && call < 64u; ++call) {
       ctr.z = call;
@@ -171,15 +174,15 @@ __device__ __forceinline__ void ray_init(const WalkParams &W, const float4 *__re
     // cell index -> (ix, iy, iz) in 32-bit unsigned arithmetic (c < ncells < 2^31)
     // with the divisors' reciprocals (exact for 31-bit dividends)
     const uint32_t n0 = (uint32_t)W.n[0], n1 = (uint32_t)W.n[1];
-    const uint32_t q0 = (uint32_t)(((unsigned long long)c * W.div_m[0]) >> W.div_s[0]);
-    const uint32_t q1 = (uint32_t)(((unsigned long long)q0 * W.div_m[1]) >> W.div_s[1]);
+    const uint32_t q0 = __umulhi(2u * c, W.div_m[0]) >> W.div_s[0];
+    const uint32_t q1 = __umulhi(2u * q0, W.div_m[1]) >> W.div_s[1];
     R.cell = (int)c;
     R.ix = (int)(c - q0 * n0);
     R.iy = (int)(q0 - q1 * n1);
     R.iz = (int)q1;
-    R.px = W.fin[0] ? __fmul_rn(__fadd_rn((float)R.ix, fx), W.h[0]) : 0.0f;
-    R.py = W.fin[1] ? __fmul_rn(__fadd_rn((float)R.iy, fy), W.h[1]) : 0.0f;
-    R.pz = W.fin[2] ? __fmul_rn(__fadd_rn((float)R.iz, fz), W.h[2]) : 0.0f;
+    R.px = W.fin[0] ? __fmul_rn(u24_plus(wx, (float)R.ix), W.h[0]) : 0.0f;
+    R.py = W.fin[1] ? __fmul_rn(u24_plus(wy, (float)R.iy), W.h[1]) : 0.0f;
+    R.pz = W.fin[2] ? __fmul_rn(u24_plus(wz, (float)R.iz), W.h[2]) : 0.0f;
     // emission weight from the table; walks without a table set it at their first step
     if (TAB) {
       const float ke = W.nT < 2 ? cd.y * node.x : cd.y * fmaf(cd.x, node.y, (1.0f - cd.x) * node.x);
