@@ -58,7 +58,7 @@ template <int TAB>
 __global__ void __launch_bounds__(256, 4)
 k_walk_batch(const EnclDev *__restrict__ E, const long long *__restrict__ item_off, int n_encl,
              long long n_items, int rays_per_item, const float4 *__restrict__ cells_all,
-             const float *__restrict__ tab, unsigned long long *__restrict__ counter) {
+             const float *__restrict__ tab, unsigned long long *__restrict__ counter, uint2 key) {
   // the current item's enclosure (walk parameters and tally pointers), one slot
   // per warp, read like the constant bank
   __shared__ __align__(16) EnclDev s_e[8];
@@ -99,7 +99,7 @@ k_walk_batch(const EnclDev *__restrict__ E, const long long *__restrict__ item_o
       if (next < last && (idle == 0xffffffffu || __popc(idle) >= kRefillIdleBatch)) {
         const unsigned rank = __popc(idle & ((1u << lane) - 1u));
         if (!active && next + rank < last) {
-          ray_init<TAB>(W, cells, tab, next + rank, false, R, &cd);
+          ray_init<TAB>(W, cells, tab, next + rank, false, R, &cd, key);
           if (TAB == 2) krow = reinterpret_cast<const float2 *>(tab) + (long long)R.j * (W.nT - 1);
           if (TAB == 1) krow1 = tab + (long long)R.j * W.nT;
           active = true;
@@ -157,6 +157,7 @@ struct rt_batch {
   long long n_items = 0, total_cells = 0;
   int rays_per_item = 0, threads = 0;
   rt::CellParams C{};
+  uint2 key{};
   rt::EnclDev *d_encl = nullptr;
   long long *d_item_off = nullptr, *d_cell_off = nullptr;
   unsigned long long *d_counter = nullptr;
@@ -245,6 +246,7 @@ static rt_status batch_build(int32_t n_encl, const rt_enclosure *encl, const rt_
   B->rays_per_item = rays_per_item;
   B->threads = threads;
   B->C = cell_params(spec, 0, 0);
+  B->key = make_uint2(H[0].W.seed_lo, H[0].W.seed_hi);
   cudaError_t e1 = cudaMemcpyAsync(B->d_encl, H.data(), b_encl, cudaMemcpyHostToDevice, st);
   cudaError_t e2 = cudaMemcpyAsync(B->d_item_off, item_off.data(), 8 * ((size_t)n_encl + 1), cudaMemcpyHostToDevice, st);
   cudaError_t e3 = cudaMemcpyAsync(B->d_cell_off, cell_off.data(), 8 * ((size_t)n_encl + 1), cudaMemcpyHostToDevice, st);
@@ -279,7 +281,7 @@ static rt_status batch_run(rt_batch *B, const float *kappa, cudaStream_t st) {
   if (v != RT_OK) return v;
   auto kern = B->layout == 2 ? k_walk_batch<2> : k_walk_batch<1>;
   kern<<<B->blocks, B->threads, 0, st>>>(B->d_encl, B->d_item_off, B->n_encl, B->n_items,
-                                         B->rays_per_item, B->d_cells, B->d_tabt, B->d_counter);
+                                         B->rays_per_item, B->d_cells, B->d_tabt, B->d_counter, B->key);
   RT_CUDA_TRY(cudaGetLastError());
   return RT_OK;
 }

@@ -128,10 +128,13 @@ struct Ray {
 // TAB: the walk table's layout (1 or 2; 0: no table).  The cell's record is loaded as soon as
 // the first draw names it and the table as soon as the record is there, so that the
 // direction's draws and the set-up arithmetic run under the two dependent gathers.
+// key: the seed, apart from W so that the batched walk, whose W is in shared memory, can pass it as
+// a kernel parameter (the key schedule then takes no instructions of the lanes: 6.24 -> 6.11 ms
+// for 48 opaque enclosures; the table walk 13.30 -> 13.11 on the 128^3 box).
 template <int TAB>
 __device__ __forceinline__ void ray_init(const WalkParams &W, const float4 *__restrict__ cells,
                                          const float *__restrict__ tab, unsigned long long rr,
-                                         bool record, Ray &R, float4 *cd_out = nullptr) {
+                                         bool record, Ray &R, float4 *cd_out, uint2 key) {
   const unsigned long long r = W.ray_begin + rr;
   float dx, dy, dz;
   if (W.mode == RT_SRC_BEAM) {
@@ -145,7 +148,7 @@ __device__ __forceinline__ void ray_init(const WalkParams &W, const float4 *__re
     R.w = 1.0f;
   } else {
     u32x4 ctr{(uint32_t)r, (uint32_t)(r >> 32), 0u, W.enclosure};
-    u32x4 v = philox4x32_10(ctr, W.seed_lo, W.seed_hi);
+    u32x4 v = philox4x32_10(ctr, key.x, key.y);
     // (draw * count) >> 32, the counts below 2^31
     const uint32_t c = __umulhi(v.x, (uint32_t)W.ncells);
     R.j = (int)__umulhi(v.y, (uint32_t)W.n_nu);
@@ -153,12 +156,12 @@ __device__ __forceinline__ void ray_init(const WalkParams &W, const float4 *__re
     float4 cd = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     if (TAB) cd = __ldg(cells + c);
     ctr.z = 1u;
-    v = philox4x32_10(ctr, W.seed_lo, W.seed_hi);
+    v = philox4x32_10(ctr, key.x, key.y);
     const uint32_t wz = v.x;
     bool ok = marsaglia(v.y, v.z, dx, dy, dz);
     for (uint32_t call = 2; !ok && call < 64u; ++call) {
       ctr.z = call;
-      v = philox4x32_10(ctr, W.seed_lo, W.seed_hi);
+      v = philox4x32_10(ctr, key.x, key.y);
       ok = marsaglia(v.x, v.y, dx, dy, dz);
       if (!ok) ok = marsaglia(v.z, v.w, dx, dy, dz);
     }
@@ -203,6 +206,13 @@ __device__ __forceinline__ void ray_init(const WalkParams &W, const float4 *__re
   R.nv = 0;
 }
 
+template <int TAB>
+__device__ __forceinline__ void ray_init(const WalkParams &W, const float4 *__restrict__ cells,
+                                         const float *__restrict__ tab, unsigned long long rr,
+                                         bool record, Ray &R, float4 *cd_out = nullptr) {
+  ray_init<TAB>(W, cells, tab, rr, record, R, cd_out, make_uint2(W.seed_lo, W.seed_hi));
+}
+
 // The wavenumber index of ray rr: the draw ray_init makes (Philox call 0, word 1),
 // for grouping rays by wavenumber before a walk.
 __device__ __forceinline__ int ray_nu_index(const WalkParams &W, unsigned long long rr) {
@@ -220,7 +230,9 @@ __device__ __forceinline__ float one_minus_exp_neg(float a) {
   p = __fmaf_rn(a, p, 1.0f / 6.0f);
   p = __fmaf_rn(a, p, -0.5f);
   p = __fmaf_rn(a, p, 1.0f);
-  return a < 0.25f ? a * p : 1.0f - __expf(-a);
+  float e;  // 2^(-a log2 e); where it would be subnormal 1 - e is 1 either way
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(__fmul_rn(a, -1.44269504088896341f)));
+  return a < 0.25f ? a * p : 1.0f - e;
 }
 
 struct NoPrefetch {
