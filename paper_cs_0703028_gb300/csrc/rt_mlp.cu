@@ -85,7 +85,7 @@ k_mlp_prep(const float *__restrict__ P, uint16_t *__restrict__ tiles, int n_mats
   tiles += (net * n_mats + m) * kTileElems;
   const int step = m < 3 ? 1 : kH;
 #pragma unroll 4
-  for (int e = threadIdx.x; e < kTileElems / 8; e += kPrepThreads) {
+  for (int e = blockIdx.z * kPrepThreads + threadIdx.x; e < kTileElems / 8; e += gridDim.z * kPrepThreads) {
     const int r = ((e >> 7) << 3) + (e & 7), k = ((e >> 3) & 15) << 3;  // e = (r / 8, k / 8, r % 8)
     const float *w = m < 3 ? P + r * kH + k : P + k * kH + r;
     float v[8];
@@ -1649,7 +1649,10 @@ Norm to_norm(const rt_mlp_norm *nm) {
 // BF16 tiles of n_nets networks: the first n_mats of W2..W4, W2^T..W4^T per network, times scale
 // (a power of two)
 rt_status mlp_prep_tiles(const float *params, uint16_t *tiles, int n_nets, int n_mats, float scale, cudaStream_t st) {
-  k_mlp_prep<<<dim3(n_mats, n_nets), kPrepThreads, 0, st>>>(params, tiles, n_mats, scale);
+  // few matrices are spread over more blocks (two steps of one network and 512 samples 138 us with
+  // a block a matrix, 133 so)
+  const int slices = (int64_t)n_nets * n_mats < 256 ? kTileElems / 8 / kPrepThreads : 1;
+  k_mlp_prep<<<dim3(n_mats, n_nets, slices), kPrepThreads, 0, st>>>(params, tiles, n_mats, scale);
   RT_CUDA_TRY(cudaGetLastError());
   return RT_OK;
 }
@@ -1758,10 +1761,12 @@ rt_status mlp_train_impl(float *params, float *m, float *v, float *grad, const f
 // the other, the separate kernels spread all tiles over the GPU.  Per step, in us, measured on
 // 1 .. 1024 networks of 1 .. 4 tiles: fused 43 for one tile and 22 for each further one, per
 // round of one network an SM; separate about 50 + 0.3 per tile (fused / separate: 1 x 1 tile 37 /
-// 59, 32 x 2 66 / 75, 32 x 4 109 / 76, 48 x 3 87 / 87, 152 x 4 119 / 248, 1024 x 2 480 / 933).
+// 59, 32 x 2 66 / 75, 32 x 4 109 / 76, 48 x 3 87 / 87, 152 x 4 119 / 248, 1024 x 2 480 / 933; 2
+// steps of 2 tiles: 1 network 138 / 135, 24 networks 151 / 159).
 bool fused_pays(int n_nets, int64_t tiles, int sms) {
   const double rounds = (double)((n_nets + sms - 1) / sms);
-  return tiles == 1 || rounds * (43.0 + 22.0 * (double)(tiles - 1)) <= 50.0 + 0.3 * (double)n_nets * (double)tiles;
+  return tiles == 1 || (tiles == 2 && n_nets >= 16) ||
+         rounds * (43.0 + 22.0 * (double)(tiles - 1)) <= 50.0 + 0.3 * (double)n_nets * (double)tiles;
 }
 
 // n_steps steps of n_nets networks (one network: nm is a host norm; an ensemble: nm
