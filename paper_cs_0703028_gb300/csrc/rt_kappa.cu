@@ -953,8 +953,29 @@ k_kappa(const float4 *__restrict__ P, const float4 *__restrict__ P2, const int4 
     // lines enter the compensated sum in pairs: the sum of two positive line
     // values is rounded once (relative error <= 2^-24 of the pair)
     auto run_general = [&](auto at, int n) {
+      int q0 = 0;
+      if (!kVoigt) {  // four lines at a time: a grid of few tiles is bound by the latency of a pair
 #pragma unroll 1
-      for (int q = 0; q < n; q += 2) {
+        for (; q0 + 4 <= n; q0 += 4) {
+          float2 v[2][kPairs], w[kPairs];
+#pragma unroll
+          for (int e = 0; e < 2; ++e) {
+            const int i = at(q0 + 2 * e), j = at(q0 + 2 * e + 1);
+            line_series(i, v[e]);
+            mask_window(i, v[e]);
+            line_series(j, w);
+            mask_window(j, w);
+#pragma unroll
+            for (int h = 0; h < kPairs; ++h) v[e][h] = __fadd2_rn(v[e][h], w[h]);
+          }
+#pragma unroll
+          for (int e = 0; e < 2; ++e)
+#pragma unroll
+            for (int h = 0; h < kPairs; ++h) kahan_add2(acc[h], cmp[h], v[e][h]);
+        }
+      }
+#pragma unroll 1
+      for (int q = q0; q < n; q += 2) {
         const bool two = q + 1 < n;
         const int i = at(q), j = two ? at(q + 1) : i;
         int fa = 0, fb = 0, na = 0, nb = 0;
