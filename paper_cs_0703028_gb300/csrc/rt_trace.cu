@@ -123,13 +123,15 @@ namespace {
 constexpr int kSetupThreads = 256;
 constexpr int kPairRows = 64;
 // Blocks of the walk's copy of a T-major table: bx over 32-wavenumber slices, by over nodes.
-// Layout 1, [nT][n_nu] -> [n_nu][nT]: 32 x 32 tiles.  Layout 2, node pairs out[j (nT - 1) + k] =
+// Layout 1, [nT][n_nu] -> [n_nu][nT]: tiles of kPairRows nodes x 32 wavenumbers, eight loads a
+// thread in flight (64 nodes x 300k wavenumbers 28.6 us; 32 x 32 tiles, four loads, 56 here and 42 in
+// a kernel of their own).  Layout 2, node pairs out[j (nT - 1) + k] =
 // {in[k][j], in[k + 1][j]}: each block stages kPairRows + 1 rows of 32 wavenumbers and writes
 // the pairs wavenumber by wavenumber.
 template <int LAYOUT>
 __device__ __forceinline__ void table_block(const float *__restrict__ in, int nT, long long n_nu,
                                             float *__restrict__ out, long long bx, int by) {
-  __shared__ float t[LAYOUT == 2 ? kPairRows + 1 : 32][33];
+  __shared__ float t[kPairRows + 1][33];
   const long long j0 = bx * 32;
   if (LAYOUT == 2) {
     const int k0 = by * kPairRows;
@@ -146,12 +148,23 @@ __device__ __forceinline__ void table_block(const float *__restrict__ in, int nT
         reinterpret_cast<float2 *>(out)[(j0 + c) * (long long)(nT - 1) + k0 + r] = make_float2(t[r][c], t[r + 1][c]);
     }
   } else {
-    const int r0 = by * 32, x = threadIdx.x & 31;
-    for (int i = threadIdx.x >> 5; i < 32; i += kSetupThreads / 32)
+    const int r0 = by * kPairRows, x = threadIdx.x & 31;
+    if (nT == 1) {  // the table itself
+      if (threadIdx.x < 32 && j0 + x < n_nu) out[j0 + x] = in[j0 + x];
+      return;
+    }
+#pragma unroll
+    for (int q = 0; q < kPairRows; q += kSetupThreads / 32) {
+      const int i = q + (threadIdx.x >> 5);
       if (r0 + i < nT && j0 + x < n_nu) t[i][x] = in[(long long)(r0 + i) * n_nu + j0 + x];
+    }
     __syncthreads();
-    for (int i = threadIdx.x >> 5; i < 32; i += kSetupThreads / 32)
-      if (r0 + x < nT && j0 + i < n_nu) out[(j0 + i) * nT + r0 + x] = t[x][i];
+    const int r = threadIdx.x % kPairRows;
+#pragma unroll
+    for (int q = 0; q < 32; q += kSetupThreads / kPairRows) {
+      const int c = q + threadIdx.x / kPairRows;
+      if (r0 + r < nT && j0 + c < n_nu) out[(j0 + c) * nT + r0 + r] = t[r][c];
+    }
   }
 }
 
@@ -181,11 +194,11 @@ __device__ __forceinline__ float4 step_bracket(const float2 c, float ktop) {
 template <int LAYOUT>
 __global__ void __launch_bounds__(kSetupThreads)
 k_walk_setup(const float *__restrict__ T, const float *__restrict__ p, const float *__restrict__ x, CellParams C,
-             float4 *__restrict__ cells, float2 *__restrict__ step_cells, uint32_t *status, long long cell_blocks,
-             const float *__restrict__ in, int nT, long long n_nu, long long slices, float *__restrict__ out) {
-  const long long b = blockIdx.x;
+             float4 *__restrict__ cells, float2 *__restrict__ step_cells, uint32_t *status, unsigned cell_blocks,
+             const float *__restrict__ in, int nT, long long n_nu, unsigned slices, float *__restrict__ out) {
+  const unsigned b = blockIdx.x;
   if (b < cell_blocks) {
-    const long long c = b * kSetupThreads + threadIdx.x;
+    const long long c = (long long)b * kSetupThreads + threadIdx.x;
     if (c < C.ncells) {
       const float4 cd = cell_prep_one(T, p, x, c, C, status);
       cells[c] = cd;
@@ -193,8 +206,8 @@ k_walk_setup(const float *__restrict__ T, const float *__restrict__ p, const flo
     }
     return;
   }
-  const long long q = b - cell_blocks;
-  table_block<LAYOUT>(in, nT, n_nu, out, q % slices, (int)(q / slices));
+  const unsigned q = b - cell_blocks, y = q / slices;
+  table_block<LAYOUT>(in, nT, n_nu, out, q - y * slices, (int)y);
 }
 
 // Four blocks of 64 registers: at five of 48 the walk spills, and more resident rays share
@@ -471,8 +484,11 @@ size_t walk_table_bytes(int layout, int nT, long long n_nu) {
   return layout == 2 ? (size_t)n_nu * (size_t)(nT - 1) * 8 : (size_t)n_nu * (size_t)nT * 4;
 }
 
+// blocks along the nodes (see table_block)
+static int walk_table_rows(int layout, int nT) { return ((layout == 2 ? nT - 1 : nT) + kPairRows - 1) / kPairRows; }
+
 rt_status launch_walk_table(int layout, const float *tab, int nT, long long n_nu, float *out, cudaStream_t st) {
-  const int ny = layout == 2 ? (nT - 1 + kPairRows - 1) / kPairRows : (nT + 31) / 32;
+  const int ny = walk_table_rows(layout, nT);
   const dim3 g((unsigned)((n_nu + 31) / 32), (unsigned)ny);
   if (layout == 2) k_walk_table<2><<<g, kSetupThreads, 0, st>>>(tab, nT, n_nu, out);
   else k_walk_table<1><<<g, kSetupThreads, 0, st>>>(tab, nT, n_nu, out);
@@ -543,13 +559,13 @@ rt_status trace_impl(const rt_grid *grid, const float *kappa, const rt_spectral 
   {
     const CellParams C = cell_params(spec, W.ncells, (grid->p_atm || grid->x) ? 1 : 0);
     const long long cb = (W.ncells + kSetupThreads - 1) / kSetupThreads, slices = (spec->n_nu + 31) / 32;
-    const long long ny = layout == 2 ? (spec->nT - 1 + kPairRows - 1) / kPairRows : (spec->nT + 31) / 32;
+    const long long ny = walk_table_rows(layout, spec->nT);
     const long long nblocks = cb + slices * ny;
     const bool one = nblocks <= 0x7FFFFFFFLL;  // else the table in a launch of its own
     auto setup = layout == 2 ? k_walk_setup<2> : k_walk_setup<1>;
     setup<<<(unsigned)(one ? nblocks : cb), kSetupThreads, 0, st>>>(grid->T, grid->p_atm, grid->x, C, cells, step_cells,
-                                                                    tally->status, cb, kappa, spec->nT, spec->n_nu,
-                                                                    slices, tabw);
+                                                                    tally->status, (unsigned)cb, kappa, spec->nT,
+                                                                    spec->n_nu, (unsigned)slices, tabw);
     RT_CUDA_TRY(cudaGetLastError());
     if (!one) {
       v = launch_walk_table(layout, kappa, spec->nT, spec->n_nu, tabw, st);
