@@ -180,10 +180,10 @@ KAPPA_LIMITERS = {
     1: {"issue_pct": 67.1, "fma_pipe_pct": 51.6, "alu_pipe_pct": 47.5, "xu_pipe_pct": 16.3},
 }
 WALK_LIMITERS = {
-    4: {"issue_pct": 68.4, "threads_per_instruction": 26.8, "alu_pipe_pct": 49.3, "dram_pct": 49.8,
-        "l2_hit_pct": 37.5, "dram_bytes_per_ray": 131},
-    1: {"issue_pct": 70.2, "threads_per_instruction": 26.8, "alu_pipe_pct": 50.3, "dram_pct": 1.8,
-        "l2_hit_pct": 85.2, "dram_bytes_per_ray": 4.6},
+    4: {"issue_pct": 67.6, "threads_per_instruction": 27.2, "alu_pipe_pct": 48.4, "dram_pct": 53.1,
+        "l2_hit_pct": 37.6, "dram_bytes_per_ray": 132},
+    1: {"issue_pct": 69.3, "threads_per_instruction": 27.2, "alu_pipe_pct": 50.0, "dram_pct": 1.9,
+        "l2_hit_pct": 85.3, "dram_bytes_per_ray": 4.6},
 }
 
 
