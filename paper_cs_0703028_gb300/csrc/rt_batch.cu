@@ -99,7 +99,7 @@ k_walk_batch(const EnclDev *__restrict__ E, const long long *__restrict__ item_o
       if (next < last && (idle == 0xffffffffu || __popc(idle) >= kRefillIdleBatch)) {
         const unsigned rank = __popc(idle & ((1u << lane) - 1u));
         if (!active && next + rank < last) {
-          ray_init<TAB>(W, cells, tab, next + rank, false, R, &cd, key);
+          ray_init<TAB, true>(W, cells, tab, next + rank, false, R, &cd, key);
           if (TAB == 2) krow = reinterpret_cast<const float2 *>(tab) + (long long)R.j * (W.nT - 1);
           if (TAB == 1) krow1 = tab + (long long)R.j * W.nT;
           active = true;

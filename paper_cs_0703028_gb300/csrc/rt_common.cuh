@@ -44,9 +44,20 @@ struct u32x4 {
   uint32_t x, y, z, w;
 };
 
+// WIDE: 64-bit products instead of a low and a high one each (the same bits).  Which compiles to
+// the faster walk differs: 48 opaque enclosures in the batched walk 6.10 ms, wide 5.98; 4e8 rays of
+// the 128^3 box in the table walk 13.07, wide 13.15.
+template <bool WIDE = false>
 __device__ __forceinline__ u32x4 philox4x32_10(u32x4 c, uint32_t k0, uint32_t k1) {
 #pragma unroll
   for (int r = 0; r < 10; ++r) {
+    if (WIDE) {
+      const unsigned long long p0 = 0xD2511F53ull * c.x, p1 = 0xCD9E8D57ull * c.z;
+      c = u32x4{(uint32_t)(p1 >> 32) ^ c.y ^ k0, (uint32_t)p1, (uint32_t)(p0 >> 32) ^ c.w ^ k1, (uint32_t)p0};
+      k0 += 0x9E3779B9u;
+      k1 += 0xBB67AE85u;
+      continue;
+    }
     const uint32_t lo0 = 0xD2511F53u * c.x, hi0 = __umulhi(0xD2511F53u, c.x);
     const uint32_t lo1 = 0xCD9E8D57u * c.z, hi1 = __umulhi(0xCD9E8D57u, c.z);
     c = u32x4{hi1 ^ c.y ^ k0, lo1, hi0 ^ c.w ^ k1, lo0};

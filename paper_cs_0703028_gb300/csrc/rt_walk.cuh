@@ -131,7 +131,7 @@ struct Ray {
 // key: the seed, apart from W so that the batched walk, whose W is in shared memory, can pass it as
 // a kernel parameter (the key schedule then takes no instructions of the lanes: 6.24 -> 6.11 ms
 // for 48 opaque enclosures; the table walk 13.30 -> 13.11 on the 128^3 box).
-template <int TAB>
+template <int TAB, bool WIDE = false>
 __device__ __forceinline__ void ray_init(const WalkParams &W, const float4 *__restrict__ cells,
                                          const float *__restrict__ tab, unsigned long long rr,
                                          bool record, Ray &R, float4 *cd_out, uint2 key) {
@@ -148,7 +148,7 @@ __device__ __forceinline__ void ray_init(const WalkParams &W, const float4 *__re
     R.w = 1.0f;
   } else {
     u32x4 ctr{(uint32_t)r, (uint32_t)(r >> 32), 0u, W.enclosure};
-    u32x4 v = philox4x32_10(ctr, key.x, key.y);
+    u32x4 v = philox4x32_10<WIDE>(ctr, key.x, key.y);
     // (draw * count) >> 32, the counts below 2^31
     const uint32_t c = __umulhi(v.x, (uint32_t)W.ncells);
     R.j = (int)__umulhi(v.y, (uint32_t)W.n_nu);
@@ -156,12 +156,12 @@ __device__ __forceinline__ void ray_init(const WalkParams &W, const float4 *__re
     float4 cd = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     if (TAB) cd = __ldg(cells + c);
     ctr.z = 1u;
-    v = philox4x32_10(ctr, key.x, key.y);
+    v = philox4x32_10<WIDE>(ctr, key.x, key.y);
     const uint32_t wz = v.x;
     bool ok = marsaglia(v.y, v.z, dx, dy, dz);
     for (uint32_t call = 2; !ok && call < 64u; ++call) {
       ctr.z = call;
-      v = philox4x32_10(ctr, key.x, key.y);
+      v = philox4x32_10<WIDE>(ctr, key.x, key.y);
       ok = marsaglia(v.x, v.y, dx, dy, dz);
       if (!ok) ok = marsaglia(v.z, v.w, dx, dy, dz);
     }
