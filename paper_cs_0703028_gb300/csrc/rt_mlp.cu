@@ -1666,21 +1666,21 @@ size_t train_scratch_bytes(int64_t n, int n_nets) {
                grid * kGradStride * sizeof(float)) + 64;
 }
 
+// the arguments of a step of n samples (touches no device; a device norm array is not read)
 rt_status validate_train(float *params, float *m, float *v, float *grad, const float *inputs,
                          const float *targets, int64_t n, int n_nets, const rt_mlp_norm *nm, bool norm_on_device,
-                         int32_t flags, float *loss) {
-  if (!params || !grad || !inputs || !targets || !loss)
-    return fail(RT_E_INVAL, "rt_mlp_train_step: NULL buffer");
+                         int32_t flags) {
+  if (!params || !grad || !inputs || !targets) return fail(RT_E_INVAL, "rt_mlp_train_step: NULL buffer");
   if (!(flags & RT_MLP_GRAD_ONLY) && (!m || !v)) return fail(RT_E_INVAL, "rt_mlp_train_step: NULL Adam state");
   if (n < 1 || n > (1LL << 26)) return fail(RT_E_INVAL, "rt_mlp_train_step: n out of range");
   if (n_nets < 1 || n_nets > 65535) return fail(RT_E_INVAL, "rt_mlp_train_steps_nets: n_nets must be in [1, 65535]");
   if ((double)n * (double)n_nets > (double)(1LL << 30))
     return fail(RT_E_INVAL, "rt_mlp_train_steps_nets: n * n_nets must not exceed 2^30 samples per step");
   if (!nm) return fail(RT_E_INVAL, "norm is NULL");
-  if (!norm_on_device) {
-    rt_status s = validate_norm(nm);
-    if (s != RT_OK) return s;
-  }
+  return norm_on_device ? RT_OK : validate_norm(nm);
+}
+
+rt_status train_kernel_attributes() {
   static std::once_flag once;
   static rt_status attr = RT_OK;
   std::call_once(once, [] {
@@ -1746,10 +1746,13 @@ rt_status mlp_train_core(float *params, float *m, float *v, float *grad, const f
 rt_status mlp_train_impl(float *params, float *m, float *v, float *grad, const float *inputs,
                          const float *targets, int64_t n, const rt_mlp_norm *nm, float lr, int32_t step,
                          int32_t flags, float *loss, uint32_t *status, cudaStream_t st) {
-  rt_status s = validate_train(params, m, v, grad, inputs, targets, n, 1, nm, false, flags, loss);
+  if (!loss) return fail(RT_E_INVAL, "rt_mlp_train_step: NULL buffer");
+  rt_status s = validate_train(params, m, v, grad, inputs, targets, n, 1, nm, false, flags);
   if (s != RT_OK) return s;
   if (!(flags & RT_MLP_GRAD_ONLY) && (step < 1 || !std::isfinite(lr) || lr < 0))
     return fail(RT_E_INVAL, "rt_mlp_train_step: step >= 1 and finite lr >= 0 required");
+  s = train_kernel_attributes();
+  if (s != RT_OK) return s;
   Scratch scr;
   s = scr.alloc(train_scratch_bytes(n, 1), st);
   if (s != RT_OK) return s;
@@ -1785,6 +1788,8 @@ rt_status mlp_train_steps_impl(float *params, float *m, float *v, float *grad, c
     return fail(RT_E_INVAL, "rt_mlp_train_steps: finite learning rates >= 0 required");
   if (n_nets < 1) return fail(RT_E_INVAL, "rt_mlp_train_steps_nets: n_nets must be >= 1");
   if (n_steps == 0) return RT_OK;
+  rt_status r = validate_train(params, m, v, grad, inputs, targets, batch, n_nets, nm, norm_on_device, 0);
+  if (r != RT_OK) return r;
   const Norm N1 = norm_on_device ? Norm{} : to_norm(nm);
   const Norm *norms = norm_on_device ? reinterpret_cast<const Norm *>(nm) : nullptr;
   const int64_t nb = n / batch;
@@ -1796,12 +1801,10 @@ rt_status mlp_train_steps_impl(float *params, float *m, float *v, float *grad, c
   if (fused_pays(n_nets, (batch + kH - 1) / kH, sms)) {
     const int blocks = std::min(n_nets, sms);
     Scratch scr;
-    rt_status r = scr.alloc(256 + (batch > kH ? (size_t)blocks * kGradStride * sizeof(float) : 0), st);
+    r = scr.alloc(256 + (batch > kH ? (size_t)blocks * kGradStride * sizeof(float) : 0), st);
     if (r != RT_OK) return r;
     float *loss = losses ? losses : scr.as<float>();
     float *gsum = scr.as<float>() + 64;
-    r = validate_train(params, m, v, grad, inputs, targets, batch, n_nets, nm, norm_on_device, 0, loss);
-    if (r != RT_OK) return r;
     static std::once_flag once;
     static rt_status attr = RT_OK;
     std::call_once(once, [] {
@@ -1829,13 +1832,12 @@ rt_status mlp_train_steps_impl(float *params, float *m, float *v, float *grad, c
   }
   // one scratch for all steps: the step's buffers, then a loss slot if none is given
   const size_t sb = (train_scratch_bytes(batch, n_nets) + 255) & ~size_t(255);
+  r = train_kernel_attributes();
+  if (r != RT_OK) return r;
   Scratch scr;
-  rt_status r = scr.alloc(sb + 256, st);
+  r = scr.alloc(sb + 256, st);
   if (r != RT_OK) return r;
   float *loss1 = reinterpret_cast<float *>(scr.as<char>() + sb);
-  r = validate_train(params, m, v, grad, inputs, targets, batch, n_nets, nm, norm_on_device, 0,
-                     losses ? losses : loss1);
-  if (r != RT_OK) return r;
   // the steps after the first take their BF16 tiles from the previous step's Adam
   // kernel, and a given loss buffer is zeroed once for all steps
   if (losses) RT_CUDA_TRY(cudaMemsetAsync(losses, 0, (size_t)n_steps * sizeof(float), st));
