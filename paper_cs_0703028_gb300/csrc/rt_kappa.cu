@@ -36,8 +36,8 @@ constexpr int kPtsPerThread = 8;
 constexpr int kTilePts = 32 * kPtsPerThread;  // 256 wavenumbers per block, one warp per T node
 constexpr int kMaxTPerBlock = 8;              // warps (T nodes) per block
 constexpr int kChunk = 192;                   // lines per staged chunk that need P only (half that with P2)
-constexpr int kStagedLines = 2048;            // host lists up to this go through pinned memory
-constexpr int kDirectPairs = 8192;            // (node, line) pairs up to which the kernels read them there
+constexpr int kArgLines = 1000;               // host lists up to this travel as kernel parameters (32 of 32,764 B)
+constexpr int kDirectPairs = 65536;           // (node, line) pairs up to which the set-up reads them there
 constexpr int kGroup = 8;                     // fast-path lines summed before one compensated add
 constexpr int kNodeGroup = 4;                 // interpolated lines a lane sums before one compensated add
 constexpr unsigned kWaitLimit = 1u << 22;     // bounded mbarrier waits
@@ -236,13 +236,26 @@ __device__ __forceinline__ void prefactors(const double *__restrict__ nu0, const
   }
 }
 
+// The lines: arrays on the GPU, or a short host list as kernel parameters, which a launch copies
+// before it returns (no allocation, no wait, nothing kept).
+struct LineArrays {
+  const double *nu0, *S, *g, *E;
+  __device__ const double *array(int q) const { return q == 0 ? nu0 : (q == 1 ? S : (q == 2 ? g : E)); }
+};
+template <int N>
+struct LineArgs {
+  double v[4][N];
+  __device__ const double *array(int q) const { return v[q]; }
+};
+
 // The lines' set-up in one launch: line_blocks blocks of k_line_geometry's work, then as many
 // for each T node's prefactors (neither reads what the other writes).
-__global__ void k_line_setup(const double *__restrict__ nu0, const double *__restrict__ S,
-                             const double *__restrict__ g, const double *__restrict__ E, GeomParams G, PrefParams Q,
+template <class Lines>
+__global__ void k_line_setup(const __grid_constant__ Lines L, GeomParams G, PrefParams Q,
                              unsigned line_blocks, int4 *__restrict__ R, float4 *__restrict__ Pout,
                              float4 *__restrict__ P2out, unsigned *__restrict__ far_bits,
                              unsigned long long *evals, uint32_t *status) {
+  const double *nu0 = L.array(0), *S = L.array(1), *g = L.array(2), *E = L.array(3);
   const unsigned y = blockIdx.x / line_blocks;
   const long long l = (long long)(blockIdx.x - y * line_blocks) * blockDim.x + threadIdx.x;
   if (y == 0) line_geometry(nu0, S, g, E, G, R, evals, status, l);
@@ -1487,115 +1500,24 @@ rt_status validate_build_args(const rt_lines *lines, const rt_spectral *spec, fl
   return RT_OK;
 }
 
-// Small host lists are handed to the GPU through pinned memory: read from there by the set-up
-// kernels where few (node, line) pairs do, else in one copy, instead of four copies out of
-// pageable memory (about 2 us of device time each; a 500-line table 41 -> 33 us).  Per host
-// thread, kSlots buffers of kStagedLines lines (64 KB each) in turn, each with an event that
-// tells when the work of its last call has read it; freed when the thread ends.
-class LineStage {
- public:
-  ~LineStage() { release(); }
-  // The four arrays packed into a slot (n values each), or nullptr: a capturing stream, whose
-  // replays would read the slot again; a list too long; no pinned memory.
-  const double *pack(const double *const (&src)[4], long long n, cudaStream_t st) {
-    const Relaxed relaxed;
-    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
-    int dev = 0;
-    if (n > kStagedLines || cudaStreamIsCapturing(st, &capture) != cudaSuccess ||
-        capture != cudaStreamCaptureStatusNone || cudaGetDevice(&dev) != cudaSuccess || !ready(dev))
-      return nullptr;
-    if (cudaEventSynchronize(ev_[next_]) != cudaSuccess) {  // its device was reset: start over
-      cudaGetLastError();
-      release();
-      return nullptr;
-    }
-    double *b = buf_ + (size_t)next_ * 4 * kStagedLines;
-    for (int q = 0; q < 4; ++q) std::memcpy(b + q * n, src[q], (size_t)n * sizeof(double));
-    return b;
-  }
-  // Everything that reads the packed slot is queued on st.
-  void queued(cudaStream_t st) {
-    const Relaxed relaxed;
-    if (cudaEventRecord(ev_[next_], st) != cudaSuccess) {
-      cudaGetLastError();
-      cudaStreamSynchronize(st);
-    }
-    next_ = (next_ + 1) % kSlots;
-  }
+template <int N>
+LineArgs<N> line_args(const double *const (&src)[4], long long n) {
+  LineArgs<N> A;
+  for (int q = 0; q < 4; ++q) std::memcpy(A.v[q], src[q], (size_t)n * sizeof(double));
+  return A;
+}
+template <int N>
+__global__ void k_line_list(const __grid_constant__ LineArgs<N> A, int n, double *__restrict__ out) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x, q = i / N;
+  if (i - q * N < n) out[q * n + i - q * N] = A.v[q][i - q * N];
+}
 
- private:
-  // another thread's capture is not disturbed by what this one does to its own buffers
-  struct Relaxed {
-    mutable cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
-    Relaxed() { cudaThreadExchangeStreamCaptureMode(&mode); }
-    ~Relaxed() { cudaThreadExchangeStreamCaptureMode(&mode); }
-  };
-  static constexpr int kSlots = 4;
-  bool ready(int dev) {
-    if (buf_ && dev == dev_) return true;
-    release();  // events belong to a device
-    if (cudaHostAlloc(&buf_, kSlots * 4 * kStagedLines * sizeof(double), cudaHostAllocPortable) != cudaSuccess) {
-      cudaGetLastError();
-      buf_ = nullptr;
-      return false;
-    }
-    for (n_ev_ = 0; n_ev_ < kSlots; ++n_ev_)
-      if (cudaEventCreateWithFlags(&ev_[n_ev_], cudaEventDisableTiming) != cudaSuccess) {
-        cudaGetLastError();
-        release();
-        return false;
-      }
-    dev_ = dev;
-    return true;
-  }
-  void release() {
-    for (int i = 0; i < n_ev_; ++i) {
-      cudaEventSynchronize(ev_[i]);
-      cudaEventDestroy(ev_[i]);
-    }
-    n_ev_ = 0;
-    if (buf_) cudaFreeHost(buf_);
-    buf_ = nullptr;
-    cudaGetLastError();
-  }
-  double *buf_ = nullptr;
-  cudaEvent_t ev_[kSlots] = {};
-  int n_ev_ = 0, next_ = 0, dev_ = -1;
-};
-
-// Everything after validation, on scratch laid out by kappa_layout.  staged: small host lists
-// may go through the thread's pinned buffers (the allocation-free entry has none).
-rt_status run_build(char *base, const KappaLayout &L, const rt_lines *lines, const rt_spectral *spec, bool staged,
+// Everything after validation, on scratch laid out by kappa_layout.
+rt_status run_build(char *base, const KappaLayout &L, const rt_lines *lines, const rt_spectral *spec,
                     float *kappa, unsigned long long *evals_out, uint32_t *status, cudaStream_t st) {
   const long long n = lines->n;
   const double *d_nu0 = lines->nu0, *d_S = lines->S_ref, *d_g = lines->gamma_ref, *d_E = lines->E_lower;
   unsigned *far_bits = reinterpret_cast<unsigned *>(base + L.off_far);
-  // a packed slot is given back once everything below that reads it is queued
-  struct SlotUser {
-    LineStage *stage = nullptr;
-    cudaStream_t st = nullptr;
-    ~SlotUser() {
-      if (stage) stage->queued(st);
-    }
-  } user;
-  if (lines->memory == RT_MEM_HOST) {
-    static thread_local LineStage stage;
-    double *d = reinterpret_cast<double *>(base);
-    const double *src[4] = {lines->nu0, lines->S_ref, lines->gamma_ref, lines->E_lower};
-    const double *slot = staged ? stage.pack(src, n, st) : nullptr;
-    if (slot) {
-      user.stage = &stage;
-      user.st = st;
-      if (n * spec->nT <= kDirectPairs)
-        d = const_cast<double *>(slot);  // read by the kernels (the address is the same on the device)
-      else
-        RT_CUDA_TRY(cudaMemcpyAsync(d, slot, 4 * (size_t)n * sizeof(double), cudaMemcpyHostToDevice, st));
-    } else {
-      for (int q = 0; q < 4; ++q)
-        RT_CUDA_TRY(cudaMemcpyAsync(d + q * n, src[q], (size_t)n * sizeof(double), cudaMemcpyHostToDevice, st));
-    }
-    d_nu0 = d; d_S = d + n; d_g = d + 2 * n; d_E = d + 3 * n;
-  }
   int4 *R = reinterpret_cast<int4 *>(base + L.off_R);
   float4 *P = reinterpret_cast<float4 *>(base + L.off_P);
   float4 *P2 = reinterpret_cast<float4 *>(base + L.off_P2);
@@ -1623,12 +1545,44 @@ rt_status run_build(char *base, const KappaLayout &L, const rt_lines *lines, con
   Q.nT = spec->nT;
   Q.profile = spec->profile;
   RT_CUDA_TRY(cudaMemsetAsync(far_bits, 0, sizeof(unsigned), st));
+  // A host list goes to the scratch in four copies (out of pageable memory about 2 us each) or, as
+  // far as a launch's parameters reach, in a launch: 500 Lorentz lines 42 us, so 32; 1000 lines 47
+  // and 35.  The set-up kernel carries the list itself, 3 us less, unless later kernels read it or
+  // many pairs do (1000 lines at 8 nodes 42 us, so 38; at 64 nodes 77 and 75, the gain falling).
+  // A capturing stream takes the copies: its replays read the caller's arrays again.
+  int carried = 0;  // capacity of the set-up kernel's list
+  if (lines->memory == RT_MEM_HOST) {
+    double *d = reinterpret_cast<double *>(base);
+    const double *src[4] = {d_nu0, d_S, d_g, d_E};
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (n <= kArgLines) RT_CUDA_TRY(cudaStreamIsCapturing(st, &capture));
+    if (n > kArgLines || capture != cudaStreamCaptureStatusNone) {
+      for (int q = 0; q < 4; ++q)
+        RT_CUDA_TRY(cudaMemcpyAsync(d + q * n, src[q], (size_t)n * sizeof(double), cudaMemcpyHostToDevice, st));
+    } else if (adaptive || n * spec->nT > kDirectPairs) {
+      const auto list = [&](auto cap) {
+        constexpr int N = decltype(cap)::value;
+        k_line_list<N><<<(4 * N + 255) / 256, 256, 0, st>>>(line_args<N>(src, n), (int)n, d);
+      };
+      if (n <= kArgLines / 2) list(std::integral_constant<int, kArgLines / 2>());
+      else list(std::integral_constant<int, kArgLines>());
+      RT_CUDA_TRY(cudaGetLastError());
+    } else {
+      carried = n <= kArgLines / 2 ? kArgLines / 2 : kArgLines;
+    }
+    d_nu0 = d; d_S = d + n; d_g = d + 2 * n; d_E = d + 3 * n;
+  }
   // with adaptive points the evaluations are counted per (node, line) window below
   unsigned long long *ev = adaptive ? nullptr : evals_out;
   const unsigned line_blocks = (unsigned)((n + tb - 1) / tb);
   if ((unsigned long long)line_blocks * (spec->nT + 1ull) <= 0x7FFFFFFFull) {
-    k_line_setup<<<line_blocks * (spec->nT + 1u), tb, 0, st>>>(d_nu0, d_S, d_g, d_E, G, Q, line_blocks, R, P, P2,
-                                                               far_bits, ev, status);
+    const auto setup = [&](const auto &list) {
+      k_line_setup<<<line_blocks * (spec->nT + 1u), tb, 0, st>>>(list, G, Q, line_blocks, R, P, P2, far_bits, ev, status);
+    };
+    const double *src[4] = {lines->nu0, lines->S_ref, lines->gamma_ref, lines->E_lower};
+    if (carried == kArgLines) setup(line_args<kArgLines>(src, n));
+    else if (carried) setup(line_args<kArgLines / 2>(src, n));
+    else setup(LineArrays{d_nu0, d_S, d_g, d_E});
     RT_CUDA_TRY(cudaGetLastError());
   } else {
     k_line_geometry<<<line_blocks, tb, 0, st>>>(d_nu0, d_S, d_g, d_E, G, R, ev, status);
@@ -1689,7 +1643,7 @@ rt_status build_kappa_impl(const rt_lines *lines, const rt_spectral *spec, float
   Scratch scr;
   v = scr.alloc(L.total, st);
   if (v != RT_OK) return v;
-  return run_build(scr.as<char>(), L, lines, spec, true, kappa, evals_out, status, st);
+  return run_build(scr.as<char>(), L, lines, spec, kappa, evals_out, status, st);
 }
 
 // ---------------------------------------------------------------------------
@@ -1741,7 +1695,7 @@ rt_status build_kappa_static_impl(const rt_lines *lines, const rt_spectral *spec
   void *scratch = nullptr;
   v = static_scratch_address(&scratch);
   if (v != RT_OK) return v;
-  return run_build(reinterpret_cast<char *>(scratch), L, lines, spec, false, kappa, evals_out, status, st);
+  return run_build(reinterpret_cast<char *>(scratch), L, lines, spec, kappa, evals_out, status, st);
 }
 
 }  // namespace rt
