@@ -319,13 +319,15 @@ __device__ __forceinline__ long long lower_bound_lo(const int4 *R, long long n, 
 // nodes).  A Lorentz-like wing 1/(u^2 + g^2) whose centre is D half-widths from the middle of
 // an interval has its poles on or outside the Bernstein ellipse of
 // rho = D + sqrt(D^2 - 1), so M nodes leave an error of order M rho^-M of the value.
-// Largest relative error of one line's value at any point (computed, g = 0 .. 20 grid
-// points; the nodes are Chebyshev's rounded to 1/16 grid point, so that u is exact):
-//   8 nodes on the tile (half-width 128 points), centre >= 704 points from it: 3.4e-8
-//  16 nodes on the tile, centre >= 141 points from it:                        1.4e-8
-//   4 nodes on a 32-point sub-block, centre >= 928 points from it:            4.9e-8
-// (an eighth of that on average over a line's points), against 6e-8 for one binary32
-// rounding.
+// The distances are those beyond which the interpolation changes no line's value by more than
+// half a binary32 rounding, 2^-25 = 3.0e-8 of it, at any point (computed in binary64 for g = 0 ..
+// 1000 grid points; the nodes are Chebyshev's rounded to 1/16 grid point, so that u is exact):
+//   8 nodes on the tile (half-width 128 points), centre >= 704 points from it: 2.7e-8
+//  16 nodes on the tile, centre >= 141 points from it:                        1.7e-8
+//   4 nodes on a 32-point sub-block, centre >= 1080 points from it:           2.9e-8
+// The tables' error is that of the values' roundings: 36 tables are 1.55e-7 from binary64 in the
+// mean, 1.60e-7 with every line at every point, 1.54e-7 with 900, 160 and 1600 points, which take
+// 4.82 instead of 4.72 ms for the 128^3 workload.
 template <int M>
 struct Nodes {
   double u[M];
@@ -334,7 +336,7 @@ constexpr Nodes<8> kNodes8{{1.9375, 21.0625, 56.375, 102.5, 152.5, 198.625, 233.
 constexpr Nodes<16> kNodes16{{0.125, 5.0, 14.625, 28.5625, 46.3125, 67.1875, 90.3125, 114.9375, 140.0625, 164.6875,
                               187.8125, 208.6875, 226.4375, 240.375, 250.0, 254.875}};
 constexpr Nodes<4> kNodes4{{0.6875, 9.375, 21.625, 30.3125}};
-constexpr int kDist8 = 704, kDist16 = 141, kDistEdge = 928;  // grid points from the tile's nearest point
+constexpr int kDist8 = 704, kDist16 = 141, kDistEdge = 1080;  // grid points from the tile's nearest point
 
 // Lagrange weights w[m][j] of the M nodes at N positions, and the nodes in binary32
 template <int M, int N>
@@ -366,8 +368,10 @@ __device__ constexpr NodeTable<8, 16> kTab8 = node_table<8, 16>(kNodes8, AtNode1
 __device__ constexpr NodeTable<4, 32> kTab4 = node_table<4, 32>(kNodes4, AtPoint{});
 
 // Weideman's series for the core points.  Its error falls fast with y: relative to Re w over
-// |z| < 8.2 (against binary64), 24 terms give 2e-8 at y = 0.1 and 4e-10 at 0.75, 16 terms 2.5e-8
-// at y = 2.3, 12 terms 1.4e-8 at y = 5; each is used from there on.
+// |z| < 8 (against binary64), 24 terms give 1.8e-8 at y = 0.1 and 4e-10 at 0.75; 16 and 12 terms
+// are used from the y on where theirs is as small, 1.5e-8 and 1.8e-8.  Fewer terms also round less
+// often: the 36 tables are 1.60e-7 from binary64 with 24 terms throughout, 1.55e-7 so.
+constexpr float kTerms16 = 2.3f, kTerms12 = 5.0f;
 struct WeidSet {
   WeidSeries<24> n24;
   WeidSeries<16> n16;
@@ -915,7 +919,7 @@ k_kappa(const float4 *__restrict__ P, const float4 *__restrict__ P2, const int4 
           const float2 x = __fmul2_rn(sd, __fadd2_rn(__fadd2_rn(first, dup2((float)e)), dg));
           // iz = -y + ix, v = 1 / (L - iz), Z = (L + iz) v; sqrt(pi) w = v (p(Z) v + 1)
           const float2 d = __ffma2_rn(dr, dr, __fmul2_rn(x, x));
-          float2 inv = rcp2(d);  // one Newton step: within a rounding of 1 / d
+          float2 inv = rcp2(d);  // one Newton step: the tables are no further from binary64 than by division
           inv = __ffma2_rn(inv, __ffma2_rn(neg2(d), inv, dup2(1.0f)), inv);
           const float2 vr = __fmul2_rn(dr, inv), vi = __fmul2_rn(x, inv);
           const float2 zr = __ffma2_rn(nr, vr, neg2(__fmul2_rn(x, vi))), zi = __ffma2_rn(nr, vi, __fmul2_rn(x, vr));
@@ -937,8 +941,8 @@ k_kappa(const float4 *__restrict__ P, const float4 *__restrict__ P2, const int4 
       };
       // fewer terms where the line is broad (warp-uniform; see WeidSet)
       const float ymin = fminf(y.x, y.y);
-      if (ymin >= 5.0f) points(ws.n12);
-      else if (ymin >= 2.3f) points(ws.n16);
+      if (ymin >= kTerms12) points(ws.n12);
+      else if (ymin >= kTerms16) points(ws.n16);
       else points(ws.n24);
       __syncwarp();
     };
