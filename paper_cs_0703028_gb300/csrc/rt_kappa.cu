@@ -748,10 +748,22 @@ k_kappa(const float4 *__restrict__ P, const float4 *__restrict__ P2, const int4 
       const float un = 32.0f * (float)sb + kTab4.u[lane & 3];
       float2 s = make_float2(0.0f, 0.0f), sc = s;
 #pragma unroll
-      for (int q = 0; q < kPtsPerThread; ++q) res[32 * q + lane] = 0.0f;
+      for (int q = 0; q < (ADAPT ? 2 : 1) * kPtsPerThread; ++q) res[32 * q + lane] = 0.0f;
       int cur = -1;
+      // the sum of the lines that end in sub-block cur joins the earlier ones': cutoff windows end
+      // in a sub-block once, windows of their own any number of times, so their sums are carried
+      // on with their roundings (the second half of res)
       auto flush = [&]() {
-        if (cur >= 0 && cur < kTilePts / 32) res[32 * cur + lane] += __fsub_rn(s.y, sc.y);
+        if (cur >= 0 && cur < kTilePts / 32) {
+          float &r = res[32 * cur + lane];
+          const float v = __fsub_rn(s.y, sc.y), t = __fadd_rn(r, v);
+          if (ADAPT) {
+            const float b = __fsub_rn(t, r);
+            float &e = res[kTilePts + 32 * cur + lane];
+            e = __fadd_rn(e, __fadd_rn(__fsub_rn(r, __fsub_rn(t, b)), __fsub_rn(v, b)));
+          }
+          r = t;
+        }
         s.y = sc.y = 0.0f;
       };
 #pragma unroll 1
@@ -788,6 +800,7 @@ k_kappa(const float4 *__restrict__ P, const float4 *__restrict__ P2, const int4 
         for (int m = 0; m < 4; ++m)
           if (m != 1)
             v = __ffma2_rn(*reinterpret_cast<const float2 *>(&kTab4.w[m][w0 + 2 * h]), dup2(fm[m] - fm[1]), v);
+        if (ADAPT) v = __fadd2_rn(v, *reinterpret_cast<const float2 *>(res + kTilePts + p0 + 2 * h));
         two_sum_add2(acc[h], cmp[h], v);
       }
       __syncwarp();  // res is the general path's next
