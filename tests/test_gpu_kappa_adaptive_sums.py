@@ -57,3 +57,18 @@ def test_window_ends_that_alternate_keep_their_sums(rt):
     ref = [okappa.kappa_table(l, spec)[0, pts] for l in (strong, lines)]
     assert (ref[1] - ref[0] > 20 * unit).all() and (got[0] >= 1.0).all() and (got[0] < 2.0).all()
     assert np.max(np.abs((got[1] - got[0]) - (ref[1] - ref[0]))) <= 2 * unit
+
+
+# A point's offset from a line centre is rounded once, so a lone line's value there is the same bits
+# wherever the grid begins, whichever lane and place of it the point falls to.
+@pytest.mark.parametrize("at,points", [(300.2718281828, 90.0), (700.4142135623, 25.0), (1023.4577215664, 120.0), (511.5772156649, 3.0)])
+def test_lone_line_is_the_same_wherever_the_grid_begins(rt, at, points):
+    lines = _lines([at], np.array([1e-2 * points ** 2]), 0.02)
+    spec = _spec(1e-2, cutoff=4.0)
+    ref = rt.build_kappa(lines, spec).cpu().numpy()[0]
+    assert 2 * int(points) - 1 <= np.count_nonzero(ref) <= 2 * int(points) + 2
+    for shift in (1, 2, 3, 5, 6, 7, 17, 100, 255):
+        s = _spec(1e-2, cutoff=4.0)
+        s.nu_min = 2000.0 + shift * DNU
+        got = rt.build_kappa(lines, s).cpu().numpy()[0]
+        assert np.array_equal(got[:spec.n_nu - shift], ref[shift:])
