@@ -190,8 +190,10 @@ size_t rt_kappa_table_elems(const rt_spectral *spec);
  * with u = x_ref p_ref / (k_B T) the absorber number density [cm^-3], S_l(T) by
  * Eq. (S) with Q(T_ref)/Q(T) = (T_ref/T)^q_exp, and f the Lorentz profile (half-width
  * gamma = gamma_ref p_ref (T_ref/T)^n_T) or the Voigt profile (that Lorentz width and
- * the Doppler half-width nu0/c sqrt(2 ln2 k_B T / m)).  Binary32 with a Kahan sum
- * over lines in ascending nu0.
+ * the Doppler half-width nu0/c sqrt(2 ln2 k_B T / m)).  Binary32 with compensated sums
+ * over the lines, near lines in ascending nu0; lines far from a run of 256 wavenumbers
+ * are summed at a few nodes and interpolated to them, which changes a line's value by less
+ * than half a binary32 rounding.
  *   kappa      device [nT * n_nu] binary32, cm^-1, written (T-major: row k is the
  *              spectrum at T_k).
  *   evals_out  optional device counter: adds the number of (T_k, line, nu_j)
@@ -296,8 +298,8 @@ rt_status rt_trace_batch(int32_t n_encl, const rt_enclosure *encl, const float *
 /*
  * Process-wide launch shapes, set by an autotuner (no effect on results):
  * kappa_t_per_block = temperature nodes per rt_build_kappa block (1..8, 0 = 8);
- * walk_blocks_per_sm = 4 or 5 (0 = 5): kept and reported; the rt_trace walk is compiled
- *   for four resident 256-thread blocks per SM either way;
+ * walk_blocks_per_sm = 4 or 5 (0 = 5): ignored, kept for rt_get_tuning; the rt_trace walk
+ *   is compiled for four resident 256-thread blocks per SM;
  * walk_refill_idle = idle lanes of a warp that trigger loading new rays in the
  *   rt_trace walk (12 or 16; 0 = 16);
  * walk_group = rays of an rt_trace call grouped by wavenumber before the walk, so

@@ -4,11 +4,11 @@
 //   k_line_geometry : per line, the binary64 grid decisions (cutoff window
 //                     [j_lo, j_hi], nearest grid index j_c and offset) and the
 //                     profile-evaluation count; validates device-resident lists.
-//   k_prefactor     : per (T node, line), Eq. (S) times the number density and
-//                     the width parameters, in binary32 with double-float
+//   k_line_setup    : that, and per (T node, line), Eq. (S) times the number density
+//                     and the width parameters, in binary32 with double-float
 //                     arithmetic for the Boltzmann exponent; for Voigt lines
 //                     also the far-wing polynomial coefficients.
-//   k_line_setup    : both in one launch.
+//   k_line_list     : a short host list, its kernel parameters, into device memory.
 //   k_adaptive_windows : with adaptive points, per (T node, line) its own window.
 //   k_tile_lines    : per 256-point wavenumber tile, the range of lines whose
 //                     windows reach it, split into segments by kind: lines far from
@@ -262,14 +262,6 @@ __global__ void k_line_setup(const __grid_constant__ Lines L, GeomParams G, Pref
   else prefactors(nu0, S, g, E, Q, Pout, P2out, far_bits, l, (int)y - 1);
 }
 
-// The prefactors alone, nodes along grid.y (sizes whose blocks exceed one grid axis).
-__global__ void k_prefactor(const double *__restrict__ nu0, const double *__restrict__ S,
-                            const double *__restrict__ g, const double *__restrict__ E,
-                            PrefParams Q, float4 *__restrict__ Pout, float4 *__restrict__ P2out,
-                            unsigned *__restrict__ far_bits) {
-  prefactors(nu0, S, g, E, Q, Pout, P2out, far_bits, (long long)blockIdx.x * blockDim.x + threadIdx.x, blockIdx.y);
-}
-
 // ---- bulk asynchronous copies global -> shared, completed on an mbarrier
 __device__ __forceinline__ uint32_t smem_u32(const void *p) {
   return (uint32_t)__cvta_generic_to_shared(p);
@@ -483,23 +475,21 @@ __global__ void k_tile_lines(const int4 *__restrict__ R, long long n, long long 
   const int next_kd = __shfl_sync(0xffffffffu, kd, above ? __ffs(above) - 1 : 0);
   const bool last = ((full >> lane) & 1u) && (!above || next_kd != kd);
   const unsigned ends = __ballot_sync(0xffffffffu, last);
-  const int nseg = __popc(ends);  // at most 12: of the 13 ranges one is always empty or joined
+  // at most 12 of the 13: the change at d8 counts among covering lines, the one at D1 among the
+  // others, and with d8 >= D1 they never both count (searches of one field end in the order of
+  // their keys, sorted lines or not)
+  const int nseg = __popc(ends);
   const int seg = __popc(ends & ((1u << lane) - 1u));
   int *o = reinterpret_cast<int *>(out + kTileInts * t);
   unsigned char *kinds = reinterpret_cast<unsigned char *>(o + 16);
   if (lane < 16) kinds[lane] = 0;
   if (lane >= nseg && lane < kMaxSegs) o[4 + lane] = ub;
   __syncwarp();
-  if (last && seg < kMaxSegs) {
+  if (last) {
     o[4 + seg] = end;
     kinds[seg] = (unsigned char)kd;
   }
-  if (lane == 0) *reinterpret_cast<int4 *>(o) = make_int4(lb, ub, min(nseg, kMaxSegs), 0);
-  if (nseg > kMaxSegs && lane == 0) {  // cannot happen; the general path holds for every line
-    __threadfence_block();
-    o[4 + kMaxSegs - 1] = ub;
-    kinds[kMaxSegs - 1] = (unsigned char)kSegGeneral;
-  }
+  if (lane == 0) *reinterpret_cast<int4 *>(o) = make_int4(lb, ub, nseg, 0);
 }
 
 __device__ __forceinline__ float rcp_approx(float x) {
@@ -541,7 +531,7 @@ __device__ __forceinline__ void two_sum_add2(float2 &s, float2 &c, float2 v) {
 // to the distance itself.
 // Voigt far wing (|z| >= 20): with t = 1/|z|^2 the three-term series is the
 // polynomial c0 t + c1 t^2 + c2 t^3 + c3 t^4 + c4 t^5 (coefficients from
-// k_prefactor).  The binary32 arithmetic runs on pairs of points, nodes or lines (f32x2
+// k_line_setup).  The binary32 arithmetic runs on pairs of points, nodes or lines (f32x2
 // instructions).  By kind: far lines at 8 or 16 nodes of the tile, several lines per warp at
 // a time; lines whose window ends in the tile at 4 nodes of the covered sub-blocks plus the
 // points of the one it ends in; fast lines at every point, kGroup per compensated add;
@@ -695,8 +685,7 @@ k_kappa(const float4 *__restrict__ P, const float4 *__restrict__ P2, const int4 
     // line i's window: its own at this node, or the cutoff's
     auto window = [&](int i) -> int2 { return ADAPT ? cW[i] : *reinterpret_cast<const int2 *>(&cR[i].x); };
 
-    // the line's value, less the factor p.x for Lorentz lines, at a pair of offsets u (grid
-    // units) from its centre; DEG 4 or 1: the far-wing series' degree
+    // the line's value at a pair of offsets u (grid units) from its centre; DEG 4 or 1: the far-wing series' degree
     auto far_value = [&](auto deg, float2 u, const float4 &p, int i) -> float2 {
       constexpr int DEG = decltype(deg)::value;
       if (!kVoigt) return __fmul2_rn(dup2(p.x), rcp2(__ffma2_rn(u, u, dup2(p.y))));
@@ -1307,7 +1296,7 @@ __device__ __noinline__ int2 adaptive_window64(double v, double S, double g, dou
   return make_int2((int)lo, (int)hi);
 }
 
-// Windows of 256 lines at kWinNodes nodes per block, after k_prefactor.  The binary32
+// Windows of 256 lines at kWinNodes nodes per block, after k_line_setup.  The binary32
 // coefficients give the half-width in grid units, sqrt(c0 / kappa_min) / (s dnu) for Voigt and
 // sqrt(P.x / kappa_min) for Lorentz lines, to a relative error below kWinTol (half that of
 // A gamma: two roundings of expf, four of powf each for q and gamma, a dozen others, 2e-6 in
@@ -1485,7 +1474,8 @@ rt_status launch_line_geometry(const double *nu0, const double *S, const double 
 namespace {
 
 // Scratch of one build: [line arrays if host-resident][R: n int4][P: nT n float4]
-// [P2: nT n float4, Voigt][tile segments: 3 int4 per 256-point tile][far-zone bound]
+// [P2: nT n float4, Voigt][tile segments: kTileInts int4 per 256-point tile][far-zone bound]
+// [adaptive windows: nT n int2]
 struct KappaLayout {
   size_t off_R, off_P, off_P2, off_tiles, off_far, off_AW, total;
 };
@@ -1599,21 +1589,15 @@ rt_status run_build(char *base, const KappaLayout &L, const rt_lines *lines, con
   // with adaptive points the evaluations are counted per (node, line) window below
   unsigned long long *ev = adaptive ? nullptr : evals_out;
   const unsigned line_blocks = (unsigned)((n + tb - 1) / tb);
-  if ((unsigned long long)line_blocks * (spec->nT + 1ull) <= 0x7FFFFFFFull) {
-    const auto setup = [&](const auto &list) {
-      k_line_setup<<<line_blocks * (spec->nT + 1u), tb, 0, st>>>(list, G, Q, line_blocks, R, P, P2, far_bits, ev, status);
-    };
-    const double *src[4] = {lines->nu0, lines->S_ref, lines->gamma_ref, lines->E_lower};
-    if (carried == kArgLines) setup(line_args<kArgLines>(src, n));
-    else if (carried) setup(line_args<kArgLines / 2>(src, n));
-    else setup(LineArrays{d_nu0, d_S, d_g, d_E});
-    RT_CUDA_TRY(cudaGetLastError());
-  } else {
-    k_line_geometry<<<line_blocks, tb, 0, st>>>(d_nu0, d_S, d_g, d_E, G, R, ev, status);
-    RT_CUDA_TRY(cudaGetLastError());
-    k_prefactor<<<dim3(line_blocks, (unsigned)spec->nT), tb, 0, st>>>(d_nu0, d_S, d_g, d_E, Q, P, P2, far_bits);
-    RT_CUDA_TRY(cudaGetLastError());
-  }
+  // (the coefficients of 2^31 blocks would take 8 TB: the scratch was refused before)
+  const auto setup = [&](const auto &list) {
+    k_line_setup<<<line_blocks * (spec->nT + 1u), tb, 0, st>>>(list, G, Q, line_blocks, R, P, P2, far_bits, ev, status);
+  };
+  const double *src[4] = {lines->nu0, lines->S_ref, lines->gamma_ref, lines->E_lower};
+  if (carried == kArgLines) setup(line_args<kArgLines>(src, n));
+  else if (carried) setup(line_args<kArgLines / 2>(src, n));
+  else setup(LineArrays{d_nu0, d_S, d_g, d_E});
+  RT_CUDA_TRY(cudaGetLastError());
 
   int2 *AW = nullptr;
   if (adaptive) {

@@ -662,13 +662,15 @@ k_grad_adam(const float *__restrict__ part, int nparts, float *__restrict__ grad
 //    there are no transposed tiles): of the per-step traffic of the separate kernels (Z 0.26 MB
 //    written and read 3 times, partials 0.2 MB twice, tiles 0.2 MB three times) only the masters
 //    and moments are left, 0.6 MB read and 0.6 MB written;
-//  - those stay in L2 from step to step (0.6 MB of one network per SM, 92 MB in all).
+//  - those are read from L2 from the second step on (0.6 MB of one network per SM, 92 MB in all);
+//    their stores reach DRAM all the same (304 networks, 8 steps: 268 MB read, 1391 of the 1468 MB
+//    stored written).
 // 8 steps of 1024 networks x 128 samples: 5.09 -> 2.26 ms, x 256 samples 7.47 -> 3.84 (the
 // separate kernels spent 0.32 ms on
 // the tiles and 0.075 + 0.22 + 0.286 ms a step on forward, backward and Adam); one network
-// 60 -> 36 us a step. Of a step's 33 us per network and SM the products take 3, the
-// elementwise passes and barriers between them 14, Adam 13; issue (16 warps an SM) and the latency
-// of Adam's loads bound it.
+// 60 -> 36 us a step. Of a step's 40 us per network with every SM busy (36 alone) the products take
+// about 3, Adam 13 to 16, the elementwise passes and barriers between the products the rest (clock
+// stamps); issue (16 warps an SM) and the latency of Adam's loads bound it.
 // Every value is formed by the same operations in the same order as in k_mlp_fwd, k_mlp_bwd
 // and k_grad_adam, so the parameters are bitwise those of the separate kernels.
 // The weight gradient is taken transposed (rows = input unit), so that a warp's 32 lanes hold
@@ -1761,11 +1763,14 @@ rt_status mlp_train_impl(float *params, float *m, float *v, float *grad, const f
 }
 
 // Whether a run's steps go to the fused kernel: its blocks take their networks' tiles one after
-// the other, the separate kernels spread all tiles over the GPU.  Per step, in us, measured on
-// 1 .. 1024 networks of 1 .. 4 tiles: fused 43 for one tile and 22 for each further one, per
-// round of one network an SM; separate about 50 + 0.3 per tile (fused / separate: 1 x 1 tile 37 /
-// 59, 32 x 2 66 / 75, 32 x 4 109 / 76, 48 x 3 87 / 87, 152 x 4 119 / 248, 1024 x 2 480 / 933; 2
-// steps of 2 tiles: 1 network 138 / 135, 24 networks 151 / 159).
+// the other, the separate kernels spread all tiles over the GPU.  Per step, in us, a model of 1 ..
+// 200 networks of 1 .. 4 tiles: fused 43 for one tile and 22 for each further one, per round of one
+// network an SM; separate about 50 + 0.3 per tile.  Measured, 8 steps in us, fused / separate: 2 tiles,
+// 12 networks 525 / 518, 16 525 / 536, 24 525 / 565, 152 589 / 1135, 200 1120 / 1695; 3 tiles, 40
+// networks 703 / 637, 48 705 / 686, 64 706 / 895; 4 tiles, 48 networks 883 / 872, 64 884 / 935, 200
+// 1839 / 2708.  The line of two tiles is that of long runs, which the model puts at 25: a run of one
+// step has it at 24 networks (79 / 79; 16 networks 79 / 74), of two at 18 (142 / 139 at 16, 142 / 146
+// at 20).
 bool fused_pays(int n_nets, int64_t tiles, int sms) {
   const double rounds = (double)((n_nets + sms - 1) / sms);
   return tiles == 1 || (tiles == 2 && n_nets >= 16) ||

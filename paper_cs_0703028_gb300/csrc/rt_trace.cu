@@ -110,7 +110,7 @@ __global__ void k_band_scatter(WalkParams W, int band_pts, unsigned long long *_
 
 }  // namespace
 
-int g_walk_blocks = 5;   // accepted launch shape (4 or 5); both run the one compiled occupancy
+int g_walk_blocks = 5;   // kept for rt_get_tuning only: no launch reads it
 int g_walk_refill = 16;  // idle lanes that trigger a refill (12 or 16)
 // Rays grouped by wavenumber only when asked for (2; 0 and 1 never): the counting passes
 // cost more than the shared table rows save.  Off / on: 1e7 rays of the opaque 32^3 box
@@ -560,17 +560,12 @@ rt_status trace_impl(const rt_grid *grid, const float *kappa, const rt_spectral 
     const CellParams C = cell_params(spec, W.ncells, (grid->p_atm || grid->x) ? 1 : 0);
     const long long cb = (W.ncells + kSetupThreads - 1) / kSetupThreads, slices = (spec->n_nu + 31) / 32;
     const long long ny = walk_table_rows(layout, spec->nT);
-    const long long nblocks = cb + slices * ny;
-    const bool one = nblocks <= 0x7FFFFFFFLL;  // else the table in a launch of its own
+    // (a table of 2^31 blocks would take 17 TB: the scratch was refused before)
     auto setup = layout == 2 ? k_walk_setup<2> : k_walk_setup<1>;
-    setup<<<(unsigned)(one ? nblocks : cb), kSetupThreads, 0, st>>>(grid->T, grid->p_atm, grid->x, C, cells, step_cells,
+    setup<<<(unsigned)(cb + slices * ny), kSetupThreads, 0, st>>>(grid->T, grid->p_atm, grid->x, C, cells, step_cells,
                                                                     tally->status, (unsigned)cb, kappa, spec->nT,
                                                                     spec->n_nu, (unsigned)slices, tabw);
     RT_CUDA_TRY(cudaGetLastError());
-    if (!one) {
-      v = launch_walk_table(layout, kappa, spec->nT, spec->n_nu, tabw, st);
-      if (v != RT_OK) return v;
-    }
   }
   int dev = 0, sms = 0;
   RT_CUDA_TRY(cudaGetDevice(&dev));
