@@ -742,19 +742,18 @@ k_kappa(const float4 *__restrict__ P, const float4 *__restrict__ P2, const int4 
 #pragma unroll
       for (int q = 0; q < (ADAPT ? 2 : 1) * kPtsPerThread; ++q) res[32 * q + lane] = 0.0f;
       int cur = -1;
-      // the sum of the lines that end in sub-block cur joins the earlier ones': cutoff windows end
-      // in a sub-block once, windows of their own any number of times, so their sums are carried
-      // on with their roundings (the second half of res)
+      // the sum of the lines that end in sub-block cur is put away: cutoff windows end in a
+      // sub-block once, windows of their own any number of times, so their sums wait with their
+      // compensation (the second half of res) for the next line that ends there
       auto flush = [&]() {
         if (cur >= 0 && cur < kTilePts / 32) {
           float &r = res[32 * cur + lane];
-          const float v = __fsub_rn(s.y, sc.y), t = __fadd_rn(r, v);
           if (ADAPT) {
-            const float b = __fsub_rn(t, r);
-            float &e = res[kTilePts + 32 * cur + lane];
-            e = __fadd_rn(e, __fadd_rn(__fsub_rn(r, __fsub_rn(t, b)), __fsub_rn(v, b)));
+            r = s.y;
+            res[kTilePts + 32 * cur + lane] = sc.y;
+          } else {
+            r += __fsub_rn(s.y, sc.y);
           }
-          r = t;
         }
         s.y = sc.y = 0.0f;
       };
@@ -769,6 +768,10 @@ k_kappa(const float4 *__restrict__ P, const float4 *__restrict__ P2, const int4 
         if (eb != cur) {  // warp-uniform; cutoff windows' ends are monotone in the line index
           flush();
           cur = eb;
+          if (ADAPT && cur >= 0 && cur < kTilePts / 32) {
+            s.y = res[32 * cur + lane];
+            sc.y = res[kTilePts + 32 * cur + lane];
+          }
         }
         const int pt = 32 * eb + lane;
         const float2 u = __fadd2_rn(__fadd2_rn(dup2((float)(jw0 - r.z)), make_float2(un, (float)pt)), dup2(__int_as_float(r.w)));
@@ -792,7 +795,7 @@ k_kappa(const float4 *__restrict__ P, const float4 *__restrict__ P2, const int4 
         for (int m = 0; m < 4; ++m)
           if (m != 1)
             v = __ffma2_rn(*reinterpret_cast<const float2 *>(&kTab4.w[m][w0 + 2 * h]), dup2(fm[m] - fm[1]), v);
-        if (ADAPT) v = __fadd2_rn(v, *reinterpret_cast<const float2 *>(res + kTilePts + p0 + 2 * h));
+        if (ADAPT) v = __fadd2_rn(v, neg2(*reinterpret_cast<const float2 *>(res + kTilePts + p0 + 2 * h)));
         two_sum_add2(acc[h], cmp[h], v);
       }
       __syncwarp();  // res is the general path's next
