@@ -17,6 +17,7 @@ from __future__ import annotations
 
 import argparse
 import json
+import math
 import os
 import statistics
 import subprocess
@@ -66,6 +67,67 @@ def alu_roofline(evals_per_s, profile, probe, n_sm, clock_mhz):
                                    "mufu": n_sm * MUFU_LANES_PER_SM * clock_mhz * 1e6 / 1e12}}
 
 
+def line_sum_values(lines, spec):
+    """What rt_build_kappa's cutoff sum evaluates, summed over tiles and T nodes, from the rules of
+    its kernel: (far-wing values, {terms of the rational series: core values})."""
+    tile, dist8, dist16, edge = 256, 704, 141, 1080  # kTilePts, kDist8, kDist16, kDistEdge
+    n, dnu = int(spec.n_nu), float(spec.dnu)
+    at = (lines.nu0 - spec.nu_min) / dnu
+    cut = spec.cutoff / dnu
+    nodes = np.linspace(spec.T_min, spec.T_max, spec.nT) if spec.nT > 1 else np.array([spec.T_min])
+    core, near, d1 = {}, 4.0, 4.0
+    if spec.profile == "voigt":
+        doppler = math.sqrt(2.0 * math.log(2.0) * 1.380649e-23 / (lines.mass_amu * 1.66053906660e-27)) / 299792458.0
+        reach = float(max(abs(spec.nu_min - spec.cutoff), abs(spec.nu_min + n * dnu + spec.cutoff)))
+        near += 20.2 * reach * math.sqrt(spec.T_max) * doppler / (math.sqrt(math.log(2.0)) * dnu) + 2.0
+        inside = (at > 0) & (at < n)
+        for T in nodes:
+            s = 0.83255461 / (lines.nu0 * math.sqrt(T) * doppler)
+            y, sd = s * lines.gamma_ref * spec.p_ref_atm * (lines.T_ref / T) ** lines.n_T, s * dnu
+            far = np.maximum(1.05 * (33554432.0 * (3.75 + 2.0 * y * y)) ** 0.25, 29.1 * np.cbrt(y)) / sd
+            d1 = max(d1, float(far.max()) + 2.0)
+            points = 2.0 * np.sqrt(np.maximum(64.0 - y * y, 0.0)) / sd
+            for terms, m in ((12, y >= 5.0), (16, (y >= 2.3) & (y < 5.0)), (24, y < 2.3)):
+                core[terms] = core.get(terms, 0.0) + float(points[m & inside].sum())
+        d1 = max(d1, near)
+    values = 0.0
+    for j0 in range(0, n, tile):
+        j1 = min(j0 + tile, n)
+        p = at[np.searchsorted(at, j0 - cut):np.searchsorted(at, j1 - 1 + cut, side="right")]
+        d = np.maximum(np.maximum(j0 - p, p - (j0 + tile - 1)), 0.0)
+        covers = (p - cut <= j0) & (p + cut >= j1 - 1)
+        c = d[covers]
+        n8, n16 = np.count_nonzero(c >= max(d1, dist8)), np.count_nonzero(c >= max(near, dist16))
+        e = d[~covers]
+        ends = np.count_nonzero(e >= max(d1, edge))
+        # a window end: 4 nodes of each of half the sub-blocks and half the points of one, in the mean
+        values += 8 * n8 + 16 * (max(n16, n8) - n8) + (j1 - j0) * (c.size - max(n16, n8) + 0.5 * (e.size - ends)) + 32 * ends
+    return values * spec.nT, core
+
+
+def line_sum_roofline(lists, spec, ms, probe):
+    """Roofline of the line sums of line lists (one after the other in ms): the binary32 and reciprocal
+    work of the values they evaluate against the measured rates; a far value takes OPS_PER_EVAL's
+    operations, a core value 4 for each further term of the series and 18 more."""
+    far, core = 0.0, {}
+    for lines in lists:
+        f, c = line_sum_values(lines, spec)
+        far += f
+        for t in c:
+            core[t] = core.get(t, 0.0) + c[t]
+    ops = OPS_PER_EVAL[spec.profile]
+    fp32 = far * ops["fp32"] + sum(v * (18 + 4 * (t - 1)) for t, v in core.items())
+    mufu = far * ops["mufu"] + sum(core.values())
+    use = {"FP32": (fp32, probe["fma_lane_ops_per_s"]), "MUFU reciprocal": (mufu, probe["rcp_lane_ops_per_s"])}
+    pipe = max(use, key=lambda k: use[k][0] / use[k][1])
+    other = next(k for k in use if k != pipe)
+    frac = {k: v[0] / v[1] / (ms * 1e-3) for k, v in use.items()}
+    return {"bound": "alu", "pipe": pipe, "achieved": use[pipe][0] / (ms * 1e-3) / 1e12, "peak": use[pipe][1] / 1e12,
+            "unit": "Tops/s", "frac": frac[pipe], "other_pipe_frac": frac[other],
+            "far_values": far, "core_values": core,
+            "peak_source": "measured by rt_alu_probe (independent chains on every SM)"}
+
+
 def _dist():
     ws = int(os.environ.get("WORLD_SIZE", "1"))
     rank = int(os.environ.get("RANK", "0"))
@@ -107,26 +169,29 @@ def _clock_summary(path, dev_index):
             "reasons": sorted(reasons), "samples": len(rows)}
 
 
-def _profiled_traffic(summary, sources):
-    """DRAM bytes per launch from a committed ncu summary, or None once the
-    kernel's sources have changed since the counters were taken."""
+def _profiled(summary, sources):
+    """(DRAM bytes per launch, what bounds the kernel) from a committed ncu summary, or
+    (None, None) once the kernel's sources have changed since the counters were taken."""
     import hashlib
     import re
     path = os.path.join(ROOT, "profiles", summary)
     try:
         text = open(path).read()
     except OSError:
-        return None
+        return None, None
     m_sha = re.search(r"source_sha: ([0-9a-f]{12})", text)
     m_tr = re.search(r"traffic_bytes_per_launch \| (\d+)", text)
+    m_lim = re.search(r"limiters: (\{.*\})", text)
     if not m_sha or not m_tr:
-        return None
+        return None, None
     h = hashlib.sha1()
     for s in sources:
         h.update(hashlib.sha1(open(os.path.join(ROOT, "paper_cs_0703028_gb300", "csrc", s), "rb")
                               .read()).hexdigest().encode() + b"  " +
                  os.path.join("paper_cs_0703028_gb300", "csrc", s).encode() + b"\n")
-    return int(m_tr.group(1)) if h.hexdigest()[:12] == m_sha.group(1) else None
+    if h.hexdigest()[:12] != m_sha.group(1):
+        return None, None
+    return int(m_tr.group(1)), {**(json.loads(m_lim.group(1)) if m_lim else {}), "source": "profiles/" + summary}
 
 
 def _peaks():
@@ -174,19 +239,6 @@ WORKLOADS = {
 }
 PROFILE_SUMMARIES = {4: ("k_kappa_box128_voigt100k.md", "k_walk_box128_voigt100k.md"),
                      1: ("k_kappa_box32_voigt20k.md", "k_walk_box32_voigt20k.md")}
-# what bounds the line sum and the walk, from those profiles
-KAPPA_LIMITERS = {
-    4: {"issue_pct": 68.3, "fma_pipe_pct": 52.7, "alu_pipe_pct": 47.5, "xu_pipe_pct": 17.4},
-    1: {"issue_pct": 67.1, "fma_pipe_pct": 51.6, "alu_pipe_pct": 47.5, "xu_pipe_pct": 16.3},
-}
-WALK_LIMITERS = {
-    4: {"issue_pct": 67.6, "threads_per_instruction": 27.2, "alu_pipe_pct": 48.4, "dram_pct": 53.1,
-        "l2_hit_pct": 37.6, "dram_bytes_per_ray": 132},
-    1: {"issue_pct": 69.3, "threads_per_instruction": 27.2, "alu_pipe_pct": 50.0, "dram_pct": 1.9,
-        "l2_hit_pct": 85.3, "dram_bytes_per_ray": 4.6},
-}
-
-
 def hot_path_line(index, args, world, rank, local, e2e=True, tau_cut=True):
     """Time the whole path (one step = build, zero, trace, [all-reduce], tally) on
     workload ``index``; returns the fields of a benchmark line (rank 0) or None."""
@@ -290,10 +342,10 @@ def hot_path_line(index, args, world, rank, local, e2e=True, tau_cut=True):
            # k_band_plan, k_band_scatter when the rays are grouped by wavenumber], k_walk;
            # k_reduce, k_final
            "gpu_launches": (8 + (3 if walk_shape[2] == 2 else 0)) * args.steps,
-           "tuning": {"walk_blocks_per_sm": walk_shape[0], "walk_refill_idle": walk_shape[1],
+           "tuning": {"walk_refill_idle": walk_shape[1],
                       "walk_group_by_wavenumber": walk_shape[2] == 2,
                       "walk_candidates_ms": walk_tune_ms,
-                      "note": "blocks,refill timed on min(rays, 1e7) ungrouped; blocks,refill,group "
+                      "note": "5,refill timed on min(rays, 1e7) ungrouped; 5,refill,group "
                               "(1 off, 2 on) on the step's rays"},
            "clocks": clk.result}
 
@@ -375,28 +427,24 @@ def hot_path_line(index, args, world, rank, local, e2e=True, tau_cut=True):
 
     if rank != 0:
         return None
-    peaks = _peaks()
-    sm_clock_mhz = peaks.get("sm_max_mhz", 2070.0)
-    props = torch.cuda.get_device_properties(local)
     probe = rt.alu_probe()  # measured FP32 and MUFU ceilings
-    roof = alu_roofline(evals_per_step / (ms_build * 1e-3), spec.profile, probe,
-                        props.multi_processor_count, sm_clock_mhz)
     prof_k, prof_w = PROFILE_SUMMARIES[index]
-    traffic = _profiled_traffic(prof_k, ["rt_kappa.cu", "rt_common.cuh"])
+    traffic, limiters = _profiled(prof_k, ["rt_kappa.cu", "rt_common.cuh"])
+    roof = line_sum_roofline([lines], spec, ms_build, probe)
     out["roofline"] = {"kernel": "k_kappa (rt_build_kappa)", **roof, "traffic": traffic,
                        "timed": "rt_build_kappa (k_kappa and its two small set-up kernels)",
-                       "limiters": {**KAPPA_LIMITERS[index], "source": "profiles/" + prof_k},
-                       "note": "evaluations are (line, point) pairs within the cutoff, as the estimate "
-                               "defines them; the sum evaluates far lines at a tile's nodes and "
-                               "interpolates, so that frac, the rate all pairs would need, exceeds 1"}
+                       "limiters": limiters,
+                       "pairs_per_s": evals_per_step / (ms_build * 1e-3),
+                       "note": "values the sum evaluates: far lines at a tile's nodes, the others at its points; "
+                               "pairs_per_s counts the (line, point) pairs within the cutoff they stand for"}
     # the walk, by rays: in an opaque gas most of a ray's steps are visits after its transmission
     # has underflowed, which are counted in closed form and move no bytes
+    traffic_w, limiters_w = _profiled(prof_w, ["rt_trace.cu", "rt_walk.cuh", "rt_common.cuh"])
     out["walk_roofline"] = {"kernel": "k_walk (rt_trace)", "bound": "issue",
                             "rays_per_s": n_rays / (ms_trace * 1e-3),   # per GPU
                             "ray_cell_steps_per_s": steps_per_step / world / (ms_trace * 1e-3),
-                            "traffic": _profiled_traffic(prof_w, ["rt_trace.cu", "rt_walk.cuh",
-                                                                  "rt_common.cuh"]),
-                            "limiters": {**WALK_LIMITERS[index], "source": "profiles/" + prof_w},
+                            "traffic": traffic_w,
+                            "limiters": limiters_w,
                             "note": "a ray's draws, set-up and one to three lit visits bound the walk; its "
                                     "visits in the dark are counted in closed form and are part of the "
                                     "ray-cell steps, as in every other count of them"}
@@ -1018,7 +1066,7 @@ def run_next(args):
     with ClockWindow(0) as clk2:
         ms2 = _ev_time(two_gas, reps=args.steps)
     out["two_gases"] = {"evals": ev2, "ms": ms2, "evals_per_s": ev2 / (ms2 * 1e-3),
-                        "roofline": alu_roofline(ev2 / (ms2 * 1e-3), "voigt", probe, n_sm, clock),
+                        "roofline": line_sum_roofline([case.lines, h2o], spec, ms2, probe),
                         "clocks": clk2.result}
     out["cutoff_build"] = {"evals": ev16_full, "ms": ms_full}
     res = {"metric": "Eq. I updates/s (marching), line-profile evals/s (variants)",
@@ -1067,10 +1115,8 @@ def run_box128(args):
            "build_ms": ms_build, "evals": ev, "line_profile_evals_per_s": ev / (ms_build * 1e-3),
            "trace_ms": ms_trace, "steps": steps, "energy_residual": float(sc[3]),
            "walk_hbm_frac_at_16B_per_step": steps * 16 / (ms_trace * 1e-3) / (hbm * 1e9),
-           "build_roofline": alu_roofline(ev / (ms_build * 1e-3), spec.profile, rt.alu_probe(),
-                                          torch.cuda.get_device_properties(0).multi_processor_count,
-                                          _peaks().get("sm_max_mhz", 2070.0)),
-           "tuning": {"walk_blocks_per_sm": walk_shape[0], "walk_refill_idle": walk_shape[1],
+           "build_roofline": line_sum_roofline([case.lines], spec, ms_build, rt.alu_probe()),
+           "tuning": {"walk_refill_idle": walk_shape[1],
                       "walk_group_by_wavenumber": walk_shape[2] == 2, "walk_candidates_ms": walk_ms},
            "clocks": {"build": clk_b.result, "trace": clk_t.result},
            "pressure_reading_error_vs_lbl": pressure_reading_error(rt, case, kap)}
