@@ -102,14 +102,14 @@ def tune_batch(grids, n_rays, spec, kappa, candidates=None, reps=2, use_cache=Tr
 
 def tune_walk(grid_struct, ncells, spec, kappa, n_rays, candidates=None, reps=2, use_cache=True,
               n_rays_group=None):
-    """Pick the walk's (resident blocks per SM, refill threshold) on the caller's trace
-    (n_rays rays, no wavenumber grouping), then, with that shape, whether grouping the
-    rays by wavenumber pays on n_rays_group rays (default n_rays): grouping costs a
-    counting pass over the rays and gains only when many rays share each wavenumber.
+    """Pick the walk's refill threshold on the caller's trace (n_rays rays, no wavenumber
+    grouping; candidates are (walk_blocks_per_sm, refill) pairs, the first of which no
+    launch reads), then, with that shape, whether grouping the rays by wavenumber pays on
+    n_rays_group rays (default n_rays).
     Returns ((blocks, refill, group), {"blocks,refill[,group]": ms}) with group 1 (off)
     or 2 (on) as rt_tuning.walk_group."""
     if candidates is None:
-        candidates = [(5, 12), (5, 16)]   # 4 and 5 blocks run the same kernel
+        candidates = [(5, 12), (5, 16)]
     ng = int(n_rays if n_rays_group is None else n_rays_group)
     key = f"walk:{ncells}:{spec.n_nu}:{spec.nT}:{int(n_rays)}:{ng}"
     cached = _load().get(key) if use_cache else None
